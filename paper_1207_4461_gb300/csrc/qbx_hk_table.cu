@@ -8,8 +8,16 @@
 // once per k on the intervals of the real-axis table, by Chebyshev
 // interpolation at QBX_HK_DEG + 1 nodes per interval, and the pair kernels
 // evaluate them like the real-axis fits (KW<cplx>).  The values at the nodes
-// come from hankel01_cplx for |z| <= 20 and from the asymptotic amplitude
-// (hankel_amp_asym_c, finite for any Im z) above.
+// are the integral
+//   B_n(z) = (2/(pi z))^{1/2} e^{-i n pi/2} / Gamma(n + 1/2)
+//            int_0^inf e^{-t} t^{n-1/2} (1 + i t/(2z))^{n-1/2} dt
+// (DLMF 10.32.8 with K_n(-iz) = (pi i/2) e^{i n pi/2} H_n(z)), t = u^2, by the
+// trapezoidal rule in u, whose error falls as e^{-2 pi |Im sqrt(2 i z)| / h}:
+// step 0.2, 32 points, 7e-16 at |z| >= 1.9 for every angle in [0, pi/2]
+// (against 90-digit values).  Nothing cancels, where the series and Miller
+// sums J + iY lose e^{2 Im z} (k = 2 + 6i on the 48-panel starfish: S off by
+// 1.4e-10 with those, 3e-15 with the integral; the table takes 56 us instead
+// of 922).
 #include <cuda_runtime.h>
 #include "qbx_apply_impl.cuh"
 #include "qbx_internal.h"
@@ -19,30 +27,46 @@ namespace {
 
 constexpr int kN = QBX_HK_DEG + 1;   // nodes and coefficients per interval
 
-__device__ cplx amp_on_ray(cplx z, int n) {
-  if (cabs_(z) > 20.0) return hankel_amp_asym_c(z, n);
-  cplx h0, h1;
-  hankel01_cplx(z, h0, h1);
-  return (n == 0 ? h0 : h1) * cexp_(mul_i(cplx{0.78539816339744830962 - z.re, -z.im}));   // e^{-i(z - pi/4)}
-}
+constexpr int kPts = 32;             // quadrature points
+constexpr double kStep = 0.2;
+constexpr int kSplit = 4;            // threads per node
+constexpr int kPerCta = 8;           // intervals per CTA
 
-// one thread per interval i of width w = 2^-LOG2_PER_UNIT in s, [i w, (i+1) w]
-__global__ void k_hk_table(double kre, double kim, double* tab) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= QBX_HK_NI) return;
+// One thread per (interval, node, quarter of the quadrature), then one per
+// interval for the fit: about 60 complex square roots deep instead of 400.
+// Interval i has width w = 2^-LOG2_PER_UNIT in s, [i w, (i+1) w].
+__global__ void __launch_bounds__(kPerCta * kN * kSplit) k_hk_table(double kre, double kim, double* tab) {
+  __shared__ cplx s_f[kPerCta][2][kN][kSplit];
   const double w = 1.0 / (double)(1 << QBX_HK_LOG2_PER_UNIT);
-  const double mid = (i + 0.5) * w, half = 0.5 * w;
-  const double ka = hypot(kre, kim);
-  const cplx dir{kre / ka, kim / ka};   // k / |k|
-  double xs[kN];
-  cplx f[2][kN];
-  for (int j = 0; j < kN; ++j) {
-    xs[j] = cos(3.14159265358979323846 * (j + 0.5) / kN);
-    const double s = mid + half * xs[j];
-    const cplx z = (1.0 / (s * s)) * dir;
-    f[0][j] = amp_on_ray(z, 0);
-    f[1][j] = amp_on_ray(z, 1);
+  const double half = 0.5 * w;
+  {
+    const int part = threadIdx.x % kSplit, j = threadIdx.x / kSplit % kN, q = threadIdx.x / (kSplit * kN);
+    const int i = min((int)blockIdx.x * kPerCta + q, QBX_HK_NI - 1);
+    const double ka = hypot(kre, kim);
+    const double s = (i + 0.5) * w + half * cos(3.14159265358979323846 * (j + 0.5) / kN);
+    const cplx iz{s * s * kre / ka, -s * s * kim / ka};   // 1/z, z = (k / |k|) / s^2
+    cplx s0{0.0, 0.0}, s1{0.0, 0.0};
+    for (int m = part; m < kPts; m += kSplit) {
+      const double u2 = (m * kStep) * (m * kStep);
+      const double wt = (m == 0 ? 1.0 : 2.0) * kStep * exp(-u2);
+      const cplx r = csqrt_(cplx{1.0 - 0.5 * u2 * iz.im, 0.5 * u2 * iz.re});
+      s0 = s0 + wt * cinv(r);
+      s1 = s1 + (wt * u2) * r;
+    }
+    const cplx pre = 0.56418958354775628695 * csqrt_(0.63661977236758134308 * iz);   // (2/(pi z))^{1/2} / Gamma(1/2)
+    const cplx b1 = pre * s1;
+    s_f[q][0][j][part] = pre * s0;
+    s_f[q][1][j][part] = cplx{2.0 * b1.im, -2.0 * b1.re};   // e^{-i pi/2} / (1/2)
   }
+  __syncthreads();
+  const int q = threadIdx.x, i = blockIdx.x * kPerCta + q;
+  if (q >= kPerCta || i >= QBX_HK_NI) return;
+  cplx f[2][kN];
+  for (int n = 0; n < 2; ++n)
+    for (int j = 0; j < kN; ++j) {
+      f[n][j] = s_f[q][n][j][0];
+      for (int c = 1; c < kSplit; ++c) f[n][j] = f[n][j] + s_f[q][n][j][c];
+    }
   // monomial coefficients of T_0 .. T_{kN-1} in x (T_{m+1} = 2 x T_m - T_{m-1})
   double T[kN][kN];
   for (int m = 0; m < kN; ++m)
@@ -91,7 +115,7 @@ __global__ void k_debug_hankel_ray(double kre, double kim, const double* tab, co
 int hk_table_doubles() { return QBX_HK_NI * kN * 4; }
 
 cudaError_t launch_hk_table(double kre, double kim, double* tab, cudaStream_t st) {
-  k_hk_table<<<(QBX_HK_NI + 63) / 64, 64, 0, st>>>(kre, kim, tab);
+  k_hk_table<<<(QBX_HK_NI + kPerCta - 1) / kPerCta, kPerCta * kN * kSplit, 0, st>>>(kre, kim, tab);
   return cudaGetLastError();
 }
 
