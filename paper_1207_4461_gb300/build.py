@@ -18,9 +18,9 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libqbx_gb300.so")
 SOURCES = ["qbx_apply_real.cu", "qbx_apply_cplx.cu", "qbx_apply_local.cu", "qbx_far.cu", "qbx_misc.cu", "qbx_capi.cu", "qbx_batch.cu",
            "qbx_adjoint.cu", "qbx_gmres.cu", "qbx_shape.cu", "qbx_assemble.cu",
-           "qbx_static.cu", "qbx_grad_d.cu", "qbx_hk_table.cu", "qbx_zgemm.cu"]
+           "qbx_static.cu", "qbx_tree.cu", "qbx_grad_d.cu", "qbx_hk_table.cu", "qbx_zgemm.cu"]
 HEADERS = ["qbx_device.cuh", "qbx_internal.h", "special_tables.h", "qbx_apply_impl.cuh",
-           "qbx_group_impl.cuh", "qbx_adjoint_impl.cuh"]
+           "qbx_group_impl.cuh", "qbx_adjoint_impl.cuh", "qbx_tree.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -32,7 +32,7 @@ __global__ void k_coef_columns(AdjArgs a) {
   const int t = c % a.n_tgt;
   double ux = a.tx[t] - cx, uy = a.ty[t] - cy;
   const double r = hypot(ux, uy);
-  besselj_seq<T>(rmul(kk, r), a.p + 1, col, 1);
+  besselj_column<T>(rmul(kk, r), a.p + 1, col, 1);
   for (int l = 0; l <= a.p; ++l) {
     const T jl = col[l];
     if (kD || kG || kX) col[P2 + l] = rmul(jl, (double)l);

@@ -5,9 +5,8 @@
 // (complex k), which instantiate it.
 //
 // One thread owns one expansion centre c with its on-surface target x
-// (x - c = r e^{i theta_t}); a CTA owns 128 consecutive centres and one
-// contiguous range of sources (a split), staged through shared memory in
-// tiles of 128.  For a pair with x_s - c = rho e^{i theta_s}, psi = theta_t -
+// (x - c = r e^{i theta_t}); a CTA owns 32 consecutive centres and one
+// share (a split) of the sources.  For a pair with x_s - c = rho e^{i theta_s}, psi = theta_t -
 // theta_s, z = k rho, the orders come from H0(z), H1(z) by the upward
 // recurrence H_{l+1} = (2l/z) H_l - H_{l-1} and from the Chebyshev recurrence
 // for cos(l psi), sin(l psi); the kernels are the truncated Graf sums folded
@@ -204,24 +203,20 @@ __host__ __device__ constexpr int ops_ncomp(int m) {
 // |l| <= p, no J_{p+1} term).
 __host__ __device__ constexpr bool keeps_jp1(int m) { return (m & OPB_G) && (m & (OPB_D | OPB_X)); }
 
-// Shared memory layout (bytes): source tile x, y [, nx, ny] ; densities
-// [nops][tile][NR] (one slot for the one-density instances) ; per-centre
-// coefficient columns of type T, kApplyThreads wide: J (J_l, l = 0..p+1;
-// J_{p+1} = 0 unless keeps_jp1),
-// then with D or grad S  L (l J_l, l = 0..p), then with grad S
-// G (J_{l-1} - J_{l+1}, l = 0..p).
-template <int OPS, typename T, int NR, bool ONEW = false>
+// Shared memory layout of the fused apply (bytes): per-centre coefficient
+// columns of type T, kApplyCentres wide: J (J_l, l = 0..p+1; J_{p+1} = 0
+// unless keeps_jp1), then with D or grad S  L (l J_l, l = 0..p), then with
+// grad S  G (J_{l-1} - J_{l+1}, l = 0..p); then the sums handed from warp to
+// warp at the end.
+template <int OPS, typename T, int NR>
 struct ApplySmem {
-  static constexpr int kNops = ONEW ? 1 : popc3(OPS);   // density slots (X shares grad S's)
-  static constexpr bool kS = OPS & OPB_S, kD = OPS & OPB_D, kG = OPS & OPB_G;
-  static constexpr int kGeo = kD ? 4 : 2;
-  static __host__ __device__ size_t tile_bytes() {
-    return (size_t)kGeo * kSrcTile * 8 + (size_t)kNops * kSrcTile * NR * 16;
-  }
+  static constexpr bool kS = OPS & OPB_S, kD = OPS & OPB_D, kG = OPS & OPB_G, kX = OPS & OPB_X;
+  static constexpr int kAcc = (kS + kD + 2 * kG + 2 * kX) * NR;   // sums per centre
   static __host__ __device__ int nslots() { return 1 + ((kD || kG) ? 1 : 0) + (kG ? 1 : 0); }
-  static __host__ __device__ size_t bytes(int p) {
-    return tile_bytes() + (size_t)((p + 2) + (nslots() - 1) * (p + 1)) * kApplyThreads * sizeof(T);
+  static __host__ __device__ size_t col_bytes(int p) {
+    return (size_t)((p + 2) + (nslots() - 1) * (p + 1)) * kApplyCentres * sizeof(T);
   }
+  static __host__ __device__ size_t bytes(int p) { return col_bytes(p) + (size_t)kAcc * kApplyCentres * 16; }
 };
 
 // The kernel values of one (centre, source) pair for the operator set OPS,
@@ -713,13 +708,16 @@ __device__ __forceinline__ void pair_direct_w(const KW<T>& kw, const T kk, doubl
   }
 }
 
-// The storage-free apply (a2-a6 fused): one thread per centre, a CTA of
-// kApplyThreads centres against one split of the sources, staged through
-// shared memory in tiles of kSrcTile; each pair's order sums go straight
-// into the centre's accumulators (split partial sums, finished by
-// k_apply_finish).  D with grad S comes from grad S's own sums and two end
-// terms (pair_kernels, pair_dsum_w), otherwise from the coefficients e_m
-// with the C_m, V_m recurrences (or S's next product, with S).
+// The storage-free apply (a2-a6 fused): a CTA of four warps owns 32
+// consecutive centres of one side, one per lane, and one share of their
+// sources, which the warps take in turn; each pair's order sums go straight
+// into the warp's accumulators, which the warps add up at the end (split
+// partial sums, finished by k_apply_finish).  Every lane of a warp reads the
+// same source, so the loads are broadcasts from L1 and nothing is staged.
+// With a near list (a.near) the sources are those of the block's near panels
+// (qbx_tree.cuh), otherwise all of them.  D with grad S comes from grad S's
+// own sums and two end terms (pair_kernels, pair_dsum_w), otherwise from the
+// coefficients e_m with the C_m, V_m recurrences (or S's next product, with S).
 // LOCAL: the near-only variant (a separate instance, so that the global
 // apply carries no per-pair test).  ONEW: one rhs and one density for all
 // operators, accumulated through weighted seeds (pair_accumulate_w,
@@ -734,37 +732,44 @@ __host__ __device__ constexpr int fused_min_ctas() {
 template <int OPS, typename T, int NR, bool LOCAL = false, bool ONEW = false>
 __global__ void __launch_bounds__(kApplyThreads, (fused_min_ctas<OPS, LOCAL, ONEW>()))
 k_apply_fused(ApplyArgs a) {
-  using L = ApplySmem<OPS, T, NR, ONEW>;
-  constexpr bool kS = L::kS, kD = L::kD, kG = L::kG, kX = OPS & OPB_X;
+  using L = ApplySmem<OPS, T, NR>;
+  constexpr bool kS = L::kS, kD = L::kD, kG = L::kG, kX = L::kX;
   static_assert(!kX || kG, "X is formed with grad S and shares its density");
   static_assert(!ONEW || (NR == 1 && !kX), "one-density instances: one rhs, no X");
+  constexpr int W = kApplyThreads / kApplyCentres;   // warps
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* s_x = reinterpret_cast<double*>(smem_raw);
-  double* s_y = s_x + kSrcTile;
-  double* s_nx = s_y + kSrcTile;            // only with D
-  double* s_ny = s_nx + kSrcTile;
-  cplx* s_wd = reinterpret_cast<cplx*>(smem_raw + (size_t)L::kGeo * kSrcTile * 8);  // [nops][tile][NR]
-  T* slot = reinterpret_cast<T*>(smem_raw + L::tile_bytes());
   const int p = a.p;
-  T* sJ = slot;                                                   // J_l, p + 2 rows
-  T* sL = slot + (p + 2) * kApplyThreads;                         // l J_l, p + 1 rows
-  T* sG = sL + ((kD || kG) ? (p + 1) * kApplyThreads : 0);        // J_{l-1} - J_{l+1}, p + 1 rows
+  T* sJ = reinterpret_cast<T*>(smem_raw);                         // J_l, p + 2 rows
+  T* sL = sJ + (p + 2) * kApplyCentres;                           // l J_l, p + 1 rows
+  T* sG = sL + ((kD || kG) ? (p + 1) * kApplyCentres : 0);        // J_{l-1} - J_{l+1}, p + 1 rows
+  cplx* s_sum = reinterpret_cast<cplx*>(smem_raw + L::col_bytes(p));   // [sums][centre]
 
-  const int tid = threadIdx.x;
-  // work item (centre block, source split): rank r = blockIdx.x / nblk;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // work item (centre block of one side, source split): rank r = blockIdx.x / nblk;
   // near-field splits first when the grids' node counts are given
-  const int nblk = (a.n_ctr + kApplyThreads - 1) / kApplyThreads;
-  const int cblk = (int)(blockIdx.x % (unsigned)nblk), rank = (int)(blockIdx.x / (unsigned)nblk);
-  const int split = a.near_q_tgt > 0 ? near_first_split(rank, (cblk * kApplyThreads + kApplyThreads / 2) % a.n_tgt,
-                                                        a.near_q_tgt, a.near_q_src, a.src_per_split, a.nsplit)
-                                     : rank;
-  const int c = cblk * kApplyThreads + tid;
-  const bool active = c < a.n_ctr;
-  const int cc = active ? c : a.n_ctr - 1;
+  const int blks = (a.n_tgt + kApplyCentres - 1) / kApplyCentres;   // per side
+  const int nblk = blks * (a.n_ctr / a.n_tgt);
+  const int unit = (int)(blockIdx.x % (unsigned)nblk), rank = (int)(blockIdx.x / (unsigned)nblk);
+  const int side = unit / blks, blk = unit - side * blks;
+  const bool active = blk * kApplyCentres + lane < a.n_tgt;
+  const int t = active ? blk * kApplyCentres + lane : a.n_tgt - 1;
+  const int c = side * a.n_tgt + t;
+  int split = rank, v0, v1;   // sources [v0, v1), numbered through the near list if there is one
+  if (a.near) {
+    const long n = (long)a.near_cnt[3 * blk] * a.near_q_src;
+    v0 = (int)(n * rank / a.nsplit);
+    v1 = (int)(n * (rank + 1) / a.nsplit);
+  } else {
+    if (a.near_q_tgt > 0)
+      split = near_first_split(rank, min(blk * kApplyCentres + kApplyCentres / 2, a.n_tgt - 1), a.near_q_tgt,
+                               a.near_q_src, a.src_per_split, a.nsplit);
+    v0 = split * a.src_per_split;
+    v1 = min(a.src.n, v0 + a.src_per_split);
+  }
+  const int* near = a.near ? a.near + (size_t)blk * a.near_stride : nullptr;
 
   // ---- per-centre set-up: target direction, J_l(k r) (a5) ----
-  const double cx = a.cx[cc], cy = a.cy[cc];
-  const int t = cc % a.n_tgt;
+  const double cx = a.cx[c], cy = a.cy[c];
   double ux = a.tx[t] - cx, uy = a.ty[t] - cy;
   const double r = hypot(ux, uy);
   const double ir = 1.0 / r;
@@ -775,25 +780,28 @@ k_apply_fused(ApplyArgs a) {
   KW<T> kw;
   kw.init(a.kre, a.kim, a.hk_tab);
   const T kk = kw.kval();
-  T* colJ = sJ + tid;
-  T* colL = sL + tid;
-  T* colG = sG + tid;
-  besselj_seq<T>(rmul(kk, r), p + 1, colJ, kApplyThreads);
-  const T J0 = colJ[0];
-  for (int l = 0; l <= p; ++l) {
-    const T jl = colJ[l * kApplyThreads];
-    if (kD || kG) colL[l * kApplyThreads] = rmul(jl, (double)l);
-    if (kG) {
-      const T jn = colJ[(l + 1) * kApplyThreads];
-      const T jp = (l == 0) ? jn : colJ[(l - 1) * kApplyThreads];
-      colG[l * kApplyThreads] = (l == 0) ? rmul(jn, -1.0) : sc_sub(jp, jn);
+  T* colJ = sJ + lane;
+  T* colL = sL + lane;
+  T* colG = sG + lane;
+  if (warp == 0) {
+    besselj_column<T>(rmul(kk, r), p + 1, colJ, kApplyCentres);
+    for (int l = 0; l <= p; ++l) {
+      const T jl = colJ[l * kApplyCentres];
+      if (kD || kG) colL[l * kApplyCentres] = rmul(jl, (double)l);
+      if (kG) {
+        const T jn = colJ[(l + 1) * kApplyCentres];
+        const T jp = (l == 0) ? jn : colJ[(l - 1) * kApplyCentres];
+        colG[l * kApplyCentres] = (l == 0) ? rmul(jn, -1.0) : sc_sub(jp, jn);
+      }
+    }
+    if (!keeps_jp1(OPS)) {
+      T z0;
+      sc_zero(z0);
+      colJ[(p + 1) * kApplyCentres] = z0;  // e_p has no J_{p+1} term (orders |l| <= p)
     }
   }
-  if (!keeps_jp1(OPS)) {
-    T z0;
-    sc_zero(z0);
-    colJ[(p + 1) * kApplyThreads] = z0;  // e_p has no J_{p+1} term (orders |l| <= p)
-  }
+  __syncthreads();
+  const T J0 = colJ[0];
   const T kneg_j0 = rmul(sc_mul(kk, J0), -1.0);  // -k J0 (D)
   T gA0;
   if (kG) gA0 = rmul(colG[0], 2.0);                // -2 J_1 (one-density grad S)
@@ -804,116 +812,114 @@ k_apply_fused(ApplyArgs a) {
 #pragma unroll
   for (int q = 0; q < NR; ++q) accS[q] = accD[q] = accA[q] = accB[q] = accX[q] = accY[q] = cplx{0.0, 0.0};
 
-  const int s_begin = split * a.src_per_split;
-  const int s_end = min(a.src.n, s_begin + a.src_per_split);
   const cplx* wdp[3] = {reinterpret_cast<const cplx*>(a.wd[0]), reinterpret_cast<const cplx*>(a.wd[1]),
                         reinterpret_cast<const cplx*>(a.wd[2])};
+  auto source = [&](int v) {   // node index of the v-th source
+    if (!near) return v;
+    const int i = v / a.near_q_src;
+    return near[i] * a.near_q_src + (v - i * a.near_q_src);
+  };
+  auto weight = [&](int o, int s, int q) {   // density of operator o
+    if (q >= a.nr) return cplx{0.0, 0.0};
+    const double2 w = __ldg(reinterpret_cast<const double2*>(wdp[o] + (size_t)s * a.nrhs + a.rhs0 + q));
+    return cplx{w.x, w.y};
+  };
+  constexpr int oW = kS ? 0 : kD ? 1 : 2;   // one-density instances: any requested operator's
+  constexpr int NP = (ONEW && kD && kG && !LOCAL) ? 2 : 1;
 
-  for (int base = s_begin; base < s_end; base += kSrcTile) {
-    const int nt = min(kSrcTile, s_end - base);
-    __syncthreads();
-    for (int i = tid; i < nt; i += kApplyThreads) {
-      s_x[i] = a.src.x[base + i];
-      s_y[i] = a.src.y[base + i];
-      if (kD) {
-        s_nx[i] = a.src.nx[base + i];
-        s_ny[i] = a.src.ny[base + i];
-      }
-    }
-    {
-      int slotn = 0;
-#pragma unroll
-      for (int o = 0; o < 3; ++o) {
-        if (!(OPS & (1 << o))) continue;
-        if (ONEW && slotn > 0) break;   // one density for all operators
-        const cplx* w = wdp[o];
-        cplx* dst = s_wd + (size_t)slotn * kSrcTile * NR;
-        for (int i = tid; i < nt * NR; i += kApplyThreads) {
-          const int s = i / NR, rr = i - s * NR;
-          dst[i] = (rr < a.nr) ? w[(size_t)(base + s) * a.nrhs + a.rhs0 + rr] : cplx{0.0, 0.0};
-        }
-        ++slotn;
-      }
-    }
-    __syncthreads();
-    if (!active) continue;
-
-    const T* cJ = colJ;
-    const T* cL = colL;
-    const T* cG = colG;
-
-    int j0 = 0;
-    if constexpr (ONEW && kD && kG && !LOCAL) {
+  for (int v = v0 + NP * warp; v < v1; v += NP * W) {
+    if constexpr (NP == 2) {
       // two sources per step: two independent recurrence chains per thread
-      for (; j0 + 2 <= nt; j0 += 2) {
+      if (v + 1 < v1) {
         double dx2[2], dy2[2], nx2[2], ny2[2];
         cplx w2[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-          dx2[q] = s_x[j0 + q] - cx;
-          dy2[q] = s_y[j0 + q] - cy;
-          nx2[q] = s_nx[j0 + q];
-          ny2[q] = s_ny[j0 + q];
-          w2[q] = s_wd[j0 + q];
+          const int s = source(v + q);
+          dx2[q] = __ldg(a.src.x + s) - cx;
+          dy2[q] = __ldg(a.src.y + s) - cy;
+          nx2[q] = __ldg(a.src.nx + s);
+          ny2[q] = __ldg(a.src.ny + s);
+          w2[q] = weight(oW, s, 0);
         }
-        pair_dsum_w<OPS, T, kApplyThreads, 2>(kw, J0, gA0, khalf, 0.5 * ir, cJ, cL, cG, p, dx2, dy2, nx2, ny2,
+        pair_dsum_w<OPS, T, kApplyCentres, 2>(kw, J0, gA0, khalf, 0.5 * ir, colJ, colL, colG, p, dx2, dy2, nx2, ny2,
                                               ux2, uy2, w2, accS[0], accD[0], accA[0], accB[0]);
-      }
-    }
-    for (int j = j0; j < nt; ++j) {
-      const double dx = s_x[j] - cx, dy = s_y[j] - cy;
-      double nx = 0.0, ny = 0.0;
-      if (kD) {
-        nx = s_nx[j];
-        ny = s_ny[j];
-      }
-      if constexpr (ONEW) {
-        if (LOCAL && fma(dx, dx, dy * dy) >= lim2) {   // near-only QBX: a distant source
-          pair_direct_w<OPS, T>(kw, kk, r * ux - dx, r * uy - dy, nx, ny, ux, uy, r, s_wd[j], accS[0], accD[0],
-                                accA[0], accB[0]);
-        } else {
-          pair_accumulate_w<OPS, T, kApplyThreads>(kw, kk, J0, kneg_j0, gA0, khalf, 0.5 * ir, cJ, cL, cG, p, dx, dy,
-                                                    nx, ny, ux2, uy2, s_wd[j], accS[0], accD[0], accA[0],
-                                                    accB[0]);
-        }
         continue;
       }
-      cplx GS, K, GA, GB, EX, EY;
+    }
+    const int s = source(v);
+    const double dx = __ldg(a.src.x + s) - cx, dy = __ldg(a.src.y + s) - cy;
+    double nx = 0.0, ny = 0.0;
+    if (kD) {
+      nx = __ldg(a.src.nx + s);
+      ny = __ldg(a.src.ny + s);
+    }
+    if constexpr (ONEW) {
+      const cplx w = weight(oW, s, 0);
       if (LOCAL && fma(dx, dx, dy * dy) >= lim2) {   // near-only QBX: a distant source
-        pair_direct<OPS, T>(kw, kk, r * ux - dx, r * uy - dy, nx, ny, ux, uy, r, GS, K, GA, GB);
+        pair_direct_w<OPS, T>(kw, kk, r * ux - dx, r * uy - dy, nx, ny, ux, uy, r, w, accS[0], accD[0], accA[0],
+                              accB[0]);
       } else {
-        pair_kernels<OPS, T, kApplyThreads>(kw, kk, J0, kneg_j0, cJ, cL, cG, p, dx, dy, nx, ny, ux, uy, ir, GS,
-                                             K, GA, GB, EX, EY);
+        pair_accumulate_w<OPS, T, kApplyCentres>(kw, kk, J0, kneg_j0, gA0, khalf, 0.5 * ir, colJ, colL, colG, p, dx,
+                                                 dy, nx, ny, ux2, uy2, w, accS[0], accD[0], accA[0], accB[0]);
       }
-      // ---- weighted densities ----
-      int slotn = 0;
-      if (kS) {
-        const cplx* w = s_wd + ((size_t)slotn * kSrcTile + j) * NR;
+      continue;
+    }
+    cplx GS, K, GA, GB, EX, EY;
+    if (LOCAL && fma(dx, dx, dy * dy) >= lim2) {   // near-only QBX: a distant source
+      pair_direct<OPS, T>(kw, kk, r * ux - dx, r * uy - dy, nx, ny, ux, uy, r, GS, K, GA, GB);
+    } else {
+      pair_kernels<OPS, T, kApplyCentres>(kw, kk, J0, kneg_j0, colJ, colL, colG, p, dx, dy, nx, ny, ux, uy, ir, GS,
+                                          K, GA, GB, EX, EY);
+    }
+    // ---- weighted densities ----
+    if (kS) {
 #pragma unroll
-        for (int q = 0; q < NR; ++q) cfma(accS[q], w[q], GS);
-        ++slotn;
-      }
-      if (kD) {
-        const cplx* w = s_wd + ((size_t)slotn * kSrcTile + j) * NR;
+      for (int q = 0; q < NR; ++q) cfma(accS[q], weight(0, s, q), GS);
+    }
+    if (kD) {
 #pragma unroll
-        for (int q = 0; q < NR; ++q) cfma(accD[q], w[q], K);
-        ++slotn;
-      }
-      if (kG) {
-        const cplx* w = s_wd + ((size_t)slotn * kSrcTile + j) * NR;
+      for (int q = 0; q < NR; ++q) cfma(accD[q], weight(1, s, q), K);
+    }
+    if (kG) {
 #pragma unroll
-        for (int q = 0; q < NR; ++q) {
-          cfma(accA[q], w[q], GA);
-          cfma(accB[q], w[q], GB);
-          if (kX) {
-            cfma(accX[q], w[q], EX);
-            cfma(accY[q], w[q], EY);
-          }
+      for (int q = 0; q < NR; ++q) {
+        const cplx w = weight(2, s, q);
+        cfma(accA[q], w, GA);
+        cfma(accB[q], w, GB);
+        if (kX) {
+          cfma(accX[q], w, EX);
+          cfma(accY[q], w, EY);
         }
       }
     }
   }
-  if (!active) return;
+  // ---- the warps' sums, in warp order ----
+  for (int w = 0; w < W; ++w) {
+    if (warp == w) {
+      int i = 0;
+      auto pass = [&](cplx& v) {
+        cplx* m = s_sum + (i++) * kApplyCentres + lane;
+        if (w > 0) v = *m + v;
+        *m = v;
+      };
+#pragma unroll
+      for (int q = 0; q < NR; ++q) {
+        if (kS) pass(accS[q]);
+        if (kD) pass(accD[q]);
+        if (kG) {
+          pass(accA[q]);
+          pass(accB[q]);
+        }
+        if (kX) {
+          pass(accX[q]);
+          pass(accY[q]);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (warp != W - 1 || !active) return;
   cplx* part = reinterpret_cast<cplx*>(a.part);
   constexpr int ncomp = ops_ncomp(OPS);
   const size_t row = ((size_t)split * a.n_ctr + c) * ncomp;
@@ -961,7 +967,7 @@ static cudaError_t onew_occupancy(K kern, size_t smem, int* n) {
 
 template <int OPS, typename T, int NR, bool LOCAL, bool ONEW = false>
 static cudaError_t launch_apply_t(const ApplyArgs& a, cudaStream_t st) {
-  const size_t smem = ApplySmem<OPS, T, NR, ONEW>::bytes(a.p);
+  const size_t smem = ApplySmem<OPS, T, NR>::bytes(a.p);
   auto kern = k_apply_fused<OPS, T, NR, LOCAL, ONEW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -971,13 +977,15 @@ static cudaError_t launch_apply_t(const ApplyArgs& a, cudaStream_t st) {
     int n = 0;
     e = onew_occupancy(kern, smem, &n);
     if (e != cudaSuccess) return e;
-    const int pct = carveout_percent(n, smem);
+    // (with a near list its arguments are small ones, which take no table, and
+    // the cluster kernels beside it on the SM need the shared memory)
+    const int pct = a.near ? 0 : carveout_percent(n, smem);
     if (pct > 0) {
       e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
       if (e != cudaSuccess) return e;
     }
   }
-  const unsigned grid = (unsigned)((a.n_ctr + kApplyThreads - 1) / kApplyThreads) * (unsigned)a.nsplit;
+  const unsigned grid = (unsigned)apply_units(a.n_ctr, a.n_tgt) * (unsigned)a.nsplit;
   kern<<<grid, kApplyThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
@@ -1026,7 +1034,7 @@ static int occupancy_t(int p, int nr, bool one_w) {
   if constexpr (!(OPS & OPB_X)) {
     if (nr <= 1 && one_w) {
       int n = 0;
-      onew_occupancy(k_apply_fused<OPS, T, 1, LOCAL, true>, ApplySmem<OPS, T, 1, true>::bytes(p), &n);
+      onew_occupancy(k_apply_fused<OPS, T, 1, LOCAL, true>, ApplySmem<OPS, T, 1>::bytes(p), &n);
       return n;
     }
   }

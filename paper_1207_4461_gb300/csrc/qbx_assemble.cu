@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kAsmLanes * kAsmWarps) k_assemble_cfie(AsmArgs
   if (warp < 2) {
     T* J = warp == 0 ? sJ : sJe;
     T* Lc = warp == 0 ? sL : sLe;
-    besselj_seq<T>(rmul(kk, warp == 0 ? r : re), p + 1, J + lane, kAsmLanes);
+    besselj_column<T>(rmul(kk, warp == 0 ? r : re), p + 1, J + lane, kAsmLanes);
     for (int l = 0; l <= p; ++l) Lc[l * kAsmLanes + lane] = rmul(J[l * kAsmLanes + lane], (double)l);
     T z0;
     sc_zero(z0);

@@ -34,6 +34,10 @@ struct qbx_plan {
   // (tab_kim = 0: none made yet)
   double* d_hk_tab;
   double tab_kre, tab_kim;
+  // the pair sums run here, beside the cluster moments on the caller's stream
+  // (forked from it and joined to it by events within every call)
+  cudaStream_t side;
+  cudaEvent_t fork, join;
 };
 
 namespace {
@@ -336,6 +340,9 @@ int qbx_plan_create(qbx_plan** plan, int device, int q_tgt, int q_src, size_t wo
   if (e == cudaSuccess) e = cudaMemcpy(p->d_wgl_tgt, wt.data(), q_tgt * sizeof(double), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(p->d_wgl_src, ws.data(), q_src * sizeof(double), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     qbx_plan_destroy(p);
     return cuda_fail(e, "qbx_plan_create");
@@ -350,6 +357,9 @@ int qbx_plan_destroy(qbx_plan* p) {
   cudaSetDevice(p->device);
   if (p->ev0) cudaEventDestroy(p->ev0);
   if (p->ev1) cudaEventDestroy(p->ev1);
+  if (p->fork) cudaEventDestroy(p->fork);
+  if (p->join) cudaEventDestroy(p->join);
+  if (p->side) cudaStreamDestroy(p->side);
   cudaFree(p->d_interp);
   cudaFree(p->d_wgl_tgt);
   cudaFree(p->d_wgl_src);
@@ -660,7 +670,7 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   // more than 32 rhs (global apply): eight warps of 8 rhs, so that the kernel
   // values of a pair are formed once per 64 rhs instead of once per 32
   const int rg = (nrhs > 32 && !(eta > 0.0)) ? kGrpRhsWide : 8;
-  const int units = group ? (nc + kGrpCentres - 1) / kGrpCentres : (nc + kApplyThreads - 1) / kApplyThreads;
+  const int units = group ? (nc + kGrpCentres - 1) / kGrpCentres : apply_units(nc, g->n_tgt);
   const bool local = eta > 0.0;
   const int chunk = local ? std::min(4, apply_chunk(ops)) : apply_chunk(ops);
   // one rhs of one density for every operator: the weighted-seed instance
@@ -682,14 +692,43 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   const int waves = local   ? std::max(p->min_waves, 4)
                     : one_w ? std::max(p->min_waves, ck ? 8 : 4)
                             : p->min_waves;
-  const int ns = host_choose_split_waves(p->num_sms, occ, units, g->n_src, per_split, avail, waves);
-  if (ns < 1) return fail(QBX_ENOMEM, "workspace too small for the apply partial sums");
+  // distant sources through cluster moments (qbx_tree.cu)
+  TreeArgs tr{};
+  size_t tree_bytes = 0;
+  int ns_far = 0;
+  if (!group && g->M >= kTreeMinPanels) {
+    tr.kre = k.re;
+    tr.kim = k.im;
+    tr.p = pp;
+    tr.pl = local ? std::max(pp, kTreeLocal) : pp;
+    tr.nd = (ops & (QBX_OPS_D | QBX_OPS_GRAD_S)) ? 1 : 0;
+    tr.eta = eta;
+    tr.n_tgt = g->n_tgt;
+    tr.n_ctr = nc;
+    tr.n_blk = apply_units(g->n_tgt, g->n_tgt);
+    tr.ops = ops;
+    tr.nrhs = nrhs;
+    tree_columns(&tr, slot_of);
+    tree_levels(g->M, g->q_src, &tr);
+    tree_bytes = tree_layout(&tr, nullptr);
+    // a few CTAs per SM share a block's far nodes; few blocks: several warps to a node
+    tr.nparts = std::max(1, std::min(4, p->num_sms * 8 / (units * 16)));
+    ns_far = std::max(2, std::min(8, (p->num_sms * 2 + units - 1) / units));
+    if (!far_clusters_fit(tr) || avail < tree_bytes + (size_t)(ns_far + 1) * per_split) ns_far = 0;
+  }
+  const bool tree = ns_far > 0;
+  if (!tree) tree_bytes = 0;
+  // (with clusters a block's near leaves are some six panels; down to two dozen sources a CTA)
+  const int ns_near = host_choose_split_waves(p->num_sms, occ, units, tree ? std::min(g->n_src, 16 * g->q_src) : g->n_src,
+                                              per_split, avail - tree_bytes - ns_far * per_split, waves);
+  if (ns_near < 1) return fail(QBX_ENOMEM, "workspace too small for the apply partial sums");
+  const int ns = ns_near + ns_far;
   if (group ? (ck ? group_smem_cplx(gops, pp, rg) : group_smem_real(gops, pp, rg)) > 220 * 1024
             : apply_smem_bytes(ops, ck, pp, chunk) > 220 * 1024)
     return fail(QBX_EINVAL, "p = %d too large", pp);
   cudaStream_t st = (cudaStream_t)stream;
   char* base = (char*)align256((size_t)p->ws);
-  void* part = base + wd_bytes;
+  void* part = base + wd_bytes + tree_bytes;
   // a1: oversample the densities
   for (int s = 0; s < nd; ++s)
     CK(launch_upsample(g->M, g->q_tgt, g->q_src, nrhs, p->d_interp, g->src_w, distinct[s], base + s * wd_one, st),
@@ -721,8 +760,8 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   a.ty = g->tgt_y;
   a.src = SrcView{g->src_x, g->src_y, g->src_nx, g->src_ny, g->n_src};
   a.nrhs = nrhs;
-  a.nsplit = ns;
-  a.src_per_split = split_len(g->n_src, ns);
+  a.nsplit = ns_near;
+  a.src_per_split = split_len(g->n_src, ns_near);
   a.part = part;
   a.eta2 = eta > 0.0 ? eta * eta : 0.0;
   a.near_q_tgt = g->q_tgt;   // near-field items first
@@ -732,6 +771,43 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     cudaError_t te;
     a.hk_tab = host_plan_hk_table(p, k, st, &te);
     CK(te, "complex-k amplitude table");
+  }
+  if (tree) {
+    tr.sx = g->src_x;
+    tr.sy = g->src_y;
+    tr.snx = g->src_nx;
+    tr.sny = g->src_ny;
+    tr.cx = a.cx;
+    tr.cy = a.cy;
+    tr.tx = g->tgt_x;
+    tr.ty = g->tgt_y;
+    tr.hk_tab = a.hk_tab;
+    for (int i = 0; i < tr.nset; ++i) tr.wd[i] = base + tr.slot[i] * wd_one;
+    tree_layout(&tr, base + wd_bytes);
+    tr.nsplit = ns_far;
+    tr.split0 = ns_near;
+    tr.part = part;
+    CK(launch_tree_lists(tr, st), "cluster lists");
+    a.near = tr.near;
+    a.near_cnt = tr.cnt;
+    a.near_stride = tr.M;
+    a.near_q_src = tr.q_src;
+    // near pairs on the side stream, clusters on the caller's: the moments'
+    // and the far sums' short launches fill in where the pair kernel leaves room
+    CK(cudaEventRecord(p->fork, st), "fork event");
+    CK(cudaStreamWaitEvent(p->side, p->fork, 0), "fork");
+    cudaError_t en = cudaSuccess;
+    for (int r0 = 0; r0 < nrhs && en == cudaSuccess; r0 += chunk) {
+      a.rhs0 = r0;
+      a.nr = std::min(chunk, nrhs - r0);
+      en = launch_apply_fused(a, p->side);
+    }
+    cudaError_t ef = launch_tree_moments(tr, st);
+    if (ef == cudaSuccess) ef = launch_far_clusters(tr, st);
+    CK(cudaEventRecord(p->join, p->side), "join event");   // (joined also after an error)
+    CK(cudaStreamWaitEvent(st, p->join, 0), "join");
+    CK(en, "apply kernel");
+    CK(ef, "far clusters");
   }
   if (group) {
     GroupArgs ga{};
@@ -773,7 +849,7 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
       CK(launch_group_local(ga, ck, rg, units * ns, st), "group kernel (near-only)");
     else
       CK(ck ? launch_group_cplx(ga, rg, units * ns, st) : launch_group_real(ga, rg, units * ns, st), "group kernel");
-  } else {
+  } else if (!tree) {
     for (int r0 = 0; r0 < nrhs; r0 += chunk) {
       a.rhs0 = r0;
       a.nr = std::min(chunk, nrhs - r0);

@@ -411,4 +411,57 @@ __host__ __device__ void besselj_seq(T z, int nmax, T* out, int stride) {
   for (int l = 0; l <= nmax; ++l) out[l * stride] = sc_mul(out[l * stride], inv);
 }
 
+// 1/(m(m+1)) and 1/m
+struct RecipTab {
+  double mm[192], m1[192];
+  constexpr RecipTab() : mm(), m1() {
+    mm[0] = m1[0] = 0.0;
+    for (int m = 1; m < 192; ++m) {
+      mm[m] = 1.0 / ((double)m * (m + 1));
+      m1[m] = 1.0 / (double)m;
+    }
+  }
+};
+static __constant__ const RecipTab c_recip = RecipTab();
+
+// J_0..J_n at z (z != 0), out[l * stride], by the backward recurrence of
+// g_m = J_m m!/(z/2)^m: g_{m-1} = g_m - (z/2)^2/(m(m+1)) g_{m+1}, of
+// magnitude about one for every z (no rescaling, no division per order),
+// normalised by J_0 + 2 sum J_2k = 1.  About 5 FP64 instructions per order.
+template <typename T>
+__device__ __forceinline__ void besselj_column(T z, int n, T* out, int stride) {
+  if (!(sc_abs(z) < 100.0)) {   // far beyond the table's orders (and not finite)
+    besselj_seq<T>(z, n, out, stride);
+    return;
+  }
+  // start: its error falls by |z|^2/(4 m^2) per order, beyond |z| only; the
+  // orders above it add nothing to the sum
+  const double az = sc_abs(z);
+  int N = az < 0.5   ? max(n + 6, 12)
+          : az < 2.0 ? max(n + 10, 20)
+                     : max(n + 16, (int)((float)az + 16.0f + 7.0f * cbrtf((float)az)));
+  N += N & 1;
+  const T hz = sc_scale(0.5, z);
+  const T t = sc_mul(hz, hz);
+  T g1, g, acc;
+  sc_set(g1, 1.0);
+  sc_set(g, 1.0);
+  sc_set(acc, 1.0);          // sum_{k >= m/2} g_2k t^k (2k)-falling weights, Horner from the top
+  for (int m = N; m >= 1; --m) {
+    const T gm = sc_sub(g, sc_mul(sc_scale(c_recip.mm[m], t), g1));   // g_{m-1}
+    if (m - 1 <= n) out[(m - 1) * stride] = gm;
+    if (m - 1 >= 2 && ((m - 1) & 1) == 0)   // J_{m+1} relative to J_{m-1}: t / (m (m+1))
+      acc = sc_add(gm, sc_mul(sc_scale(c_recip.mm[m], t), acc));
+    g1 = g;
+    g = gm;
+  }
+  // norm = g_0 + 2 (t/2) acc, acc = g_2 + g_4 t/(3 4) + ...
+  const T f = sc_inv(sc_add(g, sc_mul(t, acc)));
+  T w = f;
+  for (int l = 0; l <= n; ++l) {
+    out[l * stride] = sc_mul(out[l * stride], w);
+    w = sc_mul(w, sc_scale(c_recip.m1[l + 1], hz));
+  }
+}
+
 }  // namespace qbx

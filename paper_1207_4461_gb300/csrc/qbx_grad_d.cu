@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kGdThreads) k_grad_d_fused(ApplyArgs a) {
   T* colJ = sJ + tid;
   T* colC = sC + tid;
   T* colS = sS + tid;
-  besselj_seq<T>(rmul(kk, r), p + 1, colJ, kGdThreads);
+  besselj_column<T>(rmul(kk, r), p + 1, colJ, kGdThreads);
   for (int m = 1; m <= p - 1; ++m) {
     const T jm2 = jl_signed(colJ, m - 2), jp2 = colJ[(m + 2) * kGdThreads];
     colC[m * kGdThreads] = rmul(sadd(jm2, jp2), 0.5);

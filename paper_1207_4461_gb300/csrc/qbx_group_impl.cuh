@@ -130,7 +130,7 @@ k_apply_group(GroupArgs a) {
     T* colG = sG + lane;
     __syncthreads();   // previous item's coefficient columns are no longer read
     if (warp == 0) {
-      besselj_seq<T>(rmul(kk, r), p + 1, colJ, kGrpCentres);
+      besselj_column<T>(rmul(kk, r), p + 1, colJ, kGrpCentres);
       for (int l = 0; l <= p; ++l) {
         const T jl = colJ[l * kGrpCentres];
         if (kD || kG) colL[l * kGrpCentres] = rmul(jl, (double)l);

@@ -9,8 +9,13 @@ namespace qbx {
 
 struct cplx;
 
-constexpr int kApplyThreads = 128;   // centres per CTA of the fused apply
-constexpr int kSrcTile = 128;        // sources staged in shared memory per step
+constexpr int kApplyThreads = 128;   // threads per CTA of the fused apply (and of the far and grad D kernels)
+constexpr int kApplyCentres = 32;    // centres per CTA of the fused apply (one per lane, four warps)
+// centre blocks of a fused apply: 32 consecutive centres of one side
+inline int apply_units(int n_ctr, int n_tgt) {
+  return (n_tgt + kApplyCentres - 1) / kApplyCentres * (n_ctr / n_tgt);
+}
+constexpr int kSrcTile = 128;        // sources staged in shared memory per step (far, form and grad D kernels)
 constexpr int kFormThreads = 64;     // centres per CTA of form_locals
 constexpr int kMaxSplit = 64;        // source splits of the split reductions
 
@@ -40,6 +45,9 @@ struct ApplyArgs {
   int one_w;              // 1: wd[] of every requested operator is one array and nr = 1 (weighted
                           // seeds: the density multiplies H0, H1); 0: per-pair kernel values
   const double* hk_tab;   // complex k: the amplitude table of this k's ray (launch_hk_table), or null
+  const int *near, *near_cnt;   // near leaves of every 32-target block (near_q_src sources each; [blocks][near_stride], counts
+                                // at [blocks][3]); the launch then covers their sources only.  null: all sources
+  int near_stride;
 };
 // Amplitudes B_n = H_n(z) e^{-i(z - pi/4)}, n = 0, 1, along the ray z = k rho
 // (|z| >= 2) as piecewise polynomials in s = |z|^{-1/2}, in the layout of the
@@ -239,5 +247,70 @@ void host_plan_workspace(const qbx_plan* plan, void** ws, size_t* bytes, int* nu
 // The plan's amplitude table for complex k (made on st when k changes), or
 // null for real k.
 const double* host_plan_hk_table(qbx_plan* plan, qbx_c64 k, cudaStream_t st, cudaError_t* err);
+
+}  // namespace qbx
+
+namespace qbx {
+
+// ---- cluster moments (qbx_tree.cu) -----------------------------------------
+// Order of a cluster's outgoing expansion: admits clusters at 4.2 radii.  24
+// would leave 8.0 near panels per block instead of 6.1 (starfish, 256 panels;
+// 266k instead of 204k FP64 instructions of pairs per target), 36 6.0; a warp
+// holds one order per lane.
+constexpr int kTreeP = 30;
+constexpr int kTreeLocal = 32;    // near-only QBX: orders of a centre's expansion that stands for the smooth rule
+constexpr int kTreeMinPanels = 16;   // fewer panels: every source pair by pair (no cluster of 8 is far from any block)
+constexpr int kTreeLevels = 16;
+constexpr int kTreeSets = 4;
+// what a moment set is made of: the density itself, or dipoles along n_s, x, y
+enum { kSetMono = 0, kSetNormal = 1, kSetX = 2, kSetY = 3 };
+
+struct TreeArgs {
+  double kre, kim;
+  int p;                      // order of the centres' expansions
+  int pl;                     // orders of the list entries (p, or kTreeLocal for near-only QBX)
+  int nd;                     // 1 if a derivative is taken anywhere (D, grad S), else 0
+  double eta;                 // near-only QBX (> 0)
+  int M, q_src, n_src;        // leaves (halves of panels, or panels), sources per leaf, sources
+  const double *sx, *sy, *snx, *sny;
+  int n_tgt, n_ctr;           // n_ctr = n_tgt or 2 n_tgt centres
+  const double *cx, *cy, *tx, *ty;
+  const double* hk_tab;
+  int lev;                    // levels; node (l, j) is off[l] + j
+  int off[kTreeLevels + 1];   // off[lev]: node count
+  int n_blk;                  // 32-target blocks
+  double* node;               // [nodes + n_blk][4]: centre x, y, radius; then the blocks
+  int* near;                  // [n_blk][M] near leaves
+  int* far;                   // [n_blk][M + 1][2] far nodes: index, orders (cluster | centre << 8);
+                              // last the block's local expansion (index nodes + block, bit 16 set)
+  int* loc;                   // [n_blk][M][2] nodes of the local expansion: index, orders (cluster | block << 8)
+  int* cnt;                   // [n_blk][3] counts: near, far, loc
+  int nset, nrhs;
+  int kind[kTreeSets];
+  int slot[kTreeSets];        // which of the call's densities
+  const void* wd[kTreeSets];  // [n_src][nrhs] weighted densities
+  void* mom;                  // [lev][M][nset nrhs][kTreeP + 2][2] leaf contributions
+  int ncset;                  // coefficient column sets: a moment set, or its x, y derivative
+  int base[2 * kTreeSets], shift[2 * kTreeSets], plain[kTreeSets];
+  void* coef;                 // [nodes + n_blk][kTreeP + 1][ncset nrhs][2] coefficients
+  // evaluation (launch_far_clusters)
+  int ops;                    // OPB_* bits
+  int set_s, set_d, set_g, set_gx, set_x;   // column sets (grad S: the density's, its x derivative; y after x)
+  int rhs0, nr;
+  int nparts;                 // warps that share a far entry (1..4)
+  int nsplit, split0;         // partial-sum rows split0 .. split0 + nsplit - 1
+  void* part;                 // as ApplyArgs::part
+};
+// leaves, levels and node offsets of a run of panels; returns the node count
+int tree_levels(int panels, int q_src, TreeArgs* a);
+// device bytes of the arrays of `a` (lev, off, n_blk, nset, nrhs set); with
+// base != null also their addresses
+size_t tree_layout(TreeArgs* a, char* base);
+cudaError_t launch_tree_lists(const TreeArgs& a, cudaStream_t st);    // nodes, block lists
+cudaError_t launch_tree_moments(const TreeArgs& a, cudaStream_t st);  // moments, coefficients, local expansions
+cudaError_t launch_far_clusters(TreeArgs a, cudaStream_t st);         // partial sums of the far nodes
+bool far_clusters_fit(const TreeArgs& a);                             // whether their kernel can hold the orders
+// moment and column sets of a->ops, the densities of S, D, grad S (and X) in slots `slot`
+void tree_columns(TreeArgs* a, const int slot[3]);
 
 }  // namespace qbx

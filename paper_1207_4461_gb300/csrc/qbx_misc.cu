@@ -527,7 +527,7 @@ __global__ void k_eval(EvalArgs a) {
   const cplx eith = rho > 0.0 ? cplx{dx / rho, dy / rho} : cplx{1.0, 0.0};
   T J[QBX_MAX_P + 2];
   const T kr = make_kr<T>(a.kre, a.kim, rho);
-  if (rho > 0.0) besselj_seq<T>(kr, a.p + 1, J, 1);
+  if (rho > 0.0) besselj_column<T>(kr, a.p + 1, J, 1);
   else {
     for (int l = 0; l <= a.p + 1; ++l) sc_zero(J[l]);
     sc_set(J[0], 1.0);
@@ -622,11 +622,11 @@ __global__ void k_debug_besselj(const cplx* z, int n, int nmax, cplx* j) {
   const cplx zz = z[i];
   if (zz.im == 0.0) {
     double J[QBX_MAX_P + 2];
-    besselj_seq<double>(zz.re, nmax, J, 1);
+    besselj_column<double>(zz.re, nmax, J, 1);
     for (int l = 0; l <= nmax; ++l) j[(size_t)i * (nmax + 1) + l] = cplx{J[l], 0.0};
   } else {
     cplx J[QBX_MAX_P + 2];
-    besselj_seq<cplx>(zz, nmax, J, 1);
+    besselj_column<cplx>(zz, nmax, J, 1);
     for (int l = 0; l <= nmax; ++l) j[(size_t)i * (nmax + 1) + l] = J[l];
   }
 }

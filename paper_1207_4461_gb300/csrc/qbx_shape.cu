@@ -297,7 +297,7 @@ __global__ void k_dshape_columns(DsArgs a) {
   const double cx = a.cx[c], cy = a.cy[c];
   const int t = c % a.n_tgt;
   const double ux = a.tx[t] - cx, uy = a.ty[t] - cy, r = hypot(ux, uy);
-  besselj_seq<T>(rmul(kw.kval(), r), a.p + 1, reinterpret_cast<T*>(a.coef) + (size_t)c * (a.p + 2), 1);
+  besselj_column<T>(rmul(kw.kval(), r), a.p + 1, reinterpret_cast<T*>(a.coef) + (size_t)c * (a.p + 2), 1);
   double* geo = a.cgeo + 4 * (size_t)c;
   geo[0] = ux / r;
   geo[1] = uy / r;
@@ -579,7 +579,7 @@ static int shape_impl(int op, qbx_plan* plan, const qbx_geom* g, int side, qbx_c
   const int occ = opD ? 0
                       : (ck ? apply_occupancy_cplx(kOpsFwd, p, std::min(chunk, nrhs))
                             : apply_occupancy_real(kOpsFwd, p, std::min(chunk, nrhs)));
-  const int units = (nc + kApplyThreads - 1) / kApplyThreads;
+  const int units = opD ? (nc + 127) / 128 : apply_units(nc, n_tgt);
   int ns_fwd = host_choose_split_waves(num_sms, occ, units, n_src, per_fwd, avail / 2);
   const int tiles = opD ? (n_src + 127) / 128 : (n_src + kGrpCentres - 1) / kGrpCentres;
   int ns_adj = std::max(1, (num_sms * 6 + tiles - 1) / tiles);

@@ -163,7 +163,7 @@ extern "C" int qbx_apply_static(const qbx_geom* g, int op, int side, int limit, 
   const int chunk = apply_chunk(1 << op);
   const int occ = ck ? apply_occupancy_cplx(1 << op, p, std::min(chunk, nrhs), one_w)
                      : apply_occupancy_real(1 << op, p, std::min(chunk, nrhs), one_w);
-  const int units = (nc + kApplyThreads - 1) / kApplyThreads;
+  const int units = apply_units(nc, g->n_tgt);
   const int ns = host_choose_split_waves(s->num_sms, occ, units, g->n_src, per_split,
                                          QBX_STATIC_SCRATCH_BYTES - wd_bytes, 1);
   if (ns < 1) return invalid("no source split fits the fixed scratch");
