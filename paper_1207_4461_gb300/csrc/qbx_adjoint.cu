@@ -69,6 +69,40 @@ __global__ void k_adj_interp_t(int n_tgt, int q_tgt, int q_src, int nrhs, const 
 
 }  // namespace
 
+namespace qbx {
+// The sums over the centres (kernel a.ops) into a.part: all pair by pair, or
+// (tr) near leaves pair by pair on the plan's side stream beside the cluster
+// moments, the far sums in the row after the pair kernel's.
+cudaError_t adjoint_sums(AdjArgs& a, TreeArgs* tr, qbx_plan* plan, const qbx_geom* g, int c0, int nc, qbx_c64 k,
+                         int fops, int nd, int mode, int num_sms, char* tree_base, cudaStream_t st) {
+  const bool ck = k.im != 0.0;
+  auto pairs = [&](cudaStream_t s) { return ck ? launch_adjoint_cplx(a, s) : launch_adjoint_real(a, s); };
+  if (!tr) return pairs(st);
+  adj_tree_setup(tr, g, c0, nc, k, a.p, fops, nd, a.nrhs, a.hk_tab, a.gc, num_sms, tree_base);
+  cudaStream_t side;
+  cudaEvent_t fork, join;
+  host_plan_side(plan, &side, &fork, &join);
+  cudaError_t e = launch_tree_lists(*tr, st);
+  if (e == cudaSuccess) e = cudaEventRecord(fork, st);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork, 0);
+  if (e != cudaSuccess) return e;
+  a.near = tr->near;
+  a.near_cnt = tr->cnt;
+  a.near_stride = tr->M;
+  a.near_q = tr->q_src;
+  e = pairs(side);
+  cudaError_t ef = launch_tree_moments(*tr, ck, st);
+  if (ef == cudaSuccess) ef = launch_far_clusters(*tr, st);
+  const int ncomp = mode == 3 ? 5 : mode == 2 ? 3 : 1;
+  if (ef == cudaSuccess)
+    ef = launch_adj_far(*tr, mode, g->src_nx, g->src_ny,
+                        (cplx*)a.part + (size_t)a.nsplit * g->n_src * ncomp * a.nrhs, st);
+  cudaError_t ej = cudaEventRecord(join, side);   // (joined also after an error)
+  if (ej == cudaSuccess) ej = cudaStreamWaitEvent(st, join, 0);
+  return e != cudaSuccess ? e : ef != cudaSuccess ? ef : ej;
+}
+}  // namespace qbx
+
 extern "C" int qbx_apply_adjoint(qbx_plan* plan, const qbx_geom* g, int op, int side, int limit, qbx_c64 k,
                                  int p, const qbx_c64* gout, int nrhs, qbx_c64* gdens, void* stream) {
   if (!plan) return afail(QBX_EINVAL, "plan is NULL");
@@ -103,11 +137,18 @@ extern "C" int qbx_apply_adjoint(qbx_plan* plan, const qbx_geom* g, int op, int 
   const size_t fixed = b_gc + b_coef + b_geo + b_v + 256;
   if (ws_bytes < fixed) return afail(QBX_ENOMEM, "workspace too small");
   const size_t per_split = (size_t)g->n_src * nrhs * 16;
+  // distant centres through cluster moments (S: value; D: gradient along n_s), few columns
+  TreeArgs tr;
+  const int fops = op == QBX_OP_S ? 1 << QBX_OP_S : 1 << QBX_OP_GRAD_S;
+  size_t b_tree = nrhs <= 8 ? adj_tree_setup(&tr, g, c0, nc, k, p, fops, op == QBX_OP_D ? 1 : 0, nrhs, nullptr, nullptr,
+                                             num_sms, nullptr)
+                            : 0;
+  if (ws_bytes < fixed + b_tree + 256 + 2 * per_split) b_tree = 0;
   const int tiles = (g->n_src + kGrpCentres - 1) / kGrpCentres;
   int ns = std::max(1, (num_sms * 6 + tiles - 1) / tiles);
-  ns = std::min(ns, std::max(1, nc / kGrpTile));
+  ns = std::min(ns, std::max(1, (b_tree ? std::min(nc, 12 * q_tgt * nsides) : nc) / kGrpTile));
   ns = std::min(ns, kMaxSplit);
-  ns = std::min<long>(ns, (long)((ws_bytes - fixed) / per_split));
+  ns = std::min<long>(ns, (long)((ws_bytes - fixed - b_tree) / per_split) - (b_tree ? 1 : 0));
   if (ns < 1) return afail(QBX_ENOMEM, "workspace too small for the partial sums");
   cudaError_t e = cudaSetDevice(device);
   if (e != cudaSuccess) return acuda(e, "cudaSetDevice");
@@ -117,7 +158,7 @@ extern "C" int qbx_apply_adjoint(qbx_plan* plan, const qbx_geom* g, int op, int 
   void* coef = base + b_gc;
   double* cgeo = (double*)(base + b_gc + b_coef);
   void* v = base + b_gc + b_coef + b_geo;
-  void* part = base + b_gc + b_coef + b_geo + b_v;
+  void* part = base + b_gc + b_coef + b_geo + b_v + b_tree;
   k_adj_spread<<<(g->n_tgt * nrhs + 255) / 256, 256, 0, st>>>(g->n_tgt, nsides, nrhs, (const cplx*)gout, (cplx*)gc);
   e = cudaGetLastError();
   if (e != cudaSuccess) return acuda(e, "spread kernel");
@@ -146,9 +187,10 @@ extern "C" int qbx_apply_adjoint(qbx_plan* plan, const qbx_geom* g, int op, int 
   a.part = part;
   a.hk_tab = host_plan_hk_table(plan, k, st, &e);
   if (e != cudaSuccess) return acuda(e, "complex-k amplitude table");
-  e = ck ? launch_adjoint_cplx(a, st) : launch_adjoint_real(a, st);
+  e = adjoint_sums(a, b_tree ? &tr : nullptr, plan, g, c0, nc, k, fops, op == QBX_OP_D ? 1 : 0, op == QBX_OP_D ? 1 : 0,
+                   num_sms, base + b_gc + b_coef + b_geo + b_v, st);
   if (e != cudaSuccess) return acuda(e, "adjoint kernel");
-  k_adj_reduce<<<(g->n_src * nrhs + 255) / 256, 256, 0, st>>>(g->n_src, ns, nrhs, g->src_w, (const cplx*)part,
+  k_adj_reduce<<<(g->n_src * nrhs + 255) / 256, 256, 0, st>>>(g->n_src, ns + (b_tree ? 1 : 0), nrhs, g->src_w, (const cplx*)part,
                                                               (cplx*)v);
   // PV of D: u = lim - sg mu / 2 (sg = +1 exterior, -1 interior): adjoint adds -sg g / 2
   double jump = 0.0;

@@ -59,7 +59,7 @@ struct AdjSmem {
   static constexpr bool kD = OPS & OPB_D, kG = OPS & OPB_G, kX = OPS & OPB_X;
   static __host__ __device__ constexpr int nslots() { return 1 + ((kD || kG || kX) ? 1 : 0) + (kG ? 1 : 0); }
   static __host__ __device__ size_t bytes(int p) {
-    return 5 * kGrpTile * 8 +                                   // centre x, y, ux, uy, 1/r
+    return 5 * kGrpTile * 8 + kGrpTile * 8 +                    // centre x, y, ux, uy, 1/r; centre indices
            (size_t)kGrpTile * kGrpWarps * RG * 16 +              // gradients [centre][4 RG]
            (size_t)kNc * kGrpTile * kGrpCentres * 16 +           // kernel values [comp][centre][source]
            (size_t)nslots() * (p + 2) * kGrpTile * sizeof(T);    // coefficient columns [slot][l][centre]
@@ -81,7 +81,8 @@ k_adjoint(AdjArgs a) {
   double* s_ux = s_cy + kGrpTile;
   double* s_uy = s_ux + kGrpTile;
   double* s_ir = s_uy + kGrpTile;
-  cplx* s_g = reinterpret_cast<cplx*>(s_ir + kGrpTile);     // [centre][kRP]
+  int* s_c = reinterpret_cast<int*>(s_ir + kGrpTile);       // (8 bytes each reserved)
+  cplx* s_g = reinterpret_cast<cplx*>(s_c + 2 * kGrpTile);  // [centre][kRP]
   cplx* s_kv = s_g + kGrpTile * kRP;                         // [comp][centre][source]
   T* s_col = reinterpret_cast<T*>(s_kv + kNc * kGrpTile * kGrpCentres);  // [slot][l][centre]
   const int p = a.p, P2 = p + 2;
@@ -89,8 +90,15 @@ k_adjoint(AdjArgs a) {
 
   const int item = blockIdx.x;
   const int stile = item / a.nsplit, split = item % a.nsplit;
-  const int c_begin = split * a.ctr_per_split;
-  const int c_end = min(a.n_ctr, c_begin + a.ctr_per_split);
+  // centres [c_begin, c_end), numbered through the near list if there is one
+  int c_begin = split * a.ctr_per_split, c_end = min(a.n_ctr, c_begin + a.ctr_per_split);
+  const int per = a.near ? a.near_q * (a.n_ctr / a.n_tgt) : 1;   // centres of a leaf
+  const int* near = a.near ? a.near + (size_t)stile * a.near_stride : nullptr;
+  if (near) {
+    const long n = (long)a.near_cnt[3 * stile] * per;
+    c_begin = (int)(n * split / a.nsplit);
+    c_end = (int)(n * (split + 1) / a.nsplit);
+  }
   const int s = stile * kGrpCentres + lane;
   const bool active = s < a.n_src;
   const int ss = active ? s : a.n_src - 1;
@@ -116,19 +124,26 @@ k_adjoint(AdjArgs a) {
       const int nt = min(kGrpTile, c_end - base);
       __syncthreads();
       for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-        s_cx[i] = a.cx[base + i];
-        s_cy[i] = a.cy[base + i];
-        s_ux[i] = a.cgeo[3 * (size_t)(base + i)];
-        s_uy[i] = a.cgeo[3 * (size_t)(base + i) + 1];
-        s_ir[i] = a.cgeo[3 * (size_t)(base + i) + 2];
+        int c = base + i;
+        if (near) {
+          const int leaf = c / per, rem = c - leaf * per, sd = rem / a.near_q;
+          c = sd * a.n_tgt + near[leaf] * a.near_q + rem - sd * a.near_q;
+        }
+        s_c[i] = c;
+        s_cx[i] = a.cx[c];
+        s_cy[i] = a.cy[c];
+        s_ux[i] = a.cgeo[3 * (size_t)c];
+        s_uy[i] = a.cgeo[3 * (size_t)c + 1];
+        s_ir[i] = a.cgeo[3 * (size_t)c + 2];
       }
+      __syncthreads();
       for (int i = threadIdx.x; i < kGrpTile * kRP; i += blockDim.x) {
         const int c = i / kRP, rr = i - c * kRP;
-        s_g[i] = (c < nt && r0 + rr < a.nrhs) ? gin[(size_t)(base + c) * a.nrhs + r0 + rr] : cplx{0.0, 0.0};
+        s_g[i] = (c < nt && r0 + rr < a.nrhs) ? gin[(size_t)s_c[c] * a.nrhs + r0 + rr] : cplx{0.0, 0.0};
       }
       for (int i = threadIdx.x; i < nt * ns * P2; i += blockDim.x) {
         const int c = i / (ns * P2), rem = i - c * ns * P2;   // rem = slot * P2 + l
-        s_col[rem * kGrpTile + c] = coef[(size_t)(base + c) * ns * P2 + rem];
+        s_col[rem * kGrpTile + c] = coef[(size_t)s_c[c] * ns * P2 + rem];
       }
       __syncthreads();
       // ---- phase 1: K(c_j, x_s) for this warp's centres ----

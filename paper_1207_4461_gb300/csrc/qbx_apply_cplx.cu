@@ -15,9 +15,8 @@ int apply_occupancy_cplx(int ops, int p, int nr, bool one_w) {
 cudaError_t launch_group_cplx(const GroupArgs& a, int rg, int grid, cudaStream_t st) {
   return launch_group_any<cplx>(a, rg, grid, st);
 }
-size_t group_smem_cplx(int ops, int p, int rg) { return group_smem_any<cplx>(ops, p, rg); }
-int group_occupancy_cplx(int ops, int p, int rg) { return group_occupancy_any<cplx>(ops, p, rg); }
-const void* group_ptr_cplx(int ops, int rg) { return group_ptr_any<cplx>(ops, rg); }
+size_t group_smem_cplx(int ops, int p, int rg, int nsd) { return group_smem_any<cplx>(ops, p, rg, nsd); }
+int group_occupancy_cplx(int ops, int p, int rg, int nsd) { return group_occupancy_any<cplx>(ops, p, rg, nsd); }
 
 }  // namespace qbx
 

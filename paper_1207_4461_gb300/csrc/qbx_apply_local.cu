@@ -18,11 +18,8 @@ int apply_occupancy_local(int ops, bool ck, int p, int nr, bool one_w) {
 cudaError_t launch_group_local(const GroupArgs& a, bool ck, int rg, int grid, cudaStream_t st) {
   return ck ? launch_group_any<cplx, true>(a, rg, grid, st) : launch_group_any<double, true>(a, rg, grid, st);
 }
-int group_occupancy_local(int ops, bool ck, int p, int rg) {
-  return ck ? group_occupancy_any<cplx, true>(ops, p, rg) : group_occupancy_any<double, true>(ops, p, rg);
-}
-const void* group_ptr_local(int ops, bool ck, int rg) {
-  return ck ? group_ptr_any<cplx, true>(ops, rg) : group_ptr_any<double, true>(ops, rg);
+int group_occupancy_local(int ops, bool ck, int p, int rg, int nsd) {
+  return ck ? group_occupancy_any<cplx, true>(ops, p, rg, nsd) : group_occupancy_any<double, true>(ops, p, rg, nsd);
 }
 
 }  // namespace qbx

@@ -15,9 +15,8 @@ int apply_occupancy_real(int ops, int p, int nr, bool one_w) {
 cudaError_t launch_group_real(const GroupArgs& a, int rg, int grid, cudaStream_t st) {
   return launch_group_any<double>(a, rg, grid, st);
 }
-size_t group_smem_real(int ops, int p, int rg) { return group_smem_any<double>(ops, p, rg); }
-int group_occupancy_real(int ops, int p, int rg) { return group_occupancy_any<double>(ops, p, rg); }
-const void* group_ptr_real(int ops, int rg) { return group_ptr_any<double>(ops, rg); }
+size_t group_smem_real(int ops, int p, int rg, int nsd) { return group_smem_any<double>(ops, p, rg, nsd); }
+int group_occupancy_real(int ops, int p, int rg, int nsd) { return group_occupancy_any<double>(ops, p, rg, nsd); }
 
 }  // namespace qbx
 

@@ -1,8 +1,9 @@
 // qbx_batch.cu -- many curves (each with its own panels, wavenumber and
 // densities) applied in one persistent launch of the group kernel, run as a
 // CUDA graph: [zero the item counter] -> [oversample every curve's
-// densities] -> [group kernel over the longest-first item list] -> [scale,
-// jump terms / two-sided average into every curve's outputs].
+// densities] -> [cluster lists] -> [group kernel over the longest-first item
+// list of near sources, beside cluster moments and far sums] -> [scale, jump
+// terms / two-sided average into every curve's outputs].
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
@@ -37,6 +38,16 @@ struct qbx_batch {
   int q_tgt = 0, q_src = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
+  int nsd = 1;                      // 2: both sides of a target averaged per pair (two-sided S, D, S + D)
+  // distant sources through cluster moments (qbx_tree.cu): per-curve arguments
+  bool tree = false;
+  std::vector<qbx::TreeArgs> h_tree;
+  TreeArgs* d_tree = nullptr;
+  void* d_tree_mem = nullptr;
+  int ns_far = 0;                   // far splits of every clustered curve
+  int tree_q = 0;                   // sources per leaf
+  cudaStream_t cap[2] = {nullptr, nullptr};   // the graph's two branches are captured from these
+  cudaEvent_t ev[2] = {nullptr, nullptr};
 };
 
 namespace {
@@ -95,12 +106,12 @@ __global__ void k_batch_finish(const GroupInst* inst, int ops, int ncomp, int li
     qq -= n;
   }
   const cplx* part = reinterpret_cast<const cplx*>(in.part);
-  const int nsides = in.side == QBX_SIDE_TWO ? 2 : 1;
+  const int nsides = in.n_row / in.n_tgt;   // (merged: the sums are the two-sided average already)
   cplx res{0.0, 0.0};
   for (int sd = 0; sd < nsides; ++sd) {
     const int c = t + sd * in.n_tgt;
     cplx u{0.0, 0.0};
-    for (int k = 0; k < in.nsplit; ++k) u = u + part[(((size_t)k * in.n_ctr + c) * ncomp + q) * nrhs + r];
+    for (int k = 0; k < in.nsplit; ++k) u = u + part[(((size_t)k * in.n_row + c) * ncomp + q) * nrhs + r];
     u = mul_i(0.25 * u);
     if (in.side != QBX_SIDE_TWO && limit == QBX_LIMIT_PV) {
       const double sg = in.side == QBX_SIDE_EXT ? 1.0 : -1.0;
@@ -129,36 +140,51 @@ void destroy(qbx_batch* b) {
   cudaFree(b->d_wd);
   cudaFree(b->d_part);
   cudaFree(b->d_hk);
+  cudaFree(b->d_tree);
+  cudaFree(b->d_tree_mem);
+  for (int i = 0; i < 2; ++i) {
+    if (b->cap[i]) cudaStreamDestroy(b->cap[i]);
+    if (b->ev[i]) cudaEventDestroy(b->ev[i]);
+  }
   delete b;
 }
 
 
-// Work items of a configuration: 32 centres of one curve x a range of at
+// Sources of a work item's block: all of the curve's, or with clusters about
+// the six panels that stay near (the kernel takes the list's actual share).
+int block_sources(const GroupInst& in) {
+  return in.near ? std::min(in.n_src, 6 * (in.n_src / in.M)) : in.n_src;
+}
+
+// Work items of a configuration: 32 targets of one curve x a range of at
 // most `chunk` of its sources (equal ranges per curve), longest first.
 std::vector<GroupItem> make_items(const std::vector<GroupInst>& inst, int chunk, std::vector<int>& nsplit) {
   std::vector<GroupItem> items;
   nsplit.assign(inst.size(), 1);
   for (size_t i = 0; i < inst.size(); ++i) {
-    int ns = std::max(1, (inst[i].n_src + chunk - 1) / chunk);
-    const int len = (inst[i].n_src + ns - 1) / ns;
-    ns = (inst[i].n_src + len - 1) / len;   // every range non-empty
+    const int n = block_sources(inst[i]);
+    int ns = std::max(1, (n + chunk - 1) / chunk);
+    const int len = (n + ns - 1) / ns;
+    ns = (n + len - 1) / len;   // every range non-empty
     nsplit[i] = ns;
-    for (int c = 0; c < inst[i].n_ctr; c += kGrpCentres)
-      for (int k = 0; k < ns; ++k)
-        items.push_back(GroupItem{(int)i, c, k, k * len, std::min(inst[i].n_src, (k + 1) * len)});
+    for (int sd = 0; sd < inst[i].n_row / inst[i].n_tgt; ++sd)
+      for (int t = 0; t < inst[i].n_tgt; t += kGrpCentres)
+        for (int k = 0; k < ns; ++k)
+          items.push_back(GroupItem{(int)i, t, sd, k, k * len, std::min(n, (k + 1) * len)});
   }
   std::stable_sort(items.begin(), items.end(), [&](const GroupItem& x, const GroupItem& y) {
-    const long cx = (long)std::min(kGrpCentres, inst[x.inst].n_ctr - x.ctr0) * (x.src1 - x.src0);
-    const long cy = (long)std::min(kGrpCentres, inst[y.inst].n_ctr - y.ctr0) * (y.src1 - y.src0);
+    const long cx = (long)std::min(kGrpCentres, inst[x.inst].n_tgt - x.t0) * (x.src1 - x.src0);
+    const long cy = (long)std::min(kGrpCentres, inst[y.inst].n_tgt - y.t0) * (y.src1 - y.src0);
     return cx > cy;
   });
   return items;
 }
 
-size_t part_bytes(const std::vector<GroupInst>& inst, const std::vector<int>& nsplit, int ncomp, int nrhs) {
+// (the pair kernel's nsplit rows, and a clustered curve's ns_far more)
+size_t part_bytes(const std::vector<GroupInst>& inst, const std::vector<int>& nsplit, int ns_far, int ncomp, int nrhs) {
   size_t t = 0;
   for (size_t i = 0; i < inst.size(); ++i)
-    t += host_align256((size_t)nsplit[i] * inst[i].n_ctr * ncomp * nrhs * 16);
+    t += host_align256((size_t)(nsplit[i] + (inst[i].near ? ns_far : 0)) * inst[i].n_row * ncomp * nrhs * 16);
   return t;
 }
 
@@ -170,26 +196,29 @@ double lpt_makespan(const std::vector<GroupInst>& inst, const std::vector<GroupI
   auto cmp = [](double x, double y) { return x > y; };
   for (const GroupItem& it : items) {
     std::pop_heap(heap.begin(), heap.end(), cmp);
-    const double pairs = (double)std::min(kGrpCentres, inst[it.inst].n_ctr - it.ctr0) * (it.src1 - it.src0);
+    const double pairs = (double)std::min(kGrpCentres, inst[it.inst].n_tgt - it.t0) * (it.src1 - it.src0);
     heap.back() += pairs + 32.0 * kGrpTile;   // + one tile's worth of set-up per item
     std::push_heap(heap.begin(), heap.end(), cmp);
   }
   return *std::max_element(heap.begin(), heap.end());
 }
 
+// smallest source range of an item (with clusters a block has few hundred sources in all)
+int min_chunk(const qbx_batch* b) { return b->tree ? 64 : 512; }
+
 // The source chunk the model prefers: the smallest predicted makespan over
 // chunks 2^j * 32 (and all sources), ties to the larger chunk (fewer
 // partial sums), within the partial-sum memory budget.
 int model_chunk(const qbx_batch* b, int slots, size_t budget) {
   std::vector<int> cand{(b->max_src + kGrpTile - 1) / kGrpTile * kGrpTile};
-  for (int c = 1 << 20; c >= 512; c /= 2)
+  for (int c = 1 << 20; c >= min_chunk(b); c /= 2)
     if (c < b->max_src) cand.push_back(c);
   int best = cand[0];
   double bt = 1e300;
   std::vector<int> ns;
   for (int c : cand) {
     std::vector<GroupItem> items = make_items(b->h_inst, c, ns);
-    if (part_bytes(b->h_inst, ns, b->ncomp, b->nrhs) > budget) break;
+    if (part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs) > budget) break;
     const double t = lpt_makespan(b->h_inst, items, slots);
     if (t < bt * 0.995) {
       bt = t;
@@ -206,7 +235,7 @@ int configure(qbx_batch* b, int rg, int chunk) {
   if (e != cudaSuccess) return bcuda(e, "device");
   std::vector<int> ns;
   std::vector<GroupItem> items = make_items(b->h_inst, chunk, ns);
-  const size_t pb = part_bytes(b->h_inst, ns, b->ncomp, b->nrhs);
+  const size_t pb = part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs);
   if (pb > b->part_cap) {
     cudaFree(b->d_part);
     b->d_part = nullptr;
@@ -223,11 +252,20 @@ int configure(qbx_batch* b, int rg, int chunk) {
   }
   size_t off = 0;
   for (int i = 0; i < b->n_inst; ++i) {
-    b->h_inst[i].nsplit = ns[i];
-    b->h_inst[i].part = static_cast<char*>(b->d_part) + off;
-    off += host_align256((size_t)ns[i] * b->h_inst[i].n_ctr * b->ncomp * b->nrhs * 16);
+    GroupInst& in = b->h_inst[i];
+    in.nsplit_near = ns[i];
+    in.nsplit = ns[i] + (in.near ? b->ns_far : 0);
+    in.part = static_cast<char*>(b->d_part) + off;
+    off += host_align256((size_t)in.nsplit * in.n_row * b->ncomp * b->nrhs * 16);
+    if (b->tree) {
+      b->h_tree[i].part = in.part;
+      b->h_tree[i].split0 = ns[i];
+      b->h_tree[i].nsplit = in.near ? b->ns_far : 0;
+    }
   }
   e = cudaMemcpy(b->d_inst, b->h_inst.data(), sizeof(GroupInst) * b->n_inst, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && b->tree)
+    e = cudaMemcpy(b->d_tree, b->h_tree.data(), sizeof(TreeArgs) * b->n_inst, cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(b->d_items, items.data(), sizeof(GroupItem) * items.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return bcuda(e, "upload");
@@ -235,9 +273,10 @@ int configure(qbx_batch* b, int rg, int chunk) {
   b->rg = rg;
   b->chunk = chunk;
   const bool local = b->eta2 > 0.0;
-  const int occ = local ? group_occupancy_local(b->ops, b->ck, b->p, rg)
-                        : (b->ck ? group_occupancy_cplx(b->ops, b->p, rg) : group_occupancy_real(b->ops, b->p, rg));
-  const size_t gsmem = b->ck ? group_smem_cplx(b->ops, b->p, rg) : group_smem_real(b->ops, b->p, rg);
+  const int occ = local ? group_occupancy_local(b->ops, b->ck, b->p, rg, b->nsd)
+                        : (b->ck ? group_occupancy_cplx(b->ops, b->p, rg, b->nsd)
+                                 : group_occupancy_real(b->ops, b->p, rg, b->nsd));
+  const size_t gsmem = b->ck ? group_smem_cplx(b->ops, b->p, rg, b->nsd) : group_smem_real(b->ops, b->p, rg, b->nsd);
   if (occ < 1 || gsmem > 220 * 1024) return bfail(QBX_EINVAL, "p too large for the group kernel");
   b->grid = std::min(b->n_items, b->num_sms * occ);
   if (b->exec) cudaGraphExecDestroy(b->exec);
@@ -248,60 +287,133 @@ int configure(qbx_batch* b, int rg, int chunk) {
   ga.ops = b->ops;
   ga.p = b->p;
   ga.nrhs = b->nrhs;
+  ga.nsd = b->nsd;
   ga.inst = b->d_inst;
   ga.n_items = b->n_items;
   ga.items = b->d_items;
   ga.counter = b->d_counter;
   ga.eta2 = b->eta2;
-  const void* gk = local ? group_ptr_local(b->ops, b->ck, rg)
-                         : (b->ck ? group_ptr_cplx(b->ops, rg) : group_ptr_real(b->ops, rg));
-  if (!gk) return bfail(QBX_EINVAL, "no group kernel for this operator set");
-  e = cudaFuncSetAttribute(gk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem);
-  if (e == cudaSuccess) e = cudaGraphCreate(&b->graph, 0);
-  cudaGraphNode_t n_memset, n_up, n_group, n_fin;
-  if (e == cudaSuccess) {
-    cudaMemsetParams mp{};
-    mp.dst = b->d_counter;
-    mp.value = 0;
-    mp.elementSize = sizeof(int);
-    mp.width = 1;
-    mp.height = 1;
-    e = cudaGraphAddMemsetNode(&n_memset, b->graph, nullptr, 0, &mp);
+  // the graph, captured from two streams of the batch's own: the pair sums
+  // beside the cluster moments and far sums
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+    if (!b->cap[i]) e = cudaStreamCreateWithFlags(&b->cap[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess && !b->ev[i]) e = cudaEventCreateWithFlags(&b->ev[i], cudaEventDisableTiming);
   }
-  int q_tgt = b->q_tgt, q_src = b->q_src, nr = b->nrhs, ncomp = b->ncomp, lim = b->limit, opsv = b->ops;
-  const GroupInst* di = b->d_inst;
-  const double* P = b->d_interp;
-  int* st = b->d_status;
-  if (e == cudaSuccess) {
-    void* args[] = {(void*)&di, &q_tgt, &q_src, &nr, (void*)&P};
-    cudaKernelNodeParams kp{};
-    kp.func = (void*)k_batch_upsample;
-    kp.gridDim = dim3((b->max_src * nr + 255) / 256, b->n_inst);
-    kp.blockDim = dim3(256);
-    kp.kernelParams = args;
-    e = cudaGraphAddKernelNode(&n_up, b->graph, &n_memset, 1, &kp);
+  if (e == cudaSuccess) e = cudaStreamBeginCapture(b->cap[0], cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return bcuda(e, "graph capture");
+  cudaStream_t s0 = b->cap[0], s1 = b->tree ? b->cap[1] : b->cap[0];
+  auto ok = [&](cudaError_t x) {
+    if (e == cudaSuccess) e = x;
+  };
+  ok(cudaMemsetAsync(b->d_counter, 0, sizeof(int), s0));
+  k_batch_upsample<<<dim3((b->max_src * b->nrhs + 255) / 256, b->n_inst), 256, 0, s0>>>(b->d_inst, b->q_tgt, b->q_src,
+                                                                                       b->nrhs, b->d_interp);
+  ok(cudaGetLastError());
+  TreeArgs tr{};
+  if (b->tree) {   // launch sizes: the largest over the curves
+    tr = b->h_tree[0];
+    tr.inst = b->d_tree;
+    for (const TreeArgs& t : b->h_tree) {
+      tr.M = std::max(tr.M, t.M);
+      tr.n_blk = std::max(tr.n_blk, t.n_blk);
+      if (t.off[t.lev] > tr.off[tr.lev]) {
+        tr.lev = t.lev;
+        for (int l = 0; l <= t.lev; ++l) tr.off[l] = t.off[l];
+      }
+    }
+    tr.q_src = b->tree_q;
+    tr.nsplit = b->ns_far;
+    ok(launch_tree_lists(tr, s0, b->n_inst));
+    ok(cudaEventRecord(b->ev[0], s0));
+    ok(cudaStreamWaitEvent(s1, b->ev[0], 0));
   }
-  if (e == cudaSuccess) {
-    void* args[] = {&ga};
-    cudaKernelNodeParams kp{};
-    kp.func = const_cast<void*>(gk);
-    kp.gridDim = dim3(b->grid);
-    kp.blockDim = dim3(kGrpCentres * kGrpWarps);
-    kp.sharedMemBytes = (unsigned)gsmem;
-    kp.kernelParams = args;
-    e = cudaGraphAddKernelNode(&n_group, b->graph, &n_up, 1, &kp);
+  if (local) ok(launch_group_local(ga, b->ck, rg, b->grid, s1));
+  else ok(b->ck ? launch_group_cplx(ga, rg, b->grid, s1) : launch_group_real(ga, rg, b->grid, s1));
+  if (b->tree) {
+    ok(launch_tree_moments(tr, b->ck, s0, b->n_inst));
+    ok(launch_far_group(tr, b->ck, s0, b->n_inst));
+    ok(cudaEventRecord(b->ev[1], s1));
+    ok(cudaStreamWaitEvent(s0, b->ev[1], 0));
   }
-  if (e == cudaSuccess) {
-    void* args[] = {(void*)&di, &opsv, &ncomp, &lim, &nr, &st};
-    cudaKernelNodeParams kp{};
-    kp.func = (void*)k_batch_finish;
-    kp.gridDim = dim3((b->max_tgt * ncomp * nr + 255) / 256, b->n_inst);
-    kp.blockDim = dim3(256);
-    kp.kernelParams = args;
-    e = cudaGraphAddKernelNode(&n_fin, b->graph, &n_group, 1, &kp);
-  }
+  k_batch_finish<<<dim3((b->max_tgt * b->ncomp * b->nrhs + 255) / 256, b->n_inst), 256, 0, s0>>>(
+      b->d_inst, b->ops, b->ncomp, b->limit, b->nrhs, b->d_status);
+  ok(cudaGetLastError());
+  const cudaError_t ec = cudaStreamEndCapture(s0, &b->graph);   // (also after an error)
+  ok(ec);
   if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
   if (e != cudaSuccess) return bcuda(e, "graph construction");
+  return QBX_OK;
+}
+
+// Cluster arrays of every curve with enough panels (many columns: S, D or
+// S + D), for the batch's eta: sizes them, allocates on first use, and points
+// the curves' pair sums at their near lists.  Without memory for them, or for
+// orders the far kernel cannot hold, every pair goes pair by pair.
+int prepare_tree(qbx_batch* b, size_t budget) {
+  b->tree = false;
+  for (GroupInst& in : b->h_inst) in.near = nullptr;
+  if (b->ops == (QBX_OPS_S | QBX_OPS_D | QBX_OPS_GRAD_S)) return QBX_OK;
+  const int none[3] = {0, 0, 0};
+  std::vector<TreeArgs> v(b->n_inst);
+  size_t total = 0;
+  long blocks = 0;
+  for (int i = 0; i < b->n_inst; ++i) {
+    const GroupInst& in = b->h_inst[i];
+    TreeArgs& t = v[i];
+    t = TreeArgs{};
+    t.kre = in.kre;
+    t.kim = in.kim;
+    t.p = b->p;
+    t.pl = b->eta2 > 0.0 ? std::max(b->p, kTreeLocal) : b->p;
+    t.nd = (b->ops & QBX_OPS_D) ? 1 : 0;
+    t.eta = sqrt(b->eta2);
+    t.n_tgt = in.n_tgt;
+    t.n_ctr = in.n_ctr;
+    t.ops = b->ops;
+    t.nrhs = b->nrhs;
+    t.up = 1;
+    tree_columns(&t, none);
+    if (in.M < kTreeMinPanels) continue;   // (no levels, leaves or blocks)
+    tree_levels(in.M, b->q_src, &t);
+    b->tree_q = t.q_src;
+    t.n_blk = (in.n_tgt + kGrpCentres - 1) / kGrpCentres;
+    blocks += t.n_blk;
+    t.sx = in.sx;
+    t.sy = in.sy;
+    t.snx = in.snx;
+    t.sny = in.sny;
+    t.cx = in.cx;
+    t.cy = in.cy;
+    t.tx = in.tx;
+    t.ty = in.ty;
+    t.hk_tab = in.hk_tab;
+    for (int s = 0; s < t.nset; ++s) t.wd[s] = in.wd;
+    total += tree_layout(&t, nullptr);
+  }
+  if (total == 0 || !far_group_fit(v[0], b->ck, b->h_inst[0].n_ctr / b->h_inst[0].n_tgt)) return QBX_OK;
+  if (!b->d_tree_mem) {
+    if (total > budget) return QBX_OK;
+    cudaError_t e = cudaMalloc(&b->d_tree_mem, total);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_tree, sizeof(TreeArgs) * b->n_inst);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      cudaFree(b->d_tree_mem);
+      b->d_tree_mem = nullptr;
+      return QBX_OK;
+    }
+  }
+  b->tree = true;
+  b->ns_far = (int)std::max<long>(1, std::min<long>(4, (b->num_sms * 3 + blocks - 1) / blocks));
+  size_t off = 0;
+  for (int i = 0; i < b->n_inst; ++i) {
+    if (v[i].n_blk == 0) continue;
+    off += tree_layout(&v[i], static_cast<char*>(b->d_tree_mem) + off);
+    b->h_inst[i].near = v[i].near;
+    b->h_inst[i].near_cnt = v[i].cnt;
+    b->h_inst[i].near_stride = v[i].M;
+    b->h_inst[i].near_q = v[i].q_src;
+  }
+  b->h_tree = v;
   return QBX_OK;
 }
 
@@ -357,6 +469,7 @@ int qbx_batch_create(qbx_batch** batch, qbx_plan* plan, int n_inst, const qbx_ge
   b->nrhs = nrhs;
   b->ncomp = (ops & 1) + ((ops >> 1) & 1) + 2 * ((ops >> 2) & 1);
   b->rg = nrhs > 8 ? 8 : 2;
+  b->nsd = side == QBX_SIDE_TWO && b->ncomp <= 2 ? 2 : 1;
   // the plan's device, grid pair and interpolation matrix
   int num_sms = 0;
   host_plan_info(plan, &b->device, &b->q_tgt, &b->q_src, &b->d_interp);
@@ -399,6 +512,7 @@ int qbx_batch_create(qbx_batch** batch, qbx_plan* plan, int n_inst, const qbx_ge
     in.M = g.M;
     in.side = side;
     in.n_ctr = side == QBX_SIDE_TWO ? 2 * g.n_tgt : g.n_tgt;
+    in.n_row = b->nsd == 2 ? g.n_tgt : in.n_ctr;
     const int c0 = side == QBX_SIDE_EXT ? g.n_tgt : 0;
     in.nsplit = 1;
     in.sx = g.src_x;
@@ -454,11 +568,12 @@ int qbx_batch_create(qbx_batch** batch, qbx_plan* plan, int n_inst, const qbx_ge
     return bcuda(e, "complex-k amplitude tables");
   }
   // ---- items: the source chunk the makespan model prefers ----
-  const int occ = b->ck ? group_occupancy_cplx(ops, p, b->rg) : group_occupancy_real(ops, p, b->rg);
+  const int occ = b->ck ? group_occupancy_cplx(ops, p, b->rg, b->nsd) : group_occupancy_real(ops, p, b->rg, b->nsd);
   if (occ < 1) {
     destroy(b);
     return bfail(QBX_EINVAL, "p too large for the group kernel");
   }
+  prepare_tree(b, part_budget(b->device));
   int rg = b->rg, chunk = 0;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -471,7 +586,7 @@ int qbx_batch_create(qbx_batch** batch, qbx_plan* plan, int n_inst, const qbx_ge
   if (chunk > 0) {   // a cached choice, if its partial sums fit
     std::vector<int> ns;
     make_items(b->h_inst, chunk, ns);
-    if (part_bytes(b->h_inst, ns, b->ncomp, b->nrhs) > part_budget(b->device)) chunk = 0;
+    if (part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs) > part_budget(b->device)) chunk = 0;
   }
   if (chunk == 0) {
     rg = b->rg;
@@ -495,7 +610,7 @@ int qbx_batch_tune(qbx_batch* b, void* stream, int* rg_out, int* chunk_out) {
   const size_t budget = part_budget(b->device) + b->part_cap;
   const int c0 = b->chunk;
   std::vector<int> chunks{c0};
-  if (c0 / 2 >= 512) chunks.push_back(c0 / 2);
+  if (c0 / 2 >= min_chunk(b)) chunks.push_back(c0 / 2);
   if (c0 < b->max_src) chunks.push_back(std::min(2 * c0, (b->max_src + kGrpTile - 1) / kGrpTile * kGrpTile));
   std::vector<int> rgs{b->nrhs > 8 ? 8 : 2};
   if (b->nrhs > 2 && b->nrhs % 32 != 0) rgs.push_back(rgs[0] == 8 ? 2 : 8);
@@ -512,7 +627,7 @@ int qbx_batch_tune(qbx_batch* b, void* stream, int* rg_out, int* chunk_out) {
     for (int c : chunks) {
       std::vector<int> ns;
       make_items(b->h_inst, c, ns);
-      if (part_bytes(b->h_inst, ns, b->ncomp, b->nrhs) > budget) continue;
+      if (part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs) > budget) continue;
       if ((rc = configure(b, rg, c))) break;
       // one untimed launch, then one timed
       e = cudaGraphLaunch(b->exec, st);
@@ -551,6 +666,10 @@ int qbx_batch_set_eta(qbx_batch* b, double eta) {
   if (!b) return bfail(QBX_EINVAL, "NULL batch");
   if (!(eta >= 0.0) || !isfinite(eta)) return bfail(QBX_EINVAL, "eta must be finite and >= 0");
   b->eta2 = eta * eta;
+  const bool was = b->tree;
+  prepare_tree(b, part_budget(b->device));
+  if (was != b->tree)   // other items, other ranges
+    b->chunk = model_chunk(b, b->grid, part_budget(b->device) + b->part_cap);
   return configure(b, b->rg, b->chunk);
 }
 

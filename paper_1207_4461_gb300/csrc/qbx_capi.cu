@@ -217,6 +217,12 @@ void host_plan_workspace(const qbx_plan* plan, void** ws, size_t* bytes, int* nu
   *status = plan->d_status;
 }
 
+void host_plan_side(const qbx_plan* plan, cudaStream_t* side, cudaEvent_t* fork, cudaEvent_t* join) {
+  *side = plan->side;
+  *fork = plan->fork;
+  *join = plan->join;
+}
+
 void host_plan_info(const qbx_plan* plan, int* device, int* q_tgt, int* q_src, const double** interp) {
   *device = plan->device;
   *q_tgt = plan->q_tgt;
@@ -661,24 +667,29 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   const size_t wd_bytes = wd_one * nd + tan_bytes;
   if (p->ws_bytes < wd_bytes + 512) return fail(QBX_ENOMEM, "workspace too small (%zu < %zu)", p->ws_bytes, wd_bytes + 512);
   const size_t avail = p->ws_bytes - wd_bytes - 512;
-  const size_t per_split = (size_t)nc * ncomp * nrhs * 16;
   // many right-hand sides of one density: the group kernel (kernel values
   // formed once per pair for all rhs); otherwise the fused kernel
   const bool ck = k.im != 0.0;
   const bool group = cf || (nrhs >= 16 && nd == 1 && (ops == 1 || ops == 2 || ops == 3 || ops == 7));
   const int gops = cf ? kOpsCombined : ops;   // the group kernel's operator set
+  // both sides of a target in one lane of the group kernel, their kernel
+  // values averaged before the rhs products (64 rhs of the combined field,
+  // 256 panels: 452 -> 294 FP64 instructions per pair)
+  const bool merged = group && side == QBX_SIDE_TWO && ops != 7;
+  const int nsd = merged ? 2 : 1, nrow = merged ? g->n_tgt : nc;   // nrow: rows of the partial sums
+  const size_t per_split = (size_t)nrow * ncomp * nrhs * 16;
   // more than 32 rhs (global apply): eight warps of 8 rhs, so that the kernel
   // values of a pair are formed once per 64 rhs instead of once per 32
   const int rg = (nrhs > 32 && !(eta > 0.0)) ? kGrpRhsWide : 8;
-  const int units = group ? (nc + kGrpCentres - 1) / kGrpCentres : apply_units(nc, g->n_tgt);
+  const int units = apply_units(nrow, g->n_tgt);   // 32-target blocks, per side or merged
   const bool local = eta > 0.0;
   const int chunk = local ? std::min(4, apply_chunk(ops)) : apply_chunk(ops);
   // one rhs of one density for every operator: the weighted-seed instance
   const bool one_w = !group && nd == 1 && nrhs == 1;
   CK(cudaSetDevice(p->device), "cudaSetDevice");
   int occ;
-  if (group && local) occ = group_occupancy_local(ops, ck, pp, rg);
-  else if (group) occ = ck ? group_occupancy_cplx(gops, pp, rg) : group_occupancy_real(gops, pp, rg);
+  if (group && local) occ = group_occupancy_local(ops, ck, pp, rg, nsd);
+  else if (group) occ = ck ? group_occupancy_cplx(gops, pp, rg, nsd) : group_occupancy_real(gops, pp, rg, nsd);
   else if (local) occ = apply_occupancy_local(ops, ck, pp, std::min(chunk, nrhs), one_w);
   else occ = ck ? apply_occupancy_cplx(ops, pp, std::min(chunk, nrhs), one_w)
                 : apply_occupancy_real(ops, pp, std::min(chunk, nrhs), one_w);
@@ -696,7 +707,8 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   TreeArgs tr{};
   size_t tree_bytes = 0;
   int ns_far = 0;
-  if (!group && g->M >= kTreeMinPanels) {
+  const bool far_group = group && ops != 7;   // many columns: far values formed once for all
+  if (g->M >= kTreeMinPanels) {
     tr.kre = k.re;
     tr.kim = k.im;
     tr.p = pp;
@@ -706,24 +718,36 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     tr.n_tgt = g->n_tgt;
     tr.n_ctr = nc;
     tr.n_blk = apply_units(g->n_tgt, g->n_tgt);
-    tr.ops = ops;
+    tr.ops = gops;
     tr.nrhs = nrhs;
+    tr.up = far_group ? 1 : 0;
+    if (cf) {
+      tr.eta_re = cf_eta->re;
+      tr.eta_im = cf_eta->im;
+    }
     tree_columns(&tr, slot_of);
     tree_levels(g->M, g->q_src, &tr);
     tree_bytes = tree_layout(&tr, nullptr);
-    // a few CTAs per SM share a block's far nodes; few blocks: several warps to a node
-    tr.nparts = std::max(1, std::min(4, p->num_sms * 8 / (units * 16)));
-    ns_far = std::max(2, std::min(8, (p->num_sms * 2 + units - 1) / units));
-    if (!far_clusters_fit(tr) || avail < tree_bytes + (size_t)(ns_far + 1) * per_split) ns_far = 0;
+    if (far_group) {
+      ns_far = std::max(1, std::min(4, (p->num_sms * 3 + units - 1) / units));
+    } else {
+      // a few CTAs per SM share a block's far nodes; few blocks: several warps to a node
+      tr.nparts = std::max(1, std::min(4, p->num_sms * 8 / (units * 16)));
+      ns_far = std::max(2, std::min(8, (p->num_sms * 2 + units - 1) / units));
+    }
+    if (!(far_group ? far_group_fit(tr, ck, nsd) : far_clusters_fit(tr)) ||
+        avail < tree_bytes + (size_t)(ns_far + 1) * per_split)
+      ns_far = 0;
   }
   const bool tree = ns_far > 0;
   if (!tree) tree_bytes = 0;
   // (with clusters a block's near leaves are some six panels; down to two dozen sources a CTA)
-  const int ns_near = host_choose_split_waves(p->num_sms, occ, units, tree ? std::min(g->n_src, 16 * g->q_src) : g->n_src,
-                                              per_split, avail - tree_bytes - ns_far * per_split, waves);
+  const int ns_near =
+      host_choose_split_waves(p->num_sms, occ, units, tree ? std::min(g->n_src, (group ? 8 : 16) * g->q_src) : g->n_src,
+                              per_split, avail - tree_bytes - ns_far * per_split, waves);
   if (ns_near < 1) return fail(QBX_ENOMEM, "workspace too small for the apply partial sums");
   const int ns = ns_near + ns_far;
-  if (group ? (ck ? group_smem_cplx(gops, pp, rg) : group_smem_real(gops, pp, rg)) > 220 * 1024
+  if (group ? (ck ? group_smem_cplx(gops, pp, rg, nsd) : group_smem_real(gops, pp, rg, nsd)) > 220 * 1024
             : apply_smem_bytes(ops, ck, pp, chunk) > 220 * 1024)
     return fail(QBX_EINVAL, "p = %d too large", pp);
   cudaStream_t st = (cudaStream_t)stream;
@@ -792,28 +816,13 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     a.near_cnt = tr.cnt;
     a.near_stride = tr.M;
     a.near_q_src = tr.q_src;
-    // near pairs on the side stream, clusters on the caller's: the moments'
-    // and the far sums' short launches fill in where the pair kernel leaves room
-    CK(cudaEventRecord(p->fork, st), "fork event");
-    CK(cudaStreamWaitEvent(p->side, p->fork, 0), "fork");
-    cudaError_t en = cudaSuccess;
-    for (int r0 = 0; r0 < nrhs && en == cudaSuccess; r0 += chunk) {
-      a.rhs0 = r0;
-      a.nr = std::min(chunk, nrhs - r0);
-      en = launch_apply_fused(a, p->side);
-    }
-    cudaError_t ef = launch_tree_moments(tr, st);
-    if (ef == cudaSuccess) ef = launch_far_clusters(tr, st);
-    CK(cudaEventRecord(p->join, p->side), "join event");   // (joined also after an error)
-    CK(cudaStreamWaitEvent(st, p->join, 0), "join");
-    CK(en, "apply kernel");
-    CK(ef, "far clusters");
   }
+  GroupArgs ga{};
   if (group) {
-    GroupArgs ga{};
     ga.ops = gops;
     ga.p = pp;
     ga.nrhs = nrhs;
+    ga.nsd = nsd;
     if (cf) {
       ga.cf_re = cf_eta->re;
       ga.cf_im = cf_eta->im;
@@ -824,8 +833,10 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     in.n_src = g->n_src;
     in.n_tgt = g->n_tgt;
     in.n_ctr = nc;
+    in.n_row = nrow;
     in.side = side;
     in.nsplit = ns;
+    in.nsplit_near = ns_near;
     in.M = g->M;
     in.sx = g->src_x;
     in.sy = g->src_y;
@@ -841,33 +852,57 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     in.wd = base;
     in.part = part;
     in.hk_tab = a.hk_tab;
+    in.near = a.near;
+    in.near_cnt = a.near_cnt;
+    in.near_stride = a.near_stride;
+    in.near_q = a.near_q_src;
     ga.st_units = units;
-    ga.st_nsplit = ns;
-    ga.st_split_len = split_len(g->n_src, ns);
+    ga.st_nsplit = ns_near;
+    ga.st_split_len = split_len(g->n_src, ns_near);
     ga.eta2 = a.eta2;
-    if (local)
-      CK(launch_group_local(ga, ck, rg, units * ns, st), "group kernel (near-only)");
-    else
-      CK(ck ? launch_group_cplx(ga, rg, units * ns, st) : launch_group_real(ga, rg, units * ns, st), "group kernel");
-  } else if (!tree) {
-    for (int r0 = 0; r0 < nrhs; r0 += chunk) {
+  }
+  auto pair_sums = [&](cudaStream_t s) {
+    if (group) {
+      if (local) return launch_group_local(ga, ck, rg, units * ns_near, s);
+      return ck ? launch_group_cplx(ga, rg, units * ns_near, s) : launch_group_real(ga, rg, units * ns_near, s);
+    }
+    cudaError_t e = cudaSuccess;
+    for (int r0 = 0; r0 < nrhs && e == cudaSuccess; r0 += chunk) {
       a.rhs0 = r0;
       a.nr = std::min(chunk, nrhs - r0);
-      CK(launch_apply_fused(a, st), "apply kernel");
+      e = launch_apply_fused(a, s);
     }
+    return e;
+  };
+  if (tree) {
+    // near pairs on the side stream, clusters on the caller's: the moments'
+    // and the far sums' short launches fill in where the pair kernel leaves room
+    CK(cudaEventRecord(p->fork, st), "fork event");
+    CK(cudaStreamWaitEvent(p->side, p->fork, 0), "fork");
+    const cudaError_t en = pair_sums(p->side);
+    cudaError_t ef = launch_tree_moments(tr, ck, st);
+    if (ef == cudaSuccess) ef = far_group ? launch_far_group(tr, ck, st) : launch_far_clusters(tr, st);
+    CK(cudaEventRecord(p->join, p->side), "join event");   // (joined also after an error)
+    CK(cudaStreamWaitEvent(st, p->join, 0), "join");
+    CK(en, "pair kernel");
+    CK(ef, "far clusters");
+  } else {
+    CK(pair_sums(st), "pair kernel");
   }
   if (p->timing) CK(cudaEventRecord(p->ev1, st), "timing event");
   // a7: reduce, i/4, jumps / two-sided average, per operator (the combined
   // field: one finish, the two-sided average as for S and D)
+  // (merged: the partial sums are the average already, without a jump)
+  const int fside = merged ? QBX_SIDE_INT : side, flimit = merged ? QBX_LIMIT_ONE_SIDED : limit;
   if (cf) {
-    CK(launch_apply_finish(QBX_OP_S, side, limit, g->n_tgt, ns, nc, nrhs, 0, 1, part, dens[0], g->tgt_nx,
+    CK(launch_apply_finish(QBX_OP_S, fside, flimit, g->n_tgt, ns, nrow, nrhs, 0, 1, part, dens[0], g->tgt_nx,
                            g->tgt_ny, out[1], p->d_status, st),
        "apply finish");
     return QBX_OK;
   }
   for (int o = 0; o < 3; ++o) {
     if (!(ops >> o & 1)) continue;
-    CK(launch_apply_finish(tangent ? QBX_OP_S : o, side, limit, g->n_tgt, ns, nc, nrhs, comp0[o], ncomp, part,
+    CK(launch_apply_finish(tangent ? QBX_OP_S : o, fside, flimit, g->n_tgt, ns, nrow, nrhs, comp0[o], ncomp, part,
                            dens[o], g->tgt_nx,
                            g->tgt_ny, out[o], p->d_status, st),
        "apply finish");
@@ -907,17 +942,42 @@ static int grad_d_impl(qbx_plan* p, const qbx_geom* g, int side, int limit, qbx_
     const size_t fixed = b_wd + b_ev + 512;
     if (p->ws_bytes < fixed) return fail(QBX_ENOMEM, "workspace too small for grad D");
     const size_t per_split = (size_t)nc * 2 * nrhs * 16;
-    const int units = (nc + kApplyThreads - 1) / kApplyThreads;
+    const int units = apply_units(nc, g->n_tgt);
     CK(cudaSetDevice(p->device), "cudaSetDevice");
     const int occ = grad_d_fused_occupancy(ck, pp);
-    const int ns = host_choose_split_waves(p->num_sms, occ, units, g->n_src, per_split, p->ws_bytes - fixed,
-                                           p->min_waves);
-    if (ns < 1) return fail(QBX_ENOMEM, "workspace too small for the grad D partial sums");
+    // distant sources through cluster moments, as the applies
+    TreeArgs tr{};
+    size_t tree_bytes = 0;
+    int ns_far = 0;
+    if (g->M >= kTreeMinPanels) {
+      tr.kre = k.re;
+      tr.kim = k.im;
+      tr.p = tr.pl = pp;
+      tr.nd = 2;   // at the source and at the target
+      tr.n_tgt = g->n_tgt;
+      tr.n_ctr = nc;
+      tr.n_blk = apply_units(g->n_tgt, g->n_tgt);
+      tr.ops = QBX_OPS_GRAD_S;
+      tr.nrhs = nrhs;
+      tree_columns_grad_d(&tr, false);
+      tree_levels(g->M, g->q_src, &tr);
+      tree_bytes = tree_layout(&tr, nullptr);
+      tr.nparts = std::max(1, std::min(4, p->num_sms * 8 / (units * 16)));
+      ns_far = std::max(2, std::min(8, (p->num_sms * 2 + units - 1) / units));
+      if (!far_clusters_fit(tr) || p->ws_bytes < fixed + tree_bytes + (size_t)(ns_far + 1) * per_split) ns_far = 0;
+    }
+    const bool tree = ns_far > 0;
+    if (!tree) tree_bytes = 0;
+    const int ns_near = host_choose_split_waves(
+        p->num_sms, occ, units, tree ? std::min(g->n_src, 16 * g->q_src) : g->n_src, per_split,
+        p->ws_bytes - fixed - tree_bytes - ns_far * per_split, tree ? std::max(p->min_waves, 2) : p->min_waves);
+    if (ns_near < 1) return fail(QBX_ENOMEM, "workspace too small for the grad D partial sums");
+    const int ns = ns_near + ns_far;
     cudaStream_t st = (cudaStream_t)stream;
     char* base = (char*)align256((size_t)p->ws);
     void* wd = base;
     void* ev = base + b_wd;
-    void* part = base + b_wd + b_ev;
+    void* part = base + b_wd + b_ev + tree_bytes;
     CK(launch_upsample(g->M, g->q_tgt, g->q_src, nrhs, p->d_interp, g->src_w, dens, wd, st), "upsample");
     if (p->timing) CK(cudaEventRecord(p->ev0, st), "timing event");
     ApplyArgs a{};
@@ -934,8 +994,8 @@ static int grad_d_impl(qbx_plan* p, const qbx_geom* g, int side, int limit, qbx_
     a.wd[0] = a.wd[1] = a.wd[2] = wd;
     a.nrhs = nrhs;
     a.nr = 1;
-    a.nsplit = ns;
-    a.src_per_split = split_len(g->n_src, ns);
+    a.nsplit = ns_near;
+    a.src_per_split = split_len(g->n_src, ns_near);
     a.part = part;
     a.near_q_tgt = g->q_tgt;
     a.near_q_src = g->q_src;
@@ -944,9 +1004,45 @@ static int grad_d_impl(qbx_plan* p, const qbx_geom* g, int side, int limit, qbx_
       a.hk_tab = host_plan_hk_table(p, k, st, &te);
       CK(te, "complex-k amplitude table");
     }
-    for (int r = 0; r < nrhs; ++r) {
-      a.rhs0 = r;
-      CK(launch_grad_d_fused(a, st), "grad D kernel");
+    auto pair_sums = [&](cudaStream_t s) {
+      cudaError_t e = cudaSuccess;
+      for (int r = 0; r < nrhs && e == cudaSuccess; ++r) {
+        a.rhs0 = r;
+        e = launch_grad_d_fused(a, s);
+      }
+      return e;
+    };
+    if (tree) {
+      tr.sx = g->src_x;
+      tr.sy = g->src_y;
+      tr.snx = g->src_nx;
+      tr.sny = g->src_ny;
+      tr.cx = a.cx;
+      tr.cy = a.cy;
+      tr.tx = g->tgt_x;
+      tr.ty = g->tgt_y;
+      tr.hk_tab = a.hk_tab;
+      tr.wd[0] = wd;
+      tree_layout(&tr, base + b_wd + b_ev);
+      tr.nsplit = ns_far;
+      tr.split0 = ns_near;
+      tr.part = part;
+      CK(launch_tree_lists(tr, st), "cluster lists");
+      a.near = tr.near;
+      a.near_cnt = tr.cnt;
+      a.near_stride = tr.M;
+      a.near_q_src = tr.q_src;
+      CK(cudaEventRecord(p->fork, st), "fork event");
+      CK(cudaStreamWaitEvent(p->side, p->fork, 0), "fork");
+      const cudaError_t en = pair_sums(p->side);
+      cudaError_t ef = launch_tree_moments(tr, ck, st);
+      if (ef == cudaSuccess) ef = launch_far_clusters(tr, st);
+      CK(cudaEventRecord(p->join, p->side), "join event");   // (joined also after an error)
+      CK(cudaStreamWaitEvent(st, p->join, 0), "join");
+      CK(en, "grad D kernel");
+      CK(ef, "far clusters");
+    } else {
+      CK(pair_sums(st), "grad D kernel");
     }
     CK(launch_form_finish(nc, 2, ns, nrhs, part, ev, p->d_status, st), "grad D reduction");
     if (p->timing) CK(cudaEventRecord(p->ev1, st), "timing event");

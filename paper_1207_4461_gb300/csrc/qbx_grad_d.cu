@@ -29,47 +29,55 @@
 namespace qbx {
 namespace {
 
-constexpr int kGdThreads = kApplyThreads;   // one centre per thread, 128-centre CTAs
+constexpr int kGdWarps = 4;                  // warps per CTA, which take its sources in turn
 
-// shared memory: source tile x, y, nx, ny, w; columns J (J_0..J_{p+1}),
-// C (J_{m-2}+J_{m+2})/2 and S (J_{m-2}-J_{m+2})/2 for m = 1..p-1 (row m).
+// shared memory: columns J (J_0..J_{p+1}), C (J_{m-2}+J_{m+2})/2 and
+// S (J_{m-2}-J_{m+2})/2 for m = 1..p-1 (row m), 32 centres wide; the warps' sums
 template <typename T>
 __host__ __device__ size_t gd_smem(int p) {
-  return (size_t)kSrcTile * (4 * 8 + 16) + (size_t)((p + 2) + 2 * p) * kGdThreads * sizeof(T);
+  return (size_t)((p + 2) + 2 * p) * 32 * sizeof(T) + 2 * 32 * 16;
 }
 
 template <typename T>
 __device__ __forceinline__ T jl_signed(const T* cJ, int l) {   // J_l for l >= -1 from the column
-  return l >= 0 ? cJ[l * kGdThreads] : rmul(cJ[kGdThreads], -1.0);
+  return l >= 0 ? cJ[l * 32] : rmul(cJ[32], -1.0);
 }
 
+// A CTA owns 32 centres of one side (one per lane); its warps take its share
+// of the sources (all, or the block's near leaves: ApplyArgs::near) in turn.
 template <typename T>
-__global__ void __launch_bounds__(kGdThreads) k_grad_d_fused(ApplyArgs a) {
+__global__ void __launch_bounds__(32 * kGdWarps) k_grad_d_fused(ApplyArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* s_x = reinterpret_cast<double*>(smem_raw);
-  double* s_y = s_x + kSrcTile;
-  double* s_nx = s_y + kSrcTile;
-  double* s_ny = s_nx + kSrcTile;
-  cplx* s_w = reinterpret_cast<cplx*>(s_ny + kSrcTile);
-  T* sJ = reinterpret_cast<T*>(s_w + kSrcTile);
   const int p = a.p;
-  T* sC = sJ + (p + 2) * kGdThreads;
-  T* sS = sC + p * kGdThreads;
+  T* sJ = reinterpret_cast<T*>(smem_raw);
+  T* sC = sJ + (p + 2) * 32;
+  T* sS = sC + p * 32;
+  cplx* s_sum = reinterpret_cast<cplx*>(sS + p * 32);   // [2][32]
 
-  const int tid = threadIdx.x;
-  // work item (centre block, source split), near-field splits first
-  const int nblk = (a.n_ctr + kGdThreads - 1) / kGdThreads;
-  const int cblk = (int)(blockIdx.x % (unsigned)nblk), rank = (int)(blockIdx.x / (unsigned)nblk);
-  const int split = a.near_q_tgt > 0 ? near_first_split(rank, (cblk * kGdThreads + kGdThreads / 2) % a.n_tgt,
-                                                        a.near_q_tgt, a.near_q_src, a.src_per_split, a.nsplit)
-                                     : rank;
-  const int c = cblk * kGdThreads + tid;
-  const bool active = c < a.n_ctr;
-  const int cc = active ? c : a.n_ctr - 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // work item (centre block of one side, source split), near-field splits first
+  const int blks = (a.n_tgt + 31) / 32, nblk = blks * (a.n_ctr / a.n_tgt);
+  const int unit = (int)(blockIdx.x % (unsigned)nblk), rank = (int)(blockIdx.x / (unsigned)nblk);
+  const int side = unit / blks, blk = unit - side * blks;
+  const bool active = blk * 32 + lane < a.n_tgt;
+  const int t = active ? blk * 32 + lane : a.n_tgt - 1;
+  const int c = side * a.n_tgt + t;
+  const int* near = a.near ? a.near + (size_t)blk * a.near_stride : nullptr;
+  int split = rank, v0, v1;
+  if (near) {
+    const long n = (long)a.near_cnt[3 * blk] * a.near_q_src;
+    v0 = (int)(n * rank / a.nsplit);
+    v1 = (int)(n * (rank + 1) / a.nsplit);
+  } else {
+    if (a.near_q_tgt > 0)
+      split = near_first_split(rank, min(blk * 32 + 16, a.n_tgt - 1), a.near_q_tgt, a.near_q_src, a.src_per_split,
+                               a.nsplit);
+    v0 = split * a.src_per_split;
+    v1 = min(a.src.n, v0 + a.src_per_split);
+  }
 
   // ---- per-centre set-up ----
-  const double cx = a.cx[cc], cy = a.cy[cc];
-  const int t = cc % a.n_tgt;
+  const double cx = a.cx[c], cy = a.cy[c];
   double ux = a.tx[t] - cx, uy = a.ty[t] - cy;
   const double r = hypot(ux, uy);
   ux /= r;
@@ -77,39 +85,35 @@ __global__ void __launch_bounds__(kGdThreads) k_grad_d_fused(ApplyArgs a) {
   KW<T> kw;
   kw.init(a.kre, a.kim, a.hk_tab);
   const T kk = kw.kval();
-  T* colJ = sJ + tid;
-  T* colC = sC + tid;
-  T* colS = sS + tid;
-  besselj_column<T>(rmul(kk, r), p + 1, colJ, kGdThreads);
-  for (int m = 1; m <= p - 1; ++m) {
-    const T jm2 = jl_signed(colJ, m - 2), jp2 = colJ[(m + 2) * kGdThreads];
-    colC[m * kGdThreads] = rmul(sadd(jm2, jp2), 0.5);
-    colS[m * kGdThreads] = rmul(sc_sub(jm2, jp2), 0.5);
+  T* colJ = sJ + lane;
+  T* colC = sC + lane;
+  T* colS = sS + lane;
+  if (warp == 0) {
+    besselj_column<T>(rmul(kk, r), p + 1, colJ, 32);
+    for (int m = 1; m <= p - 1; ++m) {
+      const T jm2 = jl_signed(colJ, m - 2), jp2 = colJ[(m + 2) * 32];
+      colC[m * 32] = rmul(sadd(jm2, jp2), 0.5);
+      colS[m * 32] = rmul(sc_sub(jm2, jp2), 0.5);
+    }
   }
-  const T J0 = colJ[0], J2 = colJ[2 * kGdThreads];
+  __syncthreads();
+  const T J0 = colJ[0], J2 = colJ[2 * 32];
   // edge coefficients (halved: the Chebyshev values below are doubled)
-  const T eQ0 = rmul(colJ[p * kGdThreads], 0.5), eQ1 = rmul(colJ[(p + 1) * kGdThreads], 0.5);
-  const T eR0 = rmul(jl_signed(colJ, p - 2), 0.5), eR1 = rmul(colJ[(p - 1) * kGdThreads], 0.5);
+  const T eQ0 = rmul(colJ[p * 32], 0.5), eQ1 = rmul(colJ[(p + 1) * 32], 0.5);
+  const T eR0 = rmul(jl_signed(colJ, p - 2), 0.5), eR1 = rmul(colJ[(p - 1) * 32], 0.5);
 
   cplx accP{0.0, 0.0}, accM{0.0, 0.0};   // sums of the d and dbar brackets
-  const int s_begin = split * a.src_per_split;
-  const int s_end = min(a.src.n, s_begin + a.src_per_split);
-  const cplx* wd = reinterpret_cast<const cplx*>(a.wd[0]);
-  for (int base = s_begin; base < s_end; base += kSrcTile) {
-    const int nt = min(kSrcTile, s_end - base);
-    __syncthreads();
-    for (int i = tid; i < nt; i += kGdThreads) {
-      s_x[i] = a.src.x[base + i];
-      s_y[i] = a.src.y[base + i];
-      s_nx[i] = a.src.nx[base + i];
-      s_ny[i] = a.src.ny[base + i];
-      s_w[i] = wd[(size_t)(base + i) * a.nrhs + a.rhs0];
-    }
-    __syncthreads();
-    if (!active) continue;
-    for (int j = 0; j < nt; ++j) {
-      const double dx = s_x[j] - cx, dy = s_y[j] - cy;
-      const double nx = s_nx[j], ny = s_ny[j];
+  const double2* wd = reinterpret_cast<const double2*>(a.wd[0]) + a.rhs0;
+  {
+    for (int v = v0 + warp; v < v1; v += kGdWarps) {
+      int s_ = v;
+      if (near) {
+        const int i = v / a.near_q_src;
+        s_ = near[i] * a.near_q_src + (v - i * a.near_q_src);
+      }
+      const double dx = __ldg(a.src.x + s_) - cx, dy = __ldg(a.src.y + s_) - cy;
+      const double nx = __ldg(a.src.nx + s_), ny = __ldg(a.src.ny + s_);
+      const double2 w2 = __ldg(wd + (size_t)s_ * a.nrhs);
       const double rho2 = fma(dx, dx, dy * dy);
       double inv, rho, yq;
       kw.geom(rho2, inv, rho, yq);
@@ -119,7 +123,7 @@ __global__ void __launch_bounds__(kGdThreads) k_grad_d_fused(ApplyArgs a) {
       const double bv = fma(ny, dx, -nx * dy) * inv;  // n_s . e_theta
       cplx H0, H1;
       T twoz;
-      kw.hankel_w(rho, inv, yq, s_w[j], H0, H1, twoz);   // w H0, w H1
+      kw.hankel_w(rho, inv, yq, cplx{w2.x, w2.y}, H0, H1, twoz);   // w H0, w H1
       // core sums over m = 1..p-1 with 2 cos(m psi), 2 sin(m psi)
       cplx SQ{0.0, 0.0}, CR{0.0, 0.0}, SR{0.0, 0.0};
       const double tw = 2.0 * cs;
@@ -127,7 +131,7 @@ __global__ void __launch_bounds__(kGdThreads) k_grad_d_fused(ApplyArgs a) {
       T s = twoz;
       double cp = 2.0, cl = tw, sp = 0.0, sl = sn + sn;
       for (int m = 1; m < p; ++m) {
-        const int o = m * kGdThreads;
+        const int o = m * 32;
         madd(SQ, rmul(colJ[o], cl), H);
         madd(CR, rmul(colC[o], cl), H);
         madd(SR, rmul(colS[o], sl), H);
@@ -169,7 +173,19 @@ __global__ void __launch_bounds__(kGdThreads) k_grad_d_fused(ApplyArgs a) {
       cfma(accM, -nu, Qa + iQb);
     }
   }
-  if (!active) return;
+  // the warps' sums in warp order
+  for (int w = 0; w < kGdWarps; ++w) {
+    if (warp == w) {
+      if (w > 0) {
+        accP = s_sum[lane] + accP;
+        accM = s_sum[32 + lane] + accM;
+      }
+      s_sum[lane] = accP;
+      s_sum[32 + lane] = accM;
+    }
+    __syncthreads();
+  }
+  if (warp != kGdWarps - 1 || !active) return;
   // d D = (k^2/2) e^{-i theta_t} P, dbar D = -(k^2/2) e^{i theta_t} M (without the factor i/4)
   const cplx h = 0.5 * sc_mul(to_c(kk), to_c(kk));
   const cplx et{ux, uy};
@@ -189,8 +205,8 @@ cudaError_t launch_gd(const ApplyArgs& a, cudaStream_t st) {
   const size_t smem = gd_smem<T>(a.p);
   cudaError_t e = cudaFuncSetAttribute(k_grad_d_fused<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)((a.n_ctr + kGdThreads - 1) / kGdThreads) * (unsigned)a.nsplit;
-  k_grad_d_fused<T><<<grid, kGdThreads, smem, st>>>(a);
+  const unsigned grid = (unsigned)apply_units(a.n_ctr, a.n_tgt) * (unsigned)a.nsplit;
+  k_grad_d_fused<T><<<grid, 32 * kGdWarps, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -200,7 +216,7 @@ int occ_gd(int p) {
   int n = 0;
   if (cudaFuncSetAttribute(k_grad_d_fused<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_grad_d_fused<T>, kGdThreads, smem) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_grad_d_fused<T>, 32 * kGdWarps, smem) != cudaSuccess) return 0;
   return n;
 }
 

@@ -10,9 +10,16 @@
 // Kernel generation is therefore paid once per pair however many densities
 // there are, and each thread keeps only RG accumulators per component.
 //
-// Items (32 centres x a source range) come either from blockIdx (one curve,
+// Items (32 targets x a source range) come either from blockIdx (one curve,
 // static split of the sources) or from a longest-first item list through an
-// atomic counter (a batch: persistent CTAs, no waits between CTAs).
+// atomic counter (a batch: persistent CTAs, no waits between CTAs).  With a
+// near list (qbx_tree.cu) an item's sources are its share of the block's near
+// leaves; otherwise its range of all sources.
+//
+// Two-sided averages of S, D, S + D and the combined field (merged): a lane
+// holds a target and both its centres, whose kernel values are averaged before
+// phase 2, so the rhs products are paid once per (target, source) instead of
+// once per (centre, source).
 #pragma once
 #include "qbx_apply_impl.cuh"
 
@@ -31,11 +38,12 @@ struct GroupSmem {
   static constexpr bool k3M = kNc <= 2;
   static constexpr int kVal = k3M ? 24 : 16;   // bytes per stored complex value
   static __host__ __device__ int nslots() { return 1 + ((kD || kG) ? 1 : 0) + (kG ? 1 : 0); }
-  static __host__ __device__ size_t bytes(int p) {
-    return 4 * kGrpTile * 8 +                                  // x, y, nx, ny
+  static __host__ __device__ size_t bytes(int p, int nsd) {
+    return 4 * kGrpTile * 8 + kGrpTile * 8 +                   // x, y, nx, ny; source indices
            (size_t)kGrpTile * W * RG * kVal +                   // densities [tile][W RG]
            (size_t)kNc * kGrpTile * kGrpCentres * kVal +        // kernel values [comp][tile][centre]
-           (size_t)nslots() * (p + 2) * kGrpCentres * sizeof(T) +  // coefficient columns
+           (size_t)nsd * nslots() * (p + 2) * kGrpCentres * sizeof(T) +  // coefficient columns per side
+           (size_t)nsd * 6 * kGrpCentres * 8 +                  // centre, direction, radius, 1/radius per side
            16;                                                  // item index
   }
 };
@@ -72,13 +80,13 @@ k_apply_group(GroupArgs a) {
   double* s_ka = reinterpret_cast<double*>(k_raw);
   double* s_kb = s_ka + kNK;
   double* s_ks = s_kb + kNK;
-  T* slot = reinterpret_cast<T*>(k_raw + (size_t)kNK * L::kVal);
-  const int p = a.p;
+  const int p = a.p, nsd = a.nsd;   // nsd = 2: both sides of a target averaged
   const int P2 = (p + 2) * kGrpCentres;
-  T* sJ = slot;
-  T* sL = slot + P2;
-  T* sG = sL + ((kD || kG) ? P2 : 0);
-  int* s_item = reinterpret_cast<int*>(slot + L::nslots() * P2);
+  double* s_geo = reinterpret_cast<double*>(k_raw + (size_t)kNK * L::kVal);   // [side][6][32]
+  int* s_src = reinterpret_cast<int*>(s_geo + nsd * 6 * kGrpCentres);         // [tile] (8 bytes each reserved)
+  T* slot = reinterpret_cast<T*>(s_src + 2 * kGrpTile);                       // [side][slots][p + 2][32]
+  constexpr int kSlots = 1 + ((kD || kG) ? 1 : 0) + (kG ? 1 : 0);
+  int* s_item = reinterpret_cast<int*>(slot + nsd * kSlots * P2);
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool dynamic = a.items != nullptr;
@@ -97,39 +105,51 @@ k_apply_group(GroupArgs a) {
     if (dynamic) {
       item = a.items[it];
     } else {
-      // rank r of the launch takes the 32-centre units' splits near-field
+      // rank r of the launch takes the 32-target blocks' splits near-field
       // first, as the fused apply
+      const int blks = (a.inst0.n_tgt + kGrpCentres - 1) / kGrpCentres;
       item.inst = 0;
       const int unit = it % a.st_units, rank = it / a.st_units;
       const int q_t = a.inst0.n_tgt / a.inst0.M, q_s = a.inst0.n_src / a.inst0.M;
-      item.ctr0 = unit * kGrpCentres;
-      item.split = near_first_split(rank, (unit * kGrpCentres + kGrpCentres / 2) % a.inst0.n_tgt, q_t, q_s,
-                                    a.st_split_len, a.st_nsplit);
+      item.side = unit / blks;
+      item.t0 = (unit - item.side * blks) * kGrpCentres;
+      item.split = a.inst0.near ? rank
+                                : near_first_split(rank, min(item.t0 + kGrpCentres / 2, a.inst0.n_tgt - 1), q_t, q_s,
+                                                   a.st_split_len, a.st_nsplit);
       item.src0 = item.split * a.st_split_len;
       item.src1 = min(a.inst0.n_src, item.src0 + a.st_split_len);
     }
     const GroupInst& in = dynamic ? a.inst[item.inst] : a.inst0;
+    const int blk = item.t0 / kGrpCentres;
+    const int* near = in.near ? in.near + (size_t)blk * in.near_stride : nullptr;
+    if (near) {
+      const long n = (long)in.near_cnt[3 * blk] * in.near_q;
+      item.src0 = (int)(n * item.split / in.nsplit_near);
+      item.src1 = (int)(n * (item.split + 1) / in.nsplit_near);
+    }
 
-    // ---- per-centre set-up (every warp keeps its lane's centre geometry) ----
-    const int c = item.ctr0 + lane;
-    const bool active = c < in.n_ctr;
-    const int cc = active ? c : in.n_ctr - 1;
-    const double cx = in.cx[cc], cy = in.cy[cc];
-    const int t = cc % in.n_tgt;
-    double ux = in.tx[t] - cx, uy = in.ty[t] - cy;
-    const double r = hypot(ux, uy);
-    const double ir = 1.0 / r;
-    ux *= ir;
-    uy *= ir;
-    const double lim2 = LOCAL ? a.eta2 * r * r : INFINITY;
+    // ---- per-target set-up: warp sd forms side sd's geometry and columns ----
+    const bool active = item.t0 + lane < in.n_tgt;
+    const int t = active ? item.t0 + lane : in.n_tgt - 1;
+    const int c = item.side * in.n_tgt + t;   // row of the partial sums
     KW<T> kw;
     kw.init(in.kre, in.kim, in.hk_tab);
     const T kk = kw.kval();
-    T* colJ = sJ + lane;
-    T* colL = sL + lane;
-    T* colG = sG + lane;
     __syncthreads();   // previous item's coefficient columns are no longer read
-    if (warp == 0) {
+    if (warp < nsd) {
+      const int cc = c + warp * in.n_tgt;
+      const double cx = in.cx[cc], cy = in.cy[cc];
+      const double ux = in.tx[t] - cx, uy = in.ty[t] - cy, r = hypot(ux, uy), ir = 1.0 / r;
+      double* g = s_geo + warp * 6 * kGrpCentres + lane;
+      g[0] = cx;
+      g[kGrpCentres] = cy;
+      g[2 * kGrpCentres] = ux * ir;
+      g[3 * kGrpCentres] = uy * ir;
+      g[4 * kGrpCentres] = r;
+      g[5 * kGrpCentres] = ir;
+      T* colJ = slot + warp * kSlots * P2 + lane;
+      T* colL = colJ + P2;
+      T* colG = colL + P2;
       besselj_column<T>(rmul(kk, r), p + 1, colJ, kGrpCentres);
       for (int l = 0; l <= p; ++l) {
         const T jl = colJ[l * kGrpCentres];
@@ -147,8 +167,6 @@ k_apply_group(GroupArgs a) {
       }
     }
     __syncthreads();
-    const T J0 = colJ[0];
-    const T kneg_j0 = rmul(sc_mul(kk, J0), -1.0);
     const cplx* wd = reinterpret_cast<const cplx*>(in.wd);
 
     for (int r0 = 0; r0 < a.nrhs; r0 += kRP) {
@@ -166,17 +184,25 @@ k_apply_group(GroupArgs a) {
       for (int base = item.src0; base < item.src1; base += kGrpTile) {
         const int nt = min(kGrpTile, item.src1 - base);
         __syncthreads();   // previous tile's values consumed
+        auto source = [&](int v) {   // node index of the v-th source
+          if (!near) return v;
+          const int i = v / in.near_q;
+          return near[i] * in.near_q + (v - i * in.near_q);
+        };
         for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-          s_x[i] = in.sx[base + i];
-          s_y[i] = in.sy[base + i];
+          const int s = source(base + i);
+          s_src[i] = s;
+          s_x[i] = in.sx[s];
+          s_y[i] = in.sy[s];
           if (kD) {
-            s_nx[i] = in.snx[base + i];
-            s_ny[i] = in.sny[base + i];
+            s_nx[i] = in.snx[s];
+            s_ny[i] = in.sny[s];
           }
         }
+        __syncthreads();
         for (int i = threadIdx.x; i < kGrpTile * kRP; i += blockDim.x) {
           const int s = i / kRP, rr = i - s * kRP;
-          const cplx v = (s < nt && r0 + rr < a.nrhs) ? wd[(size_t)(base + s) * a.nrhs + r0 + rr] : cplx{0.0, 0.0};
+          const cplx v = (s < nt && r0 + rr < a.nrhs) ? wd[(size_t)s_src[s] * a.nrhs + r0 + rr] : cplx{0.0, 0.0};
           if constexpr (k3M) {
             s_wa[i] = v.re;
             s_wb[i] = v.im;
@@ -188,18 +214,34 @@ k_apply_group(GroupArgs a) {
         __syncthreads();
         // ---- phase 1: kernel values of this warp's sources ----
         for (int j = warp; j < nt; j += W) {
-          const double dx = s_x[j] - cx, dy = s_y[j] - cy;
           double nx = 0.0, ny = 0.0;
           if (kD) {
             nx = s_nx[j];
             ny = s_ny[j];
           }
-          cplx GS, K, GA, GB, EX, EY;
-          if (LOCAL && fma(dx, dx, dy * dy) >= lim2) {   // near-only QBX: a distant source
-            pair_direct<PK, T>(kw, kk, r * ux - dx, r * uy - dy, nx, ny, ux, uy, r, GS, K, GA, GB);
-          } else {
-            pair_kernels<PK, T, kGrpCentres>(kw, kk, J0, kneg_j0, colJ, colL, colG, p, dx, dy, nx, ny, ux,
-                                             uy, ir, GS, K, GA, GB, EX, EY);
+          cplx GS, K, GA, GB, EX, EY, GS1, K1;
+          for (int sd = 0; sd < nsd; ++sd) {
+            const double* g = s_geo + sd * 6 * kGrpCentres + lane;
+            const T* colJ = slot + sd * kSlots * P2 + lane;
+            const T* colL = colJ + P2;
+            const T* colG = colL + P2;
+            const double dx = s_x[j] - g[0], dy = s_y[j] - g[kGrpCentres];
+            const double ux = g[2 * kGrpCentres], uy = g[3 * kGrpCentres], r = g[4 * kGrpCentres];
+            const T J0 = colJ[0];
+            if (sd > 0) {
+              GS1 = GS;
+              K1 = K;
+            }
+            if (LOCAL && fma(dx, dx, dy * dy) >= a.eta2 * r * r) {   // near-only QBX: a distant source
+              pair_direct<PK, T>(kw, kk, r * ux - dx, r * uy - dy, nx, ny, ux, uy, r, GS, K, GA, GB);
+            } else {
+              pair_kernels<PK, T, kGrpCentres>(kw, kk, J0, rmul(sc_mul(kk, J0), -1.0), colJ, colL, colG, p, dx, dy, nx,
+                                               ny, ux, uy, g[5 * kGrpCentres], GS, K, GA, GB, EX, EY);
+            }
+            if (sd > 0) {   // the two sides' average
+              if (kS) GS = 0.5 * (GS1 + GS);
+              if (kD) K = 0.5 * (K1 + K);
+            }
           }
           auto put = [&](int q, cplx v) {
             const int idx = (q * kGrpTile + j) * kGrpCentres + lane;
@@ -264,7 +306,7 @@ k_apply_group(GroupArgs a) {
       // ---- raw sums of this item (grad S already turned into x, y) ----
       if (active) {
         cplx* part = reinterpret_cast<cplx*>(in.part);
-        const size_t row = ((size_t)item.split * in.n_ctr + c) * kNc;
+        const size_t row = ((size_t)item.split * in.n_row + c) * kNc;
 #pragma unroll
         for (int g = 0; g < RG; ++g) {
           const int rr = r0 + warp * RG + g;
@@ -283,6 +325,8 @@ k_apply_group(GroupArgs a) {
             ++q;
           }
           if (kG) {
+            const double ux = s_geo[2 * kGrpCentres + lane], uy = s_geo[3 * kGrpCentres + lane];
+            const double ir = s_geo[5 * kGrpCentres + lane];
             const cplx kA = smul(kk, acc[q][g]);
             const cplx Bi = acc[q + 1][g] * (2.0 * ir);
             part[(row + q) * a.nrhs + rr] = kA * ux + Bi * uy;
@@ -297,7 +341,7 @@ k_apply_group(GroupArgs a) {
 
 template <int OPS, typename T, int RG, bool LOCAL = false, int W = kGrpWarps>
 static cudaError_t launch_group_t(const GroupArgs& a, int grid, cudaStream_t st) {
-  const size_t smem = GroupSmem<OPS, T, RG, W>::bytes(a.p);
+  const size_t smem = GroupSmem<OPS, T, RG, W>::bytes(a.p, a.nsd);
   auto kern = k_apply_group<OPS, T, RG, LOCAL, W>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -339,15 +383,15 @@ static cudaError_t launch_group_any(const GroupArgs& a, int rg, int grid, cudaSt
 }
 
 template <typename T, bool LOCAL = false>
-static int group_occupancy_any(int ops, int p, int rg) {
+static int group_occupancy_any(int ops, int p, int rg, int nsd) {
   int n = 0;
   if constexpr (!LOCAL) {
     if (rg == kGrpRhsWide) {
 #define X(O, TT, R)                                                                                               \
   cudaFuncSetAttribute(k_apply_group<O, TT, R, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
-                       (int)GroupSmem<O, TT, R, 8>::bytes(p));                                                   \
+                       (int)GroupSmem<O, TT, R, 8>::bytes(p, nsd));                                                   \
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_apply_group<O, TT, R, false, 8>, kGrpCentres * 8,          \
-                                                GroupSmem<O, TT, R, 8>::bytes(p));                               \
+                                                GroupSmem<O, TT, R, 8>::bytes(p, nsd));                               \
   return n
       QBX_GROUP_OPS(X, T, 8)
 #undef X
@@ -356,9 +400,9 @@ static int group_occupancy_any(int ops, int p, int rg) {
   }
 #define X(O, TT, R)                                                                                         \
   cudaFuncSetAttribute(k_apply_group<O, TT, R, LOCAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
-                       (int)GroupSmem<O, TT, R>::bytes(p));                                                 \
+                       (int)GroupSmem<O, TT, R>::bytes(p, nsd));                                                 \
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_apply_group<O, TT, R, LOCAL>, kGrpCentres * kGrpWarps, \
-                                                GroupSmem<O, TT, R>::bytes(p));                             \
+                                                GroupSmem<O, TT, R>::bytes(p, nsd));                             \
   return n
   if (rg == 8) {
     QBX_GROUP_OPS(X, T, 8)
@@ -369,27 +413,15 @@ static int group_occupancy_any(int ops, int p, int rg) {
   return 0;
 }
 
-template <typename T, bool LOCAL = false>
-static const void* group_ptr_any(int ops, int rg) {
-#define X(O, TT, R) return (const void*)k_apply_group<O, TT, R, LOCAL>
-  if (rg == 8) {
-    QBX_GROUP_OPS(X, T, 8)
-  } else {
-    QBX_GROUP_OPS(X, T, 2)
-  }
-#undef X
-  return nullptr;
-}
-
 template <typename T>
-static size_t group_smem_any(int ops, int p, int rg) {
+static size_t group_smem_any(int ops, int p, int rg, int nsd) {
   if (rg == kGrpRhsWide) {
-#define X(O, TT, R) return GroupSmem<O, TT, R, 8>::bytes(p)
+#define X(O, TT, R) return GroupSmem<O, TT, R, 8>::bytes(p, nsd)
     QBX_GROUP_OPS(X, T, 8)
 #undef X
     return 0;
   }
-#define X(O, TT, R) return GroupSmem<O, TT, R>::bytes(p)
+#define X(O, TT, R) return GroupSmem<O, TT, R>::bytes(p, nsd)
   if (rg == 8) {
     QBX_GROUP_OPS(X, T, 8)
   } else {

@@ -183,23 +183,29 @@ constexpr int kGrpTile = 32;      // sources per shared-memory tile
 struct GroupInst {
   double kre, kim;
   int n_src, n_tgt, n_ctr;        // n_ctr: centres of the side set
-  int side, nsplit, M;
+  int n_row;                      // rows of the partial sums: n_ctr, or n_tgt with both sides merged
+  int side, nsplit, M;            // nsplit: partial sums of all kernels
+  int nsplit_near;                // of the pair kernel
+  const int *near, *near_cnt;     // near leaves per 32-target block, as ApplyArgs::near; null: all sources
+  int near_stride, near_q;        // list stride, sources per leaf
   const double *sx, *sy, *snx, *sny, *sw;
   const double *cx, *cy;          // centres of the side set
   const double *tx, *ty, *tnx, *tny;
   const void* wd;                 // [n_src][nrhs] oversampled weighted density
   const void* dens;               // [n_tgt][nrhs] density on the target grid (jump terms)
-  void* part;                     // [nsplit][n_ctr][ncomp][nrhs] raw sums
+  void* part;                     // [nsplit][n_row][ncomp][nrhs] raw sums
   void* out[3];                   // per operator (S, D, grad S) outputs, for the finish
   const double* hk_tab;           // complex k: the amplitude table of this curve's k, or null
 };
-// A work item: 32 centres from ctr0 of instance inst, sources [src0, src1),
-// partial-sum slot `split`.
+// A work item: 32 targets from t0 of instance inst, one side's centres (both
+// when merged: side 0), sources [src0, src1) or the split's share of the near
+// leaves, partial-sum slot `split`.
 struct GroupItem {
-  int inst, ctr0, split, src0, src1;
+  int inst, t0, side, split, src0, src1;
 };
 struct GroupArgs {
   int ops, p, nrhs;
+  int nsd;                        // 2: both sides of a target averaged per pair (S, D, S + D, D - i eta S), else 1
   const GroupInst* inst;          // dynamic mode: instance table
   GroupInst inst0;                // static mode: the one instance
   int n_items;
@@ -212,21 +218,19 @@ struct GroupArgs {
 };
 cudaError_t launch_group_real(const GroupArgs& a, int rg, int grid, cudaStream_t st);
 cudaError_t launch_group_cplx(const GroupArgs& a, int rg, int grid, cudaStream_t st);
-size_t group_smem_real(int ops, int p, int rg);
-size_t group_smem_cplx(int ops, int p, int rg);
-int group_occupancy_real(int ops, int p, int rg);
-int group_occupancy_cplx(int ops, int p, int rg);
-const void* group_ptr_real(int ops, int rg);
-const void* group_ptr_cplx(int ops, int rg);
+size_t group_smem_real(int ops, int p, int rg, int nsd);
+size_t group_smem_cplx(int ops, int p, int rg, int nsd);
+int group_occupancy_real(int ops, int p, int rg, int nsd);
+int group_occupancy_cplx(int ops, int p, int rg, int nsd);
 // near-only instances of the group kernel (GroupArgs::eta2 > 0)
 cudaError_t launch_group_local(const GroupArgs& a, bool ck, int rg, int grid, cudaStream_t st);
-int group_occupancy_local(int ops, bool ck, int p, int rg);
-const void* group_ptr_local(int ops, bool ck, int rg);
+int group_occupancy_local(int ops, bool ck, int p, int rg, int nsd);
 
 }  // namespace qbx
 
 namespace qbx {
 
+struct TreeArgs;
 // ---- adjoint (transposed sweep) -------------------------------------------
 struct AdjArgs {
   int ops, p, nrhs;
@@ -238,12 +242,18 @@ struct AdjArgs {
   void* coef;            // [n_ctr][nslots][p+2] coefficient columns (workspace)
   double* cgeo;          // [n_ctr][3] target direction and 1/r (workspace)
   int nsplit, ctr_per_split;
-  void* part;            // [nsplit][n_src][1][nrhs]
+  const int *near, *near_cnt;   // near leaves of every 32-source block (near_q targets each, all their centres);
+  int near_stride, near_q;      // null: every centre
+  void* part;            // [nsplit][n_src][ncomp][nrhs]
   const double* hk_tab;  // complex k: the amplitude table of this k's ray, or null
 };
 cudaError_t launch_adjoint_real(const AdjArgs& a, cudaStream_t st);
 cudaError_t launch_adjoint_cplx(const AdjArgs& a, cudaStream_t st);
+// the plan's side stream and the events that fork it from and join it to a call's stream
+void host_plan_side(const qbx_plan* plan, cudaStream_t* side, cudaEvent_t* fork, cudaEvent_t* join);
 void host_plan_workspace(const qbx_plan* plan, void** ws, size_t* bytes, int* num_sms, int** status);
+cudaError_t adjoint_sums(AdjArgs& a, TreeArgs* tr, qbx_plan* plan, const qbx_geom* g, int c0, int nc, qbx_c64 k,
+                         int fops, int nd, int mode, int num_sms, char* tree_base, cudaStream_t st);
 // The plan's amplitude table for complex k (made on st when k changes), or
 // null for real k.
 const double* host_plan_hk_table(qbx_plan* plan, qbx_c64 k, cudaStream_t st, cudaError_t* err);
@@ -263,16 +273,22 @@ constexpr int kTreeMinPanels = 16;   // fewer panels: every source pair by pair 
 constexpr int kTreeLevels = 16;
 constexpr int kTreeSets = 4;
 // what a moment set is made of: the density itself, or dipoles along n_s, x, y
-enum { kSetMono = 0, kSetNormal = 1, kSetX = 2, kSetY = 3 };
+enum { kSetMono = 0, kSetNormal = 1, kSetX = 2, kSetY = 3, kSetCombined = 4,
+       kSetQuadX = 5, kSetQuadY = 6 };   // (the dipoles' derivatives along x, y)
 
 struct TreeArgs {
+  const TreeArgs* inst;       // a batch: one entry per curve (device memory), blockIdx.z the curve; else null
   double kre, kim;
   int p;                      // order of the centres' expansions
   int pl;                     // orders of the list entries (p, or kTreeLocal for near-only QBX)
-  int nd;                     // 1 if a derivative is taken anywhere (D, grad S), else 0
+  int nd;                     // derivatives taken on one side of a kernel (D, grad S: 1)
   double eta;                 // near-only QBX (> 0)
   int M, q_src, n_src;        // leaves (halves of panels, or panels), sources per leaf, sources
   const double *sx, *sy, *snx, *sny;
+  // adjoint sweeps: the nodes hold the discs of n_ctr_n centres (dcx, dcy) of
+  // the targets (sx, sy), and the blocks evaluation points (tx = cx)
+  int discs, n_ctr_n;
+  const double *dcx, *dcy;
   int n_tgt, n_ctr;           // n_ctr = n_tgt or 2 n_tgt centres
   const double *cx, *cy, *tx, *ty;
   const double* hk_tab;
@@ -289,10 +305,13 @@ struct TreeArgs {
   int kind[kTreeSets];
   int slot[kTreeSets];        // which of the call's densities
   const void* wd[kTreeSets];  // [n_src][nrhs] weighted densities
-  void* mom;                  // [lev][M][nset nrhs][kTreeP + 2][2] leaf contributions
+  int up;                     // many columns: the leaves' coefficients, carried upward node by node;
+                              // few: leaf contributions to every level
+  double eta_re, eta_im;      // kSetCombined: dipoles - i eta density
+  void* mom;                  // few columns: [lev][M][nset nrhs][kTreeP + 2][2] leaf contributions
   int ncset;                  // coefficient column sets: a moment set, or its x, y derivative
   int base[2 * kTreeSets], shift[2 * kTreeSets], plain[kTreeSets];
-  void* coef;                 // [nodes + n_blk][kTreeP + 1][ncset nrhs][2] coefficients
+  void* coef;                 // [nodes + n_blk][kTreeP + 2][ncset nrhs][2] coefficients
   // evaluation (launch_far_clusters)
   int ops;                    // OPB_* bits
   int set_s, set_d, set_g, set_gx, set_x;   // column sets (grad S: the density's, its x derivative; y after x)
@@ -306,11 +325,28 @@ int tree_levels(int panels, int q_src, TreeArgs* a);
 // device bytes of the arrays of `a` (lev, off, n_blk, nset, nrhs set); with
 // base != null also their addresses
 size_t tree_layout(TreeArgs* a, char* base);
-cudaError_t launch_tree_lists(const TreeArgs& a, cudaStream_t st);    // nodes, block lists
-cudaError_t launch_tree_moments(const TreeArgs& a, cudaStream_t st);  // moments, coefficients, local expansions
+// (several curves: a.inst and n_inst; a then holds the largest M, n_blk, node
+// count and levels over the curves)
+cudaError_t launch_tree_lists(const TreeArgs& a, cudaStream_t st, int n_inst = 1);    // nodes, block lists
+// moments, coefficients, local expansions; ck: complex k
+cudaError_t launch_tree_moments(const TreeArgs& a, bool ck, cudaStream_t st, int n_inst = 1);
 cudaError_t launch_far_clusters(TreeArgs a, cudaStream_t st);         // partial sums of the far nodes
 bool far_clusters_fit(const TreeArgs& a);                             // whether their kernel can hold the orders
+// the same for many columns of S, D or the combined field (both sides of a
+// target averaged when n_ctr = 2 n_tgt)
+cudaError_t launch_far_group(const TreeArgs& a, bool ck, cudaStream_t st, int n_inst = 1);
+bool far_group_fit(const TreeArgs& a, bool ck, int nsd);
+// adjoint sweeps: the tree over the discs of the centres, evaluated at the
+// source nodes (columns by ops: value, gradient, second derivatives), its
+// arrays and far sums at `base`; returns their bytes (base null: only those),
+// 0 where no clusters are formed
+size_t adj_tree_setup(TreeArgs* t, const qbx_geom* g, int c0, int nc, qbx_c64 k, int p, int ops, int nd, int nrhs,
+                      const double* hk_tab, const void* gc, int num_sms, char* base);
+cudaError_t launch_adj_far(const TreeArgs& a, int mode, const double* snx, const double* sny, void* row,
+                           cudaStream_t st);
 // moment and column sets of a->ops, the densities of S, D, grad S (and X) in slots `slot`
 void tree_columns(TreeArgs* a, const int slot[3]);
+void tree_columns_grad_d(TreeArgs* a, bool sources);   // grad D (OPB_G); with sources also the dipoles' derivatives (OPB_X)
+void tree_columns_discs(TreeArgs* a);                  // adjoint: value (S), gradient (G), d_xx and d_xy (X)
 
 }  // namespace qbx

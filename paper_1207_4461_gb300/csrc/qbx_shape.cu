@@ -269,8 +269,7 @@ __device__ __forceinline__ void dshape_pair(const KW<T>& kw, const T kk, const T
   Ty = mul_i(0.5 * (dxK - dbxK));
 }
 
-constexpr int kDsTile = 64;     // sources per shared-memory tile (forward), centres (transposed)
-constexpr int kDsNR = 4;        // rhs per pass
+constexpr int kDsWarps = 4;     // warps per CTA of 32 centres (forward) or sources (transposed)
 constexpr int kNcFwdD = 4, kNcAdjD = 5;
 
 struct DsArgs {
@@ -285,8 +284,28 @@ struct DsArgs {
   void* coef;         // [n_ctr][p+2] J_0..J_{p+1} (written by k_dshape_columns)
   double* cgeo;       // [n_ctr][4] ux, uy, r, unused (written by k_dshape_columns)
   int nsplit, per_split;
+  // near leaves of every 32-target (forward: near_q sources each) or 32-source
+  // block (transposed: near_q targets each, all their centres); null: all
+  const int *near, *near_cnt;
+  int near_stride, near_q;
   cplx* part;
 };
+
+// the warps' sums in warp order; the last warp's lanes return true with the totals
+template <int N>
+__device__ __forceinline__ bool warps_total(cplx (&acc)[N], cplx* s_sum, int lane, int warp) {
+  for (int w = 0; w < kDsWarps; ++w) {
+    __syncthreads();
+    if (warp == w) {
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        if (w > 0) acc[q] = s_sum[q * 32 + lane] + acc[q];
+        s_sum[q * 32 + lane] = acc[q];
+      }
+    }
+  }
+  return warp == kDsWarps - 1;
+}
 
 template <typename T>
 __global__ void k_dshape_columns(DsArgs a) {
@@ -305,140 +324,117 @@ __global__ void k_dshape_columns(DsArgs a) {
   geo[3] = 0.0;
 }
 
-// lanes = centres: F = sum_s (w mu)_s grad_x K_D, E = sum_s (w mu)_s grad_y K_D
-template <typename T>
-__global__ void __launch_bounds__(128) k_dshape_fwd(DsArgs a) {
+// lanes = centres of one side: F = sum_s (w mu)_s grad_x K_D, E = sum_s (w mu)_s
+// grad_y K_D; the four warps take the sources in turn
+template <typename T, int NR>
+__global__ void __launch_bounds__(32 * kDsWarps) k_dshape_fwd(DsArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* s_x = reinterpret_cast<double*>(smem_raw);
-  double* s_y = s_x + kDsTile;
-  double* s_nx = s_y + kDsTile;
-  double* s_ny = s_nx + kDsTile;
-  cplx* s_w = reinterpret_cast<cplx*>(s_ny + kDsTile);            // [tile][kDsNR]
-  T* s_col = reinterpret_cast<T*>(s_w + kDsTile * kDsNR);          // [p+2][128]
-  const int nblk = (a.n_ctr + 127) / 128;
-  const int cb = blockIdx.x % nblk, split = blockIdx.x / nblk;
-  const int c = cb * 128 + threadIdx.x;
-  const bool active = c < a.n_ctr;
-  const int cc = active ? c : a.n_ctr - 1;
+  T* s_col = reinterpret_cast<T*>(smem_raw);                                     // [p+2][32]
+  cplx* s_sum = reinterpret_cast<cplx*>(smem_raw + (size_t)(a.p + 2) * 32 * sizeof(T));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int blks = (a.n_tgt + 31) / 32, units = blks * (a.n_ctr / a.n_tgt);
+  const int unit = blockIdx.x % units, split = blockIdx.x / units;
+  const int side = unit / blks, blk = unit - side * blks;
+  const bool active = blk * 32 + lane < a.n_tgt;
+  const int c = side * a.n_tgt + (active ? blk * 32 + lane : a.n_tgt - 1);
+  const int* near = a.near ? a.near + (size_t)blk * a.near_stride : nullptr;
+  int s0 = split * a.per_split, s1 = min(a.n_src, s0 + a.per_split);
+  if (near) {
+    const long n = (long)a.near_cnt[3 * blk] * a.near_q;
+    s0 = (int)(n * split / a.nsplit);
+    s1 = (int)(n * (split + 1) / a.nsplit);
+  }
   KW<T> kw;
   kw.init(a.kre, a.kim, a.hk_tab);
   const T kk = kw.kval();
-  const T* coef = reinterpret_cast<const T*>(a.coef) + (size_t)cc * (a.p + 2);
-  for (int l = 0; l <= a.p + 1; ++l) s_col[l * 128 + threadIdx.x] = coef[l];
-  const double cx = a.cx[cc], cy = a.cy[cc];
-  const double ux = a.cgeo[4 * (size_t)cc], uy = a.cgeo[4 * (size_t)cc + 1];
-  cplx acc[kNcFwdD][kDsNR];
+  const T* coef = reinterpret_cast<const T*>(a.coef) + (size_t)c * (a.p + 2);
+  for (int l = warp; l <= a.p + 1; l += kDsWarps) s_col[l * 32 + lane] = coef[l];
+  __syncthreads();
+  const double cx = a.cx[c], cy = a.cy[c];
+  const double ux = a.cgeo[4 * (size_t)c], uy = a.cgeo[4 * (size_t)c + 1];
+  cplx acc[kNcFwdD * NR];
 #pragma unroll
-  for (int q = 0; q < kNcFwdD; ++q)
-#pragma unroll
-    for (int r = 0; r < kDsNR; ++r) acc[q][r] = cplx{0.0, 0.0};
-  const int s0 = split * a.per_split, s1 = min(a.n_src, s0 + a.per_split);
-  for (int base = s0; base < s1; base += kDsTile) {
-    const int nt = min(kDsTile, s1 - base);
-    __syncthreads();
-    for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-      s_x[i] = a.sx[base + i];
-      s_y[i] = a.sy[base + i];
-      s_nx[i] = a.snx[base + i];
-      s_ny[i] = a.sny[base + i];
+  for (int q = 0; q < kNcFwdD * NR; ++q) acc[q] = cplx{0.0, 0.0};
+  for (int v = s0 + warp; v < s1; v += kDsWarps) {
+    int s = v;
+    if (near) {
+      const int i = v / a.near_q;
+      s = near[i] * a.near_q + (v - i * a.near_q);
     }
-    for (int i = threadIdx.x; i < nt * kDsNR; i += blockDim.x) {
-      const int j = i / kDsNR, r = i - j * kDsNR;
-      s_w[i] = r < a.nr ? a.wd[(size_t)(base + j) * a.nrhs + a.rhs0 + r] : cplx{0.0, 0.0};
-    }
-    __syncthreads();
-    if (!active) continue;
-    for (int j = 0; j < nt; ++j) {
-      cplx K, Gx, Gy, Sx, Sy, Tx, Ty;
-      dshape_pair<T>(kw, kk, s_col + threadIdx.x, 128, a.p, s_x[j] - cx, s_y[j] - cy, s_nx[j], s_ny[j], ux, uy,
-                     K, Gx, Gy, Sx, Sy, Tx, Ty);
+    cplx K, Gx, Gy, Sx, Sy, Tx, Ty;
+    dshape_pair<T>(kw, kk, s_col + lane, 32, a.p, __ldg(a.sx + s) - cx, __ldg(a.sy + s) - cy, __ldg(a.snx + s),
+                   __ldg(a.sny + s), ux, uy, K, Gx, Gy, Sx, Sy, Tx, Ty);
 #pragma unroll
-      for (int r = 0; r < kDsNR; ++r) {
-        const cplx w = s_w[j * kDsNR + r];
-        cfma(acc[0][r], w, Tx);
-        cfma(acc[1][r], w, Ty);
-        cfma(acc[2][r], w, Sx);
-        cfma(acc[3][r], w, Sy);
-      }
+    for (int r = 0; r < NR; ++r) {
+      if (r >= a.nr) break;
+      const cplx w = a.wd[(size_t)s * a.nrhs + a.rhs0 + r];
+      cfma(acc[r], w, Tx);
+      cfma(acc[NR + r], w, Ty);
+      cfma(acc[2 * NR + r], w, Sx);
+      cfma(acc[3 * NR + r], w, Sy);
     }
   }
-  if (!active) return;
+  if (!warps_total(acc, s_sum, lane, warp) || !active) return;
   const size_t row = ((size_t)split * a.n_ctr + c) * kNcFwdD;
 #pragma unroll
-  for (int r = 0; r < kDsNR; ++r) {
+  for (int r = 0; r < NR; ++r) {
     if (r >= a.nr) break;
 #pragma unroll
-    for (int q = 0; q < kNcFwdD; ++q) a.part[(row + q) * a.nrhs + a.rhs0 + r] = acc[q][r];
+    for (int q = 0; q < kNcFwdD; ++q) a.part[(row + q) * a.nrhs + a.rhs0 + r] = acc[q * NR + r];
   }
 }
 
 // lanes = sources: Psi = sum_c g_c conj(K_D), Xi = sum_c g_c conj(grad_y K_D),
-// N = sum_c g_c conj(grad_y G)
-template <typename T>
-__global__ void __launch_bounds__(128) k_dshape_adj(DsArgs a) {
+// N = sum_c g_c conj(grad_y G); the four warps take the centres in turn
+template <typename T, int NR>
+__global__ void __launch_bounds__(32 * kDsWarps) k_dshape_adj(DsArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* s_cx = reinterpret_cast<double*>(smem_raw);
-  double* s_cy = s_cx + kDsTile;
-  double* s_ux = s_cy + kDsTile;
-  double* s_uy = s_ux + kDsTile;
-  cplx* s_g = reinterpret_cast<cplx*>(s_uy + kDsTile);              // [tile][kDsNR]
-  T* s_col = reinterpret_cast<T*>(s_g + kDsTile * kDsNR);            // [p+2][tile]
-  const int nblk = (a.n_src + 127) / 128;
-  const int sb = blockIdx.x % nblk, split = blockIdx.x / nblk;
-  const int s = sb * 128 + threadIdx.x;
-  const bool active = s < a.n_src;
-  const int ss = active ? s : a.n_src - 1;
+  cplx* s_sum = reinterpret_cast<cplx*>(smem_raw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int blks = (a.n_src + 31) / 32;
+  const int blk = blockIdx.x % blks, split = blockIdx.x / blks;
+  const bool active = blk * 32 + lane < a.n_src;
+  const int s = active ? blk * 32 + lane : a.n_src - 1;
+  const int per = a.near ? a.near_q * (a.n_ctr / a.n_tgt) : 1;   // centres of a leaf
+  const int* near = a.near ? a.near + (size_t)blk * a.near_stride : nullptr;
+  int c0 = split * a.per_split, c1 = min(a.n_ctr, c0 + a.per_split);
+  if (near) {
+    const long n = (long)a.near_cnt[3 * blk] * per;
+    c0 = (int)(n * split / a.nsplit);
+    c1 = (int)(n * (split + 1) / a.nsplit);
+  }
   KW<T> kw;
   kw.init(a.kre, a.kim, a.hk_tab);
   const T kk = kw.kval();
-  const double sx = a.sx[ss], sy = a.sy[ss], snx = a.snx[ss], sny = a.sny[ss];
-  const int P2 = a.p + 2;
-  cplx acc[kNcAdjD][kDsNR];
+  const double sx = a.sx[s], sy = a.sy[s], snx = a.snx[s], sny = a.sny[s];
+  cplx acc[kNcAdjD * NR];
 #pragma unroll
-  for (int q = 0; q < kNcAdjD; ++q)
-#pragma unroll
-    for (int r = 0; r < kDsNR; ++r) acc[q][r] = cplx{0.0, 0.0};
-  const int c0 = split * a.per_split, c1 = min(a.n_ctr, c0 + a.per_split);
-  for (int base = c0; base < c1; base += kDsTile) {
-    const int nt = min(kDsTile, c1 - base);
-    __syncthreads();
-    for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-      s_cx[i] = a.cx[base + i];
-      s_cy[i] = a.cy[base + i];
-      s_ux[i] = a.cgeo[4 * (size_t)(base + i)];
-      s_uy[i] = a.cgeo[4 * (size_t)(base + i) + 1];
+  for (int q = 0; q < kNcAdjD * NR; ++q) acc[q] = cplx{0.0, 0.0};
+  for (int v = c0 + warp; v < c1; v += kDsWarps) {
+    int c = v;
+    if (near) {
+      const int leaf = v / per, rem = v - leaf * per, sd = rem / a.near_q;
+      c = sd * a.n_tgt + near[leaf] * a.near_q + rem - sd * a.near_q;
     }
-    for (int i = threadIdx.x; i < nt * kDsNR; i += blockDim.x) {
-      const int j = i / kDsNR, r = i - j * kDsNR;
-      s_g[i] = r < a.nr ? a.gc[(size_t)(base + j) * a.nrhs + a.rhs0 + r] : cplx{0.0, 0.0};
-    }
-    const T* coef = reinterpret_cast<const T*>(a.coef);
-    for (int i = threadIdx.x; i < nt * P2; i += blockDim.x) {
-      const int j = i / P2, l = i - j * P2;
-      s_col[l * kDsTile + j] = coef[(size_t)(base + j) * P2 + l];
-    }
-    __syncthreads();
-    if (!active) continue;
-    for (int j = 0; j < nt; ++j) {
-      cplx K, Gx, Gy, Sx, Sy, Tx, Ty;
-      dshape_pair<T>(kw, kk, s_col + j, kDsTile, a.p, sx - s_cx[j], sy - s_cy[j], snx, sny, s_ux[j], s_uy[j], K,
-                     Gx, Gy, Sx, Sy, Tx, Ty);
-      const cplx v[kNcAdjD] = {conj(K), conj(Sx), conj(Sy), conj(Gx), conj(Gy)};
+    cplx K, Gx, Gy, Sx, Sy, Tx, Ty;
+    dshape_pair<T>(kw, kk, reinterpret_cast<const T*>(a.coef) + (size_t)c * (a.p + 2), 1, a.p, sx - a.cx[c],
+                   sy - a.cy[c], snx, sny, a.cgeo[4 * (size_t)c], a.cgeo[4 * (size_t)c + 1], K, Gx, Gy, Sx, Sy, Tx, Ty);
+    const cplx k5[kNcAdjD] = {conj(K), conj(Sx), conj(Sy), conj(Gx), conj(Gy)};
 #pragma unroll
-      for (int r = 0; r < kDsNR; ++r) {
-        const cplx g = s_g[j * kDsNR + r];
+    for (int r = 0; r < NR; ++r) {
+      if (r >= a.nr) break;
+      const cplx g = a.gc[(size_t)c * a.nrhs + a.rhs0 + r];
 #pragma unroll
-        for (int q = 0; q < kNcAdjD; ++q) cfma(acc[q][r], g, v[q]);
-      }
+      for (int q = 0; q < kNcAdjD; ++q) cfma(acc[q * NR + r], g, k5[q]);
     }
   }
-  if (!active) return;
+  if (!warps_total(acc, s_sum, lane, warp) || !active) return;
   const size_t row = ((size_t)split * a.n_src + s) * kNcAdjD;
 #pragma unroll
-  for (int r = 0; r < kDsNR; ++r) {
+  for (int r = 0; r < NR; ++r) {
     if (r >= a.nr) break;
 #pragma unroll
-    for (int q = 0; q < kNcAdjD; ++q) a.part[(row + q) * a.nrhs + a.rhs0 + r] = acc[q][r];
+    for (int q = 0; q < kNcAdjD; ++q) a.part[(row + q) * a.nrhs + a.rhs0 + r] = acc[q * NR + r];
   }
 }
 
@@ -478,21 +474,24 @@ __global__ void k_shape_sources_d(int n_src, int q_src, int nsplit, int nrhs, co
   g_dgam[2 * s + 1] = f * vy - gt * ny / sp;
 }
 
+template <typename T, int NR>
+cudaError_t launch_dshape_nr(const DsArgs& a, bool fwd, cudaStream_t st) {
+  const size_t smem = fwd ? (size_t)(a.p + 2) * 32 * sizeof(T) + kNcFwdD * NR * 32 * 16 : (size_t)kNcAdjD * NR * 32 * 16;
+  auto kern = fwd ? k_dshape_fwd<T, NR> : k_dshape_adj<T, NR>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const unsigned units = fwd ? apply_units(a.n_ctr, a.n_tgt) : (a.n_src + 31) / 32;
+  kern<<<units * (unsigned)a.nsplit, 32 * kDsWarps, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_dshape(const DsArgs& a0, bool fwd, cudaStream_t st) {
   DsArgs a = a0;
-  const size_t col = (size_t)(a.p + 2) * (fwd ? 128 : kDsTile) * sizeof(T);
-  const size_t smem = 4 * kDsTile * 8 + (size_t)kDsTile * kDsNR * 16 + col;
-  auto kern = fwd ? k_dshape_fwd<T> : k_dshape_adj<T>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const int lanes = fwd ? a.n_ctr : a.n_src;
-  const unsigned grid = (unsigned)((lanes + 127) / 128) * (unsigned)a.nsplit;
-  for (int r0 = 0; r0 < a.nrhs; r0 += kDsNR) {
+  for (int r0 = 0; r0 < a.nrhs; r0 += 4) {
     a.rhs0 = r0;
-    a.nr = std::min(kDsNR, a.nrhs - r0);
-    kern<<<grid, 128, smem, st>>>(a);
-    e = cudaGetLastError();
+    a.nr = std::min(4, a.nrhs - r0);
+    const cudaError_t e = a.nr == 1 ? launch_dshape_nr<T, 1>(a, fwd, st) : launch_dshape_nr<T, 4>(a, fwd, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -574,29 +573,98 @@ static int shape_impl(int op, qbx_plan* plan, const qbx_geom* g, int side, qbx_c
   // sweep about six CTAs per SM; both shrink to fit the workspace
   const Layout L0 = layout(g->M, q_tgt, q_src, nc, p, nrhs, ck, 0, 0, nc_adj);
   if (ws_bytes < L0.total + 512) return sfail(QBX_ENOMEM, "workspace too small");
-  const size_t avail = ws_bytes - L0.total - 512;
   const size_t per_fwd = (size_t)nc * kNcFwd * nrhs * 16, per_adj = (size_t)n_src * nc_adj * nrhs * 16;
-  const int occ = opD ? 0
+  // distant pairs of both sweeps through cluster moments (few columns): the
+  // sources' tree for the forward sums, the centres' discs for the transposed
+  TreeArgs tf, ta;
+  const int fops = kOpsFwd, aops = (1 << QBX_OP_S) | (1 << QBX_OP_GRAD_S) | (opD ? 8 : 0);
+  size_t b_tf = 0, b_ta = 0;
+  int ns_far = 0;
+  auto set_fwd_tree = [&](char* at, const void* wdens, const double* tab, void* part, int split0) {
+    tf = TreeArgs{};
+    tf.kre = k.re;
+    tf.kim = k.im;
+    tf.p = tf.pl = p;
+    tf.nd = opD ? 2 : 1;
+    tf.ops = fops;
+    tf.nrhs = nrhs;
+    tf.n_tgt = n_tgt;
+    tf.n_ctr = nc;
+    tf.n_blk = apply_units(n_tgt, n_tgt);
+    tf.sx = g->src_x;
+    tf.sy = g->src_y;
+    tf.snx = g->src_nx;
+    tf.sny = g->src_ny;
+    tf.cx = g->ctr_x + c0;
+    tf.cy = g->ctr_y + c0;
+    tf.tx = g->tgt_x;
+    tf.ty = g->tgt_y;
+    tf.hk_tab = tab;
+    const int none[3] = {0, 0, 0};
+    if (opD) tree_columns_grad_d(&tf, true);
+    else tree_columns(&tf, none);
+    for (int i = 0; i < tf.nset; ++i) tf.wd[i] = wdens;
+    tree_levels(g->M, q_src, &tf);
+    const int units = apply_units(nc, n_tgt);
+    tf.nparts = std::max(1, std::min(4, num_sms * 8 / (units * 16)));
+    tf.nsplit = ns_far = std::max(2, std::min(8, (num_sms * 2 + units - 1) / units));
+    tf.part = part;
+    tf.split0 = split0;
+    return tree_layout(&tf, at);
+  };
+  if (g->M >= kTreeMinPanels && nrhs <= 8) {
+    b_tf = set_fwd_tree(nullptr, nullptr, nullptr, nullptr, 0);
+    if (!far_clusters_fit(tf)) b_tf = 0;
+    if (b_tf) b_ta = adj_tree_setup(&ta, g, c0, nc, k, p, aops, opD ? 2 : 1, nrhs, nullptr, nullptr, num_sms, nullptr);
+    if (!b_ta || ws_bytes < L0.total + 512 + b_tf + b_ta + (size_t)(ns_far + 2) * per_fwd + 2 * per_adj) b_tf = b_ta = 0;
+  }
+  const bool tree = b_tf > 0;
+  if (!tree) ns_far = 0;
+  const size_t avail = ws_bytes - L0.total - 512 - b_tf - b_ta - (tree ? (size_t)ns_far * per_fwd + per_adj : 0);
+  const int occ = opD ? 3
                       : (ck ? apply_occupancy_cplx(kOpsFwd, p, std::min(chunk, nrhs))
                             : apply_occupancy_real(kOpsFwd, p, std::min(chunk, nrhs)));
-  const int units = opD ? (nc + 127) / 128 : apply_units(nc, n_tgt);
-  int ns_fwd = host_choose_split_waves(num_sms, occ, units, n_src, per_fwd, avail / 2);
-  const int tiles = opD ? (n_src + 127) / 128 : (n_src + kGrpCentres - 1) / kGrpCentres;
+  const int units = apply_units(nc, n_tgt);
+  int ns_fwd = host_choose_split_waves(num_sms, occ, units, tree ? std::min(n_src, 16 * q_src) : n_src, per_fwd, avail / 2,
+                                       tree ? 2 : 1);
+  const int tiles = (n_src + kGrpCentres - 1) / kGrpCentres;
   int ns_adj = std::max(1, (num_sms * 6 + tiles - 1) / tiles);
-  ns_adj = std::min(ns_adj, std::max(1, nc / (opD ? kDsTile : kGrpTile)));
+  ns_adj = std::min(ns_adj, std::max(1, (tree ? std::min(nc, 12 * q_tgt * nsides) : nc) / kGrpTile));
   ns_adj = std::min(ns_adj, kMaxSplit);
   ns_adj = (int)std::min<size_t>((size_t)ns_adj, (avail - std::min(avail, (size_t)ns_fwd * per_fwd)) / per_adj);
   if (ns_fwd < 1 || ns_adj < 1) return sfail(QBX_ENOMEM, "workspace too small for the partial sums");
-  const Layout L = layout(g->M, q_tgt, q_src, nc, p, nrhs, ck, ns_fwd, ns_adj, nc_adj);
-  if (L.total > ws_bytes) return sfail(QBX_ENOMEM, "workspace too small");
+  // (rows: the pair kernels' splits, then the far sums)
+  const int nr_fwd = ns_fwd + ns_far, nr_adj = ns_adj + (tree ? 1 : 0);
+  const Layout L = layout(g->M, q_tgt, q_src, nc, p, nrhs, ck, nr_fwd, nr_adj, nc_adj);
+  if (L.total + 512 + b_tf + b_ta > ws_bytes) return sfail(QBX_ENOMEM, "workspace too small");
   cudaStream_t st = (cudaStream_t)stream;
   char* base = (char*)host_align256((size_t)ws);
   void* wd = base + L.wd;
+  char* at_tf = base + host_align256(L.total);
+  char* at_ta = at_tf + b_tf;
+  cudaStream_t side_st;
+  cudaEvent_t ev_fork, ev_join;
+  host_plan_side(plan, &side_st, &ev_fork, &ev_join);
+  // forward sums: pairs(stream) beside the far sums, joined on st
+  auto fwd_sums = [&](auto&& pairs) -> cudaError_t {
+    if (!tree) return pairs(st);
+    cudaError_t x = launch_tree_lists(tf, st);
+    if (x == cudaSuccess) x = cudaEventRecord(ev_fork, st);
+    if (x == cudaSuccess) x = cudaStreamWaitEvent(side_st, ev_fork, 0);
+    if (x != cudaSuccess) return x;
+    x = pairs(side_st);
+    cudaError_t y = launch_tree_moments(tf, ck, st);
+    if (y == cudaSuccess) y = launch_far_clusters(tf, st);
+    cudaError_t z = cudaEventRecord(ev_join, side_st);   // (joined also after an error)
+    if (z == cudaSuccess) z = cudaStreamWaitEvent(st, ev_join, 0);
+    return x != cudaSuccess ? x : y != cudaSuccess ? y : z;
+  };
   // (w sigma)_s
   e = launch_upsample(g->M, q_tgt, q_src, nrhs, P, g->src_w, dens_tgt, wd, st);
   if (e != cudaSuccess) return scuda(e, "upsample");
   const double* hk_tab = host_plan_hk_table(plan, k, st, &e);
   if (e != cudaSuccess) return scuda(e, "complex-k amplitude table");
+  if (tree) set_fwd_tree(at_tf, wd, hk_tab, base + L.fpart, ns_fwd);
   if (opD) {
     DsArgs d{};
     d.p = p;
@@ -628,7 +696,13 @@ static int shape_impl(int op, qbx_plan* plan, const qbx_geom* g, int side, qbx_c
     d.nsplit = ns_fwd;
     d.per_split = host_split_len(n_src, ns_fwd);
     d.part = (cplx*)(base + L.fpart);
-    e = ck ? launch_dshape<cplx>(d, true, st) : launch_dshape<double>(d, true, st);
+    if (tree) {
+      d.near = tf.near;
+      d.near_cnt = tf.cnt;
+      d.near_stride = tf.M;
+      d.near_q = tf.q_src;
+    }
+    e = fwd_sums([&](cudaStream_t s) { return ck ? launch_dshape<cplx>(d, true, s) : launch_dshape<double>(d, true, s); });
     if (e != cudaSuccess) return scuda(e, "forward sweep (D)");
     k_shape_spread<<<(n_tgt * nrhs + 255) / 256, 256, 0, st>>>(n_tgt, nsides, nrhs, (const cplx*)gout,
                                                                (cplx*)(base + L.gc));
@@ -638,16 +712,36 @@ static int shape_impl(int op, qbx_plan* plan, const qbx_geom* g, int side, qbx_c
     d.nsplit = ns_adj;
     d.per_split = (nc + ns_adj - 1) / ns_adj;
     d.part = (cplx*)(base + L.apart);
-    e = ck ? launch_dshape<cplx>(d, false, st) : launch_dshape<double>(d, false, st);
+    d.near = nullptr;
+    if (tree) {
+      adj_tree_setup(&ta, g, c0, nc, k, p, aops, 2, nrhs, hk_tab, base + L.gc, num_sms, at_ta);
+      e = launch_tree_lists(ta, st);
+      d.near = ta.near;
+      d.near_cnt = ta.cnt;
+      d.near_stride = ta.M;
+      d.near_q = ta.q_src;
+      if (e == cudaSuccess) e = cudaEventRecord(ev_fork, st);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(side_st, ev_fork, 0);
+      if (e != cudaSuccess) return scuda(e, "transposed sweep (D)");
+      e = ck ? launch_dshape<cplx>(d, false, side_st) : launch_dshape<double>(d, false, side_st);
+      cudaError_t y = launch_tree_moments(ta, ck, st);
+      if (y == cudaSuccess) y = launch_far_clusters(ta, st);
+      if (y == cudaSuccess) y = launch_adj_far(ta, 3, g->src_nx, g->src_ny, d.part + (size_t)ns_adj * n_src * nc_adj * nrhs, st);
+      cudaError_t z = cudaEventRecord(ev_join, side_st);   // (joined also after an error)
+      if (z == cudaSuccess) z = cudaStreamWaitEvent(st, ev_join, 0);
+      e = e != cudaSuccess ? e : y != cudaSuccess ? y : z;
+    } else {
+      e = ck ? launch_dshape<cplx>(d, false, st) : launch_dshape<double>(d, false, st);
+    }
     if (e != cudaSuccess) return scuda(e, "transposed sweep (D)");
     double* qh = (double*)(base + L.qh);
     double* dh = (double*)(base + L.dh);
-    k_shape_targets<<<(n_tgt + 127) / 128, 128, 0, st>>>(n_tgt, q_tgt, nsides, side0, ns_fwd, nrhs,
+    k_shape_targets<<<(n_tgt + 127) / 128, 128, 0, st>>>(n_tgt, q_tgt, nsides, side0, nr_fwd, nrhs,
                                                          (const cplx*)(base + L.fpart), (const cplx*)gout,
                                                          g->tgt_nx, g->tgt_ny, g->ctr_r, g->panel_h, dgam_tgt,
                                                          g_gam_tgt, g_dgam_tgt, qh);
     k_shape_panels<<<(g->M + 127) / 128, 128, 0, st>>>(g->M, q_tgt, qh, dh);
-    k_shape_sources_d<<<(n_src + 127) / 128, 128, 0, st>>>(n_src, q_src, ns_adj, nrhs, (const cplx*)(base + L.apart),
+    k_shape_sources_d<<<(n_src + 127) / 128, 128, 0, st>>>(n_src, q_src, nr_adj, nrhs, (const cplx*)(base + L.apart),
                                                            (const cplx*)wd, g->src_w, g->src_nx, g->src_ny, dh,
                                                            dgam_src, g_gam_src, g_dgam_src);
     e = cudaGetLastError();
@@ -673,12 +767,22 @@ static int shape_impl(int op, qbx_plan* plan, const qbx_geom* g, int side, qbx_c
   a.src_per_split = host_split_len(n_src, ns_fwd);
   a.part = base + L.fpart;
   a.hk_tab = hk_tab;
-  for (int r0 = 0; r0 < nrhs; r0 += chunk) {
-    a.rhs0 = r0;
-    a.nr = std::min(chunk, nrhs - r0);
-    e = launch_apply_fused(a, st);
-    if (e != cudaSuccess) return scuda(e, "forward sweep");
+  if (tree) {
+    a.near = tf.near;
+    a.near_cnt = tf.cnt;
+    a.near_stride = tf.M;
+    a.near_q_src = tf.q_src;
   }
+  e = fwd_sums([&](cudaStream_t s) {
+    cudaError_t x = cudaSuccess;
+    for (int r0 = 0; r0 < nrhs && x == cudaSuccess; r0 += chunk) {
+      a.rhs0 = r0;
+      a.nr = std::min(chunk, nrhs - r0);
+      x = launch_apply_fused(a, s);
+    }
+    return x;
+  });
+  if (e != cudaSuccess) return scuda(e, "forward sweep");
   // transposed sums Psi, Xi
   k_shape_spread<<<(n_tgt * nrhs + 255) / 256, 256, 0, st>>>(n_tgt, nsides, nrhs, (const cplx*)gout,
                                                              (cplx*)(base + L.gc));
@@ -708,17 +812,17 @@ static int shape_impl(int op, qbx_plan* plan, const qbx_geom* g, int side, qbx_c
   b.ctr_per_split = (nc + ns_adj - 1) / ns_adj;
   b.part = base + L.apart;
   b.hk_tab = a.hk_tab;
-  e = ck ? launch_adjoint_cplx(b, st) : launch_adjoint_real(b, st);
+  e = adjoint_sums(b, tree ? &ta : nullptr, plan, g, c0, nc, k, aops, 1, 2, num_sms, at_ta, st);
   if (e != cudaSuccess) return scuda(e, "transposed sweep");
   // chain rule to the curve samples
   double* qh = (double*)(base + L.qh);
   double* dh = (double*)(base + L.dh);
-  k_shape_targets<<<(n_tgt + 127) / 128, 128, 0, st>>>(n_tgt, q_tgt, nsides, side0, ns_fwd, nrhs,
+  k_shape_targets<<<(n_tgt + 127) / 128, 128, 0, st>>>(n_tgt, q_tgt, nsides, side0, nr_fwd, nrhs,
                                                        (const cplx*)(base + L.fpart), (const cplx*)gout,
                                                        g->tgt_nx, g->tgt_ny, g->ctr_r, g->panel_h, dgam_tgt,
                                                        g_gam_tgt, g_dgam_tgt, qh);
   k_shape_panels<<<(g->M + 127) / 128, 128, 0, st>>>(g->M, q_tgt, qh, dh);
-  k_shape_sources<<<(n_src + 127) / 128, 128, 0, st>>>(n_src, q_src, ns_adj, nrhs, (const cplx*)(base + L.apart),
+  k_shape_sources<<<(n_src + 127) / 128, 128, 0, st>>>(n_src, q_src, nr_adj, nrhs, (const cplx*)(base + L.apart),
                                                        (const cplx*)wd, g->src_w, dh, dgam_src, g_gam_src,
                                                        g_dgam_src);
   e = cudaGetLastError();

@@ -29,40 +29,58 @@ __device__ __forceinline__ float block_reduce_max(float v, float* s, int n_warps
 // more than) the largest distance from it.  One CTA per node; the points
 // relative to the node's first one in FP32 (the centre may be any point, its
 // radius has to hold for it), so the FP64 pipe sees four subtractions a point.
-__global__ void __launch_bounds__(256) k_tree_nodes(TreeArgs a) {
+__global__ void __launch_bounds__(256) k_tree_nodes(TreeArgs q) {
+  const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
   __shared__ float s_red[8];
   const int id = blockIdx.x;
+  if (id >= a.off[a.lev]) return;
   int l = 0;
   while (id >= a.off[l + 1]) ++l;
   const int j = id - a.off[l];
   const int s0 = (j << l) * a.q_src, s1 = min(a.M, (j + 1) << l) * a.q_src;
-  const double x0 = a.sx[s0], y0 = a.sy[s0];
-  float xa = 0.0f, xb = 0.0f, ya = 0.0f, yb = 0.0f, bad = 0.0f;   // max of -x, x, -y, y
-  for (int s = s0 + threadIdx.x; s < s1; s += 256) {
-    const float x = (float)(a.sx[s] - x0), y = (float)(a.sy[s] - y0);
-    if (!(fabsf(x) < 1e30f && fabsf(y) < 1e30f)) bad = 1.0f;   // a node with such a point is never far
-    xa = fmaxf(xa, -x);
-    xb = fmaxf(xb, x);
-    ya = fmaxf(ya, -y);
-    yb = fmaxf(yb, y);
-  }
+  // discs: the node's points are the targets, each with its centres' discs
+  const int nd = a.discs ? a.n_ctr_n / a.n_src : 1;
+  const double* px = a.discs ? a.dcx : a.sx;
+  const double* py = a.discs ? a.dcy : a.sy;
+  const double x0 = px[s0], y0 = py[s0];
+  float xa = -INFINITY, xb = -INFINITY, ya = -INFINITY, yb = -INFINITY, bad = 0.0f;   // max of -x, x, -y, y
+  for (int sd = 0; sd < nd; ++sd)
+    for (int s = s0 + threadIdx.x; s < s1; s += 256) {
+      const float x = (float)(px[sd * a.n_src + s] - x0), y = (float)(py[sd * a.n_src + s] - y0);
+      if (!(fabsf(x) < 1e30f && fabsf(y) < 1e30f)) bad = 1.0f;   // a node with such a point is never far
+      xa = fmaxf(xa, -x);
+      xb = fmaxf(xb, x);
+      ya = fmaxf(ya, -y);
+      yb = fmaxf(yb, y);
+    }
   xa = block_reduce_max(xa, s_red, 8);
   xb = block_reduce_max(xb, s_red, 8);
   ya = block_reduce_max(ya, s_red, 8);
   yb = block_reduce_max(yb, s_red, 8);
-  bad = block_reduce_max(bad, s_red, 8);
   const double zx = x0 + (double)(0.5f * (xb - xa)), zy = y0 + (double)(0.5f * (yb - ya));
   float r = 0.0f;
   for (int s = s0 + threadIdx.x; s < s1; s += 256) {
-    const float dx = (float)(a.sx[s] - zx), dy = (float)(a.sy[s] - zy);
-    r = fmaxf(r, fmaf(dx, dx, dy * dy));
+    if (!a.discs) {
+      const float dx = (float)(a.sx[s] - zx), dy = (float)(a.sy[s] - zy);
+      r = fmaxf(r, sqrtf(fmaf(dx, dx, dy * dy)));
+      continue;
+    }
+    for (int sd = 0; sd < nd; ++sd) {
+      const double cx = a.dcx[sd * a.n_src + s], cy = a.dcy[sd * a.n_src + s];
+      const float dx = (float)(cx - zx), dy = (float)(cy - zy);
+      const float ex = (float)(a.sx[s] - cx), ey = (float)(a.sy[s] - cy);
+      const float v = sqrtf(fmaf(dx, dx, dy * dy)) + sqrtf(fmaf(ex, ex, ey * ey));
+      if (!(v < 1e30f)) bad = 1.0f;
+      r = fmaxf(r, v);
+    }
   }
   r = block_reduce_max(r, s_red, 8);
+  bad = block_reduce_max(bad, s_red, 8);
   if (threadIdx.x == 0) {
     double* n = a.node + 4 * (size_t)id;
     n[0] = zx;
     n[1] = zy;
-    n[2] = bad > 0.0f ? INFINITY : (double)(sqrtf(r) * 1.00001f);
+    n[2] = bad > 0.0f ? INFINITY : (double)(r * 1.00001f);
     n[3] = 0.0;
   }
 }
@@ -72,7 +90,9 @@ __global__ void __launch_bounds__(256) k_tree_nodes(TreeArgs a) {
 // block; the first leaf of that node names it.  In leaf order, so the sums
 // do not depend on timing.
 constexpr int kListWarps = 8;
-__global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs a) {
+__global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs q) {
+  const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
+  if (blockIdx.x >= a.n_blk) return;
   __shared__ float s_c[64][3];                   // the centres (both sides) from the block's centre, their radii
   __shared__ double s_z[2];
   __shared__ float s_blk[3];                     // radius of all discs about it; largest, smallest radius
@@ -155,7 +175,8 @@ __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs a) {
     if (!(dm > 1.34f * R) || !(rho > 1.34f * rm)) return 0;
     const int om = series_order(ka * R, ka * dm, R / dm, damp, a.nd, kTreeP);
     if (om > kTreeP) return 0;
-    int ol = series_order(ka * rm, ka * rho, rm / rho, expf(2.0f * ki * rm), a.nd, a.pl);
+    // (evaluation points, rm = 0: the field itself)
+    int ol = rm > 0.0f ? series_order(ka * rm, ka * rho, rm / rho, expf(2.0f * ki * rm), a.nd, a.pl) : 0;
     // local expansion about the block's centre, good in all its discs
     const float dl = 0.99999f * (d - R);
     int oq = dl > 1.34f * rd ? series_order(ka * rd, ka * dl, rd / dl, expf(2.0f * ki * rd), a.nd, kTreeP) : kTreeP + 1;
@@ -233,6 +254,175 @@ __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs a) {
   }
 }
 
+// J_0..J_n at z as complex values of stride 32
+template <typename T>
+__device__ __forceinline__ void besselj_wave(T z, int n, cplx* out) {
+  if constexpr (IsCplx<T>::value) {
+    besselj_column<cplx>(z, n, out, 32);
+  } else {
+    besselj_column<double>(z, n, reinterpret_cast<double*>(out), 64);
+    for (int i = 0; i <= n; ++i) out[i * 32].im = 0.0;
+  }
+}
+
+// Waves of one far entry (index, orders om | ol << 8 | local << 16) at this
+// lane's centre, v = c - z: H_n(k d), or J_n(k d) for a local expansion,
+// n <= om + ol + 1, stride 32; the direction Theta of v; and for m = lane the
+// orders l that order m needs.
+template <typename T>
+__device__ __forceinline__ void far_waves(const KW<T>& kw, const T kk, float ka, int2 ent, int nder, double kim,
+                                          const double* nd, double vx, double vy, double r, cplx* sH, double& ct,
+                                          double& st, int& lmax) {
+  const int om = ent.y & 0xff, ol = ent.y >> 8 & 0xff, lane = threadIdx.x & 31;
+  const bool local = ent.y >> 16;
+  const int nH = om + ol + 1;   // (pairs of orders and the cut reach one further)
+  const double d2 = fma(vx, vx, vy * vy);
+  lmax = ol;
+  if (local) {
+    const double rho = sqrt(d2);
+    const bool off = rho > 0.0;   // (the centre may be the block's)
+    ct = off ? vx / rho : 1.0;
+    st = off ? vy / rho : 0.0;
+    besselj_wave<T>(rmul(kk, rho), nH, sH);
+    return;
+  }
+  double inv, rho, yq;
+  kw.geom(d2, inv, rho, yq);
+  cplx h0, h1;
+  T twoz;
+  kw.hankel(rho, inv, yq, h0, h1, twoz);
+  ct = vx * inv;
+  st = vy * inv;
+  T s = twoz;
+  sH[0] = h0;
+  for (int i = 1; i <= nH; ++i) {
+    sH[i * 32] = h1;
+    const cplx h2 = hrec(s, h1, h0);
+    h0 = h1;
+    h1 = h2;
+    s = sadd(s, twoz);
+  }
+  // Orders l that order m needs (lane = m): the terms (kR/2)^m/m!
+  // (kr/2)^l/l! |H_{m+l}| of the nearest centre against |H_nd|, dropped
+  // below 2^-61 (their count is below 2^6); in exponents, FP32.
+  const float rf = (float)rho, rmin = warp_min(rf), rc = warp_max((float)r);
+  const int nl = __ffs(__ballot_sync(0xffffffffu, rf == rmin)) - 1;
+  __syncwarp();
+  const cplx* col = sH - lane + nl;
+  auto ex = [&](int n) {
+    const cplx h = col[n * 32];
+    return (float)(max(__double2hiint(h.re) >> 20 & 0x7ff, __double2hiint(h.im) >> 20 & 0x7ff) - 1022);
+  };
+  if (lane <= om) {
+    const float R = (float)nd[2], fm = (float)lane;
+    const float lr = __log2f(0.5f * ka * rc);
+    float base = fm * __log2f(0.5f * ka * R) - lgammaf(fm + 1.0f) * 1.442695f - ex(nder) + 3.0f +
+                 1.442695f * (float)kim * (R + rc);
+    const float wm = nder ? fm / (ka * R) : 1.0f, wl = nder && rc > 0.0f ? 1.0f / (ka * rc) : 0.0f;
+    lmax = 0;
+    for (int l = 1; l <= ol; ++l) {
+      base += lr - __log2f((float)l);
+      if (base + ex(lane + l) + (nder == 2 ? 2.0f : 1.0f) * __log2f(fmaxf(wm, wl * (float)l)) > -61.0f) lmax = l;
+    }
+  }
+  __syncwarp();
+}
+
+// J_l cos(l psi), J_l sin(l psi) for l = 1..ol; optionally cos, sin of ol psi
+template <typename T>
+__device__ __forceinline__ void far_orders(double cp, double sp, int ol, const T* colJ, T* sF, double* cl = nullptr,
+                                           double* sl = nullptr) {
+  double c = 1.0, s = 0.0;
+  for (int l = 1; l <= ol; ++l) {
+    const double cn = fma(c, cp, -s * sp);
+    s = fma(s, cp, c * sp);
+    c = cn;
+    const T j = colJ[l * 32];
+    sF[(l - 1) * 64] = rmul(j, c);
+    sF[(l - 1) * 64 + 32] = rmul(j, s);
+  }
+  if (cl) {
+    *cl = c;
+    *sl = s;
+  }
+}
+
+// X, Y of the orders m and m + 1, l <= lm: their waves overlap (H_{m+l+1}
+// serves both at consecutive l), and the sums are eight independent chains.
+template <typename T>
+__device__ __forceinline__ void far_pair(const cplx* sH, const T* sF, const T J0, int m, int lm, cplx& X0, cplx& Y0,
+                                         cplx& X1, cplx& Y1) {
+  cplx lo1 = sH[m * 32], hi0 = lo1, hi1 = sH[(m + 1) * 32];   // H_{m+1-l}, H_{m+l}, H_{m+1+l}
+  X0 = smul(J0, hi0);
+  X1 = smul(J0, hi1);
+  Y0 = Y1 = cplx{0.0, 0.0};
+  auto order = [&](int l, bool odd) {
+    const int n = m - l;
+    const cplx lo0 = neg_if(n < 0 && (n & 1), sH[(n < 0 ? -n : n) * 32]);   // H_{m-l}
+    hi0 = hi1;
+    hi1 = sH[(m + 1 + l) * 32];
+    const T jc = sF[(l - 1) * 64], js = sF[(l - 1) * 64 + 32];
+    const cplx s0 = lo0 + hi0, d0 = lo0 - hi0, s1 = lo1 + hi1, d1 = lo1 - hi1;
+    madd(X0, jc, odd ? d0 : s0);
+    madd(Y0, js, odd ? s0 : d0);
+    madd(X1, jc, odd ? d1 : s1);
+    madd(Y1, js, odd ? s1 : d1);
+    lo1 = lo0;
+  };
+  int l = 1;
+  for (; l < lm; l += 2) {
+    order(l, true);
+    order(l + 1, false);
+  }
+  if (l <= lm) order(l, true);
+}
+
+// cos, sin of lane times the angle of (ct, st), by squaring
+__device__ __forceinline__ void lane_power(int lane, double ct, double st, double& cl, double& sl) {
+  double c = ct, s = st;
+  cl = 1.0;
+  sl = 0.0;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    if (lane >> i & 1) {
+      const double cn = fma(cl, c, -sl * s);
+      sl = fma(sl, c, cl * s);
+      cl = cn;
+    }
+    const double c2 = fma(c, c, -s * s);
+    s = 2.0 * c * s;
+    c = c2;
+  }
+}
+
+// Output order q = lane of a translation (k_tree_local has the formulas): W_n
+// the waves (H or J), sd the rows s_m, d_m of NC columns, m <= om.
+template <int NC>
+__device__ __forceinline__ void translate(const cplx* W, const cplx (*sd)[32], int om, int nc, int lane, double cl,
+                                          double sl, cplx* accA, cplx* accB) {
+  cplx S[NC], D[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) S[c] = D[c] = cplx{0.0, 0.0};
+  for (int m = 0; m <= om; ++m) {
+    const int d = m - lane;
+    const cplx ha = neg_if(d < 0 && (d & 1), W[d < 0 ? -d : d]);
+    const cplx hb = neg_if(lane & 1, W[m + lane]);
+    const cplx hp = ha + hb, hm = ha - hb;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (c >= nc) break;
+      cfma(S[c], sd[2 * c][m], hp);
+      cfma(D[c], sd[2 * c + 1][m], hm);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    // A' += cos S - i sin D, B' += sin S + i cos D
+    accA[c] = accA[c] + cplx{fma(cl, S[c].re, sl * D[c].im), fma(cl, S[c].im, -sl * D[c].re)};
+    accB[c] = accB[c] + cplx{fma(sl, S[c].re, -cl * D[c].im), fma(sl, S[c].im, cl * D[c].re)};
+  }
+}
+
 // Moments of one leaf about the centre of one of its nodes (blockIdx = leaf,
 // level): with C_m = J_m(k rho) cos(m theta), S_m = J_m(k rho) sin(m theta) of
 // the source's position about it,
@@ -242,11 +432,13 @@ __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs a) {
 // m > 0 in k_tree_fold).  Phase 1: one thread per source forms its columns in
 // shared memory; phase 2: one thread per (set, rhs, m) sums over the sources.
 template <typename T>
-__global__ void __launch_bounds__(128) k_tree_moments(TreeArgs a) {
+__global__ void __launch_bounds__(128) k_tree_moments(TreeArgs b) {
+  const TreeArgs& a = b.inst ? b.inst[blockIdx.z] : b;
+  if (blockIdx.x >= a.M) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int q = a.q_src, Q = q | 1, P = kTreeP;
-  T* sC = reinterpret_cast<T*>(smem_raw);    // [P + 3][Q]
-  T* sS = sC + (P + 3) * Q;
+  T* sC = reinterpret_cast<T*>(smem_raw);    // [P + 4][Q]
+  T* sS = sC + (P + 4) * Q;
   const int panel = blockIdx.x, l = blockIdx.y;
   const double* n = a.node + 4 * (size_t)(a.off[l] + (panel >> l));
   const double zx = n[0], zy = n[1];
@@ -258,10 +450,10 @@ __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs a) {
   for (int i = threadIdx.x; i < q; i += 128) {
     const double dx = a.sx[panel * q + i] - zx, dy = a.sy[panel * q + i] - zy;
     const double rho = sqrt(dx * dx + dy * dy);
-    besselj_column<T>(rmul(kk, rho), P + 2, sC + i, Q);
+    besselj_column<T>(rmul(kk, rho), P + 3, sC + i, Q);
     const double cs = rho > 0.0 ? dx / rho : 1.0, sn = rho > 0.0 ? dy / rho : 0.0;
     double c = 1.0, s = 0.0;
-    for (int m = 0; m <= P + 2; ++m) {
+    for (int m = 0; m <= P + 3; ++m) {
       const T j = sC[m * Q + i];
       sC[m * Q + i] = rmul(j, c);
       sS[m * Q + i] = rmul(j, s);
@@ -272,7 +464,9 @@ __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs a) {
   }
   __syncthreads();
   const int ncol = a.nset * a.nrhs;
-  cplx* out = reinterpret_cast<cplx*>(a.mom) + (size_t)(l * a.M + panel) * ncol * (P + 2) * 2;
+  // few columns: [leaf, level][col][m][2]; many: the leaf's own rows of the coefficients
+  cplx* out = a.up ? reinterpret_cast<cplx*>(a.coef) + (size_t)panel * (P + 2) * ncol * 2
+                   : reinterpret_cast<cplx*>(a.mom) + (size_t)(l * a.M + panel) * ncol * (P + 2) * 2;
   const T hk = rmul(kk, 0.5);
   for (int e = threadIdx.x; e < ncol * (P + 2); e += 128) {
     const int col = e / (P + 2), m = e - col * (P + 2);
@@ -284,14 +478,41 @@ __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs a) {
         madd(A, sC[m * Q + i], w[(size_t)i * a.nrhs]);
         madd(B, sS[m * Q + i], w[(size_t)i * a.nrhs]);
       }
+    } else if (kind == kSetQuadX || kind == kSetQuadY) {
+      // n . grad of d/dx or d/dy: with F = C, S and F_{m-2}, F_m, F_{m+2}
+      //   d_xx F = (k^2/4)(F_{m-2} - 2 F_m + F_{m+2}), d_yy F = -(k^2/4)(F_{m-2} + 2 F_m + F_{m+2}),
+      //   d_xy C = -(k^2/4)(S_{m-2} - S_{m+2}), d_xy S = (k^2/4)(C_{m-2} - C_{m+2})
+      const double* px = a.snx + (size_t)panel * q;
+      const double* py = a.sny + (size_t)panel * q;
+      const int mm = m >= 2 ? m - 2 : 2 - m;
+      const double sc = m == 1 ? -1.0 : 1.0, ss = m == 0 ? -1.0 : 1.0;   // C_{-n} = (-1)^n C_n, S_{-n} = -(-1)^n S_n
+      for (int i = 0; i < q; ++i) {
+        const T cm = rmul(sC[mm * Q + i], sc), c0 = sC[m * Q + i], cp = sC[(m + 2) * Q + i];
+        const T sm = rmul(sS[mm * Q + i], ss), s0 = sS[m * Q + i], sp = sS[(m + 2) * Q + i];
+        const T cxy = sc_sub(sp, sm), sxy = sc_sub(cm, cp);
+        const double nx = px[i], ny = py[i];
+        const cplx v = w[(size_t)i * a.nrhs];
+        if (kind == kSetQuadX) {
+          const T cxx = sc_sub(sadd(cm, cp), rmul(c0, 2.0)), sxx = sc_sub(sadd(sm, sp), rmul(s0, 2.0));
+          madd(A, sadd(rmul(cxx, nx), rmul(cxy, ny)), v);
+          madd(B, sadd(rmul(sxx, nx), rmul(sxy, ny)), v);
+        } else {
+          const T cyy = sadd(sadd(cm, cp), rmul(c0, 2.0)), syy = sadd(sadd(sm, sp), rmul(s0, 2.0));
+          madd(A, sc_sub(rmul(cxy, nx), rmul(cyy, ny)), v);
+          madd(B, sc_sub(rmul(sxy, nx), rmul(syy, ny)), v);
+        }
+      }
+      const T k2 = sc_mul(hk, hk);
+      A = smul(k2, A);
+      B = smul(k2, B);
     } else {
       const double* px = a.snx + (size_t)panel * q;
       const double* py = a.sny + (size_t)panel * q;
       const int mm = m > 0 ? m - 1 : 1;
       const double sg = m > 0 ? 1.0 : -1.0;   // C_{-1} = -C_1, S_{-1} = S_1
       for (int i = 0; i < q; ++i) {
-        const double nx = kind == kSetNormal ? px[i] : kind == kSetX ? 1.0 : 0.0;
-        const double ny = kind == kSetNormal ? py[i] : kind == kSetY ? 1.0 : 0.0;
+        const double nx = kind == kSetX ? 1.0 : kind == kSetY ? 0.0 : px[i];
+        const double ny = kind == kSetY ? 1.0 : kind == kSetX ? 0.0 : py[i];
         const T cm = rmul(sC[mm * Q + i], sg), cp = sC[(m + 1) * Q + i];
         const T sm = sS[mm * Q + i], sp = sS[(m + 1) * Q + i];
         const cplx v = w[(size_t)i * a.nrhs];
@@ -300,9 +521,164 @@ __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs a) {
       }
       A = smul(hk, A);
       B = smul(hk, B);
+      if (kind == kSetCombined) {   // - i eta times the density's own
+        cplx A1{0.0, 0.0}, B1{0.0, 0.0};
+        for (int i = 0; i < q; ++i) {
+          madd(A1, sC[m * Q + i], w[(size_t)i * a.nrhs]);
+          madd(B1, sS[m * Q + i], w[(size_t)i * a.nrhs]);
+        }
+        const cplx f{a.eta_im, -a.eta_re};
+        cfma(A, f, A1);
+        cfma(B, f, B1);
+      }
     }
-    out[(size_t)e * 2] = A;
-    out[(size_t)e * 2 + 1] = B;
+    const double f = a.up && m > 0 ? 2.0 : 1.0;
+    cplx* o = out + (a.up ? (size_t)m * ncol + col : (size_t)e) * 2;
+    o[0] = f * A;
+    o[1] = f * B;
+  }
+}
+
+// Moments of the centres of one leaf (adjoint sweeps: a centre with gradient g
+// sends conj(g) times its truncated expansion to the sources).  As a function
+// of the source position the truncated Graf sum of a centre c is the outgoing
+// field sum_{|n|<=p} J_n(kr) e^{-i n theta_t} H_n e^{i n theta} about c; carried
+// to the node's centre its coefficients of H_m cos, H_m sin are the values
+// that k_far_clusters forms, with J_n(k |c - z|) in the place of H_n.  One
+// centre per lane, a warp per 32 centres of the leaf (blockIdx = leaf, level);
+// the lanes' products are added up over the leaf.
+template <typename T>
+__global__ void __launch_bounds__(32) k_tree_disc_moments(TreeArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int P = kTreeP, p = a.p, lane = threadIdx.x;
+  cplx* sH = reinterpret_cast<cplx*>(smem_raw) + lane;                     // [P + p + 4][32]
+  T* colJ = reinterpret_cast<T*>(sH - lane + (P + p + 4) * 32) + lane;     // [p + 2][32]
+  T* sF = colJ + (p + 2) * 32;                                             // [p][2][32]
+  const int leaf = blockIdx.x, l = blockIdx.y;
+  const double* n = a.node + 4 * (size_t)(a.off[l] + (leaf >> l));
+  KW<T> kw;
+  kw.init(a.kre, a.kim, a.hk_tab);
+  const T kk = kw.kval();
+  const float kr = (float)sc_abs(kk) * (float)n[2];   // orders at any distance beyond kTreeP: in no list
+  if (!(kr < 64.0f) || series_order(kr, 1e4f * kr + 1e4f, 1e-4f, 1.0f, 0, kTreeP) > kTreeP) return;
+  const int nside = a.n_ctr_n / a.n_src, nc = a.q_src * nside, ncol = a.nset * a.nrhs;
+  cplx* out = reinterpret_cast<cplx*>(a.mom) + (size_t)(l * a.M + leaf) * ncol * (P + 2) * 2;
+  for (int c0 = 0; c0 < nc; c0 += 32) {
+    const bool active = c0 + lane < nc;
+    const int i = active ? c0 + lane : 0, sd = i / a.q_src, t = leaf * a.q_src + i - sd * a.q_src;
+    const int c = sd * a.n_src + t;
+    const double cx = a.dcx[c], cy = a.dcy[c];
+    double ux = a.sx[t] - cx, uy = a.sy[t] - cy;
+    const double r = hypot(ux, uy);
+    ux /= r;
+    uy /= r;
+    besselj_column<T>(rmul(kk, r), p + 1, colJ, 32);
+    const double vx = cx - n[0], vy = cy - n[1], d = sqrt(fma(vx, vx, vy * vy));
+    const double ct = d > 0.0 ? vx / d : 1.0, st = d > 0.0 ? vy / d : 0.0;
+    besselj_wave<T>(rmul(kk, d), P + p + 3, sH);
+    far_orders<T>(fma(ux, ct, uy * st), fma(uy, ct, -ux * st), p, colJ, sF);
+    const T J0 = colJ[0];
+    double cm = 1.0, sm = 0.0;
+    for (int m = 0; m <= P + 1; m += 2) {
+      cplx X0, Y0, X1, Y1;
+      far_pair<T>(sH, sF, J0, m, p, X0, Y0, X1, Y1);
+      for (int h = 0; h < 2; ++h) {
+        const cplx X = h ? X1 : X0, Y = h ? Y1 : Y0;
+        const cplx fc = lin2(cm, X, -sm, Y), fs = lin2(sm, X, cm, Y);
+        for (int col = 0; col < ncol; ++col) {
+          cplx A{0.0, 0.0}, B{0.0, 0.0};
+          if (active) {
+            const cplx g = conj(reinterpret_cast<const cplx*>(a.wd[0])[(size_t)c * a.nrhs + col]);
+            A = g * fc;
+            B = g * fs;
+          }
+          for (int o = 16; o > 0; o >>= 1) {
+            A.re += __shfl_xor_sync(0xffffffffu, A.re, o);
+            A.im += __shfl_xor_sync(0xffffffffu, A.im, o);
+            B.re += __shfl_xor_sync(0xffffffffu, B.re, o);
+            B.im += __shfl_xor_sync(0xffffffffu, B.im, o);
+          }
+          if (lane == 0) {
+            cplx* v = out + ((size_t)col * (P + 2) + m + h) * 2;
+            v[0] = c0 ? v[0] + A : A;
+            v[1] = c0 ? v[1] + B : B;
+          }
+        }
+        const double cn = fma(cm, ct, -sm * st);
+        sm = fma(sm, ct, cm * st);
+        cm = cn;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// Node moments upward (many columns): a node's moments from its two children's
+// (the addition theorem for outgoing waves about a new centre z', V = z' - z:
+// M'_q = sum_m M_m J_{m-q}(k|V|) e^{i(m-q) arg V}), in the form of k_tree_local
+// with J in the place of H.  One launch per level; a CTA per (node, 32
+// columns), warp = 4 columns, lane = q.  Per column 1/16 of the FP64 work of
+// summing the sources again at every level.
+constexpr int kUpWarps = 8, kUpCols = 4;
+template <typename T>
+__global__ void __launch_bounds__(32 * kUpWarps) k_tree_up(TreeArgs q, int l) {
+  const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
+  if (l >= a.lev || blockIdx.x >= a.off[l + 1] - a.off[l]) return;
+  constexpr int NC = kUpCols, N = kTreeP + 2;
+  static_assert(N == 32, "one lane per order");
+  __shared__ cplx s_w[2][2 * N];
+  __shared__ cplx s_sd[kUpWarps][2 * NC][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int id = a.off[l] + blockIdx.x, c0 = a.off[l - 1] + 2 * blockIdx.x;
+  const int nch = min(2, a.off[l] - c0);
+  const int ncol = a.nset * a.nrhs;
+  KW<T> kw;
+  kw.init(a.kre, a.kim, a.hk_tab);
+  const T kk = kw.kval();
+  const double* z = a.node + 4 * (size_t)id;
+  const float kr = (float)sc_abs(kk) * (float)z[2];
+  if (!(kr < 64.0f) || series_order(kr, 1e4f * kr + 1e4f, 1e-4f, 1.0f, 0, kTreeP) > kTreeP) return;   // in no list
+  if (warp < nch && lane == 0) {
+    const double* y = a.node + 4 * (size_t)(c0 + warp);
+    const double vx = z[0] - y[0], vy = z[1] - y[1];
+    if constexpr (IsCplx<T>::value) {
+      besselj_column<cplx>(rmul(kk, sqrt(vx * vx + vy * vy)), 2 * N - 2, s_w[warp], 1);
+    } else {
+      besselj_column<double>(kk * sqrt(vx * vx + vy * vy), 2 * N - 2, reinterpret_cast<double*>(s_w[warp]), 2);
+      for (int i = 0; i < 2 * N - 1; ++i) s_w[warp][i].im = 0.0;
+    }
+  }
+  __syncthreads();
+  for (int col0 = (blockIdx.y * kUpWarps + warp) * NC; col0 < ncol; col0 += gridDim.y * kUpWarps * NC) {
+    const int nc = min(NC, ncol - col0);
+    cplx accA[NC], accB[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) accA[c] = accB[c] = cplx{0.0, 0.0};
+    for (int ch = 0; ch < nch; ++ch) {
+      const double* y = a.node + 4 * (size_t)(c0 + ch);
+      const double vx = z[0] - y[0], vy = z[1] - y[1], d = sqrt(vx * vx + vy * vy);
+      const double ct = d > 0.0 ? vx / d : 1.0, st = d > 0.0 ? vy / d : 0.0;
+      double cl, sl;
+      lane_power(lane, ct, st, cl, sl);
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (c >= nc) break;
+        const cplx* m = reinterpret_cast<const cplx*>(a.coef) + (((size_t)(c0 + ch) * N + lane) * ncol + col0 + c) * 2;
+        const cplx A = m[0], B = m[1];
+        s_sd[warp][2 * c][lane] = cplx{fma(A.re, cl, B.re * sl), fma(A.im, cl, B.im * sl)};
+        s_sd[warp][2 * c + 1][lane] = cplx{fma(B.im, cl, -A.im * sl), fma(A.re, sl, -B.re * cl)};
+      }
+      __syncwarp();
+      translate<NC>(s_w[ch], s_sd[warp], N - 1, nc, lane, cl, sl, accA, accB);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (c >= nc) break;
+      cplx* m = reinterpret_cast<cplx*>(a.coef) + (((size_t)id * N + lane) * ncol + col0 + c) * 2;
+      m[0] = (lane > 0 ? 1.0 : 0.5) * accA[c];
+      m[1] = lane > 0 ? accB[c] : cplx{0.0, 0.0};
+    }
   }
 }
 
@@ -325,6 +701,27 @@ __device__ __forceinline__ void shifted_coef(const TreeArgs& a, int set, const c
     return;
   }
   const cplx hk{0.5 * a.kre, 0.5 * a.kim};
+  if (sh >= 3) {
+    // second derivatives along x, x (3) and x, y (4): the x derivative's
+    // coefficients at m - 1 and m + 1, shifted again
+    auto dx = [&](int i, cplx* v) {
+      const double f = i == 1 ? 2.0 : 1.0;
+      v[0] = i < 0 ? cplx{0.0, 0.0} : hk * (at(i + 1, 0) - f * at(i - 1, 0));
+      v[1] = i < 1 ? cplx{0.0, 0.0} : hk * (at(i + 1, 1) - at(i - 1, 1));
+    };
+    cplx p[2], q[2];
+    dx(m + 1, p);
+    dx(m - 1, q);
+    const double f = m == 1 ? 2.0 : 1.0;
+    if (sh == 3) {
+      out[0] = hk * (p[0] - f * q[0]);
+      out[1] = m ? hk * (p[1] - q[1]) : cplx{0.0, 0.0};
+    } else {
+      out[0] = hk * (p[1] + q[1]);
+      out[1] = m ? -(hk * (p[0] + f * q[0])) : cplx{0.0, 0.0};
+    }
+    return;
+  }
   const double f = m == 1 ? 2.0 : 1.0;
   const cplx Ap = at(m + 1, 0), Bp = at(m + 1, 1), Am = f * at(m - 1, 0), Bm = at(m - 1, 1);
   if (sh == 1) {
@@ -358,7 +755,7 @@ __global__ void __launch_bounds__(64) k_tree_fold(TreeArgs a) {
     const int cs = i / (kTreeP + 1), m = i - cs * (kTreeP + 1);
     if (a.base[cs] != set) continue;
     shifted_coef(a, cs, &s_m[0][0], 2, kTreeP + 1, m,
-                 reinterpret_cast<cplx*>(a.coef) + (((size_t)id * (kTreeP + 1) + m) * a.ncset * a.nrhs + cs * a.nrhs + r) * 2);
+                 reinterpret_cast<cplx*>(a.coef) + (((size_t)id * (kTreeP + 2) + m) * a.ncset * a.nrhs + cs * a.nrhs + r) * 2);
   }
 }
 
@@ -372,10 +769,11 @@ __global__ void __launch_bounds__(64) k_tree_fold(TreeArgs a) {
 //   A'_q = cos(q Theta) S_q - i sin(q Theta) T_q,  B'_q = sin(q Theta) S_q + i cos(q Theta) T_q
 // (A'_0 halved).  One warp per node, lane = q: a tenth of the FP64 work of
 // taking the node through each of the block's 32 or 64 centres.
-constexpr int kLocWarps = 8, kLocCols = 2;   // moment columns per CTA
-template <typename T>
-__global__ void __launch_bounds__(32 * kLocWarps) k_tree_local(TreeArgs a) {
-  constexpr int NC = kLocCols;
+// NC moment columns per CTA of kLocWarps warps.
+template <typename T, int NC, int kLocWarps>
+__global__ void __launch_bounds__(32 * kLocWarps) k_tree_local(TreeArgs q) {
+  const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
+  if (blockIdx.x >= a.n_blk) return;
   __shared__ cplx s_h[kLocWarps][2 * kTreeP + 2];
   __shared__ cplx s_sd[kLocWarps][2 * NC][32];
   static_assert(kTreeP < 32, "one lane per order");
@@ -408,21 +806,8 @@ __global__ void __launch_bounds__(32 * kLocWarps) k_tree_local(TreeArgs a) {
     T twoz;
     kw.hankel(rho, inv, yq, h0, h1, twoz);
     const double ct = vx * inv, st = vy * inv;
-    double cl = 1.0, sl = 0.0;   // cos, sin of lane * Theta, by squaring
-    {
-      double c = ct, s = st;
-#pragma unroll
-      for (int i = 0; i < 5; ++i) {
-        if (lane >> i & 1) {
-          const double cn = fma(cl, c, -sl * s);
-          sl = fma(sl, c, cl * s);
-          cl = cn;
-        }
-        const double c2 = fma(c, c, -s * s);
-        s = 2.0 * c * s;
-        c = c2;
-      }
-    }
+    double cl, sl;   // lane * Theta
+    lane_power(lane, ct, st, cl, sl);
     __syncwarp();   // the previous node's tables are no longer read
     if (lane == 0) s_h[warp][0] = h0;
     T s = twoz;
@@ -434,7 +819,7 @@ __global__ void __launch_bounds__(32 * kLocWarps) k_tree_local(TreeArgs a) {
       s = sadd(s, twoz);
     }
     if (lane <= om) {
-      const double2* co = reinterpret_cast<const double2*>(a.coef) + ((size_t)ent.x * (kTreeP + 1) + lane) * ncol * 2;
+      const double2* co = reinterpret_cast<const double2*>(a.coef) + ((size_t)ent.x * (kTreeP + 2) + lane) * ncol * 2;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         if (c >= nc) break;
@@ -444,29 +829,7 @@ __global__ void __launch_bounds__(32 * kLocWarps) k_tree_local(TreeArgs a) {
       }
     }
     __syncwarp();
-    if (lane <= oq) {
-      cplx S[NC], D[NC];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) S[c] = D[c] = cplx{0.0, 0.0};
-      for (int m = 0; m <= om; ++m) {
-        const int d = m - lane;
-        const cplx ha = neg_if(d < 0 && (d & 1), s_h[warp][d < 0 ? -d : d]);
-        const cplx hb = neg_if(lane & 1, s_h[warp][m + lane]);
-        const cplx hp = ha + hb, hm = ha - hb;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          if (c >= nc) break;
-          cfma(S[c], s_sd[warp][2 * c][m], hp);
-          cfma(D[c], s_sd[warp][2 * c + 1][m], hm);
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        // A' += cos S - i sin D, B' += sin S + i cos D
-        accA[c] = accA[c] + cplx{fma(cl, S[c].re, sl * D[c].im), fma(cl, S[c].im, -sl * D[c].re)};
-        accB[c] = accB[c] + cplx{fma(sl, S[c].re, -cl * D[c].im), fma(sl, S[c].im, cl * D[c].re)};
-      }
-    }
+    if (lane <= oq) translate<NC>(s_h[warp], s_sd[warp], om, nc, lane, cl, sl, accA, accB);
   }
   // the warps' sums, in warp order
   __shared__ cplx s_sum[2 * NC][32], s_mom[NC][kTreeP + 1][2];
@@ -492,24 +855,13 @@ __global__ void __launch_bounds__(32 * kLocWarps) k_tree_local(TreeArgs a) {
     }
   }
   __syncthreads();
-  cplx* out = reinterpret_cast<cplx*>(a.coef) + (size_t)(a.off[a.lev] + b) * (kTreeP + 1) * ncol * 2;
+  cplx* out = reinterpret_cast<cplx*>(a.coef) + (size_t)(a.off[a.lev] + b) * (kTreeP + 2) * ncol * 2;
   for (int i = threadIdx.x; i < nc * a.ncset * (kTreeP + 1); i += 32 * kLocWarps) {
     const int c = i / (a.ncset * (kTreeP + 1)), rem = i - c * a.ncset * (kTreeP + 1);
     const int cs = rem / (kTreeP + 1), m = rem - cs * (kTreeP + 1);
     const int set = (col0 + c) / a.nrhs, r = col0 + c - set * a.nrhs;
     if (a.base[cs] == set)
       shifted_coef(a, cs, &s_mom[c][0][0], 2, kTreeP, m, out + ((size_t)m * ncol + cs * a.nrhs + r) * 2);
-  }
-}
-
-// J_0..J_n at z as complex values of stride 32
-template <typename T>
-__device__ __forceinline__ void besselj_wave(T z, int n, cplx* out) {
-  if constexpr (IsCplx<T>::value) {
-    besselj_column<cplx>(z, n, out, 32);
-  } else {
-    besselj_column<double>(z, n, reinterpret_cast<double*>(out), 64);
-    for (int i = 0; i <= n; ++i) out[i * 32].im = 0.0;
   }
 }
 
@@ -599,77 +951,17 @@ __global__ void __launch_bounds__(128) k_far_clusters(TreeArgs a) {
     const int mpart = e % np;
     const int2 ent = far[cnt - 1 - e / np];   // the local expansion, the longest entry, first
     const int om = ent.y & 0xff, ol = ent.y >> 8 & 0xff;
-    const bool local = ent.y >> 16;
-    int lmax = ol;   // of order m = lane
+    int lmax;   // of order m = lane
     const double* nd = a.node + 4 * (size_t)ent.x;
-    const double vx = cx - nd[0], vy = cy - nd[1];
-    double inv, rho, yq;
-    const double d2 = fma(vx, vx, vy * vy);
     double ct, st;   // Theta
-    const int nH = om + ol + 1;   // (pairs of orders and the cut reach one further)
-    if (local) {
-      // regular waves: J_n(k d) in the place of H_n
-      rho = sqrt(d2);
-      const bool off = rho > 0.0;   // (the centre may be the block's)
-      ct = off ? vx / rho : 1.0;
-      st = off ? vy / rho : 0.0;
-      besselj_wave<T>(rmul(kk, rho), nH, sH);
-    } else {
-      kw.geom(d2, inv, rho, yq);
-      cplx h0, h1;
-      T twoz;
-      kw.hankel(rho, inv, yq, h0, h1, twoz);
-      ct = vx * inv;
-      st = vy * inv;
-      T s = twoz;
-      sH[0] = h0;
-      for (int i = 1; i <= nH; ++i) {
-        sH[i * 32] = h1;
-        const cplx h2 = hrec(s, h1, h0);
-        h0 = h1;
-        h1 = h2;
-        s = sadd(s, twoz);
-      }
-      // Orders l that order m needs (lane = m): the terms (kR/2)^m/m!
-      // (kr/2)^l/l! |H_{m+l}| of the nearest centre against |H_nd|, dropped
-      // below 2^-61 (their count is below 2^6); in exponents, FP32.
-      const float rf = (float)rho, rmin = warp_min(rf), rc = warp_max((float)r);
-      const int nl = __ffs(__ballot_sync(0xffffffffu, rf == rmin)) - 1;
-      __syncwarp();
-      const cplx* col = sH - lane + nl;
-      auto ex = [&](int n) {
-        const cplx h = col[n * 32];
-        return (float)(max(__double2hiint(h.re) >> 20 & 0x7ff, __double2hiint(h.im) >> 20 & 0x7ff) - 1022);
-      };
-      if (lane <= om) {
-        const float R = (float)nd[2], fm = (float)lane;
-        const float lr = __log2f(0.5f * ka * rc);
-        float base = fm * __log2f(0.5f * ka * R) - lgammaf(fm + 1.0f) * 1.442695f - ex(a.nd) + 3.0f +
-                     1.442695f * (float)a.kim * (R + rc);
-        const float wm = a.nd ? fm / (ka * R) : 1.0f, wl = a.nd ? 1.0f / (ka * rc) : 0.0f;
-        lmax = 0;
-        for (int l = 1; l <= ol; ++l) {
-          base += lr - __log2f((float)l);
-          if (base + ex(lane + l) + __log2f(fmaxf(wm, wl * (float)l)) > -61.0f) lmax = l;
-        }
-      }
-      __syncwarp();
-    }
+    far_waves<T>(kw, kk, ka, ent, a.nd, a.kim, nd, cx - nd[0], cy - nd[1], r, sH, ct, st, lmax);
     // orders m whose expansions reach the cut at l = p (grad S)
-    const unsigned cut = ol == p ? __ballot_sync(0xffffffffu, lane <= om && lmax >= p) : 0u;
+    const unsigned cut = !a.discs && ol == p ? __ballot_sync(0xffffffffu, lane <= om && lmax >= p) : 0u;
     const int mcut = cut ? 32 - __clz(cut) : -1;   // one order further: the derivative shifts m by one
     const double cp = fma(ux, ct, uy * st), sp = fma(uy, ct, -ux * st);   // psi
-    double cP = 1.0, sP = 0.0;   // p psi, after the loop for ol == p
-    for (int l = 1; l <= ol; ++l) {
-      const double cn = fma(cP, cp, -sP * sp);
-      sP = fma(sP, cp, cP * sp);
-      cP = cn;
-      const T j = colJ[l * 32];
-      T* f = sF + (l - 1) * 64;
-      f[0] = rmul(j, cP);
-      f[32] = rmul(j, sP);
-    }
-    const cplx* co = reinterpret_cast<const cplx*>(a.coef) + ((size_t)ent.x * (kTreeP + 1) * ncol + a.rhs0) * 2;
+    double cP, sP;   // cos, sin of ol psi (= p psi where the cut is reached)
+    far_orders<T>(cp, sp, ol, colJ, sF, &cP, &sP);
+    const cplx* co = reinterpret_cast<const cplx*>(a.coef) + ((size_t)ent.x * (kTreeP + 2) * ncol + a.rhs0) * 2;
     cplx U0[NR], V0[NR], U1[NR], V1[NR];
     if (kG) {
 #pragma unroll
@@ -726,32 +1018,11 @@ __global__ void __launch_bounds__(128) k_far_clusters(TreeArgs a) {
         }
       }
     };
-    // two orders m, m + 1 at a time: their waves overlap (H_{m+l+1} serves both
-    // at consecutive l), and the sums are eight independent chains
     for (int m = 2 * mpart; m <= om; m += 2 * np) {
       const bool two = m < om;
-      cplx lo1 = sH[m * 32], hi0 = lo1, hi1 = sH[(m + 1) * 32];   // H_{m+1-l}, H_{m+l}, H_{m+1+l}
-      cplx X0 = smul(J0, hi0), X1 = smul(J0, hi1), Y0{0.0, 0.0}, Y1{0.0, 0.0};
-      const int lm = max(__shfl_sync(0xffffffffu, lmax, m), __shfl_sync(0xffffffffu, lmax, min(m + 1, om)));
-      auto order = [&](int l, bool odd) {
-        // lo0 = H_{m-l}, lo1 = H_{m+1-l}, hi0 = H_{m+l}, hi1 = H_{m+1+l}
-        const cplx lo0 = wave(m - l);
-        hi0 = hi1;
-        hi1 = sH[(m + 1 + l) * 32];
-        const T jc = sF[(l - 1) * 64], js = sF[(l - 1) * 64 + 32];
-        const cplx s0 = lo0 + hi0, d0 = lo0 - hi0, s1 = lo1 + hi1, d1 = lo1 - hi1;
-        madd(X0, jc, odd ? d0 : s0);
-        madd(Y0, js, odd ? s0 : d0);
-        madd(X1, jc, odd ? d1 : s1);
-        madd(Y1, js, odd ? s1 : d1);
-        lo1 = lo0;
-      };
-      int l = 1;
-      for (; l < lm; l += 2) {
-        order(l, true);
-        order(l + 1, false);
-      }
-      if (l <= lm) order(l, true);
+      cplx X0, Y0, X1, Y1;
+      far_pair<T>(sH, sF, J0, m, max(__shfl_sync(0xffffffffu, lmax, m), __shfl_sync(0xffffffffu, lmax, min(m + 1, om))),
+                  X0, Y0, X1, Y1);
       finish(m, cm, sm, X0, Y0);
       if (two) finish(m + 1, fma(cm, ct, -sm * st), fma(sm, ct, cm * st), X1, Y1);
       const double cn = fma(cm, cstep, -sm * sstep);
@@ -801,6 +1072,138 @@ __global__ void __launch_bounds__(128) k_far_clusters(TreeArgs a) {
   }
 }
 
+// Far sums for many columns (S, D, S + D or the combined field, 16 or more
+// rhs): a CTA of eight warps holds 32 targets; for every far node of the block
+// the warps form the values of H_m cos(m Theta), H_m sin(m Theta) through the
+// target's centre (or the average over its two centres) in shared memory, as
+// k_far_clusters does, and then multiply them into RG columns each.  A column
+// costs 8 FP64 instructions per order where the pairs of a leaf cost 96.
+template <typename T>
+struct FarGroupSmem {
+  static __host__ __device__ size_t rows(int pl) { return (size_t)kTreeP + pl + 2; }
+  static __host__ __device__ size_t bytes(int pl, int nsd) {
+    return (size_t)nsd * ((pl + 2) * sizeof(T) + rows(pl) * 16 + (size_t)pl * 2 * sizeof(T) + 2 * 8 + 4) * 32 +
+           (size_t)2 * (kTreeP + 1) * 32 * 16;
+  }
+};
+constexpr int kFgWarps = 8;
+
+template <typename T, int RG>
+__global__ void __launch_bounds__(32 * kFgWarps) k_far_group(TreeArgs q) {
+  const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
+  const int pl = a.pl, nsd = a.n_ctr / a.n_tgt;
+  const int blk = (int)blockIdx.x % q.n_blk, split = (int)blockIdx.x / q.n_blk;   // q: the largest n_blk
+  if (blk >= a.n_blk || split >= a.nsplit) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const size_t rows = FarGroupSmem<T>::rows(pl);
+  cplx* sB = reinterpret_cast<cplx*>(smem_raw);                        // [2 (kTreeP + 1)][32] values
+  cplx* sH = sB + 2 * (kTreeP + 1) * 32;                               // [side][rows][32]
+  T* sJ = reinterpret_cast<T*>(sH + nsd * rows * 32);                  // [side][pl + 2][32]
+  T* sF = sJ + (size_t)nsd * (pl + 2) * 32;                            // [side][pl][2][32]
+  double* sT = reinterpret_cast<double*>(sF + (size_t)nsd * pl * 64);  // [side][2][32] Theta
+  int* sL = reinterpret_cast<int*>(sT + nsd * 64);                     // [side][32] orders l by m
+  const bool active = blk * 32 + lane < a.n_tgt;
+  const int t = active ? blk * 32 + lane : a.n_tgt - 1;
+  KW<T> kw;
+  kw.init(a.kre, a.kim, a.hk_tab);
+  const T kk = kw.kval();
+  const float ka = (float)sc_abs(kk);
+  double cx = 0.0, cy = 0.0, ux = 0.0, uy = 0.0, r = 0.0;   // of side `warp`
+  if (warp < nsd) {
+    cx = a.cx[warp * a.n_tgt + t];
+    cy = a.cy[warp * a.n_tgt + t];
+    ux = a.tx[t] - cx;
+    uy = a.ty[t] - cy;
+    r = hypot(ux, uy);
+    ux /= r;
+    uy /= r;
+    besselj_column<T>(rmul(kk, r), pl + 1, sJ + (size_t)warp * (pl + 2) * 32 + lane, 32);
+  }
+  const int ncomp = (a.ops & OPB_C) ? 1 : popc3(a.ops), ncols = ncomp * a.nrhs;
+  const int ccol = a.ncset * a.nrhs;
+  const int cnt = a.cnt[3 * blk + 1];
+  const int2* far = reinterpret_cast<const int2*>(a.far) + (size_t)blk * (a.M + 1);
+  // columns in the coefficient rows: S's set, then D's (or the combined one)
+  const int set0 = (a.ops & OPB_S) ? a.set_s : a.set_d, set1 = a.set_d;
+  for (int g0 = 0; g0 < ncols; g0 += kFgWarps * RG) {
+    cplx acc[RG];
+#pragma unroll
+    for (int i = 0; i < RG; ++i) acc[i] = cplx{0.0, 0.0};
+    const int mycol = g0 + warp * RG;
+    for (int e = split; e < cnt; e += a.nsplit) {
+      const int2 ent = far[cnt - 1 - e];
+      const int om = ent.y & 0xff, ol = ent.y >> 8 & 0xff;
+      __syncthreads();   // the previous node's waves and values are no longer read
+      if (warp < nsd) {
+        cplx* H = sH + (size_t)warp * rows * 32 + lane;
+        const double* nd = a.node + 4 * (size_t)ent.x;
+        double ct, st;
+        int lmax;
+        far_waves<T>(kw, kk, ka, ent, a.nd, a.kim, nd, cx - nd[0], cy - nd[1], r, H, ct, st, lmax);
+        sT[warp * 64 + lane] = ct;
+        sT[warp * 64 + 32 + lane] = st;
+        sL[warp * 32 + lane] = lmax;
+        far_orders<T>(fma(ux, ct, uy * st), fma(uy, ct, -ux * st), ol, sJ + (size_t)warp * (pl + 2) * 32 + lane,
+                      sF + (size_t)warp * pl * 64 + lane);
+      }
+      __syncthreads();
+      for (int m = 2 * warp; m <= om; m += 2 * kFgWarps) {
+        cplx c0{0.0, 0.0}, s0 = c0, c1 = c0, s1 = c0;
+        const double wgt = nsd == 2 ? 0.5 : 1.0;
+        for (int sd = 0; sd < nsd; ++sd) {
+          const cplx* H = sH + (size_t)sd * rows * 32 + lane;
+          cplx X0, Y0, X1, Y1;
+          far_pair<T>(H, sF + (size_t)sd * pl * 64 + lane, sJ[(size_t)sd * (pl + 2) * 32 + lane], m,
+                      max(sL[sd * 32 + m], sL[sd * 32 + min(m + 1, om)]), X0, Y0, X1, Y1);
+          const double ct = sT[sd * 64 + lane], st = sT[sd * 64 + 32 + lane];
+          double cm, sm;
+          lane_power(m, ct, st, cm, sm);
+          cm *= wgt;
+          sm *= wgt;
+          const double cn = fma(cm, ct, -sm * st), sn = fma(sm, ct, cm * st);
+          c0 = c0 + lin2(cm, X0, -sm, Y0);
+          s0 = s0 + lin2(sm, X0, cm, Y0);
+          c1 = c1 + lin2(cn, X1, -sn, Y1);
+          s1 = s1 + lin2(sn, X1, cn, Y1);
+        }
+        sB[(2 * m) * 32 + lane] = c0;
+        sB[(2 * m + 1) * 32 + lane] = s0;
+        if (m < om) {
+          sB[(2 * m + 2) * 32 + lane] = c1;
+          sB[(2 * m + 3) * 32 + lane] = s1;
+        }
+      }
+      __syncthreads();
+      if (mycol < ncols) {
+        const double2* co = reinterpret_cast<const double2*>(a.coef) + (size_t)ent.x * (kTreeP + 2) * ccol * 2;
+        int at[RG];
+#pragma unroll
+        for (int i = 0; i < RG; ++i) {
+          const int c = min(mycol + i, ncols - 1), comp = c / a.nrhs;
+          at[i] = 2 * ((comp ? set1 : set0) * a.nrhs + c - comp * a.nrhs);
+        }
+        for (int m = 0; m <= om; ++m) {
+          const cplx fc = sB[(2 * m) * 32 + lane], fs = sB[(2 * m + 1) * 32 + lane];
+          const double2* v = co + (size_t)m * ccol * 2;
+#pragma unroll
+          for (int i = 0; i < RG; ++i) {
+            const double2 A = __ldg(v + at[i]), B = __ldg(v + at[i] + 1);
+            cfma(acc[i], cplx{A.x, A.y}, fc);
+            cfma(acc[i], cplx{B.x, B.y}, fs);
+          }
+        }
+      }
+    }
+    if (active) {
+      cplx* part = reinterpret_cast<cplx*>(a.part) + ((size_t)(a.split0 + split) * a.n_tgt + t) * ncols;
+#pragma unroll
+      for (int i = 0; i < RG; ++i)
+        if (mycol + i < ncols) part[mycol + i] = acc[i];
+    }
+  }
+}
+
 // warps per CTA with the most warps on an SM (at least two CTAs on it, where
 // that many fit), and the CTA's shared memory; 0: none fits
 template <typename T>
@@ -844,7 +1247,7 @@ template <typename T>
 cudaError_t launch_far_ops(const TreeArgs& a, cudaStream_t st) {
 #define QBX_FAR(O) case O: return a.nr <= 1 ? launch_far_t<O, T, 1>(a, st) : launch_far_t<O, T, far_nr(O)>(a, st);
   switch (a.ops) {
-    QBX_FAR(1) QBX_FAR(2) QBX_FAR(3) QBX_FAR(4) QBX_FAR(5) QBX_FAR(6) QBX_FAR(7) QBX_FAR(12)
+    QBX_FAR(1) QBX_FAR(2) QBX_FAR(3) QBX_FAR(4) QBX_FAR(5) QBX_FAR(6) QBX_FAR(7) QBX_FAR(12) QBX_FAR(13)
     default: return cudaErrorInvalidValue;
   }
 #undef QBX_FAR
@@ -852,26 +1255,45 @@ cudaError_t launch_far_ops(const TreeArgs& a, cudaStream_t st) {
 
 template <typename T>
 size_t moments_smem(int q_src) {
-  return (size_t)2 * (kTreeP + 3) * (q_src | 1) * sizeof(T);
+  return (size_t)2 * (kTreeP + 4) * (q_src | 1) * sizeof(T);
 }
 
 template <typename T>
-cudaError_t launch_moments_t(const TreeArgs& a, cudaStream_t st) {
-  const size_t smem = moments_smem<T>(a.q_src);
-  cudaError_t e = cudaFuncSetAttribute(k_tree_moments<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_tree_moments<T><<<dim3(a.M, a.lev), 128, smem, st>>>(a);
-  k_tree_fold<<<dim3(a.off[a.lev], a.nset * a.nrhs), 64, 0, st>>>(a);
-  k_tree_local<T><<<dim3(a.n_blk, (a.nset * a.nrhs + kLocCols - 1) / kLocCols), 32 * kLocWarps, 0, st>>>(a);
+size_t disc_moments_smem(int p) {
+  return (size_t)(kTreeP + p + 4) * 32 * 16 + (size_t)(3 * p + 2) * 32 * sizeof(T);
+}
+
+template <typename T>
+cudaError_t launch_moments_t(const TreeArgs& a, cudaStream_t st, int n_inst) {
+  const int ncol = a.nset * a.nrhs;
+  if (a.discs) {
+    const size_t smem = disc_moments_smem<T>(a.p);
+    cudaError_t e = cudaFuncSetAttribute(k_tree_disc_moments<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_tree_disc_moments<T><<<dim3(a.M, a.lev), 32, smem, st>>>(a);
+  } else {
+    const size_t smem = moments_smem<T>(a.q_src);
+    cudaError_t e = cudaFuncSetAttribute(k_tree_moments<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_tree_moments<T><<<dim3(a.M, a.up ? 1 : a.lev, n_inst), 128, smem, st>>>(a);
+  }
+  if (a.up)
+    for (int l = 1; l < a.lev; ++l)
+      k_tree_up<T><<<dim3((a.M + (1 << l) - 1) >> l, (ncol + kUpWarps * kUpCols - 1) / (kUpWarps * kUpCols), n_inst),
+                     32 * kUpWarps, 0, st>>>(a, l);
+  if (!a.up) k_tree_fold<<<dim3(a.off[a.lev], ncol), 64, 0, st>>>(a);
+  if (a.up) k_tree_local<T, 4, 4><<<dim3(a.n_blk, (ncol + 3) / 4, n_inst), 32 * 4, 0, st>>>(a);
+  else k_tree_local<T, 2, 8><<<dim3(a.n_blk, (ncol + 1) / 2, n_inst), 32 * 8, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 int tree_levels(int panels, int q_src, TreeArgs* a) {
+  // (the discs of an adjoint's leaves reach past half a panel: whole panels there)
   // half panels as leaves where that leaves them 16 sources or more: near
   // pairs 2.05 -> 1.65 ms, far nodes 0.77 -> 0.99 ms (starfish, 256 panels)
-  const int half = q_src % 2 == 0 && q_src >= 32;
+  const int half = q_src % 2 == 0 && q_src >= 32 && !a->discs;
   const int M = panels << half;
   a->M = M;
   a->q_src = q_src >> half;
@@ -900,19 +1322,19 @@ size_t tree_layout(TreeArgs* a, char* base) {
   a->far = (int*)take((size_t)a->n_blk * (a->M + 1) * 8);
   a->loc = (int*)take((size_t)a->n_blk * a->M * 8);
   a->cnt = (int*)take((size_t)a->n_blk * 12);
-  a->mom = take((size_t)a->lev * a->M * a->nset * a->nrhs * (kTreeP + 2) * 2 * 16);
-  a->coef = take(nodes * ncol * (kTreeP + 1) * 2 * 16);
+  a->mom = take(a->up ? 0 : (size_t)a->lev * a->M * a->nset * a->nrhs * (kTreeP + 2) * 2 * 16);
+  a->coef = take(nodes * ncol * (kTreeP + 2) * 2 * 16);
   return at;
 }
 
-cudaError_t launch_tree_lists(const TreeArgs& a, cudaStream_t st) {
-  k_tree_nodes<<<a.off[a.lev], 256, 0, st>>>(a);
-  k_tree_lists<<<a.n_blk, 32 * kListWarps, 0, st>>>(a);
+cudaError_t launch_tree_lists(const TreeArgs& a, cudaStream_t st, int n_inst) {
+  k_tree_nodes<<<dim3(a.off[a.lev], 1, n_inst), 256, 0, st>>>(a);
+  k_tree_lists<<<dim3(a.n_blk, 1, n_inst), 32 * kListWarps, 0, st>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_moments(const TreeArgs& a, cudaStream_t st) {
-  return a.kim != 0.0 ? launch_moments_t<cplx>(a, st) : launch_moments_t<double>(a, st);
+cudaError_t launch_tree_moments(const TreeArgs& a, bool ck, cudaStream_t st, int n_inst) {
+  return ck ? launch_moments_t<cplx>(a, st, n_inst) : launch_moments_t<double>(a, st, n_inst);
 }
 
 cudaError_t launch_far_clusters(TreeArgs a, cudaStream_t st) {
@@ -924,6 +1346,105 @@ cudaError_t launch_far_clusters(TreeArgs a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+// Far sums of the adjoint sweeps (columns [split][source][ncol][nrhs]: value,
+// gradient, d_xx, d_xy of the field of conj(g), as ops asks) to one row of
+// their partial sums: conj of the value (S); of n . gradient (D); of value and
+// gradient (S with the source-position gradient); of K_D = n . grad, grad K_D
+// and grad (D's shape sweep, d_yy = -k^2 value - d_xx).
+__global__ void k_adj_far(int mode, int n_src, int nsplit, int ncol, int nrhs, cplx k2, const cplx* in,
+                          const double* snx, const double* sny, cplx* out) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n_src * nrhs) return;
+  const int s = idx / nrhs, r = idx - s * nrhs;
+  cplx v[5];
+  for (int q = 0; q < ncol; ++q) {
+    v[q] = cplx{0.0, 0.0};
+    for (int i = 0; i < nsplit; ++i) v[q] = v[q] + in[(((size_t)i * n_src + s) * ncol + q) * nrhs + r];
+  }
+  const double nx = snx[s], ny = sny[s];
+  cplx o[5];
+  int n = 0;
+  if (mode == 0) {
+    o[n++] = v[0];
+  } else if (mode == 1) {
+    o[n++] = nx * v[0] + ny * v[1];
+  } else if (mode == 2) {
+    for (int q = 0; q < 3; ++q) o[n++] = v[q];
+  } else {
+    const cplx yy = -(k2 * v[0]) - v[3];
+    o[n++] = nx * v[1] + ny * v[2];
+    o[n++] = nx * v[3] + ny * v[4];
+    o[n++] = nx * v[4] + ny * yy;
+    o[n++] = v[1];
+    o[n++] = v[2];
+  }
+  for (int q = 0; q < n; ++q) out[((size_t)s * n + q) * nrhs + r] = conj(o[q]);
+}
+
+cudaError_t launch_adj_far(const TreeArgs& a, int mode, const double* snx, const double* sny, void* row,
+                           cudaStream_t st) {
+  const int ncol = (a.ops & 1) + 2 * (a.ops >> 2 & 1) + 2 * (a.ops >> 3 & 1);
+  const cplx k{a.kre, a.kim};
+  k_adj_far<<<(a.n_tgt * a.nrhs + 127) / 128, 128, 0, st>>>(mode, a.n_tgt, a.nsplit, ncol, a.nrhs, k * k,
+                                                           (const cplx*)a.part, snx, sny, (cplx*)row);
+  return cudaGetLastError();
+}
+
+size_t adj_tree_setup(TreeArgs* t, const qbx_geom* g, int c0, int nc, qbx_c64 k, int p, int ops, int nd, int nrhs,
+                      const double* hk_tab, const void* gc, int num_sms, char* base) {
+  *t = TreeArgs{};
+  if (g->M < kTreeMinPanels) return 0;
+  t->kre = k.re;
+  t->kim = k.im;
+  t->p = p;
+  t->pl = 0;
+  t->nd = nd;
+  t->ops = ops;
+  t->nrhs = nrhs;
+  t->discs = 1;
+  t->sx = g->tgt_x;
+  t->sy = g->tgt_y;
+  t->dcx = g->ctr_x + c0;
+  t->dcy = g->ctr_y + c0;
+  t->n_ctr_n = nc;
+  t->tx = t->cx = g->src_x;
+  t->ty = t->cy = g->src_y;
+  t->n_tgt = t->n_ctr = g->n_src;
+  t->n_blk = (g->n_src + 31) / 32;
+  t->hk_tab = hk_tab;
+  t->wd[0] = gc;
+  tree_columns_discs(t);
+  tree_levels(g->M, g->q_tgt, t);
+  const size_t smem = k.im != 0.0 ? disc_moments_smem<cplx>(p) : disc_moments_smem<double>(p);
+  if (smem > 220 * 1024 || !far_clusters_fit(*t)) return 0;
+  t->nparts = std::max(1, std::min(4, num_sms * 8 / (t->n_blk * 16)));
+  t->nsplit = std::max(1, std::min(4, (num_sms * 2 + t->n_blk - 1) / t->n_blk));
+  size_t at = tree_layout(t, base);
+  const int ncol = (ops & 1) + 2 * (ops >> 2 & 1) + 2 * (ops >> 3 & 1);
+  t->part = base ? base + at : nullptr;
+  return at + host_align256((size_t)t->nsplit * g->n_src * ncol * nrhs * 16);
+}
+
+bool far_group_fit(const TreeArgs& a, bool ck, int nsd) {
+  return (ck ? FarGroupSmem<cplx>::bytes(a.pl, nsd) : FarGroupSmem<double>::bytes(a.pl, nsd)) <= 220 * 1024;
+}
+
+template <typename T, int RG>
+static cudaError_t launch_far_group_t(const TreeArgs& a, cudaStream_t st, int n_inst) {
+  const size_t smem = FarGroupSmem<T>::bytes(a.pl, a.n_ctr / a.n_tgt);
+  auto kern = k_far_group<T, RG>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3((unsigned)a.n_blk * a.nsplit, 1, n_inst), 32 * kFgWarps, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_far_group(const TreeArgs& a, bool ck, cudaStream_t st, int n_inst) {
+  const int cols = ((a.ops & OPB_C) ? 1 : popc3(a.ops)) * a.nrhs;
+  if (cols > 32) return ck ? launch_far_group_t<cplx, 8>(a, st, n_inst) : launch_far_group_t<double, 8>(a, st, n_inst);
+  return ck ? launch_far_group_t<cplx, 4>(a, st, n_inst) : launch_far_group_t<double, 4>(a, st, n_inst);
 }
 
 bool far_clusters_fit(const TreeArgs& a) {
@@ -946,18 +1467,51 @@ static int moment_set(TreeArgs* a, int kind, int slot) {
   return i;
 }
 
+static int shift_set(TreeArgs* a, int moment, int sh) {
+  a->base[a->ncset] = moment;
+  a->shift[a->ncset] = sh;
+  return a->ncset++;
+}
+
+void tree_columns_grad_d(TreeArgs* a, bool sources) {
+  a->nset = a->ncset = 0;
+  const int m = moment_set(a, kSetNormal, 0);
+  a->set_g = a->plain[m];
+  a->set_gx = shift_set(a, m, 1);
+  shift_set(a, m, 2);
+  if (sources) {
+    a->set_x = a->plain[moment_set(a, kSetQuadX, 0)];
+    moment_set(a, kSetQuadY, 0);
+  }
+}
+
+void tree_columns_discs(TreeArgs* a) {
+  a->nset = a->ncset = 0;
+  const int m = moment_set(a, kSetMono, 0);
+  a->set_s = a->set_g = a->plain[m];
+  if (a->ops & OPB_G) {
+    a->set_gx = shift_set(a, m, 1);
+    shift_set(a, m, 2);
+  }
+  if (a->ops & OPB_X) {
+    a->set_x = shift_set(a, m, 3);
+    shift_set(a, m, 4);
+  }
+}
+
 void tree_columns(TreeArgs* a, const int slot[3]) {
   a->nset = a->ncset = 0;
+  if (a->ops & OPB_C) {
+    a->set_d = a->plain[moment_set(a, kSetCombined, slot[1])];
+    return;
+  }
   if (a->ops & OPB_S) a->set_s = a->plain[moment_set(a, kSetMono, slot[0])];
   if (a->ops & OPB_D) a->set_d = a->plain[moment_set(a, kSetNormal, slot[1])];
   if (a->ops & OPB_G) {
     const int m = moment_set(a, kSetMono, slot[2]);
     a->set_g = a->plain[m];
-    a->set_gx = a->ncset;
-    for (int sh = 1; sh <= 2; ++sh) {
-      a->base[a->ncset] = m;
-      a->shift[a->ncset++] = sh;
-    }
+    a->set_gx = shift_set(a, m, 1);
+    shift_set(a, m, 2);
   }
   if (a->ops & OPB_X) {
     a->set_x = a->plain[moment_set(a, kSetX, slot[2])];

@@ -48,12 +48,13 @@ constexpr float kTreeTol = 5e-17f;
 __device__ __forceinline__ int series_order(float kr, float z, float q, float damp, int nd, int limit) {
   if (!(q < 0.75f)) return limit + 1;   // (NaN too)
   const float a = 0.5f * kr, iz = 1.0f / z;
-  const float qlo = fmaxf(1.0f, 0.5f * iz / (1.0f + log1pf(iz)));   // <= |H1/H0|
-  const float fac = 2.0f * damp / (1.0f - q), dw = nd ? 1.0f / (kr * qlo) : 1.0f;
+  // <= |H_nd/H0| (|H_1/H_0| > 1/(2 z (1 + log(1 + 1/z))), |H_2/H_0| > 1/(z^2 (1 + log(1 + 1/z))))
+  const float qlo = fmaxf(1.0f, (nd == 2 ? iz * iz : 0.5f * iz) / (1.0f + log1pf(iz)));
+  const float fac = 2.0f * damp / (1.0f - q), dw = nd == 2 ? 1.0f / (kr * kr * qlo) : nd ? 1.0f / (kr * qlo) : 1.0f;
   float g0 = 1.0f, g1 = a * (1.0f + iz);
   int last = 0;
   for (int l = 1; l <= limit + 1; ++l) {
-    const float w = g1 * fac * (nd ? (float)l * dw : 1.0f);
+    const float w = g1 * fac * (nd == 2 ? (float)(l * l) * dw : nd ? (float)l * dw : 1.0f);
     if (!(w <= kTreeTol)) last = l;
     const float g2 = __fdividef(a, (float)(l + 1)) * (2.0f * l * iz * g1 + __fdividef(a, (float)l) * g0);
     g0 = g1;

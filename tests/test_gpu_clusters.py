@@ -80,6 +80,67 @@ def test_clusters_match_pairs(cuda, case):
         check(got[o], ref[o], (case, o))
 
 
+GROUP = [
+    # M, q_tgt, q_src, k, p, ops ("cfie": the combined field), side, limit, nrhs, eta
+    (16, 16, 64, 5.0, 8, (0,), "int", 0, 16, None),          # fewest panels and columns
+    (19, 12, 40, 9.0, 10, (1,), "ext", 1, 17, None),         # blocks across panels, a ragged column group
+    (37, 7, 33, 7.0, 6, (0, 1), "two", 0, 33, None),         # both sides averaged per pair, 66 columns: two passes
+    (40, 16, 64, 6.0, 12, (0, 1, 2), "two", 0, 16, None),    # with grad S: sides kept apart
+    (40, 16, 64, 3 + 0.5j, 9, (0, 1), "two", 0, 20, None),
+    (36, 16, 64, 6.0, 40, (0, 1), "two", 0, 16, None),       # highest order
+    (33, 16, 64, 8.0, 0, (0, 1), "two", 0, 16, None),        # lowest
+    (64, 16, 64, 12.0, 10, (0, 1), "two", 0, 16, 6.0),       # near-only
+    (64, 16, 64, 100.0, 10, (1,), "int", 0, 24, None),       # no cluster of more than a panel
+    (48, 16, 64, 11.0, 14, "cfie", "two", 0, 1, None),       # one column
+    (48, 16, 64, 11.0, 14, "cfie", "two", 0, 65, None),
+    (48, 16, 64, 4 + 0.3j, 10, "cfie", "two", 0, 9, None),
+]
+
+
+@pytest.mark.parametrize("case", GROUP)
+def test_many_columns_match_pairs(cuda, case):
+    M, qt, qs, k, p, ops, side, limit, nrhs, eta = case
+    side = {"int": qbx.SIDE_INT, "ext": qbx.SIDE_EXT, "two": qbx.SIDE_TWO}[side]
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(qt, qs, n_src=M * qs, n_ctr=2 * M * qt, ncoef=4, nrhs=nrhs)
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M + p, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    pp = pair_plan(g, qt, qs, nrhs, 1 if ops == "cfie" else sum(2 if o == 2 else 1 for o in ops))
+    run = lambda pl: ([qbx.qbx_apply_cfie(pl, g, k, k - 0.5j, p, d)] if ops == "cfie" else
+                      list(qbx.qbx_apply_ops(pl, g, ops, side, limit, k, p, d, eta=eta).values()))
+    got = run(plan)
+    qbx.qbx_sync_status(plan)
+    for i, (a, b) in enumerate(zip(got, run(pp))):
+        check(a, b, (case, i))
+
+
+@pytest.mark.parametrize("side,limit,ops,eta,ck", [("int", 1, (0, 1), 0.0, False), ("two", 0, (0, 1), 0.0, False),
+                                                   ("ext", 0, (1,), 7.0, False), ("two", 0, (0,), 0.0, True)])
+def test_batch_clusters_match_single_curves(cuda, side, limit, ops, eta, ck):
+    """A batch of curves with and without clusters (2 and 9 panels form none)
+    against each curve alone, pair by pair; twice, for the kept counter."""
+    side = {"int": qbx.SIDE_INT, "ext": qbx.SIDE_EXT, "two": qbx.SIDE_TWO}[side]
+    Ms, ks = (40, 9, 64, 16, 12, 33), [5.0, 9.0, 14.0, 3.0, 2.0, 7.0]
+    if ck:
+        ks = [v * (1 + 0.05j) if i % 2 else v for i, v in enumerate(ks)]
+    nrhs, p = 12, 9
+    plan = qbx.Plan(16, 64, n_src=64 * max(Ms), n_ctr=32 * max(Ms), ncoef=2, nrhs=nrhs)
+    cur = W.starfish(0.15, 3)
+    gs = [qbx.qbx_geometry(plan, cur, cur.edges(M)) for M in Ms]
+    ds = [torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+          for M, g in zip(Ms, gs)]
+    b = qbx.Batch(plan, gs, ks, p, ops, side, limit, ds)
+    if eta:
+        b.set_eta(eta)
+    b.apply()
+    out = b.apply()
+    b.status()
+    for g, k, d, o in zip(gs, ks, ds, out):
+        ref = qbx.qbx_apply_ops(pair_plan(g, 16, 64, nrhs, len(ops)), g, ops, side, limit, k, p, d, eta=eta or None)
+        for i in ops:
+            check(o[i], ref[i], (g.M, i))
+
+
 @pytest.mark.parametrize("order", ["dyadic", "shuffled"])
 def test_clusters_on_uneven_and_unordered_panels(cuda, order):
     """Panels refined towards a corner (lengths over a factor of 64), and panels
@@ -102,6 +163,62 @@ def test_clusters_on_uneven_and_unordered_panels(cuda, order):
     ref = qbx.qbx_apply_ops(pair_plan(g, 16, 64, 1, 4), g, (0, 1, 2), qbx.SIDE_EXT, 0, k, p, d)
     for o in (0, 1, 2):
         check(got[o], ref[o], (order, o))
+
+
+ADJ = [
+    # M, q_tgt, q_src, k, p, side, limit, nrhs
+    (16, 16, 64, 5.0, 8, "int", 0, 1),
+    (19, 7, 33, 9.0, 10, "ext", 1, 3),
+    (40, 16, 64, 8.0, 0, "two", 0, 1),
+    (40, 16, 64, 6.0, 40, "two", 0, 1),
+    (48, 12, 40, 4 + 0.5j, 9, "two", 1, 2),
+    (64, 16, 64, 60.0, 12, "int", 0, 1),
+    (96, 16, 64, 12.0, 10, "ext", 0, 8),
+]
+
+
+@pytest.mark.parametrize("case", ADJ)
+@pytest.mark.parametrize("op", [qbx.OP_S, qbx.OP_D])
+def test_adjoint_clusters_match_pairs(cuda, case, op):
+    """The transposed sweep, and the shape gradients, with and without clusters
+    of the centres' discs (and of the sources, second derivatives included)."""
+    M, qt, qs, k, p, side, limit, nrhs = case
+    side = {"int": qbx.SIDE_INT, "ext": qbx.SIDE_EXT, "two": qbx.SIDE_TWO}[side]
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(qt, qs, workspace_bytes=qbx.qbx_shape_adjoint_workspace_bytes(M, qt, qs, p, nrhs))
+    g = geometry(plan, cur, cur.edges(M))
+    d, go = (torch.as_tensor(W.complex_gaussian(M + p + i, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+             for i in (0, 1))
+    al = lambda b: (b + 255) // 256 * 256
+    ck = 16 if isinstance(k, complex) else 8
+    nc = g.n_tgt * (2 if side == qbx.SIDE_TWO else 1)
+    # room for the fixed arrays and two splits of either sweep only
+    small = (2 * al(g.n_src * nrhs * 16) + al(nc * nrhs * 16) + al(nc * 2 * (p + 2) * ck) + al(nc * 32) + al(g.n_tgt * 8)
+             + al(M * 8) + 2 * 2 * nc * 4 * nrhs * 16 + 2 * g.n_src * 5 * nrhs * 16 + 2048)
+    pp = qbx.Plan(qt, qs, workspace_bytes=small)
+    check(qbx.qbx_apply_adjoint(plan, g, op, side, limit, k, p, go),
+          qbx.qbx_apply_adjoint(pp, g, op, side, limit, k, p, go), (case, op))
+    got = qbx.qbx_apply_shape_adjoint(plan, g, side, k, p, d, go, op=op)
+    ref = qbx.qbx_apply_shape_adjoint(pp, g, side, k, p, d, go, op=op)
+    for i, (a, b) in enumerate(zip(got, ref)):
+        # gradients through r = h/2 and the normals: a derivative of the order-p sums more, p/r times their rounding
+        err = float((a - b).abs().max() / b.abs().max())
+        assert np.isfinite(err) and err < 1e-11, (case, op, i, err)
+
+
+@pytest.mark.parametrize("case", [c for c in ADJ if c[4] >= 1])
+def test_grad_d_clusters_match_pairs(cuda, case):
+    M, qt, qs, k, p, side, limit, nrhs = case
+    nrhs = min(nrhs, 3)
+    side = {"int": qbx.SIDE_INT, "ext": qbx.SIDE_EXT, "two": qbx.SIDE_TWO}[side]
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(qt, qs, n_src=M * qs, n_ctr=2 * M * qt, ncoef=4, nrhs=nrhs)
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M + p, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    got = qbx.qbx_apply(plan, g, qbx.OP_GRAD_D, side, limit, k, p, d)
+    qbx.qbx_sync_status(plan)
+    pp = qbx.Plan(qt, qs, workspace_bytes=(g.n_src * nrhs + 2 * g.n_tgt * 2 * nrhs * 3) * 16 + 2048)
+    check(got, qbx.qbx_apply(pp, g, qbx.OP_GRAD_D, side, limit, k, p, d), case)
 
 
 def test_clusters_separate_densities_and_streams(cuda):
