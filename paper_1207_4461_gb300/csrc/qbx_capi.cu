@@ -474,29 +474,96 @@ int qbx_form_locals(qbx_plan* p, const qbx_geom* g, int kind, int side, qbx_c64 
   while (nr > 1 && form_smem_bytes(pp, nr) > 160 * 1024) nr = (nr + 1) / 2;
   if (form_smem_bytes(pp, nr) > 200 * 1024) return fail(QBX_EINVAL, "p = %d too large for form_locals", pp);
   const size_t per_split = (size_t)nc * ncoef * nrhs * 16;
-  const int units = (nc + kFormThreads - 1) / kFormThreads;
-  const int ns = choose_split(p, units, g->n_src, per_split, p->ws_bytes > 256 ? p->ws_bytes - 256 : 0);
-  if (ns < 1) return fail(QBX_ENOMEM, "workspace too small for form_locals (need %zu bytes)", per_split);
+  const int units = apply_units(nc, g->n_tgt);
+  const size_t avail = p->ws_bytes > 256 ? p->ws_bytes - 256 : 0;
+  // distant sources through cluster moments (few columns)
+  TreeArgs tr{};
+  size_t tree_bytes = 0;
+  int ns_far = 0;
+  if (g->M >= kTreeMinPanels && nrhs <= 8) {
+    tr.kre = k.re;
+    tr.kim = k.im;
+    tr.p = tr.pl = pp;
+    tr.nd = kind == QBX_OP_D ? 1 : 0;
+    tr.n_tgt = g->n_tgt;
+    tr.n_ctr = nc;
+    tr.n_blk = apply_units(g->n_tgt, g->n_tgt);
+    tr.ops = QBX_OPS_S;
+    tr.nrhs = nrhs;
+    const int none[3] = {0, 0, 0};
+    tree_columns(&tr, none);
+    if (kind == QBX_OP_D) tr.kind[0] = kSetNormal;
+    tree_levels(g->M, g->q_src, &tr);
+    tree_bytes = align256(tree_layout(&tr, nullptr));
+    ns_far = std::max(1, std::min(8, (p->num_sms * 4 + units - 1) / units));
+    if (!form_far_fit(tr) || avail < tree_bytes + (size_t)(ns_far + 1) * per_split) ns_far = 0;
+  }
+  const bool tree = ns_far > 0;
+  if (!tree) tree_bytes = 0;
+  const int ns_near = choose_split(p, tree ? units / 2 + 1 : units, tree ? std::min(g->n_src, 16 * g->q_src) : g->n_src,
+                                   per_split, avail - tree_bytes - ns_far * per_split);
+  if (ns_near < 1) return fail(QBX_ENOMEM, "workspace too small for form_locals (need %zu bytes)", per_split);
+  const int ns = ns_near + ns_far;
   cudaStream_t st = (cudaStream_t)stream;
-  void* part = (void*)align256((size_t)p->ws);
+  char* base = (char*)align256((size_t)p->ws);
+  void* part = base + tree_bytes;
   FormArgs a{};
   a.kind = kind;
   a.p = pp;
   a.kre = k.re;
   a.kim = k.im;
   a.n_ctr = nc;
+  a.n_tgt = g->n_tgt;
   a.cx = g->ctr_x + c0;
   a.cy = g->ctr_y + c0;
   a.src = SrcView{g->src_x, g->src_y, g->src_nx, g->src_ny, g->n_src};
   a.wd = wdens_src;
   a.nrhs = nrhs;
-  a.nsplit = ns;
-  a.src_per_split = split_len(g->n_src, ns);
+  a.nsplit = ns_near;
+  a.src_per_split = split_len(g->n_src, ns_near);
   a.part = part;
-  for (int r0 = 0; r0 < nrhs; r0 += nr) {
-    a.rhs0 = r0;
-    a.nr = std::min(nr, nrhs - r0);
-    CK(launch_form(a, st), "form kernel");
+  auto pair_sums = [&](cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    for (int r0 = 0; r0 < nrhs && e == cudaSuccess; r0 += nr) {
+      a.rhs0 = r0;
+      a.nr = std::min(nr, nrhs - r0);
+      e = launch_form(a, s);
+    }
+    return e;
+  };
+  if (tree) {
+    tr.sx = g->src_x;
+    tr.sy = g->src_y;
+    tr.snx = g->src_nx;
+    tr.sny = g->src_ny;
+    tr.cx = a.cx;
+    tr.cy = a.cy;
+    tr.tx = g->tgt_x;
+    tr.ty = g->tgt_y;
+    cudaError_t te;
+    tr.hk_tab = host_plan_hk_table(p, k, st, &te);
+    CK(te, "complex-k amplitude table");
+    tr.wd[0] = wdens_src;
+    tree_layout(&tr, base);
+    tr.nsplit = ns_far;
+    tr.split0 = ns_near;
+    tr.part = part;
+    CK(launch_tree_lists(tr, st), "cluster lists");
+    a.near = tr.near;
+    a.near_cnt = tr.cnt;
+    a.near_stride = tr.M;
+    a.near_q = tr.q_src;
+    CK(cudaEventRecord(p->fork, st), "fork event");
+    CK(cudaStreamWaitEvent(p->side, p->fork, 0), "fork");
+    const cudaError_t en = pair_sums(p->side);
+    cudaError_t ef = launch_tree_moments(tr, k.im != 0.0, st);
+    if (ef == cudaSuccess) ef = launch_form_far(tr, st);
+    CK(cudaEventRecord(p->join, p->side), "join event");   // (joined also after an error)
+    CK(cudaStreamWaitEvent(st, p->join, 0), "join");
+    CK(en, "form kernel");
+    CK(ef, "far clusters");
+  } else {
+    CK(pair_sums(st), "form kernel");
   }
   CK(launch_form_finish(nc, ncoef, ns, nrhs, part, alpha, p->d_status, st), "form finish");
   return QBX_OK;
@@ -552,6 +619,50 @@ static int far_impl(qbx_plan* p, const qbx_geom* g, int op, qbx_c64 k, const qbx
   const int ncomp = op == QBX_OP_GRAD_S ? 2 : 1;
   const size_t per_split = (size_t)n_far * ncomp * nrhs * 16;
   const int units = (n_far + kApplyThreads - 1) / kApplyThreads;
+  // clusters pay from about four million pairs on (their moments cost some
+  // 0.15 ms; four million pairs one by one 0.4 ms), for few columns
+  if (g->M >= kTreeMinPanels && nrhs <= 8 && (double)n_far * g->n_src >= 4e6) {
+    FarPointArgs f{};
+    TreeArgs& t = f.t;
+    t.kre = k.re;
+    t.kim = k.im;
+    t.nd = op == QBX_OP_S ? 0 : 1;
+    t.ops = op == QBX_OP_GRAD_S ? QBX_OPS_GRAD_S : QBX_OPS_S;   // D: the value of the dipoles
+    t.nrhs = nrhs;
+    t.sx = g->src_x;
+    t.sy = g->src_y;
+    t.snx = g->src_nx;
+    t.sny = g->src_ny;
+    t.n_tgt = t.n_ctr = 1;
+    const int none[3] = {0, 0, 0};
+    tree_columns(&t, none);
+    if (op == QBX_OP_D) t.kind[0] = kSetNormal;
+    tree_levels(g->M, g->q_src, &t);
+    t.wd[0] = wd;
+    const size_t tb = tree_layout(&t, nullptr);
+    const int ntop = t.off[t.lev] - t.off[t.lev - 1];
+    f.nsplit = std::max(1, std::min(ntop, (p->num_sms * 4 + units - 1) / units));
+    if (avail >= tb + 256 + f.nsplit * per_split) {
+      char* base = (char*)align256((size_t)part);
+      tree_layout(&t, base);
+      f.part = base + tb;
+      f.grad = op == QBX_OP_GRAD_S;
+      f.dip = op == QBX_OP_D;
+      f.n_far = n_far;
+      f.xy = x_far;
+      f.wd = wd;
+      cudaError_t te;
+      t.hk_tab = host_plan_hk_table(p, k, st, &te);
+      CK(te, "complex-k amplitude table");
+      CK(launch_tree_nodes(t, st), "cluster nodes");
+      CK(launch_tree_moments(t, k.im != 0.0, st), "cluster moments");
+      CK(launch_far_points(f, st), "far points");
+      // (the sums carry D's and grad S's factor k already)
+      CK(launch_far_finish(QBX_OP_S, k.re, k.im, n_far, f.nsplit, nrhs * ncomp, f.part, out, p->d_status, st),
+         "far finish");
+      return QBX_OK;
+    }
+  }
   const int ns = choose_split(p, units, g->n_src, per_split, avail);
   if (ns < 1) return fail(QBX_ENOMEM, "workspace too small for the far targets");
   FarArgs a{};
@@ -911,7 +1022,7 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   if (n_far > 0) {
     int op = 0;
     while (!(ops >> op & 1)) ++op;
-    return far_impl(p, g, op, k, (const qbx_c64*)wd, nrhs, n_far, x_far, out_far, part, avail, st);
+    return far_impl(p, g, op, k, (const qbx_c64*)wd, nrhs, n_far, x_far, out_far, base + wd_bytes, avail, st);
   }
   return QBX_OK;
 }
@@ -1063,7 +1174,7 @@ static int grad_d_impl(qbx_plan* p, const qbx_geom* g, int side, int limit, qbx_
   const size_t fixed = b_wd + b_al + b_ev + 512;
   if (p->ws_bytes < fixed) return fail(QBX_ENOMEM, "workspace too small for grad D");
   const size_t per_split = (size_t)nc * ncoef * nrhs * 16;
-  const int units = (nc + kFormThreads - 1) / kFormThreads;
+  const int units = apply_units(nc, g->n_tgt);
   const int ns = choose_split(p, units, g->n_src, per_split, p->ws_bytes - fixed);
   if (ns < 1) return fail(QBX_ENOMEM, "workspace too small for the grad D partial sums");
   CK(cudaSetDevice(p->device), "cudaSetDevice");
@@ -1081,6 +1192,7 @@ static int grad_d_impl(qbx_plan* p, const qbx_geom* g, int side, int limit, qbx_
   a.kre = k.re;
   a.kim = k.im;
   a.n_ctr = nc;
+  a.n_tgt = g->n_tgt;
   a.cx = g->ctr_x + c0;
   a.cy = g->ctr_y + c0;
   a.src = SrcView{g->src_x, g->src_y, g->src_nx, g->src_ny, g->n_src};

@@ -16,7 +16,7 @@ inline int apply_units(int n_ctr, int n_tgt) {
   return (n_tgt + kApplyCentres - 1) / kApplyCentres * (n_ctr / n_tgt);
 }
 constexpr int kSrcTile = 128;        // sources staged in shared memory per step (far, form and grad D kernels)
-constexpr int kFormThreads = 64;     // centres per CTA of form_locals
+constexpr int kFormThreads = 64;     // threads per CTA of form_locals (two warps for 32 centres)
 constexpr int kMaxSplit = 64;        // source splits of the split reductions
 
 struct SrcView {
@@ -94,8 +94,10 @@ cudaError_t launch_far(const FarArgs& a, cudaStream_t st);
 struct FormArgs {
   int kind, p;
   double kre, kim;
-  int n_ctr;
+  int n_ctr, n_tgt;
   const double *cx, *cy;
+  const int *near, *near_cnt;   // near leaves per 32-target block, as ApplyArgs::near (near_q sources each); null: all
+  int near_stride, near_q;
   SrcView src;
   const void* wd;
   int nrhs, rhs0, nr;
@@ -336,6 +338,23 @@ bool far_clusters_fit(const TreeArgs& a);                             // whether
 // target averaged when n_ctr = 2 n_tgt)
 cudaError_t launch_far_group(const TreeArgs& a, bool ck, cudaStream_t st, int n_inst = 1);
 bool far_group_fit(const TreeArgs& a, bool ck, int nsd);
+// Coefficients alpha_l of every centre from its block's far nodes (column set
+// set_s): partial sums [split][n_ctr][2p+1][nrhs] at split0 as FormArgs::part
+cudaError_t launch_form_far(const TreeArgs& a, cudaStream_t st);
+bool form_far_fit(const TreeArgs& a);
+// Plain quadrature at points that share no blocks: every point walks the nodes
+// on its own (columns set_s, or set_gx and the next for the gradient)
+struct FarPointArgs {
+  TreeArgs t;          // nodes and coefficients (no lists)
+  int grad, dip;       // gradient; the pairs of near leaves: D kernel
+  int n_far, nsplit, rhs0, nr;
+  const double* xy;
+  const void* wd;
+  void* part;          // as FarArgs::part
+};
+cudaError_t launch_far_points(FarPointArgs a, cudaStream_t st);
+// nodes and coefficients only
+cudaError_t launch_tree_nodes(const TreeArgs& a, cudaStream_t st);
 // adjoint sweeps: the tree over the discs of the centres, evaluated at the
 // source nodes (columns by ops: value, gradient, second derivatives), its
 // arrays and far sums at `base`; returns their bytes (base null: only those),

@@ -88,28 +88,65 @@ __global__ void k_cap_radius(int n_tgt, const double* tx, const double* ty, cons
   }
 }
 
-// ratio = min_s |x_s - c| / r  (eq. x-c-closest)
-__global__ void k_ratio(int n_ctr, const double* cx, const double* cy, const double* cr, int n_src,
-                        const double* sx, const double* sy, double* ratio) {
-  __shared__ double bx[256], by[256];
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  const int cc = c < n_ctr ? c : n_ctr - 1;
-  const double x = cx[cc], y = cy[cc];
-  double best = INFINITY;
-  for (int base = 0; base < n_src; base += 256) {
-    const int nt = min(256, n_src - base);
-    __syncthreads();
-    for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-      bx[i] = sx[base + i];
-      by[i] = sy[base + i];
+// ratio = min_s |x_s - c| / r  (eq. x-c-closest).  A CTA of eight warps holds
+// 32 centres, one per lane, and the warps share the sources.  The distances are
+// first taken in FP32 relative to the CTA's first centre, with a bound of their
+// error; only sources that can be the closest are then measured in FP64 (the
+// FP32 pipe has 64 times the FP64 rate here).  The all-FP64 loop of one thread
+// per centre: 2.94 ms at 128 panels (4096 centres, 8192 sources).
+constexpr int kRatioWarps = 8, kRatioTile = 128;
+__global__ void __launch_bounds__(32 * kRatioWarps)
+k_ratio(int n_ctr, const double* cx, const double* cy, const double* cr, int n_src, const double* sx, const double* sy,
+        double* ratio) {
+  __shared__ float s_p[kRatioWarps][kRatioTile][3];   // position, its error bound
+  __shared__ float s_ub[kRatioWarps][32];
+  __shared__ double s_best[kRatioWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.x * 32 + lane, cc = min(c, n_ctr - 1), c0 = blockIdx.x * 32;
+  const double x0 = cx[c0], y0 = cy[c0], x = cx[cc], y = cy[cc];
+  const float fx = (float)(x - x0), fy = (float)(y - y0);
+  const float ec = 4e-7f * (fabsf(fx) + fabsf(fy));
+  auto stage = [&](int base) {
+    __syncwarp();
+    for (int i = lane; i < kRatioTile && base + i < n_src; i += 32) {
+      const float bx = (float)(sx[base + i] - x0), by = (float)(sy[base + i] - y0);
+      s_p[warp][i][0] = bx;
+      s_p[warp][i][1] = by;
+      s_p[warp][i][2] = 4e-7f * (fabsf(bx) + fabsf(by));
     }
-    __syncthreads();
+    __syncwarp();
+    return min(kRatioTile, n_src - base);
+  };
+  // upper bound of the smallest distance
+  float ub = INFINITY;
+  for (int base = warp * kRatioTile; base < n_src; base += kRatioWarps * kRatioTile) {
+    const int nt = stage(base);
     for (int j = 0; j < nt; ++j) {
-      const double dx = bx[j] - x, dy = by[j] - y;
-      best = fmin(best, fma(dx, dx, dy * dy));
+      const float dx = s_p[warp][j][0] - fx, dy = s_p[warp][j][1] - fy;
+      ub = fminf(ub, sqrtf(fmaf(dx, dx, dy * dy)) + s_p[warp][j][2]);
     }
   }
-  if (c < n_ctr) ratio[c] = sqrt(best) / cr[c];
+  s_ub[warp][lane] = ub;
+  __syncthreads();
+  for (int w = 0; w < kRatioWarps; ++w) ub = fminf(ub, s_ub[w][lane]);
+  ub = (ub + 2.0f * ec) * 1.000001f;
+  // the sources that may be closer, in FP64 (also those whose FP32 distance is no number)
+  double best = INFINITY;
+  for (int base = warp * kRatioTile; base < n_src; base += kRatioWarps * kRatioTile) {
+    const int nt = stage(base);
+    for (int j = 0; j < nt; ++j) {
+      const float dx = s_p[warp][j][0] - fx, dy = s_p[warp][j][1] - fy;
+      if (sqrtf(fmaf(dx, dx, dy * dy)) - s_p[warp][j][2] > ub) continue;
+      const double ex = sx[base + j] - x, ey = sy[base + j] - y;
+      best = fmin(best, fma(ex, ex, ey * ey));
+    }
+  }
+  s_best[warp][lane] = best;
+  __syncthreads();
+  if (warp == 0 && c < n_ctr) {
+    for (int w = 1; w < kRatioWarps; ++w) best = fmin(best, s_best[w][lane]);
+    ratio[c] = sqrt(best) / cr[c];
+  }
 }
 
 cudaError_t launch_geometry(int M, int q_tgt, int q_src, const double* t_edges,
@@ -128,7 +165,7 @@ cudaError_t launch_geometry(int M, int q_tgt, int q_src, const double* t_edges,
   if (rule == QBX_RADIUS_ADMISSIBLE)
     k_cap_radius<<<(2 * n_t + 255) / 256, 256, 0, st>>>(n_t, g.tgt_x, g.tgt_y, g.tgt_nx, g.tgt_ny, n_s, g.src_x,
                                                        g.src_y, g.ctr_x, g.ctr_y, g.ctr_r);
-  k_ratio<<<(2 * n_t + 255) / 256, 256, 0, st>>>(2 * n_t, g.ctr_x, g.ctr_y, g.ctr_r, n_s, g.src_x,
+  k_ratio<<<(2 * n_t + 31) / 32, 32 * kRatioWarps, 0, st>>>(2 * n_t, g.ctr_x, g.ctr_y, g.ctr_r, n_s, g.src_x,
                                                 g.src_y, g.ctr_ratio);
   return cudaGetLastError();
 }
@@ -311,8 +348,10 @@ cudaError_t launch_far_finish(int op, double kre, double kim, int n_far, int nsp
 }
 
 // ---------------------------------------------------------------------------
-// a4 Unfused coefficients (Sec. 3.3 step 4b).  One thread per centre,
-// accumulators for the 2p+1 orders of `nr` rhs in shared memory.
+// a4 Unfused coefficients (Sec. 3.3 step 4b).  A CTA holds 32 centres of one
+// side, one per lane; its two warps take the sources (all, or the block's near
+// leaves) in turn, with accumulators for the 2p+1 orders of `nr` rhs in shared
+// memory, added up at the end.
 //   S: alpha_l += wd H_l e^{-i l theta},  alpha_{-l} += wd (-1)^l H_l e^{i l theta}
 //   D: alpha^D_l += wd (-1)^l (k/2) [nu F_{-l-1} - conj(nu) F_{-l+1}],
 //      F_m = H_m e^{i m theta}, F_{-m} = (-1)^m H_m e^{-i m theta}
@@ -329,33 +368,44 @@ k_form(FormArgs a) {
   cplx* s_wd = reinterpret_cast<cplx*>(s_ny + kSrcTile);        // [tile][nr]
   cplx* s_acc = s_wd + kSrcTile * nr;                          // [(2p+1)*nr][threads]
   const int tid = threadIdx.x;
-  const int c = blockIdx.x * kFormThreads + tid;
-  const bool active = c < a.n_ctr;
-  const int cc = active ? c : a.n_ctr - 1;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int blks = (a.n_tgt + 31) / 32, side = blockIdx.x / blks, blk = blockIdx.x - side * blks;
+  const bool active = blk * 32 + lane < a.n_tgt;
+  const int c = side * a.n_tgt + (active ? blk * 32 + lane : a.n_tgt - 1);
   const int p = a.p, nl = 2 * p + 1;
   for (int i = 0; i < nl * nr; ++i) s_acc[i * kFormThreads + tid] = cplx{0.0, 0.0};
-  const double cx = a.cx[cc], cy = a.cy[cc];
+  const double cx = a.cx[c], cy = a.cy[c];
   const cplx k = cplx{a.kre, a.kim};
   const cplx hk = 0.5 * k;
-  const int s_begin = blockIdx.y * a.src_per_split;
-  const int s_end = min(a.src.n, s_begin + a.src_per_split);
+  const int* near = a.near ? a.near + (size_t)blk * a.near_stride : nullptr;
+  int s_begin = blockIdx.y * a.src_per_split, s_end = min(a.src.n, s_begin + a.src_per_split);
+  if (near) {
+    const long n = (long)a.near_cnt[3 * blk] * a.near_q;
+    s_begin = (int)(n * blockIdx.y / a.nsplit);
+    s_end = (int)(n * (blockIdx.y + 1) / a.nsplit);
+  }
+  auto source = [&](int v) {   // node index of the v-th source
+    if (!near) return v;
+    const int i = v / a.near_q;
+    return near[i] * a.near_q + (v - i * a.near_q);
+  };
   const cplx* wd = reinterpret_cast<const cplx*>(a.wd);
   for (int base = s_begin; base < s_end; base += kSrcTile) {
     const int nt = min(kSrcTile, s_end - base);
     __syncthreads();
     for (int i = tid; i < nt; i += kFormThreads) {
-      s_x[i] = a.src.x[base + i];
-      s_y[i] = a.src.y[base + i];
-      s_nx[i] = a.src.nx[base + i];
-      s_ny[i] = a.src.ny[base + i];
+      const int s = source(base + i);
+      s_x[i] = a.src.x[s];
+      s_y[i] = a.src.y[s];
+      s_nx[i] = a.src.nx[s];
+      s_ny[i] = a.src.ny[s];
     }
     for (int i = tid; i < nt * nr; i += kFormThreads) {
       const int s = i / nr, rr = i - s * nr;
-      s_wd[i] = wd[(size_t)(base + s) * a.nrhs + a.rhs0 + rr];
+      s_wd[i] = wd[(size_t)source(base + s) * a.nrhs + a.rhs0 + rr];
     }
     __syncthreads();
-    if (!active) continue;
-    for (int j = 0; j < nt; ++j) {
+    for (int j = warp; j < nt; j += kFormThreads / 32) {
       const double dx = s_x[j] - cx, dy = s_y[j] - cy;
       const double rho2 = fma(dx, dx, dy * dy);
       const double inv = rsqrt(rho2);
@@ -439,12 +489,15 @@ k_form(FormArgs a) {
       }
     }
   }
+  __syncthreads();
   if (!active) return;
   cplx* part = reinterpret_cast<cplx*>(a.part);
-  for (int l = 0; l < nl; ++l)
-    for (int rr = 0; rr < nr; ++rr)
-      part[(((size_t)blockIdx.y * a.n_ctr + c) * nl + l) * a.nrhs + a.rhs0 + rr] =
-          s_acc[((size_t)l * nr + rr) * kFormThreads + tid];
+  for (int i = warp; i < nl * nr; i += kFormThreads / 32) {   // the warps' sums in warp order
+    cplx u = s_acc[(size_t)i * kFormThreads + lane];
+    for (int w = 1; w < kFormThreads / 32; ++w) u = u + s_acc[(size_t)i * kFormThreads + 32 * w + lane];
+    const int l = i / nr, rr = i - l * nr;
+    part[(((size_t)blockIdx.y * a.n_ctr + c) * nl + l) * a.nrhs + a.rhs0 + rr] = u;
+  }
 }
 
 size_t form_smem_bytes(int p, int nr) {
@@ -457,7 +510,7 @@ cudaError_t launch_form(const FormArgs& a, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_form, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((a.n_ctr + kFormThreads - 1) / kFormThreads, a.nsplit);
+  dim3 grid(apply_units(a.n_ctr, a.n_tgt), a.nsplit);
   k_form<<<grid, kFormThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
@@ -579,26 +632,64 @@ cudaError_t launch_eval(const EvalArgs& a, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // Centre assignment for off-surface points (smallest |x-c|/r <= 1, lowest index).
 // ---------------------------------------------------------------------------
-__global__ void k_assign(int n, const double* xy, int n_ctr, const double* cx, const double* cy,
-                         const double* cr, int* out) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  const double x = xy[2 * e], y = xy[2 * e + 1];
+// A CTA of eight warps holds 32 points, one per lane, and the warps share the
+// centres; a centre is measured in FP64 only where FP32 (relative to the CTA's
+// first point) leaves open whether its disc holds the point.  The all-FP64
+// loop of one thread per point: 2.28 ms for 2048 points and centres.
+constexpr int kAssignWarps = 8;
+__global__ void __launch_bounds__(32 * kAssignWarps)
+k_assign(int n, const double* xy, int n_ctr, const double* cx, const double* cy, const double* cr, int* out) {
+  __shared__ float s_p[kAssignWarps][32][3];
+  __shared__ double s_q[kAssignWarps][32];
+  __shared__ int s_i[kAssignWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane, ee = min(e, n - 1), e0 = blockIdx.x * 32;
+  const double x0 = xy[2 * e0], y0 = xy[2 * e0 + 1], x = xy[2 * ee], y = xy[2 * ee + 1];
+  const float fx = (float)(x - x0), fy = (float)(y - y0);
   int best = -1;
   double bq = INFINITY;
-  for (int c = 0; c < n_ctr; ++c) {
-    const double q = hypot(x - cx[c], y - cy[c]) / cr[c];
-    if (q <= 1.0 && q < bq) {
-      bq = q;
-      best = c;
+  for (int base = warp * 32; base < n_ctr; base += kAssignWarps * 32) {
+    __syncwarp();
+    if (base + lane < n_ctr) {
+      const float bx = (float)(cx[base + lane] - x0), by = (float)(cy[base + lane] - y0);
+      s_p[warp][lane][0] = bx;
+      s_p[warp][lane][1] = by;
+      // a distance beyond this cannot lie inside the disc
+      const float r = (float)cr[base + lane];
+      s_p[warp][lane][2] = r > 0.0f ? r * 1.00001f + 4e-7f * (fabsf(bx) + fabsf(by)) : INFINITY;
+    }
+    __syncwarp();
+    const float ex = 8e-7f * (fabsf(fx) + fabsf(fy));
+    for (int j = 0; j < min(32, n_ctr - base); ++j) {
+      const float dx = s_p[warp][j][0] - fx, dy = s_p[warp][j][1] - fy;
+      if (sqrtf(fmaf(dx, dx, dy * dy)) > s_p[warp][j][2] + ex) continue;
+      const int c = base + j;
+      const double q = hypot(x - cx[c], y - cy[c]) / cr[c];
+      if (q <= 1.0 && q < bq) {
+        bq = q;
+        best = c;
+      }
     }
   }
-  out[e] = best;
+  s_q[warp][lane] = bq;
+  s_i[warp][lane] = best;
+  __syncthreads();
+  if (warp == 0 && e < n) {
+    for (int w = 1; w < kAssignWarps; ++w) {   // ties to the lowest index
+      const double q = s_q[w][lane];
+      const int i = s_i[w][lane];
+      if (i >= 0 && (best < 0 || q < bq || (q == bq && i < best))) {
+        bq = q;
+        best = i;
+      }
+    }
+    out[e] = best;
+  }
 }
 
 cudaError_t launch_assign(int n, const double* xy, int n_ctr, const double* cx, const double* cy,
                           const double* cr, int* out, cudaStream_t st) {
-  k_assign<<<(n + 127) / 128, 128, 0, st>>>(n, xy, n_ctr, cx, cy, cr, out);
+  k_assign<<<(n + 31) / 32, 32 * kAssignWarps, 0, st>>>(n, xy, n_ctr, cx, cy, cr, out);
   return cudaGetLastError();
 }
 

@@ -1204,6 +1204,218 @@ __global__ void __launch_bounds__(32 * kFgWarps) k_far_group(TreeArgs q) {
   }
 }
 
+// Coefficients alpha_l, |l| <= p, of every centre from the far nodes of its
+// block: the translation of k_tree_local to each centre (lane), with the
+// directions Theta of the lanes apart,
+//   alpha_l = e^{-il Theta} (S_l + T_l)/2, alpha_{-l} = (-1)^l e^{il Theta} (S_l - T_l)/2.
+template <typename T>
+__host__ __device__ size_t form_far_bytes(int p) {   // per warp: waves, s_m and d_m, the sums
+  return ((size_t)(kTreeP + p + 2) + 2 * (kTreeP + 1) + (2 * p + 1)) * 32 * 16;
+}
+template <typename T>
+__global__ void __launch_bounds__(64) k_form_far(TreeArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int p = a.p, nl = 2 * p + 1, W = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  cplx* sH = reinterpret_cast<cplx*>(smem_raw + (size_t)warp * form_far_bytes<T>(p)) + lane;
+  cplx* sD = sH + (kTreeP + p + 2) * 32;          // [kTreeP + 1][2][32]
+  cplx* sA = sD + 2 * (kTreeP + 1) * 32;          // [2p + 1][32]
+  const int units = a.n_blk * (a.n_ctr / a.n_tgt);
+  const int unit = blockIdx.x % units, split = blockIdx.x / units, r = blockIdx.y;
+  const int side = unit / a.n_blk, blk = unit - side * a.n_blk;
+  const bool active = blk * 32 + lane < a.n_tgt;
+  const int t = active ? blk * 32 + lane : a.n_tgt - 1, c = side * a.n_tgt + t;
+  const double cx = a.cx[c], cy = a.cy[c], rad = hypot(a.tx[t] - cx, a.ty[t] - cy);
+  KW<T> kw;
+  kw.init(a.kre, a.kim, a.hk_tab);
+  const T kk = kw.kval();
+  const float ka = (float)sc_abs(kk);
+  for (int l = 0; l < nl; ++l) sA[l * 32] = cplx{0.0, 0.0};
+  const int cnt = a.cnt[3 * blk + 1], ncol = a.ncset * a.nrhs;
+  const int2* far = reinterpret_cast<const int2*>(a.far) + (size_t)blk * (a.M + 1);
+  for (int e = split * W + warp; e < cnt; e += a.nsplit * W) {
+    int2 ent = far[cnt - 1 - e];
+    const int om = ent.y & 0xff;
+    ent.y = (ent.y & ~0xff00) | p << 8;   // every order l <= p
+    const double* nd = a.node + 4 * (size_t)ent.x;
+    double ct, st;
+    int lmax;
+    __syncwarp();
+    far_waves<T>(kw, kk, ka, ent, a.nd, a.kim, nd, cx - nd[0], cy - nd[1], rad, sH, ct, st, lmax);
+    const double2* co = reinterpret_cast<const double2*>(a.coef) +
+                        ((size_t)ent.x * (kTreeP + 2) * ncol + (size_t)a.set_s * a.nrhs + r) * 2;
+    double cm = 1.0, sm = 0.0;
+    for (int m = 0; m <= om; ++m) {
+      const double2 A = __ldg(co + (size_t)m * ncol * 2), B = __ldg(co + (size_t)m * ncol * 2 + 1);
+      sD[(2 * m) * 32] = cplx{fma(A.x, cm, B.x * sm), fma(A.y, cm, B.y * sm)};
+      sD[(2 * m + 1) * 32] = cplx{fma(B.y, cm, -A.y * sm), fma(A.x, sm, -B.x * cm)};
+      const double cn = fma(cm, ct, -sm * st);
+      sm = fma(sm, ct, cm * st);
+      cm = cn;
+    }
+    double cl = 0.5, sl = 0.0;   // e^{i l Theta} / 2
+    for (int l = 0; l <= p; ++l) {
+      cplx S{0.0, 0.0}, D{0.0, 0.0};
+      for (int m = 0; m <= om; ++m) {
+        const int d = m - l;
+        const cplx ha = neg_if(d < 0 && (d & 1), sH[(d < 0 ? -d : d) * 32]);
+        const cplx hb = neg_if(l & 1, sH[(m + l) * 32]);
+        cfma(S, sD[(2 * m) * 32], ha + hb);
+        cfma(D, sD[(2 * m + 1) * 32], ha - hb);
+      }
+      const cplx e{cl, sl};
+      sA[(p + l) * 32] = sA[(p + l) * 32] + conj(e) * (S + D);
+      if (l > 0) sA[(p - l) * 32] = sA[(p - l) * 32] + neg_if(l & 1, e * (S - D));
+      const double cn = fma(cl, ct, -sl * st);
+      sl = fma(sl, ct, cl * st);
+      cl = cn;
+    }
+  }
+  __syncthreads();
+  if (!active) return;
+  cplx* part = reinterpret_cast<cplx*>(a.part) + ((size_t)(a.split0 + split) * a.n_ctr + c) * nl * a.nrhs + r;
+  for (int l = warp; l < nl; l += W) {   // the warps' sums in warp order
+    const cplx* v = reinterpret_cast<const cplx*>(smem_raw) + ((kTreeP + p + 2) + 2 * (kTreeP + 1) + l) * 32 + lane;
+    cplx u = *v;
+    for (int w = 1; w < W; ++w) u = u + v[w * (form_far_bytes<T>(p) / 16)];
+    part[(size_t)l * a.nrhs] = u;
+  }
+}
+
+// Plain quadrature at points anywhere: a lane owns a point and walks the nodes
+// from the top of its share of the curve, taking a node whose disc is far
+// enough through its moments, descending otherwise, and a leaf that never is
+// source by source.  The lanes of a warp step together: each finds its next
+// node, then all evaluate theirs (points in random order share no node, so
+// lists per block would hold every leaf).  About 15 FP64 instructions per order
+// of a node, 100 per source of a leaf.
+template <typename T, int NR, bool GRAD>
+__global__ void __launch_bounds__(128) k_far_points(FarPointArgs q) {
+  const TreeArgs& a = q.t;
+  constexpr int kC = GRAD ? 2 : 1;
+  const int chunks = (q.n_far + 127) / 128;
+  const int e = (int)(blockIdx.x % chunks) * 128 + threadIdx.x, split = blockIdx.x / chunks;
+  const bool active = e < q.n_far;
+  const int ee = active ? e : q.n_far - 1;
+  const double x = q.xy[2 * ee], y = q.xy[2 * ee + 1];
+  KW<T> kw;
+  kw.init(a.kre, a.kim, a.hk_tab);
+  const T kk = kw.kval();
+  const float ka = (float)sc_abs(kk), ki = (float)a.kim;
+  cplx acc[kC][NR];
+#pragma unroll
+  for (int g = 0; g < kC; ++g)
+#pragma unroll
+    for (int i = 0; i < NR; ++i) acc[g][i] = cplx{0.0, 0.0};
+  const int top = a.lev - 1, ntop = a.off[top + 1] - a.off[top], ncol = a.ncset * a.nrhs;
+  int l = top, j = (int)((long)ntop * split / q.nsplit);
+  const int jend = (int)((long)ntop * (split + 1) / q.nsplit);   // of the top level
+  const int set = GRAD ? a.set_gx : a.set_s;
+  const cplx* wd = reinterpret_cast<const cplx*>(q.wd);
+  for (;;) {
+    // ---- the next node to take: om >= 0 through its moments, -1 a near leaf ----
+    int om = 0, id = -1;
+    while ((j << l) < a.M && (j >> (top - l)) < jend) {
+      const double* n = a.node + 4 * (size_t)(a.off[l] + j);
+      const float dx = (float)(x - n[0]), dy = (float)(y - n[1]), R = (float)n[2] * 1.00001f;
+      const float d = 0.99999f * sqrtf(fmaf(dx, dx, dy * dy));
+      om = kTreeP + 1;
+      if (d > 1.34f * R) {
+        om = series_order(ka * R, ka * d, R / d, expf(2.0f * ki * R), a.nd, kTreeP);
+        if (om <= kTreeP) {
+          const float o = (float)om;   // H and the moments of order om stay in range
+          if (!(o * log10f(fmaxf(2.0f * o / (2.7f * ka * d), 1.0f)) < 280.0f) ||
+              !(o * log10f(fmaxf(2.0f * o / (2.7f * ka * R), 1.0f)) < 280.0f))
+            om = kTreeP + 1;
+        }
+      }
+      if (om > kTreeP && l > 0) {   // descend
+        --l;
+        j <<= 1;
+        continue;
+      }
+      id = a.off[l] + j;
+      if (om > kTreeP) om = -1;
+      ++j;
+      while (l < top && !(j & 1)) {
+        j >>= 1;
+        ++l;
+      }
+      break;
+    }
+    if (!__any_sync(0xffffffffu, id >= 0)) break;
+    if (id < 0) continue;
+    if (om >= 0) {
+      const double* n = a.node + 4 * (size_t)id;
+      const double vx = x - n[0], vy = y - n[1];
+      double inv, rho, yq;
+      kw.geom(fma(vx, vx, vy * vy), inv, rho, yq);
+      cplx h, h1;
+      T twoz;
+      kw.hankel(rho, inv, yq, h, h1, twoz);
+      const double ct = vx * inv, st = vy * inv;
+      T s = twoz;
+      double cm = 1.0, sm = 0.0;
+      const double2* co =
+          reinterpret_cast<const double2*>(a.coef) + ((size_t)id * (kTreeP + 2) * ncol + (size_t)set * a.nrhs + q.rhs0) * 2;
+      for (int m = 0; m <= om; ++m) {
+        const cplx fc = cm * h, fs = sm * h;
+#pragma unroll
+        for (int g = 0; g < kC; ++g)
+#pragma unroll
+          for (int i = 0; i < NR; ++i) {
+            if (i > 0 && i >= q.nr) break;
+            const double2* v = co + ((size_t)m * ncol + (size_t)g * a.nrhs + i) * 2;
+            const double2 A = __ldg(v), B = __ldg(v + 1);
+            cfma(acc[g][i], cplx{A.x, A.y}, fc);
+            cfma(acc[g][i], cplx{B.x, B.y}, fs);
+          }
+        const cplx h2 = hrec(s, h1, h);
+        h = h1;
+        h1 = h2;
+        s = sadd(s, twoz);
+        const double cn = fma(cm, ct, -sm * st);
+        sm = fma(sm, ct, cm * st);
+        cm = cn;
+      }
+    } else {
+      const int s0 = (id - a.off[0]) * a.q_src;
+      for (int i0 = 0; i0 < a.q_src; ++i0) {
+        const int sr = s0 + i0;
+        const double rx = x - __ldg(a.sx + sr), ry = y - __ldg(a.sy + sr);
+        double inv, d, yq;
+        kw.geom(fma(rx, rx, ry * ry), inv, d, yq);
+        cplx h0, h1;
+        T twoz;
+        kw.hankel(d, inv, yq, h0, h1, twoz);
+        cplx v[2];
+        if (GRAD) {
+          const cplx g = -smul(kk, h1);
+          v[0] = (rx * inv) * g;
+          v[1] = (ry * inv) * g;
+        } else {
+          v[0] = q.dip ? smul(rmul(kk, fma(rx, __ldg(a.snx + sr), ry * __ldg(a.sny + sr)) * inv), h1) : h0;
+        }
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+          if (i > 0 && i >= q.nr) break;
+          const cplx w = wd[(size_t)sr * a.nrhs + q.rhs0 + i];
+#pragma unroll
+          for (int g = 0; g < kC; ++g) cfma(acc[g][i], w, v[g]);
+        }
+      }
+    }
+  }
+  if (!active) return;
+  cplx* part = reinterpret_cast<cplx*>(q.part);
+#pragma unroll
+  for (int g = 0; g < kC; ++g)
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      if (i >= q.nr) break;
+      part[(((size_t)split * q.n_far + e) * kC + g) * a.nrhs + q.rhs0 + i] = acc[g][i];
+    }
+}
+
 // warps per CTA with the most warps on an SM (at least two CTAs on it, where
 // that many fit), and the CTA's shared memory; 0: none fits
 template <typename T>
@@ -1282,6 +1494,7 @@ cudaError_t launch_moments_t(const TreeArgs& a, cudaStream_t st, int n_inst) {
       k_tree_up<T><<<dim3((a.M + (1 << l) - 1) >> l, (ncol + kUpWarps * kUpCols - 1) / (kUpWarps * kUpCols), n_inst),
                      32 * kUpWarps, 0, st>>>(a, l);
   if (!a.up) k_tree_fold<<<dim3(a.off[a.lev], ncol), 64, 0, st>>>(a);
+  if (a.n_blk == 0) return cudaGetLastError();
   if (a.up) k_tree_local<T, 4, 4><<<dim3(a.n_blk, (ncol + 3) / 4, n_inst), 32 * 4, 0, st>>>(a);
   else k_tree_local<T, 2, 8><<<dim3(a.n_blk, (ncol + 1) / 2, n_inst), 32 * 8, 0, st>>>(a);
   return cudaGetLastError();
@@ -1343,6 +1556,47 @@ cudaError_t launch_far_clusters(TreeArgs a, cudaStream_t st) {
     a.rhs0 = r0;
     a.nr = std::min(n, a.nrhs - r0);
     const cudaError_t e = a.kim != 0.0 ? launch_far_ops<cplx>(a, st) : launch_far_ops<double>(a, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_tree_nodes(const TreeArgs& a, cudaStream_t st) {
+  k_tree_nodes<<<a.off[a.lev], 256, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <typename T>
+static int form_far_warps(int p) { return 2 * form_far_bytes<T>(p) <= 200 * 1024 ? 2 : form_far_bytes<T>(p) <= 200 * 1024 ? 1 : 0; }
+bool form_far_fit(const TreeArgs& a) { return form_far_warps<double>(a.p) > 0; }
+
+template <typename T>
+static cudaError_t launch_form_far_t(const TreeArgs& a, cudaStream_t st) {
+  const int w = form_far_warps<T>(a.p);
+  const size_t smem = w * form_far_bytes<T>(a.p);
+  cudaError_t e = cudaFuncSetAttribute(k_form_far<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_form_far<T><<<dim3((unsigned)(a.n_blk * (a.n_ctr / a.n_tgt)) * a.nsplit, a.nrhs), 32 * w, smem, st>>>(a);
+  return cudaGetLastError();
+}
+cudaError_t launch_form_far(const TreeArgs& a, cudaStream_t st) {
+  return a.kim != 0.0 ? launch_form_far_t<cplx>(a, st) : launch_form_far_t<double>(a, st);
+}
+
+template <typename T, int NR>
+static cudaError_t launch_far_points_t(const FarPointArgs& a, cudaStream_t st) {
+  const unsigned grid = (unsigned)((a.n_far + 127) / 128) * (unsigned)a.nsplit;
+  if (a.grad) k_far_points<T, NR, true><<<grid, 128, 0, st>>>(a);
+  else k_far_points<T, NR, false><<<grid, 128, 0, st>>>(a);
+  return cudaGetLastError();
+}
+cudaError_t launch_far_points(FarPointArgs a, cudaStream_t st) {
+  for (int r0 = 0; r0 < a.t.nrhs; r0 += 4) {
+    a.rhs0 = r0;
+    a.nr = std::min(4, a.t.nrhs - r0);
+    cudaError_t e;
+    if (a.t.kim != 0.0) e = a.nr == 1 ? launch_far_points_t<cplx, 1>(a, st) : launch_far_points_t<cplx, 4>(a, st);
+    else e = a.nr == 1 ? launch_far_points_t<double, 1>(a, st) : launch_far_points_t<double, 4>(a, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -221,6 +221,90 @@ def test_grad_d_clusters_match_pairs(cuda, case):
     check(got, qbx.qbx_apply(pp, g, qbx.OP_GRAD_D, side, limit, k, p, d), case)
 
 
+@pytest.mark.parametrize("M,qt,qs,k,p,kind,side,nrhs", [
+    (16, 16, 64, 5.0, 8, 0, "int", 1), (33, 7, 33, 9.0, 10, 1, "ext", 3), (40, 16, 64, 6.0, 40, 1, "two", 1),
+    (40, 16, 64, 8.0, 0, 0, "two", 8), (48, 12, 40, 4 + 0.5j, 9, 1, "two", 2), (64, 16, 64, 70.0, 12, 0, "int", 1)])
+def test_locals_clusters_match_pairs(cuda, M, qt, qs, k, p, kind, side, nrhs):
+    """Stored coefficients, each order against its own largest value, and the
+    expansions evaluated at half the radius."""
+    side = {"int": qbx.SIDE_INT, "ext": qbx.SIDE_EXT, "two": qbx.SIDE_TWO}[side]
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(qt, qs, n_src=M * qs, n_ctr=2 * M * qt, ncoef=2 * p + 1, nrhs=nrhs)
+    g = geometry(plan, cur, cur.edges(M))
+    w = torch.as_tensor(W.complex_gaussian(M + p, g.n_src * nrhs).reshape(g.n_src, nrhs), device="cuda")
+    nc = g.n_tgt * (2 if side == qbx.SIDE_TWO else 1)
+    pp = qbx.Plan(qt, qs, workspace_bytes=nc * (2 * p + 1) * nrhs * 16 * 2 + 1024)
+    got, ref = (qbx.qbx_form_locals(pl, g, kind, side, k, p, w) for pl in (plan, pp))
+    qbx.qbx_sync_status(plan)
+    for l in range(2 * p + 1):
+        check(got[:, l], ref[:, l], (M, p, l - p))
+    e = torch.arange(0, nc, 3, device="cuda", dtype=torch.int32)
+    o = g.n_tgt if side == qbx.SIDE_EXT else 0
+    ex = (g["ctr_x"][o:o + nc] + 0.5 * g["ctr_r"][o:o + nc])[e.long()].contiguous()
+    ey = g["ctr_y"][o:o + nc][e.long()].contiguous()
+    ev = [qbx.qbx_eval_locals(plan, g, side, k, p, a, ex=ex, ey=ey, ectr=e) for a in (got, ref)]
+    check(ev[0], ev[1], (M, p))
+
+
+@pytest.mark.parametrize("op,k,nrhs", [(qbx.OP_S, 9.0, 1), (qbx.OP_D, 9.0, 3), (qbx.OP_GRAD_S, 20.0, 1),
+                                       (qbx.OP_R, 5 + 0.5j, 5), (qbx.OP_GRAD_S, 3 + 0.2j, 8), (qbx.OP_S, 150.0, 2)])
+def test_far_points_clusters_match_pairs(cuda, op, k, nrhs):
+    """Points in random order, from 1e-3 off the curve to far away, and one on a
+    cluster's centre, where no cluster of it may be used."""
+    M = 64
+    plan = qbx.Plan(16, 64, n_src=M * 64, n_ctr=4000, ncoef=2, nrhs=nrhs)
+    cur = W.starfish(0.2, 3)
+    g = geometry(plan, cur, cur.edges(M))
+    rng = np.random.default_rng(4)
+    t = rng.uniform(0, 2 * np.pi, 1999)
+    xy = cur(t)[0] * (1.0 + 10.0 ** rng.uniform(-3, 1.5, t.size))[:, None]
+    xy[0] = [float(g["src_x"][:64].mean()), float(g["src_y"][:64].mean())]
+    x = torch.as_tensor(xy, device="cuda")
+    w = torch.as_tensor(W.complex_gaussian(7, g.n_src * nrhs).reshape(g.n_src, nrhs), device="cuda")
+    comp = 2 if op == qbx.OP_GRAD_S else 1
+    got = qbx.qbx_far(plan, g, op, k, w, x)
+    qbx.qbx_sync_status(plan)
+    pp = qbx.Plan(16, 64, workspace_bytes=len(t) * comp * nrhs * 16 * 2 + 2048 + g.n_src * 16)
+    check(got, qbx.qbx_far(pp, g, op, k, w, x), (op, k))
+
+
+def test_on_surface_with_far_points_fills_one_workspace(cuda):
+    """Far points of an on-surface call share its workspace with the clusters."""
+    M, n = 40, 3000
+    plan = qbx.Plan(16, 64, n_src=M * 64, n_ctr=n, ncoef=2, nrhs=1)
+    cur = W.starfish()
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(2, g.n_tgt).reshape(-1, 1), device="cuda")
+    th = torch.linspace(0, 6.28, n, dtype=torch.float64, device="cuda")
+    x = torch.stack([2 * torch.cos(th), 2 * torch.sin(th)], 1)
+    on, far = qbx.qbx_apply(plan, g, qbx.OP_GRAD_S, qbx.SIDE_TWO, 0, 7.0, 8, d, x_far=x)
+    pp = pair_plan(g, 16, 64, 1, 2)
+    check(on, qbx.qbx_apply(pp, g, qbx.OP_GRAD_S, qbx.SIDE_TWO, 0, 7.0, 8, d), "on")
+    p2 = qbx.Plan(16, 64, workspace_bytes=n * 2 * 16 * 2 + 2048)
+    check(far, qbx.qbx_far(p2, g, qbx.OP_GRAD_S, 7.0, qbx.qbx_upsample(plan, g, d), x), "far")
+
+
+def test_ratio_and_assignment_on_refined_panels(cuda):
+    """Nearest-source ratios and disc assignment against numpy over panels whose
+    lengths differ by 2^10 (the FP32 screening must not lose the nearest)."""
+    edges = W.dyadic_edges(10, 10)
+    M = len(edges) - 1
+    plan = qbx.Plan(16, 64, workspace_bytes=1 << 20)
+    g = qbx.qbx_geometry(plan, W.teardrop(), edges)
+    c = np.stack([g["ctr_x"].cpu().numpy(), g["ctr_y"].cpu().numpy()], 1)
+    s = np.stack([g["src_x"].cpu().numpy(), g["src_y"].cpu().numpy()], 1)
+    r = g["ctr_r"].cpu().numpy()
+    ref = np.array([np.sqrt(((s - q) ** 2).sum(1).min()) for q in c]) / r
+    assert np.abs(g["ctr_ratio"].cpu().numpy() / ref - 1).max() < 1e-14
+    rng = np.random.default_rng(1)
+    i = rng.integers(0, g.n_tgt, 700)
+    xy = c[i] + r[i, None] * rng.uniform(-0.9, 0.9, (700, 2))
+    got = qbx.qbx_assign_centres(plan, g, qbx.SIDE_INT, torch.as_tensor(xy, device="cuda")).cpu().numpy()
+    q = np.hypot(xy[:, None, 0] - c[None, :g.n_tgt, 0], xy[:, None, 1] - c[None, :g.n_tgt, 1]) / r[None, :g.n_tgt]
+    want = np.where(q.min(1) <= 1.0, q.argmin(1), -1)
+    assert np.array_equal(got, want)
+
+
 def test_clusters_separate_densities_and_streams(cuda):
     """One density per operator, and the call on a stream of its own followed
     by work on that stream (the pair sums run beside it and join it)."""
