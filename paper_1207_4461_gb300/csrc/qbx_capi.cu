@@ -522,6 +522,11 @@ int qbx_form_locals(qbx_plan* p, const qbx_geom* g, int kind, int side, qbx_c64 
   a.nsplit = ns_near;
   a.src_per_split = split_len(g->n_src, ns_near);
   a.part = part;
+  {
+    cudaError_t te;
+    a.hk_tab = host_plan_hk_table(p, k, st, &te);
+    CK(te, "complex-k amplitude table");
+  }
   auto pair_sums = [&](cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     for (int r0 = 0; r0 < nrhs && e == cudaSuccess; r0 += nr) {
@@ -540,9 +545,7 @@ int qbx_form_locals(qbx_plan* p, const qbx_geom* g, int kind, int side, qbx_c64 
     tr.cy = a.cy;
     tr.tx = g->tgt_x;
     tr.ty = g->tgt_y;
-    cudaError_t te;
-    tr.hk_tab = host_plan_hk_table(p, k, st, &te);
-    CK(te, "complex-k amplitude table");
+    tr.hk_tab = a.hk_tab;
     tr.wd[0] = wdens_src;
     tree_layout(&tr, base);
     tr.nsplit = ns_far;
@@ -1201,6 +1204,11 @@ static int grad_d_impl(qbx_plan* p, const qbx_geom* g, int side, int limit, qbx_
   a.nsplit = ns;
   a.src_per_split = split_len(g->n_src, ns);
   a.part = part;
+  {
+    cudaError_t te;
+    a.hk_tab = host_plan_hk_table(p, k, st, &te);
+    CK(te, "complex-k amplitude table");
+  }
   for (int r0 = 0; r0 < nrhs; r0 += nr) {
     a.rhs0 = r0;
     a.nr = std::min(nr, nrhs - r0);

@@ -103,6 +103,7 @@ struct FormArgs {
   int nrhs, rhs0, nr;
   int nsplit, src_per_split;
   void* part;             // [nsplit][n_ctr][2p+1][nrhs]
+  const double* hk_tab;   // complex k: the amplitude table of this k's ray, or null
 };
 cudaError_t launch_form(const FormArgs& a, cudaStream_t st);
 size_t form_smem_bytes(int p, int nr);

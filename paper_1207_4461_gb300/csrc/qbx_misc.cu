@@ -3,7 +3,7 @@
 // with the jump epilogue (a7), centre assignment and diagnostics.
 #include <cuda_runtime.h>
 #include <stdint.h>
-#include "qbx_device.cuh"
+#include "qbx_apply_impl.cuh"
 #include "qbx_internal.h"
 
 namespace qbx {
@@ -98,45 +98,63 @@ constexpr int kRatioWarps = 8, kRatioTile = 128;
 __global__ void __launch_bounds__(32 * kRatioWarps)
 k_ratio(int n_ctr, const double* cx, const double* cy, const double* cr, int n_src, const double* sx, const double* sy,
         double* ratio) {
-  __shared__ float s_p[kRatioWarps][kRatioTile][3];   // position, its error bound
+  __shared__ float2 s_p[kRatioWarps][kRatioTile];
   __shared__ float s_ub[kRatioWarps][32];
   __shared__ double s_best[kRatioWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane, cc = min(c, n_ctr - 1), c0 = blockIdx.x * 32;
   const double x0 = cx[c0], y0 = cy[c0], x = cx[cc], y = cy[cc];
   const float fx = (float)(x - x0), fy = (float)(y - y0);
-  const float ec = 4e-7f * (fabsf(fx) + fabsf(fy));
+  float ec = 4e-7f * (fabsf(fx) + fabsf(fy));
+  for (int o = 16; o > 0; o >>= 1) ec = fmaxf(ec, __shfl_xor_sync(0xffffffffu, ec, o));
+  // one tile of sources relative to the first centre; returns the error bound
+  // of its distances (to any of the centres)
   auto stage = [&](int base) {
     __syncwarp();
+    float e = 0.0f;
     for (int i = lane; i < kRatioTile && base + i < n_src; i += 32) {
       const float bx = (float)(sx[base + i] - x0), by = (float)(sy[base + i] - y0);
-      s_p[warp][i][0] = bx;
-      s_p[warp][i][1] = by;
-      s_p[warp][i][2] = 4e-7f * (fabsf(bx) + fabsf(by));
+      s_p[warp][i] = make_float2(bx, by);
+      e = fmaxf(e, 4e-7f * (fabsf(bx) + fabsf(by)));
     }
+    for (int o = 16; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
     __syncwarp();
-    return min(kRatioTile, n_src - base);
+    return e + ec;
+  };
+  auto dist2 = [&](int j) {
+    const float2 v = s_p[warp][j];
+    const float dx = v.x - fx, dy = v.y - fy;
+    return fmaf(dx, dx, dy * dy);
   };
   // upper bound of the smallest distance
   float ub = INFINITY;
   for (int base = warp * kRatioTile; base < n_src; base += kRatioWarps * kRatioTile) {
-    const int nt = stage(base);
-    for (int j = 0; j < nt; ++j) {
-      const float dx = s_p[warp][j][0] - fx, dy = s_p[warp][j][1] - fy;
-      ub = fminf(ub, sqrtf(fmaf(dx, dx, dy * dy)) + s_p[warp][j][2]);
-    }
+    const float e = stage(base);
+    const int nt = min(kRatioTile, n_src - base);
+    float m = INFINITY;
+#pragma unroll 8
+    for (int j = 0; j < nt; ++j) m = fminf(m, dist2(j));
+    ub = fminf(ub, sqrtf(m) + e);
   }
   s_ub[warp][lane] = ub;
   __syncthreads();
   for (int w = 0; w < kRatioWarps; ++w) ub = fminf(ub, s_ub[w][lane]);
-  ub = (ub + 2.0f * ec) * 1.000001f;
   // the sources that may be closer, in FP64 (also those whose FP32 distance is no number)
   double best = INFINITY;
   for (int base = warp * kRatioTile; base < n_src; base += kRatioWarps * kRatioTile) {
-    const int nt = stage(base);
+    const float e = stage(base), t = (ub + e) * 1.000001f, t2 = t * t;
+    const int nt = min(kRatioTile, n_src - base);
+    float m = INFINITY;   // a tile with none, at the price of the minimum
+    bool odd = false;
+#pragma unroll 8
     for (int j = 0; j < nt; ++j) {
-      const float dx = s_p[warp][j][0] - fx, dy = s_p[warp][j][1] - fy;
-      if (sqrtf(fmaf(dx, dx, dy * dy)) - s_p[warp][j][2] > ub) continue;
+      const float v = dist2(j);
+      odd |= !(v <= 3e38f);
+      m = fminf(m, v);
+    }
+    if (!odd && m > t2) continue;
+    for (int j = 0; j < nt; ++j) {
+      if (dist2(j) > t2) continue;
       const double ex = sx[base + j] - x, ey = sy[base + j] - y;
       best = fmin(best, fma(ex, ex, ey * ey));
     }
@@ -352,167 +370,140 @@ cudaError_t launch_far_finish(int op, double kre, double kim, int n_far, int nsp
 // side, one per lane; its two warps take the sources (all, or the block's near
 // leaves) in turn, with accumulators for the 2p+1 orders of `nr` rhs in shared
 // memory, added up at the end.
-//   S: alpha_l += wd H_l e^{-i l theta},  alpha_{-l} += wd (-1)^l H_l e^{i l theta}
-//   D: alpha^D_l += wd (-1)^l (k/2) [nu F_{-l-1} - conj(nu) F_{-l+1}],
-//      F_m = H_m e^{i m theta}, F_{-m} = (-1)^m H_m e^{-i m theta}
 // (factor i/4 in the finishing kernel).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kFormThreads)
-k_form(FormArgs a) {
+// With E_n = H_n e^{-i n theta}, E_{-n} = (-1)^n H_n e^{i n theta}:
+//   S: alpha_l += w E_l;  D: alpha_l += w (k/2)[conj(nu) E_{l-1} - nu E_{l+1}]
+// (the factor k/2 on the sums).  ONE: a single rhs, w folded into the seeds
+// H_0, H_1; otherwise one product per rhs.
+template <typename T, bool ONE>
+__global__ void __launch_bounds__(kFormThreads) k_form(FormArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* s_x = reinterpret_cast<double*>(smem_raw);
-  double* s_y = s_x + kSrcTile;
-  double* s_nx = s_y + kSrcTile;
-  double* s_ny = s_nx + kSrcTile;
-  const int nr = a.nr;
-  cplx* s_wd = reinterpret_cast<cplx*>(s_ny + kSrcTile);        // [tile][nr]
-  cplx* s_acc = s_wd + kSrcTile * nr;                          // [(2p+1)*nr][threads]
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
+  cplx* s_acc = reinterpret_cast<cplx*>(smem_raw);              // [(2p+1)*nr][threads]
+  const int nr = ONE ? 1 : a.nr;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int blks = (a.n_tgt + 31) / 32, side = blockIdx.x / blks, blk = blockIdx.x - side * blks;
   const bool active = blk * 32 + lane < a.n_tgt;
   const int c = side * a.n_tgt + (active ? blk * 32 + lane : a.n_tgt - 1);
   const int p = a.p, nl = 2 * p + 1;
   for (int i = 0; i < nl * nr; ++i) s_acc[i * kFormThreads + tid] = cplx{0.0, 0.0};
   const double cx = a.cx[c], cy = a.cy[c];
-  const cplx k = cplx{a.kre, a.kim};
-  const cplx hk = 0.5 * k;
+  KW<T> kw;
+  kw.init(a.kre, a.kim, a.hk_tab);
   const int* near = a.near ? a.near + (size_t)blk * a.near_stride : nullptr;
-  int s_begin = blockIdx.y * a.src_per_split, s_end = min(a.src.n, s_begin + a.src_per_split);
+  int v0 = blockIdx.y * a.src_per_split, v1 = min(a.src.n, v0 + a.src_per_split);
   if (near) {
     const long n = (long)a.near_cnt[3 * blk] * a.near_q;
-    s_begin = (int)(n * blockIdx.y / a.nsplit);
-    s_end = (int)(n * (blockIdx.y + 1) / a.nsplit);
+    v0 = (int)(n * blockIdx.y / a.nsplit);
+    v1 = (int)(n * (blockIdx.y + 1) / a.nsplit);
   }
-  auto source = [&](int v) {   // node index of the v-th source
-    if (!near) return v;
-    const int i = v / a.near_q;
-    return near[i] * a.near_q + (v - i * a.near_q);
-  };
-  const cplx* wd = reinterpret_cast<const cplx*>(a.wd);
-  for (int base = s_begin; base < s_end; base += kSrcTile) {
-    const int nt = min(kSrcTile, s_end - base);
-    __syncthreads();
-    for (int i = tid; i < nt; i += kFormThreads) {
-      const int s = source(base + i);
-      s_x[i] = a.src.x[s];
-      s_y[i] = a.src.y[s];
-      s_nx[i] = a.src.nx[s];
-      s_ny[i] = a.src.ny[s];
+  const double2* wd = reinterpret_cast<const double2*>(a.wd) + a.rhs0;
+  for (int v = v0 + warp; v < v1; v += kFormThreads / 32) {
+    int s = v;
+    if (near) {
+      const int i = v / a.near_q;
+      s = near[i] * a.near_q + (v - i * a.near_q);
     }
-    for (int i = tid; i < nt * nr; i += kFormThreads) {
-      const int s = i / nr, rr = i - s * nr;
-      s_wd[i] = wd[(size_t)source(base + s) * a.nrhs + a.rhs0 + rr];
+    const double dx = __ldg(a.src.x + s) - cx, dy = __ldg(a.src.y + s) - cy;
+    double inv, rho, yq;
+    kw.geom(fma(dx, dx, dy * dy), inv, rho, yq);
+    const double ct = dx * inv, st = dy * inv;
+    cplx Hm, H;   // H_{n-1}, H_n
+    T twoz;
+    if constexpr (ONE) {
+      const double2 w = __ldg(wd + (size_t)s * a.nrhs);
+      kw.hankel_w(rho, inv, yq, cplx{w.x, w.y}, Hm, H, twoz);
+    } else {
+      kw.hankel(rho, inv, yq, Hm, H, twoz);
     }
-    __syncthreads();
-    for (int j = warp; j < nt; j += kFormThreads / 32) {
-      const double dx = s_x[j] - cx, dy = s_y[j] - cy;
-      const double rho2 = fma(dx, dx, dy * dy);
-      const double inv = rsqrt(rho2);
-      const double rho = rho2 * inv;
-      const cplx e1 = cplx{dx * inv, -dy * inv};   // e^{-i theta}
-      cplx H0, H1;
-      cplx twoz;
-      if (a.kim == 0.0) {
-        const double z = a.kre * rho, invz = inv / a.kre;
-        hankel01_real(z, invz, sqrt(invz), H0, H1);
-        twoz = cplx{2.0 * invz, 0.0};
-      } else {
-        const cplx z = cplx{a.kre * rho, a.kim * rho};
-        hankel01_cplx(z, H0, H1);
-        twoz = 2.0 * cinv(z);
+    auto add = [&](int l, cplx v_) {   // alpha_l, l = -p..p
+#pragma unroll 1
+      for (int rr = 0; rr < nr; ++rr) {
+        cplx* A = s_acc + ((size_t)(l + p) * nr + rr) * kFormThreads + tid;
+        if constexpr (ONE) {
+          *A = *A + v_;
+        } else {
+          const double2 w = __ldg(wd + (size_t)s * a.nrhs + rr);
+          cplx u = *A;
+          cfma(u, cplx{w.x, w.y}, v_);
+          *A = u;
+        }
       }
-      if (a.kind == QBX_OP_S) {
-        cplx Hm = H0, H = H1, E = cplx{1.0, 0.0};   // E = e^{-i l theta}
-        cplx s = twoz;
-        for (int l = 0; l <= p; ++l) {
-          const cplx Hl = (l == 0) ? H0 : H;
-          const cplx Kp = Hl * E;                          // H_l e^{-i l theta}
-          const cplx Km = ((l & 1) ? -1.0 : 1.0) * (Hl * conj(E));
-          for (int rr = 0; rr < nr; ++rr) {
-            const cplx w = s_wd[j * nr + rr];
-            cplx* A = s_acc + ((size_t)(l + p) * nr + rr) * kFormThreads + tid;
-            *A = *A + w * Kp;
-            if (l > 0) {
-              cplx* B = s_acc + ((size_t)(p - l) * nr + rr) * kFormThreads + tid;
-              *B = *B + w * Km;
-            }
-          }
-          E = E * e1;
-          if (l >= 1) {
-            const cplx Hn = s * H - Hm;
-            Hm = H;
-            H = Hn;
-            s = s + twoz;
-          }
+    };
+    double cn = ct, sn = st;   // n theta
+    T sz = twoz;
+    auto waves = [&](cplx& Ep, cplx& En, int n) {   // E_n, E_{-n} of H
+      const cplx hc = cn * H, hs = sn * H;
+      Ep = cplx{hc.re + hs.im, hc.im - hs.re};      // H (cos - i sin)
+      En = cplx{hc.re - hs.im, hc.im + hs.re};
+      if (n & 1) En = -En;
+    };
+    auto step = [&] {
+      const cplx h = hrec(sz, H, Hm);
+      Hm = H;
+      H = h;
+      sz = sadd(sz, twoz);
+      const double c2 = fma(cn, ct, -sn * st);
+      sn = fma(sn, ct, cn * st);
+      cn = c2;
+    };
+    if (a.kind == QBX_OP_S) {
+      add(0, Hm);
+      for (int n = 1; n <= p; ++n) {
+        cplx Ep, En;
+        waves(Ep, En, n);
+        add(n, Ep);
+        add(-n, En);
+        if (n < p) step();
+      }
+    } else {
+      const double nx = __ldg(a.src.nx + s), ny = __ldg(a.src.ny + s);
+      const cplx nu{nx, ny}, nub{nx, -ny};
+      // at n: E_{+-n}, E_{+-(n-1)}, E_{+-(n-2)}; alpha_{n-1} and alpha_{-(n-1)} complete
+      cplx E1p = Hm, E1n = Hm, E2p{0.0, 0.0}, E2n{0.0, 0.0};
+      for (int n = 1; n <= p + 1; ++n) {
+        cplx Ep, En;
+        waves(Ep, En, n);
+        if (n == 1) {
+          add(0, nub * En - nu * Ep);
+        } else {
+          add(n - 1, nub * E2p - nu * Ep);
+          add(1 - n, nub * En - nu * E2n);
         }
-      } else {
-        // sliding window of F_{+n}, F_{-n} for n, n-1, n-2
-        const cplx nu = cplx{s_nx[j], s_ny[j]};
-        const cplx nub = conj(nu);
-        cplx Hm = H0, H = H1;
-        cplx s = twoz;
-        cplx E = cplx{1.0, 0.0};          // e^{-i n theta}
-        cplx Fp0{0, 0}, Fm0{0, 0}, Fp1{0, 0}, Fm1{0, 0}, Fp2{0, 0}, Fm2{0, 0};   // index n, n-1, n-2
-        for (int n = 0; n <= p + 1; ++n) {
-          const cplx Hn_ = (n == 0) ? H0 : H;
-          const double sg = (n & 1) ? -1.0 : 1.0;
-          Fp2 = Fp1; Fm2 = Fm1; Fp1 = Fp0; Fm1 = Fm0;
-          Fp0 = Hn_ * conj(E);              // F_{+n} = H_n e^{i n theta}
-          Fm0 = sg * (Hn_ * E);             // F_{-n} = (-1)^n H_n e^{-i n theta}
-          if (n >= 1) {
-            const int l = n - 1;
-            const double sl = (l & 1) ? -1.0 : 1.0;
-            // alpha^D_l (l >= 0): nu F_{-l-1} - conj(nu) F_{-l+1}
-            const cplx Fl1 = (l == 0) ? Fp0 : Fm2;   // F_{-l+1}: l = 0 -> F_{+1}
-            const cplx kp = (sl * hk) * (nu * Fm0 - nub * Fl1);
-            cplx km{0, 0};
-            if (l >= 1) km = (sl * hk) * (nu * Fp2 - nub * Fp0);   // l' = -l: F_{l-1}, F_{l+1}
-            for (int rr = 0; rr < nr; ++rr) {
-              const cplx w = s_wd[j * nr + rr];
-              cplx* A = s_acc + ((size_t)(l + p) * nr + rr) * kFormThreads + tid;
-              *A = *A + w * kp;
-              if (l >= 1) {
-                cplx* B = s_acc + ((size_t)(p - l) * nr + rr) * kFormThreads + tid;
-                *B = *B + w * km;
-              }
-            }
-          }
-          E = E * e1;
-          if (n >= 1) {
-            const cplx Hn = s * H - Hm;
-            Hm = H;
-            H = Hn;
-            s = s + twoz;
-          }
-        }
+        E2p = E1p;
+        E2n = E1n;
+        E1p = Ep;
+        E1n = En;
+        if (n <= p) step();
       }
     }
   }
   __syncthreads();
   if (!active) return;
+  const cplx f = a.kind == QBX_OP_S ? cplx{1.0, 0.0} : cplx{0.5 * a.kre, 0.5 * a.kim};
   cplx* part = reinterpret_cast<cplx*>(a.part);
   for (int i = warp; i < nl * nr; i += kFormThreads / 32) {   // the warps' sums in warp order
     cplx u = s_acc[(size_t)i * kFormThreads + lane];
     for (int w = 1; w < kFormThreads / 32; ++w) u = u + s_acc[(size_t)i * kFormThreads + 32 * w + lane];
     const int l = i / nr, rr = i - l * nr;
-    part[(((size_t)blockIdx.y * a.n_ctr + c) * nl + l) * a.nrhs + a.rhs0 + rr] = u;
+    part[(((size_t)blockIdx.y * a.n_ctr + c) * nl + l) * a.nrhs + a.rhs0 + rr] = f * u;
   }
 }
 
-size_t form_smem_bytes(int p, int nr) {
-  return 4 * kSrcTile * sizeof(double) + (size_t)kSrcTile * nr * 16 +
-         (size_t)(2 * p + 1) * nr * kFormThreads * 16;
+size_t form_smem_bytes(int p, int nr) { return (size_t)(2 * p + 1) * nr * kFormThreads * 16; }
+
+template <typename T>
+static cudaError_t launch_form_t(const FormArgs& a, cudaStream_t st) {
+  const size_t smem = form_smem_bytes(a.p, a.nr);
+  auto kern = a.nr == 1 ? k_form<T, true> : k_form<T, false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(apply_units(a.n_ctr, a.n_tgt), a.nsplit), kFormThreads, smem, st>>>(a);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_form(const FormArgs& a, cudaStream_t st) {
-  const size_t smem = form_smem_bytes(a.p, a.nr);
-  cudaError_t e = cudaFuncSetAttribute(k_form, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(apply_units(a.n_ctr, a.n_tgt), a.nsplit);
-  k_form<<<grid, kFormThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  return a.kim != 0.0 ? launch_form_t<cplx>(a, st) : launch_form_t<double>(a, st);
 }
 
 __global__ void k_form_finish(int n_ctr, int ncoef, int nsplit, int nrhs, const cplx* part,
