@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
+#include <cooperative_groups.h>
+#include <algorithm>
 #include "../../include/qbx.h"
 #include "qbx_device.cuh"
 #include "qbx_internal.h"
@@ -74,12 +76,17 @@ __global__ void k_dots_pass1(int n, int nrhs, int nv, const cplx* V, const cplx*
   }
 }
 
+// one warp per product: its lanes take every 32nd partial sum, then a tree
 __global__ void k_dots_pass2(int nblocks, int nrhs, int nv, const cplx* part, cplx* out) {
-  const int jr = blockIdx.x * blockDim.x + threadIdx.x;
+  const int jr = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (jr >= nv * nrhs) return;
   cplx acc{0.0, 0.0};
-  for (int b = 0; b < nblocks; ++b) acc = acc + part[(size_t)b * nv * nrhs + jr];
-  out[jr] = acc;
+  for (int b = lane; b < nblocks; b += 32) acc = acc + part[(size_t)b * nv * nrhs + jr];
+  for (int o = 16; o > 0; o >>= 1) {
+    acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
+    acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
+  }
+  if (lane == 0) out[jr] = acc;
 }
 
 // w -= sum_j V_j h[j][r]
@@ -155,7 +162,7 @@ int qbx_vec_dots(int n, int nrhs, int nv, const qbx_c64* V, const qbx_c64* w, qb
   cudaStream_t st = (cudaStream_t)stream;
   k_dots_pass1<<<dim3(kRedBlocks, nv), kRedThreads, kRedThreads * sizeof(cplx), st>>>(n, nrhs, nv, (const cplx*)V,
                                                                             (const cplx*)w, (cplx*)work);
-  k_dots_pass2<<<blocks((long)nv * nrhs), 256, 0, st>>>(kRedBlocks, nrhs, nv, (const cplx*)work, (cplx*)out);
+  k_dots_pass2<<<blocks(32 * (long)nv * nrhs), 256, 0, st>>>(kRedBlocks, nrhs, nv, (const cplx*)work, (cplx*)out);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? QBX_OK : gcuda(e, "dot kernels");
 }
@@ -207,7 +214,7 @@ int qbx_vec_combine(int n, int nrhs, int nv, const qbx_c64* V, const qbx_c64* y,
 namespace {
 
 // control block
-enum { C_J = 0, C_DONE, C_TOTAL, C_MAXITER, C_M, C_ACTIVE, C_NOTCONV, C_JDONE, C_N };
+enum { C_J = 0, C_DONE, C_TOTAL, C_MAXITER, C_M, C_ACTIVE, C_NOTCONV, C_JDONE, C_TICKET, C_N };
 
 struct Dev {
   void* p = nullptr;
@@ -225,134 +232,237 @@ struct GraphGuard {
   }
 };
 
-// start of a step: is it active?
-__global__ void k_gate(int* ctl) {
+// after ctl[C_J], C_DONE or C_TOTAL changed: does the next step run?
+__device__ void set_active(int* ctl) {
   ctl[C_ACTIVE] = (!ctl[C_DONE] && ctl[C_TOTAL] < ctl[C_MAXITER] && ctl[C_J] < ctl[C_M]) ? 1 : 0;
 }
 
-// out = V_{j + off} (dir 0) or V_{j + off} = in (dir 1)
-__global__ void k_basis_copy(long vec, const cplx* V, cplx* Vw, const int* ctl, int off, int dir, const cplx* in,
-                             cplx* out) {
-  if (!ctl[C_ACTIVE]) return;
-  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= vec) return;
-  const long b = (long)(ctl[C_J] + off) * vec;
-  if (dir == 0) out[idx] = V[b + idx];
-  else Vw[b + idx] = in[idx];
+// s[0 .. R) = the sums over q < S of s[q R + .] in a fixed order (a tree over
+// q); sub = this thread's q (threads with sub >= S only take part in the barriers)
+template <typename V>
+__device__ __forceinline__ void tree_sum(V* s, int R, int S, int sub) {
+  for (int h = S; h > 1;) {
+    const int half = (h + 1) >> 1;
+    __syncthreads();
+    if (sub < h - half) s[threadIdx.x] = s[threadIdx.x] + s[threadIdx.x + half * R];
+    h = half;
+  }
+  __syncthreads();
 }
 
-// partial dots of the step: which = 0: V_0..V_j against V_{j+1} (nv = j + 1);
-// which = 1: V_{j+1} against itself (nv = 1).  Same decomposition and order
-// as k_dots_pass1; blocks beyond nv return.
-__global__ void k_dots_step1(int n, int nrhs, const cplx* V, const int* ctl, int which, cplx* part) {
+constexpr int kDotCluster = 8, kDotThreads = 256, kDotRows = 76;   // CTAs per vector; threads; clusters
+
+// h[jv][r] = <V_jv, V_{j+1}>, jv <= j.  A cluster of 8 CTAs per vector, its
+// CTAs' sums added in rank order through distributed shared memory, so that
+// one launch gives the finished products; 76 clusters (all resident at once)
+// take the vectors in turn.  FP64-bound from some 20 vectors on (4 multiply-
+// adds per element).  With 152 row ranges x (m + 1) vectors of CTAs, most of
+// which had nothing to do, and a second kernel for the 152 sums, the products
+// of one step at n = 1152, 16 right-hand sides took 23 us, now 8.
+__global__ void __cluster_dims__(kDotCluster, 1, 1) __launch_bounds__(kDotThreads)
+k_dots_step(int n, int nrhs, const cplx* __restrict__ V, const int* ctl, cplx* h) {
   if (!ctl[C_ACTIVE]) return;
-  const int j = ctl[C_J];
-  const int nv = which == 0 ? j + 1 : 1;
-  const int jv = blockIdx.y;
-  if (jv >= nv) return;
-  extern __shared__ cplx sred[];
+  __shared__ cplx sred[kDotThreads];
+  __shared__ cplx stot[2][kDotThreads];
+  auto cluster = cooperative_groups::this_cluster();
+  const int nv = ctl[C_J] + 1, rank = blockIdx.x;
   const size_t vec = (size_t)n * nrhs;
-  const cplx* Vj = V + (which == 0 ? (size_t)jv : (size_t)(j + 1)) * vec;
-  const cplx* w = V + (size_t)(j + 1) * vec;
+  const cplx* w = V + (size_t)nv * vec;
+  const int per = (n + kDotCluster - 1) / kDotCluster;
+  const int i0 = min(n, rank * per), i1 = min(n, i0 + per);
+  const int R = min(nrhs, kDotThreads), S = kDotThreads / R;
+  const int rr = threadIdx.x % R, sub = threadIdx.x / R;
+  int buf = 0;
+  for (int jv = blockIdx.y; jv < nv; jv += gridDim.y) {
+    const cplx* Vj = V + (size_t)jv * vec;
+    for (int r0 = 0; r0 < nrhs; r0 += R) {
+      const int r = r0 + rr;
+      cplx acc{0.0, 0.0};
+      if (sub < S && r < nrhs) {
+#pragma unroll 4
+        for (int i = i0 + sub; i < i1; i += S) acc = acc + conj(Vj[(size_t)i * nrhs + r]) * w[(size_t)i * nrhs + r];
+      }
+      sred[threadIdx.x] = acc;
+      tree_sum(sred, R, S, sub);
+      if (sub == 0) stot[buf][rr] = sred[rr];
+      cluster.sync();   // (a buffer is written again only after the next one's barrier)
+      if (rank == 0 && sub == 0 && r < nrhs) {
+        cplx tot = stot[buf][rr];
+#pragma unroll
+        for (int q = 1; q < kDotCluster; ++q) tot = tot + cluster.map_shared_rank(stot[buf], q)[rr];
+        h[(size_t)jv * nrhs + r] = tot;
+      }
+      buf ^= 1;
+    }
+  }
+  cluster.sync();   // rank 0 has read the others' shared memory
+}
+
+constexpr int kOrthThreads = 512;
+
+// V_{j+1} -= sum_{i <= j} V_i h[i][r]; NORM: also the partial ||V_{j+1}||^2 of
+// the CTA's rows, part[block][r].  152 row ranges; where a range has fewer
+// rows than the CTA has room for, up to 8 threads share an element's vectors
+// (one warp alone reaches an eighth of the FP64 rate).
+template <bool NORM>
+__global__ void __launch_bounds__(kOrthThreads) k_orth_step(int n, int nrhs, cplx* __restrict__ V,
+                                                            const cplx* __restrict__ h, const int* ctl, double* part) {
+  if (!ctl[C_ACTIVE]) return;
+  __shared__ cplx sred[kOrthThreads];
+  __shared__ double snrm[kOrthThreads];
+  const int nv = ctl[C_J] + 1;
+  const size_t vec = (size_t)n * nrhs;
+  cplx* w = V + (size_t)nv * vec;
   const int per = (n + gridDim.x - 1) / gridDim.x;
-  const int i0 = blockIdx.x * per, i1 = min(n, i0 + per);
-  const int R = min(nrhs, (int)blockDim.x), S = blockDim.x / R;
+  const int i0 = min(n, (int)blockIdx.x * per), i1 = min(n, i0 + per);
+  const int R = min(nrhs, kOrthThreads), S = kOrthThreads / R;
+  const int rows = min(per, S), Q = min(8, S / rows);   // rows per pass, threads per element
+  const int rr = threadIdx.x % R, sub = threadIdx.x / R, row = sub % rows, qp = sub / rows;
+  for (int r0 = 0; r0 < nrhs; r0 += R) {
+    const int r = r0 + rr;
+    double nrm = 0.0;
+    for (int ib = i0; ib < i1; ib += rows) {
+      const int i = ib + row;
+      const bool act = qp < Q && r < nrhs && i < i1;
+      const size_t idx = (size_t)i * nrhs + r;
+      cplx acc{0.0, 0.0};
+      if (act) {
+        if (qp == 0) acc = w[idx];
+#pragma unroll 4
+        for (int q = qp; q < nv; q += Q) acc = acc - V[(size_t)q * vec + idx] * h[(size_t)q * nrhs + r];
+      }
+      if (Q > 1) {
+        sred[threadIdx.x] = acc;
+        __syncthreads();
+        if (act && qp == 0)
+          for (int q = 1; q < Q; ++q) acc = acc + sred[threadIdx.x + q * rows * R];
+        __syncthreads();
+      }
+      if (act && qp == 0) {
+        w[idx] = acc;
+        if (NORM) nrm += abs2(acc);
+      }
+    }
+    if (NORM) {
+      snrm[threadIdx.x] = nrm;
+      tree_sum(snrm, R, S, sub);
+      if (sub == 0 && r < nrhs) part[(size_t)blockIdx.x * nrhs + r] = snrm[rr];
+      __syncthreads();
+    }
+  }
+}
+
+// End of a step.  Every CTA adds the partial norms (in a fixed order) and
+// scales its rows, V_{j+1} *= 1 / ||V_{j+1}|| (0 where not finite); the CTA
+// that finishes last then takes the Hessenberg column of every system: h(i) =
+// h1 + h2 (i <= j), h(j+1) = ||V_{j+1}||; the earlier rotations, a new one
+// zeroing h(j+1), the updated g, the residual estimate |g_{j+1}| / ||f|| and
+// the convergence test.  A rotation is (a, b) -> (conj(c) a + s b, c b - s a)
+// with s real (h(j+1) is); only a <- c b - s a is a chain, two multiply-adds
+// per rotation in one warp, the products around it are formed by all threads.
+// One thread per system for the whole column, with the column in global
+// memory, took 21 us at j = 30, in registers 14; now 4.
+constexpr int kRotItems = 1024, kRotRhs = 128;
+__global__ void __launch_bounds__(256) k_finish_step(int n, int nrhs, int m, cplx* __restrict__ V,
+                                                     const double* __restrict__ part, int npart, const cplx* __restrict__ h1,
+                                                     const cplx* __restrict__ h2, double* hn, cplx* __restrict__ Hm,
+                                                     cplx* __restrict__ cs, cplx* __restrict__ sn, cplx* gv, const double* fnorm, double* rel, double tol,
+                                                     int* ctl) {
+  if (!ctl[C_ACTIVE]) return;
+  __shared__ double s[256];
+  __shared__ int s_last;
+  const int j = ctl[C_J];
+  cplx* w = V + (size_t)(j + 1) * n * nrhs;
+  const int per = (n + gridDim.x - 1) / gridDim.x;
+  const int i0 = min(n, (int)blockIdx.x * per), i1 = min(n, i0 + per);
+  const int R = min(nrhs, 256), S = 256 / R;
   const int rr = threadIdx.x % R, sub = threadIdx.x / R;
   for (int r0 = 0; r0 < nrhs; r0 += R) {
     const int r = r0 + rr;
-    cplx acc{0.0, 0.0};
+    double acc = 0.0;
     if (sub < S && r < nrhs) {
 #pragma unroll 4
-      for (int i = i0 + sub; i < i1; i += S) acc = acc + conj(Vj[(size_t)i * nrhs + r]) * w[(size_t)i * nrhs + r];
+      for (int b = sub; b < npart; b += S) acc += part[(size_t)b * nrhs + r];
     }
-    sred[threadIdx.x] = acc;
-    __syncthreads();
-    if (sub == 0 && r < nrhs) {
-      cplx tot = sred[rr];
-      for (int q = 1; q < S; ++q) tot = tot + sred[q * R + rr];
-      part[((size_t)blockIdx.x * gridDim.y + jv) * nrhs + r] = tot;
+    s[threadIdx.x] = acc;
+    tree_sum(s, R, S, sub);
+    const double hnn = sqrt(fmax(s[rr], 0.0));
+    const double a = hnn > 0.0 ? 1.0 / hnn : 0.0;
+    if (sub < S && r < nrhs) {
+      if (blockIdx.x == 0 && sub == 0) hn[r] = hnn;
+      for (int i = i0 + sub; i < i1; i += S) {
+        const size_t idx = (size_t)i * nrhs + r;
+        w[idx] = isfinite(a) ? a * w[idx] : cplx{0.0, 0.0};
+      }
     }
     __syncthreads();
   }
-}
-
-__global__ void k_dots_step2(int nblocks, int nrhs, int nvmax, const cplx* part, const int* ctl, int which,
-                             cplx* out) {
-  if (!ctl[C_ACTIVE]) return;
-  const int nv = which == 0 ? ctl[C_J] + 1 : 1;
-  const int jr = blockIdx.x * blockDim.x + threadIdx.x;
-  if (jr >= nv * nrhs) return;
-  cplx acc{0.0, 0.0};
-  for (int b = 0; b < nblocks; ++b) acc = acc + part[(size_t)b * nvmax * nrhs + jr];
-  out[jr] = acc;
-}
-
-// V_{j+1} -= sum_{i <= j} V_i h[i][r]
-__global__ void k_orth_step(int n, int nrhs, cplx* V, const cplx* h, const int* ctl) {
-  if (!ctl[C_ACTIVE]) return;
-  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long)n * nrhs) return;
-  const int r = (int)(idx % nrhs), nv = ctl[C_J] + 1;
-  const size_t vec = (size_t)n * nrhs;
-  cplx acc = V[(size_t)nv * vec + idx];
-  for (int q = 0; q < nv; ++q) acc = acc - V[(size_t)q * vec + idx] * h[(size_t)q * nrhs + r];
-  V[(size_t)nv * vec + idx] = acc;
-}
-
-// Hessenberg column j of every system: h(i) = h1 + h2 (i <= j), h(j+1) =
-// ||V_{j+1}||; the earlier rotations, a new one zeroing h(j+1), the updated
-// g and the residual estimate |g_{j+1}| / ||f||; scl = 1 / ||V_{j+1}||.
-__global__ void k_givens(int nrhs, int m, const cplx* h1, const cplx* h2, const cplx* hn, cplx* Hm, cplx* cs,
-                         cplx* sn, cplx* gv, const double* fnorm, double* rel, double* scl, double tol, int* ctl) {
-  if (!ctl[C_ACTIVE]) return;
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrhs) return;
-  const int j = ctl[C_J];
-  auto H = [&](int i) -> cplx& { return Hm[((size_t)i * m + j) * nrhs + r]; };
-  for (int i = 0; i <= j; ++i) H(i) = h1[(size_t)i * nrhs + r] + h2[(size_t)i * nrhs + r];
-  const double hnn = sqrt(fmax(hn[r].re, 0.0));
-  H(j + 1) = cplx{hnn, 0.0};
-  scl[r] = hnn > 0.0 ? 1.0 / hnn : 0.0;
-  for (int i = 0; i < j; ++i) {   // previous rotations
-    const cplx c = cs[(size_t)i * nrhs + r], s = sn[(size_t)i * nrhs + r];
-    const cplx a = H(i), b = H(i + 1);
-    H(i) = conj(c) * a + conj(s) * b;
-    H(i + 1) = c * b - s * a;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&ctl[C_TICKET], 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  __shared__ cplx s_u[kRotItems], s_a[kRotItems + kRotRhs];   // c b, a before and after each rotation: [i][r]
+  __shared__ double s_d[kRotItems];
+  int open = 0;
+  for (int r0 = 0; r0 < nrhs; r0 += kRotRhs) {
+    const int nt = min(kRotRhs, nrhs - r0), I = kRotItems / nt;   // systems, rotations at a time
+    auto hcol = [&](int i, int r) { return h1[(size_t)i * nrhs + r] + h2[(size_t)i * nrhs + r]; };
+    __syncthreads();
+    if (threadIdx.x < nt) s_a[threadIdx.x] = hcol(0, r0 + threadIdx.x);
+    for (int ib = 0; ib < j; ib += I) {
+      const int ni = min(I, j - ib);
+      for (int e = threadIdx.x; e < ni * nt; e += 256) {
+        const int i = ib + e / nt, r = r0 + e % nt;
+        s_u[e] = cs[(size_t)i * nrhs + r] * hcol(i + 1, r);
+        s_d[e] = sn[(size_t)i * nrhs + r].re;
+      }
+      __syncthreads();
+      if (threadIdx.x < nt) {
+        cplx a = s_a[threadIdx.x];
+        for (int e = threadIdx.x; e < ni * nt; e += nt) {
+          a = cplx{fma(-s_d[e], a.re, s_u[e].re), fma(-s_d[e], a.im, s_u[e].im)};
+          s_a[e + nt] = a;
+        }
+      }
+      __syncthreads();
+      for (int e = threadIdx.x; e < ni * nt; e += 256) {
+        const int i = ib + e / nt, r = r0 + e % nt;
+        Hm[((size_t)i * m + j) * nrhs + r] = conj(cs[(size_t)i * nrhs + r]) * s_a[e] + s_d[e] * hcol(i + 1, r);
+      }
+      __syncthreads();
+      if (threadIdx.x < nt) s_a[threadIdx.x] = s_a[ni * nt + threadIdx.x];
+    }
+    if (threadIdx.x < nt) {
+      const int r = r0 + threadIdx.x;
+      const cplx a = s_a[threadIdx.x];
+      const double hnn = __ldcg(hn + r);
+      const double den = sqrt(abs2(a) + hnn * hnn);
+      const cplx c = den > 0.0 ? (1.0 / den) * a : cplx{1.0, 0.0};
+      const double d = den > 0.0 ? hnn / den : 0.0;
+      cs[(size_t)j * nrhs + r] = c;
+      sn[(size_t)j * nrhs + r] = cplx{d, 0.0};
+      Hm[((size_t)j * m + j) * nrhs + r] = conj(c) * a + cplx{d * hnn, 0.0};
+      Hm[((size_t)(j + 1) * m + j) * nrhs + r] = cplx{0.0, 0.0};
+      const cplx gj = gv[(size_t)j * nrhs + r];
+      gv[(size_t)j * nrhs + r] = conj(c) * gj;
+      const cplx gn = -(d * gj);
+      gv[(size_t)(j + 1) * nrhs + r] = gn;
+      const double e = fnorm[r] > 0.0 ? sqrt(abs2(gn)) / fnorm[r] : 0.0;
+      rel[r] = e;
+      if (!(e <= tol)) open = 1;
+    }
   }
-  const cplx a = H(j), b = H(j + 1);
-  const double den = sqrt(abs2(a) + abs2(b));
-  const cplx c = den > 0.0 ? (1.0 / den) * a : cplx{1.0, 0.0};
-  const cplx s = den > 0.0 ? (1.0 / den) * b : cplx{0.0, 0.0};
-  cs[(size_t)j * nrhs + r] = c;
-  sn[(size_t)j * nrhs + r] = s;
-  H(j) = conj(c) * a + conj(s) * b;
-  H(j + 1) = cplx{0.0, 0.0};
-  const cplx gj = gv[(size_t)j * nrhs + r];
-  gv[(size_t)j * nrhs + r] = conj(c) * gj;
-  const cplx gn = -(s * gj);
-  gv[(size_t)(j + 1) * nrhs + r] = gn;
-  const double e = fnorm[r] > 0.0 ? sqrt(abs2(gn)) / fnorm[r] : 0.0;
-  rel[r] = e;
-  if (!(e <= tol)) atomicAdd(&ctl[C_NOTCONV], 1);
-}
-
-// V_{j+1} *= scl (per rhs; 0 where not finite)
-__global__ void k_scale_step(int n, int nrhs, cplx* V, const double* scl, const int* ctl) {
-  if (!ctl[C_ACTIVE]) return;
-  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long)n * nrhs) return;
-  const double a = scl[idx % nrhs];
-  cplx* v = V + (size_t)(ctl[C_J] + 1) * n * nrhs;
-  v[idx] = isfinite(a) ? a * v[idx] : cplx{0.0, 0.0};
-}
-
-__global__ void k_step_end(int* ctl) {
-  if (!ctl[C_ACTIVE]) return;
-  ctl[C_J] += 1;
-  ctl[C_TOTAL] += 1;
-  ctl[C_JDONE] = ctl[C_J];
-  ctl[C_DONE] = ctl[C_NOTCONV] == 0;
-  ctl[C_NOTCONV] = 0;
+  open = __syncthreads_or(open);
+  if (threadIdx.x == 0) {
+    ctl[C_J] = j + 1;
+    ctl[C_TOTAL] += 1;
+    ctl[C_JDONE] = j + 1;
+    ctl[C_DONE] = !open;
+    ctl[C_TICKET] = 0;
+    set_active(ctl);
+  }
 }
 
 // start of a restart cycle, from hn = ||f~ - A x~||^2 per rhs: beta, the
@@ -375,6 +485,7 @@ __global__ void k_cycle_init2(int* ctl) {
   ctl[C_JDONE] = 0;
   ctl[C_DONE] = ctl[C_NOTCONV] == 0;
   ctl[C_NOTCONV] = 0;
+  set_active(ctl);
 }
 
 __global__ void k_fnorm(int nrhs, const cplx* hn, double* fnorm) {
@@ -382,16 +493,38 @@ __global__ void k_fnorm(int nrhs, const cplx* hn, double* fnorm) {
   if (r < nrhs) fnorm[r] = sqrt(fmax(hn[r].re, 0.0));
 }
 
-// y = H^{-1} g per system (upper triangular, jdone columns)
-__global__ void k_backsolve(int nrhs, int m, const cplx* Hm, const cplx* gv, cplx* y, const int* ctl) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrhs) return;
-  const int jd = ctl[C_JDONE];
-  for (int i = jd - 1; i >= 0; --i) {
-    cplx s = gv[(size_t)i * nrhs + r];
-    for (int l = i + 1; l < jd; ++l) s = s - Hm[((size_t)i * m + l) * nrhs + r] * y[(size_t)l * nrhs + r];
+// y = H^{-1} g per system (upper triangular, jdone columns).  A CTA per system:
+// with y_i known every thread takes its rows' product from g, so that the chain
+// is one complex product and two barriers per column (one thread per system for
+// the whole triangle: 266 us at 60 columns).  y holds g, then y.
+__global__ void __launch_bounds__(128) k_backsolve(int nrhs, int m, const cplx* __restrict__ Hm,
+                                                   const cplx* __restrict__ gv, cplx* y, const int* ctl) {
+  const int r = blockIdx.x, jd = ctl[C_JDONE];
+  __shared__ cplx s_y;
+  // row l of thread l (mod 128): the running g_l, and 1 / H_ll of its first row
+  for (int l = threadIdx.x; l < jd; l += 128) y[(size_t)l * nrhs + r] = gv[(size_t)l * nrhs + r];
+  auto inv = [&](int i) {
     const cplx d = Hm[((size_t)i * m + i) * nrhs + r];
-    y[(size_t)i * nrhs + r] = abs2(d) > 0.0 ? cdiv(s, d) : cplx{0.0, 0.0};
+    return abs2(d) > 0.0 ? cdiv(cplx{1.0, 0.0}, d) : cplx{0.0, 0.0};
+  };
+  cplx own{0.0, 0.0}, id{0.0, 0.0};
+  if (threadIdx.x < jd) {
+    own = y[(size_t)threadIdx.x * nrhs + r];
+    id = inv(threadIdx.x);
+  }
+  for (int i = jd - 1; i >= 0; --i) {
+    cplx h{0.0, 0.0};
+    if (threadIdx.x < i) h = Hm[((size_t)threadIdx.x * m + i) * nrhs + r];
+    if (threadIdx.x == (i & 127)) {
+      s_y = i < 128 ? own * id : y[(size_t)i * nrhs + r] * inv(i);
+      y[(size_t)i * nrhs + r] = s_y;
+    }
+    __syncthreads();
+    const cplx v = s_y;
+    if (threadIdx.x < i) own = own - h * v;
+    for (int l = threadIdx.x + 128; l < i; l += 128)
+      y[(size_t)l * nrhs + r] = y[(size_t)l * nrhs + r] - Hm[((size_t)l * m + i) * nrhs + r] * v;
+    __syncthreads();
   }
 }
 
@@ -426,36 +559,44 @@ static int solve_impl(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, qbx_c64 eta,
   const int m = restart;
   const size_t zw = Adense ? qbx_matmul_cm_work_bytes(n, nrhs) : 0;
   if (Adense && zw == 0) return gfail(QBX_ECUDA, "matrix product set-up failed");
-  Dev V, W, X, F, DEN, DM, WORK, ST, ZW, CTL;
-  // small state: h1, h2 [(m+1)][nrhs], hn [nrhs], Hm [(m+1)][m][nrhs], cs, sn [m][nrhs],
-  // gv [(m+1)][nrhs], y [m][nrhs] (complex); fnorm, rel, scl [nrhs] (real)
-  const size_t nst = (size_t)nrhs * (2 * (m + 1) + 1 + (size_t)(m + 1) * m + 2 * m + (m + 1) + m);
-  cudaError_t e = cudaMalloc(&V.p, (size_t)(m + 1) * vec * 16);
-  if (e == cudaSuccess) e = cudaMalloc(&W.p, vec * 16);
-  if (e == cudaSuccess) e = cudaMalloc(&X.p, vec * 16);
-  if (e == cudaSuccess) e = cudaMalloc(&F.p, vec * 16);
-  if (e == cudaSuccess) e = cudaMalloc(&DEN.p, vec * 16);
-  if (e == cudaSuccess && !Adense) e = cudaMalloc(&DM.p, vec * 16);   // (D - i eta S) of the density
-  if (e == cudaSuccess) e = cudaMalloc(&WORK.p, qbx_vec_dots_work_bytes(nrhs, m + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&ST.p, nst * 16 + 3 * (size_t)nrhs * 8);
-  if (e == cudaSuccess && Adense) e = cudaMalloc(&ZW.p, zw);
-  if (e == cudaSuccess) e = cudaMalloc(&CTL.p, C_N * sizeof(int));
+  // one allocation: the basis, W, X~, F~, matrix-free: the density and
+  // (D - i eta S) of it; the reductions' partial sums; small state: h1, h2
+  // [(m+1)][nrhs], Hm [(m+1)][m][nrhs], cs, sn [m][nrhs], gv [(m+1)][nrhs],
+  // y [m][nrhs], hn [nrhs] (complex); fnorm, rel, scl, hnorm [nrhs] (real);
+  // the matrix product's splits; the control block
+  const size_t nst = (size_t)nrhs * (2 * (m + 1) + (size_t)(m + 1) * m + 2 * m + (m + 1) + m + 1);
+  Dev mem;
+  size_t total_bytes = 0;
+  auto room = [&](size_t b) {
+    const size_t o = total_bytes;
+    total_bytes += (b + 255) / 256 * 256;
+    return o;
+  };
+  const size_t oV = room((size_t)(m + 1) * vec * 16), oW = room(vec * 16), oX = room(vec * 16), oF = room(vec * 16);
+  const size_t oDEN = room(Adense ? 0 : vec * 16), oDM = room(Adense ? 0 : vec * 16);
+  const size_t oWORK = room(qbx_vec_dots_work_bytes(nrhs, 1)), oST = room(nst * 16 + 4 * (size_t)nrhs * 8);
+  const size_t oZW = room(zw), oCTL = room(C_N * sizeof(int));
+  cudaError_t e = cudaMalloc(&mem.p, total_bytes);
   if (e != cudaSuccess) return gcuda(e, "allocation");
-  cplx* Vb = (cplx*)V.p;
-  cplx* h1 = (cplx*)ST.p;
+  char* base = (char*)mem.p;
+  cplx *Vb = (cplx*)(base + oV), *W = (cplx*)(base + oW), *X = (cplx*)(base + oX), *F = (cplx*)(base + oF);
+  cplx *DEN = (cplx*)(base + oDEN), *DM = (cplx*)(base + oDM), *WORK = (cplx*)(base + oWORK);
+  void* ZW = base + oZW;
+  cplx* h1 = (cplx*)(base + oST);
   cplx* h2 = h1 + (size_t)(m + 1) * nrhs;
-  cplx* hn = h2 + (size_t)(m + 1) * nrhs;
-  cplx* Hm = hn + nrhs;
+  cplx* Hm = h2 + (size_t)(m + 1) * nrhs;
   cplx* cs = Hm + (size_t)(m + 1) * m * nrhs;
   cplx* sn = cs + (size_t)m * nrhs;
   cplx* gv = sn + (size_t)m * nrhs;
   cplx* yv = gv + (size_t)(m + 1) * nrhs;
-  double* fnorm = (double*)(yv + (size_t)m * nrhs);
+  cplx* hn = yv + (size_t)m * nrhs;
+  double* fnorm = (double*)(hn + nrhs);
   double* rel = fnorm + nrhs;
   double* scl = rel + nrhs;
-  int* ctl = (int*)CTL.p;
+  double* hnorm = scl + nrhs;
+  int* ctl = (int*)(base + oCTL);
   {
-    const int init[C_N] = {0, 0, 0, maxiter, m, 0, 0, 0};
+    const int init[C_N] = {0, 0, 0, maxiter, m, 0, 0, 0, 0};
     e = cudaMemcpyAsync(ctl, init, sizeof(init), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // (init lives on the host stack)
     if (e != cudaSuccess) return gcuda(e, "control block");
@@ -463,51 +604,41 @@ static int solve_impl(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, qbx_c64 eta,
   const unsigned ebl = blocks((long)vec), rbl = (unsigned)((nrhs + 127) / 128);
   int rc;
   // scaled right-hand side and initial guess: f~ = sqrt(w) f, x~ = sqrt(w) mu
-  if ((rc = qbx_vec_scale_sqrtw(n, nrhs, g->tgt_w, f, (qbx_c64*)F.p, 0, stream))) return rc;
-  if ((rc = qbx_vec_scale_sqrtw(n, nrhs, g->tgt_w, mu, (qbx_c64*)X.p, 0, stream))) return rc;
+  if ((rc = qbx_vec_scale_sqrtw(n, nrhs, g->tgt_w, f, (qbx_c64*)F, 0, stream))) return rc;
+  if ((rc = qbx_vec_scale_sqrtw(n, nrhs, g->tgt_w, mu, (qbx_c64*)X, 0, stream))) return rc;
   // y = A~ x~ : density x~/sqrt(w), (D - i eta S) two-sided with the two
   // kernel values of each pair combined (qbx_apply_cfie), plus x/2; or one
   // complex matrix product with the assembled A~ (qbx_matmul_cm)
   auto matvec = [&](const qbx_c64* xs, qbx_c64* y, cudaStream_t s) -> int {
     int r;
-    if (Adense) return qbx_matmul_cm(n, nrhs, Adense, xs, y, ZW.p, zw, s);
-    if ((r = qbx_vec_scale_sqrtw(n, nrhs, g->tgt_w, xs, (qbx_c64*)DEN.p, 1, s))) return r;
-    if ((r = qbx_apply_cfie(plan, g, k, eta, p, (qbx_c64*)DEN.p, nrhs, (qbx_c64*)DM.p, s))) return r;
-    return qbx_cfie_combine(n, nrhs, g->tgt_w, (qbx_c64*)DEN.p, (qbx_c64*)DM.p, nullptr, eta, y, s);
+    if (Adense) return qbx_matmul_cm(n, nrhs, Adense, xs, y, ZW, zw, s);
+    if ((r = qbx_vec_scale_sqrtw(n, nrhs, g->tgt_w, xs, (qbx_c64*)DEN, 1, s))) return r;
+    if ((r = qbx_apply_cfie(plan, g, k, eta, p, (qbx_c64*)DEN, nrhs, (qbx_c64*)DM, s))) return r;
+    return qbx_cfie_combine(n, nrhs, g->tgt_w, (qbx_c64*)DEN, (qbx_c64*)DM, nullptr, eta, y, s);
   };
   // one Arnoldi step on stream s, every kernel gated by the control block:
-  // V_j -> W, W = A~ W, W -> V_{j+1}, CGS2 against V_0..V_j, the norm, the
-  // Givens update and the convergence count, V_{j+1} normalised
-  auto step = [&](cudaStream_t s) -> int {
-    k_gate<<<1, 1, 0, s>>>(ctl);
-    k_basis_copy<<<ebl, 256, 0, s>>>((long)vec, Vb, Vb, ctl, 0, 0, nullptr, (cplx*)W.p);
+  // V_{j+1} = A~ V_j, CGS2 against V_0..V_j, the norm, V_{j+1} normalised, the
+  // Givens update and the convergence test.  jh: the step's j where the host
+  // has to know it (matrix-free).
+  auto step = [&](cudaStream_t s, int jh) -> int {
     if (Adense) {
-      if (int r = matmul_cm_gated(n, nrhs, Adense, (qbx_c64*)W.p, (qbx_c64*)DEN.p, ZW.p, zw, ctl + C_ACTIVE, s))
-        return r;
-      k_basis_copy<<<ebl, 256, 0, s>>>((long)vec, Vb, Vb, ctl, 1, 1, (const cplx*)DEN.p, nullptr);
+      if (int r = matmul_cm_step(n, nrhs, Adense, (qbx_c64*)Vb, ZW, zw, ctl + C_ACTIVE, ctl + C_J, s)) return r;
     } else {
-      if (int r = matvec((qbx_c64*)W.p, (qbx_c64*)W.p, s)) return r;   // (host-checked: runs only when active)
-      k_basis_copy<<<ebl, 256, 0, s>>>((long)vec, Vb, Vb, ctl, 1, 1, (const cplx*)W.p, nullptr);
+      cplx* vj = Vb + (size_t)jh * vec;
+      if (int r = matvec((qbx_c64*)vj, (qbx_c64*)(vj + vec), s)) return r;   // (host-checked: runs only when active)
     }
-    for (int pass = 0; pass < 2; ++pass) {   // CGS2
-      cplx* hh = pass == 0 ? h1 : h2;
-      k_dots_step1<<<dim3(kRedBlocks, m + 1), kRedThreads, kRedThreads * sizeof(cplx), s>>>(n, nrhs, Vb, ctl, 0,
-                                                                                         (cplx*)WORK.p);
-      k_dots_step2<<<blocks((long)(m + 1) * nrhs), 256, 0, s>>>(kRedBlocks, nrhs, m + 1, (const cplx*)WORK.p, ctl, 0,
-                                                               hh);
-      k_orth_step<<<ebl, 256, 0, s>>>(n, nrhs, Vb, hh, ctl);
-    }
-    k_dots_step1<<<dim3(kRedBlocks, m + 1), kRedThreads, kRedThreads * sizeof(cplx), s>>>(n, nrhs, Vb, ctl, 1,
-                                                                                       (cplx*)WORK.p);
-    k_dots_step2<<<blocks(nrhs), 256, 0, s>>>(kRedBlocks, nrhs, m + 1, (const cplx*)WORK.p, ctl, 1, hn);
-    k_givens<<<rbl, 128, 0, s>>>(nrhs, m, h1, h2, hn, Hm, cs, sn, gv, fnorm, rel, scl, tol, ctl);
-    k_scale_step<<<ebl, 256, 0, s>>>(n, nrhs, Vb, scl, ctl);
-    k_step_end<<<1, 1, 0, s>>>(ctl);
+    const dim3 dots(kDotCluster, (unsigned)std::min(m, kDotRows));
+    k_dots_step<<<dots, kDotThreads, 0, s>>>(n, nrhs, Vb, ctl, h1);   // CGS2
+    k_orth_step<false><<<kRedBlocks, kOrthThreads, 0, s>>>(n, nrhs, Vb, h1, ctl, nullptr);
+    k_dots_step<<<dots, kDotThreads, 0, s>>>(n, nrhs, Vb, ctl, h2);
+    k_orth_step<true><<<kRedBlocks, kOrthThreads, 0, s>>>(n, nrhs, Vb, h2, ctl, (double*)WORK);
+    k_finish_step<<<kRedBlocks, 256, 0, s>>>(n, nrhs, m, Vb, (const double*)WORK, kRedBlocks, h1, h2, hnorm, Hm, cs, sn,
+                                             gv, fnorm, rel, tol, ctl);
     cudaError_t ee = cudaGetLastError();
     return ee == cudaSuccess ? QBX_OK : gcuda(ee, "Arnoldi step kernels");
   };
   // ||f~|| per rhs
-  if ((rc = qbx_vec_dots(n, nrhs, 1, (qbx_c64*)F.p, (qbx_c64*)F.p, (qbx_c64*)WORK.p, (qbx_c64*)hn, stream)))
+  if ((rc = qbx_vec_dots(n, nrhs, 1, (qbx_c64*)F, (qbx_c64*)F, (qbx_c64*)WORK, (qbx_c64*)hn, stream)))
     return rc;
   k_fnorm<<<rbl, 128, 0, st>>>(nrhs, hn, fnorm);
   // the assembled operator: one Arnoldi step as a CUDA graph
@@ -516,7 +647,7 @@ static int solve_impl(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, qbx_c64 eta,
     e = cudaStreamCreateWithFlags(&gg.cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(gg.cap, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return gcuda(e, "graph capture");
-    rc = step(gg.cap);
+    rc = step(gg.cap, 0);
     e = cudaStreamEndCapture(gg.cap, &gg.g);
     if (rc) return rc;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&gg.x, gg.g, 0);
@@ -527,9 +658,9 @@ static int solve_impl(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, qbx_c64 eta,
   int total = 0;
   while (!done && total < maxiter) {
     // r = f~ - A~ x~, beta, V_0 = r / beta, g = beta e_1
-    if ((rc = matvec((qbx_c64*)X.p, (qbx_c64*)W.p, st))) return rc;
-    k_sub<<<ebl, 256, 0, st>>>((long)vec, (const cplx*)F.p, (const cplx*)W.p, Vb);
-    if ((rc = qbx_vec_dots(n, nrhs, 1, (qbx_c64*)Vb, (qbx_c64*)Vb, (qbx_c64*)WORK.p, (qbx_c64*)hn, stream)))
+    if ((rc = matvec((qbx_c64*)X, (qbx_c64*)W, st))) return rc;
+    k_sub<<<ebl, 256, 0, st>>>((long)vec, (const cplx*)F, (const cplx*)W, Vb);
+    if ((rc = qbx_vec_dots(n, nrhs, 1, (qbx_c64*)Vb, (qbx_c64*)Vb, (qbx_c64*)WORK, (qbx_c64*)hn, stream)))
       return rc;
     k_cycle_init<<<rbl, 128, 0, st>>>(nrhs, m, hn, fnorm, rel, scl, gv, tol, ctl);
     k_cycle_init2<<<1, 1, 0, st>>>(ctl);
@@ -545,12 +676,12 @@ static int solve_impl(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, qbx_c64 eta,
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return gcuda(e, "control block copy");
         if (hctl[C_DONE] || hctl[C_TOTAL] >= maxiter || hctl[C_J] >= m) break;
-        if ((rc = step(st))) return rc;
+        if ((rc = step(st, hctl[C_J]))) return rc;
       }
     }
     // y = H^{-1} g per system; x~ += V y
-    k_backsolve<<<rbl, 128, 0, st>>>(nrhs, m, Hm, gv, yv, ctl);
-    k_combine_cycle<<<ebl, 256, 0, st>>>(n, nrhs, Vb, yv, (cplx*)X.p, ctl);
+    k_backsolve<<<nrhs, 128, 0, st>>>(nrhs, m, Hm, gv, yv, ctl);
+    k_combine_cycle<<<ebl, 256, 0, st>>>(n, nrhs, Vb, yv, (cplx*)X, ctl);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(hctl, ctl, sizeof(hctl), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the one wait of the cycle
@@ -559,7 +690,7 @@ static int solve_impl(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, qbx_c64 eta,
     total = hctl[C_TOTAL];
   }
   // mu = x~ / sqrt(w); residual estimates of the last cycle
-  if ((rc = qbx_vec_scale_sqrtw(n, nrhs, g->tgt_w, (qbx_c64*)X.p, mu, 1, stream))) return rc;
+  if ((rc = qbx_vec_scale_sqrtw(n, nrhs, g->tgt_w, (qbx_c64*)X, mu, 1, stream))) return rc;
   if (resid) e = cudaMemcpyAsync(resid, rel, (size_t)nrhs * 8, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return gcuda(e, "final sync");

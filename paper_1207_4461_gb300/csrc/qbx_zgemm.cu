@@ -32,8 +32,9 @@ constexpr int kBM = 64, kBK = 16, kThreads = 256, kTM = 4;
 template <int TN>
 __global__ void __launch_bounds__(kThreads, 2)
 k_zgemm3m(int n, int nrhs, const cplx* __restrict__ A, const cplx* __restrict__ x, cplx* __restrict__ part,
-          int kchunk, const int* gate) {
+          int kchunk, const int* gate, const int* step) {
   if (gate && !*gate) return;
+  if (step) x += (size_t)*step * n * nrhs;   // vector *step of a basis
   constexpr int BN = 16 * TN;
   __shared__ double sA[3][kBK][kBM];
   __shared__ double sX[3][kBK][BN];
@@ -113,8 +114,9 @@ k_zgemm3m(int n, int nrhs, const cplx* __restrict__ A, const cplx* __restrict__ 
 }
 
 // y = sum over splits in order
-__global__ void k_zgemm_reduce(long nel, int nsplit, const cplx* part, cplx* y, const int* gate) {
+__global__ void k_zgemm_reduce(long nel, int nsplit, const cplx* part, cplx* y, const int* gate, const int* step) {
   if (gate && !*gate) return;
+  if (step) y += (size_t)(*step + 1) * nel;
   const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= nel) return;
   cplx acc = part[idx];
@@ -181,10 +183,11 @@ extern "C" size_t qbx_matmul_cm_work_bytes(int n, int nrhs) {
   return ns < 1 ? 0 : (size_t)ns * n * nrhs * 16;
 }
 
-namespace qbx {
+namespace {
 
-int matmul_cm_gated(int n, int nrhs, const qbx_c64* A, const qbx_c64* x, qbx_c64* y, void* work,
-                    size_t work_bytes, const int* gate, void* stream) {
+// y = A x; with `step` (device): y = basis vector *step + 1, x = basis vector *step, x = y = the basis
+int matmul_cm(int n, int nrhs, const qbx_c64* A, const qbx_c64* x, qbx_c64* y, void* work, size_t work_bytes,
+              const int* gate, const int* step, void* stream) {
   if (n < 1 || nrhs < 1 || !A || !x || !y || !work) return zfail(QBX_EINVAL, "bad arguments");
   int kchunk = 0;
   const int ns = choose_splits(n, nrhs, &kchunk);
@@ -194,20 +197,26 @@ int matmul_cm_gated(int n, int nrhs, const qbx_c64* A, const qbx_c64* x, qbx_c64
   const int BN = 16 * tn_of(nrhs);
   const dim3 grid((unsigned)((n + kBM - 1) / kBM), (unsigned)((nrhs + BN - 1) / BN), (unsigned)ns);
   if (tn_of(nrhs) == 1)
-    k_zgemm3m<1><<<grid, kThreads, 0, st>>>(n, nrhs, (const cplx*)A, (const cplx*)x, (cplx*)work, kchunk, gate);
+    k_zgemm3m<1><<<grid, kThreads, 0, st>>>(n, nrhs, (const cplx*)A, (const cplx*)x, (cplx*)work, kchunk, gate, step);
   else
-    k_zgemm3m<4><<<grid, kThreads, 0, st>>>(n, nrhs, (const cplx*)A, (const cplx*)x, (cplx*)work, kchunk, gate);
+    k_zgemm3m<4><<<grid, kThreads, 0, st>>>(n, nrhs, (const cplx*)A, (const cplx*)x, (cplx*)work, kchunk, gate, step);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return zcuda(e, "product kernel");
   const long nel = (long)n * nrhs;
-  k_zgemm_reduce<<<(unsigned)((nel + 255) / 256), 256, 0, st>>>(nel, ns, (const cplx*)work, (cplx*)y, gate);
+  k_zgemm_reduce<<<(unsigned)((nel + 255) / 256), 256, 0, st>>>(nel, ns, (const cplx*)work, (cplx*)y, gate,
+                                                                 step);
   e = cudaGetLastError();
   return e == cudaSuccess ? QBX_OK : zcuda(e, "reduction kernel");
 }
 
-}  // namespace qbx
+}  // namespace
+
+int qbx::matmul_cm_step(int n, int nrhs, const qbx_c64* A, qbx_c64* V, void* work, size_t work_bytes, const int* gate,
+                        const int* step, void* stream) {
+  return matmul_cm(n, nrhs, A, V, V, work, work_bytes, gate, step, stream);
+}
 
 extern "C" int qbx_matmul_cm(int n, int nrhs, const qbx_c64* A, const qbx_c64* x, qbx_c64* y, void* work,
                              size_t work_bytes, void* stream) {
-  return qbx::matmul_cm_gated(n, nrhs, A, x, y, work, work_bytes, nullptr, stream);
+  return matmul_cm(n, nrhs, A, x, y, work, work_bytes, nullptr, nullptr, stream);
 }
