@@ -428,32 +428,102 @@ __device__ __forceinline__ void lane_power(int lane, double ct, double st, doubl
   }
 }
 
-// Output order q = lane of a translation (k_tree_local has the formulas): W_n
-// the waves (H or J), sd the rows s_m, d_m of NC columns, m <= om.
-template <int NC>
-__device__ __forceinline__ void translate(const cplx* W, const cplx (*sd)[32], int om, int nc, int lane, double cl,
-                                          double sl, cplx* accA, cplx* accB) {
-  cplx S[NC], D[NC];
+// Output orders q of a translation (k_tree_local has the formulas), lane = q:
+// W_n the waves (H or J), sd the rows s_m, d_m of NC columns, m <= om, ss their
+// Re + Im.  Complex waves: three real products per complex one (Re + Im of the
+// waves formed once for all columns): 6 + 6 NC instructions per order m instead
+// of 4 + 8 NC.  Real waves (J at real k): 2 + 4 NC.  Up to q = 15 the
+// two halves of the warp share the orders m.
+template <int NC, typename TW>
+__device__ __forceinline__ void translate(const TW* W, const cplx (*sd)[32], const double (*ss)[32], int om, int oq,
+                                          int nc, int lane, double cl, double sl, cplx* accA, cplx* accB) {
+  constexpr bool kC = IsCplx<TW>::value;
+  constexpr int K = kC ? 3 : 2;
+  const bool half = oq < 16;
+  const int q = half ? lane & 15 : lane, dm = half ? 2 : 1;
+  double S[NC][K], D[NC][K];
 #pragma unroll
-  for (int c = 0; c < NC; ++c) S[c] = D[c] = cplx{0.0, 0.0};
-  for (int m = 0; m <= om; ++m) {
-    const int d = m - lane;
-    const cplx ha = neg_if(d < 0 && (d & 1), W[d < 0 ? -d : d]);
-    const cplx hb = neg_if(lane & 1, W[m + lane]);
-    const cplx hp = ha + hb, hm = ha - hb;
+  for (int c = 0; c < NC; ++c)
+#pragma unroll
+    for (int i = 0; i < K; ++i) S[c][i] = D[c][i] = 0.0;
+  for (int m = half ? lane >> 4 : 0; m <= om; m += dm) {
+    const int d = m - q;
+    const TW ha = neg_if(d < 0 && (d & 1), W[d < 0 ? -d : d]);
+    const TW hb = neg_if(q & 1, W[m + q]);
+    const TW hp = sadd(ha, hb), hm = sc_sub(ha, hb);
+    if constexpr (kC) {
+      const double tp = hp.re + hp.im, tm = hm.re + hm.im;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (c >= nc) break;
+        const cplx u = sd[2 * c][m], v = sd[2 * c + 1][m];
+        S[c][0] = fma(u.re, hp.re, S[c][0]);
+        S[c][1] = fma(u.im, hp.im, S[c][1]);
+        S[c][2] = fma(ss[2 * c][m], tp, S[c][2]);
+        D[c][0] = fma(v.re, hm.re, D[c][0]);
+        D[c][1] = fma(v.im, hm.im, D[c][1]);
+        D[c][2] = fma(ss[2 * c + 1][m], tm, D[c][2]);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (c >= nc) break;
+        const cplx u = sd[2 * c][m], v = sd[2 * c + 1][m];
+        S[c][0] = fma(u.re, hp, S[c][0]);
+        S[c][1] = fma(u.im, hp, S[c][1]);
+        D[c][0] = fma(v.re, hm, D[c][0]);
+        D[c][1] = fma(v.im, hm, D[c][1]);
+      }
+    }
+  }
+  __syncwarp();
+  if (half) {
+    cl = __shfl_sync(0xffffffffu, cl, q);
+    sl = __shfl_sync(0xffffffffu, sl, q);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       if (c >= nc) break;
-      cfma(S[c], sd[2 * c][m], hp);
-      cfma(D[c], sd[2 * c + 1][m], hm);
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        S[c][i] += __shfl_xor_sync(0xffffffffu, S[c][i], 16);
+        D[c][i] += __shfl_xor_sync(0xffffffffu, D[c][i], 16);
+      }
     }
   }
+  if (lane > oq) return;
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
+    if constexpr (kC) {
+      S[c][2] -= S[c][0] + S[c][1];
+      S[c][0] -= S[c][1];
+      S[c][1] = S[c][2];
+      D[c][2] -= D[c][0] + D[c][1];
+      D[c][0] -= D[c][1];
+      D[c][1] = D[c][2];
+    }
     // A' += cos S - i sin D, B' += sin S + i cos D
-    accA[c] = accA[c] + cplx{fma(cl, S[c].re, sl * D[c].im), fma(cl, S[c].im, -sl * D[c].re)};
-    accB[c] = accB[c] + cplx{fma(sl, S[c].re, -cl * D[c].im), fma(sl, S[c].im, cl * D[c].re)};
+    accA[c] = accA[c] + cplx{fma(cl, S[c][0], sl * D[c][1]), fma(cl, S[c][1], -sl * D[c][0])};
+    accB[c] = accB[c] + cplx{fma(sl, S[c][0], -cl * D[c][1]), fma(sl, S[c][1], cl * D[c][0])};
   }
+}
+
+// s_m, d_m of the order m = lane of one column from its coefficients A, B
+__device__ __forceinline__ void rotate_in(const cplx A, const cplx B, double cl, double sl, cplx* s, cplx* d, double* ss,
+                                          double* ds) {
+  const cplx u{fma(A.re, cl, B.re * sl), fma(A.im, cl, B.im * sl)};
+  const cplx v{fma(B.im, cl, -A.im * sl), fma(A.re, sl, -B.re * cl)};
+  *s = u;
+  *d = v;
+  if (ss) {
+    *ss = u.re + u.im;
+    *ds = v.re + v.im;
+  }
+}
+
+// whether k_tree_moments has room for the dipoles' columns (complex k: up to 99 sources a leaf)
+template <typename T>
+__host__ __device__ constexpr bool dipole_rows(int q) {
+  return (size_t)(4 * kTreeP + 12) * (q | 1) * sizeof(T) <= 210 * 1024;
 }
 
 // Moments of one leaf about the centre of one of its nodes (blockIdx = leaf,
@@ -463,7 +533,9 @@ __device__ __forceinline__ void translate(const cplx* W, const cplx (*sd)[32], i
 //   the source's direction, (k/2)(C_{m-1} - C_{m+1}) along x and so on),
 // the coefficients of H_m cos(m Theta) and H_m sin(m Theta) (the factor 2 of
 // m > 0 in k_tree_fold).  Phase 1: one thread per source forms its columns in
-// shared memory; phase 2: one thread per (set, rhs, m) sums over the sources.
+// shared memory, then the normal dipoles' columns from them (formed anew for
+// every right-hand side they were two thirds of the kernel: 12 curves, 24
+// columns 3.4 ms, now 1.6); phase 2: one thread per (set, rhs, m) sums over the sources.
 template <typename T>
 __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs b) {
   const TreeArgs& a = b.inst ? b.inst[blockIdx.z] : b;
@@ -472,6 +544,8 @@ __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs b) {
   const int q = a.q_src, Q = q | 1, P = kTreeP;
   T* sC = reinterpret_cast<T*>(smem_raw);    // [P + 4][Q]
   T* sS = sC + (P + 4) * Q;
+  T* dC = sS + (P + 4) * Q;                  // dipoles along the sources' normals: [P + 2][Q]
+  T* dS = dC + (P + 2) * Q;
   const int panel = blockIdx.x, l = blockIdx.y;
   const double* n = a.node + 4 * (size_t)(a.off[l] + (panel >> l));
   const double zx = n[0], zy = n[1];
@@ -496,6 +570,20 @@ __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs b) {
     }
   }
   __syncthreads();
+  bool dip = false;
+  for (int i = 0; i < a.nset; ++i) dip |= a.kind[i] == kSetNormal || a.kind[i] == kSetCombined;
+  dip = dip && dipole_rows<T>(q);
+  if (dip) {
+    for (int e = threadIdx.x; e < q * (P + 2); e += 128) {
+      const int m = e / q, i = e - m * q, mm = m > 0 ? m - 1 : 1;
+      const double nx = a.snx[(size_t)panel * q + i], ny = a.sny[(size_t)panel * q + i];
+      const T cm = rmul(sC[mm * Q + i], m > 0 ? 1.0 : -1.0), cp = sC[(m + 1) * Q + i];   // C_{-1} = -C_1, S_{-1} = S_1
+      const T sm = sS[mm * Q + i], sp = sS[(m + 1) * Q + i];
+      dC[m * Q + i] = sc_sub(rmul(sc_sub(cm, cp), nx), rmul(sadd(sm, sp), ny));
+      dS[m * Q + i] = sadd(rmul(sc_sub(sm, sp), nx), rmul(sadd(cm, cp), ny));
+    }
+    __syncthreads();
+  }
   const int ncol = a.nset * a.nrhs;
   // few columns: [leaf, level][col][m][2]; many: the leaf's own rows of the coefficients
   cplx* out = a.up ? reinterpret_cast<cplx*>(a.coef) + (size_t)panel * (P + 2) * ncol * 2
@@ -539,18 +627,26 @@ __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs b) {
       A = smul(k2, A);
       B = smul(k2, B);
     } else {
-      const double* px = a.snx + (size_t)panel * q;
-      const double* py = a.sny + (size_t)panel * q;
-      const int mm = m > 0 ? m - 1 : 1;
-      const double sg = m > 0 ? 1.0 : -1.0;   // C_{-1} = -C_1, S_{-1} = S_1
-      for (int i = 0; i < q; ++i) {
-        const double nx = kind == kSetX ? 1.0 : kind == kSetY ? 0.0 : px[i];
-        const double ny = kind == kSetY ? 1.0 : kind == kSetX ? 0.0 : py[i];
-        const T cm = rmul(sC[mm * Q + i], sg), cp = sC[(m + 1) * Q + i];
-        const T sm = sS[mm * Q + i], sp = sS[(m + 1) * Q + i];
-        const cplx v = w[(size_t)i * a.nrhs];
-        madd(A, sc_sub(rmul(sc_sub(cm, cp), nx), rmul(sadd(sm, sp), ny)), v);
-        madd(B, sadd(rmul(sc_sub(sm, sp), nx), rmul(sadd(cm, cp), ny)), v);
+      if (dip && (kind == kSetNormal || kind == kSetCombined)) {
+        for (int i = 0; i < q; ++i) {
+          const cplx v = w[(size_t)i * a.nrhs];
+          madd(A, dC[m * Q + i], v);
+          madd(B, dS[m * Q + i], v);
+        }
+      } else {
+        const double* px = a.snx + (size_t)panel * q;
+        const double* py = a.sny + (size_t)panel * q;
+        const int mm = m > 0 ? m - 1 : 1;
+        const double sg = m > 0 ? 1.0 : -1.0;   // C_{-1} = -C_1, S_{-1} = S_1
+        for (int i = 0; i < q; ++i) {
+          const double nx = kind == kSetX ? 1.0 : kind == kSetY ? 0.0 : px[i];
+          const double ny = kind == kSetY ? 1.0 : kind == kSetX ? 0.0 : py[i];
+          const T cm = rmul(sC[mm * Q + i], sg), cp = sC[(m + 1) * Q + i];
+          const T sm = sS[mm * Q + i], sp = sS[(m + 1) * Q + i];
+          const cplx v = w[(size_t)i * a.nrhs];
+          madd(A, sc_sub(rmul(sc_sub(cm, cp), nx), rmul(sadd(sm, sp), ny)), v);
+          madd(B, sadd(rmul(sc_sub(sm, sp), nx), rmul(sadd(cm, cp), ny)), v);
+        }
       }
       A = smul(hk, A);
       B = smul(hk, B);
@@ -659,8 +755,9 @@ __global__ void __launch_bounds__(32 * kUpWarps) k_tree_up(TreeArgs q, int l) {
   if (l >= a.lev || blockIdx.x >= a.off[l + 1] - a.off[l]) return;
   constexpr int NC = kUpCols, N = kTreeP + 2;
   static_assert(N == 32, "one lane per order");
-  __shared__ cplx s_w[2][2 * N];
+  __shared__ T s_w[2][2 * N];
   __shared__ cplx s_sd[kUpWarps][2 * NC][32];
+  __shared__ double s_ss[kUpWarps][IsCplx<T>::value ? 2 * NC : 1][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int id = a.off[l] + blockIdx.x, c0 = a.off[l - 1] + 2 * blockIdx.x;
   const int nch = min(2, a.off[l] - c0);
@@ -674,12 +771,7 @@ __global__ void __launch_bounds__(32 * kUpWarps) k_tree_up(TreeArgs q, int l) {
   if (warp < nch && lane == 0) {
     const double* y = a.node + 4 * (size_t)(c0 + warp);
     const double vx = z[0] - y[0], vy = z[1] - y[1];
-    if constexpr (IsCplx<T>::value) {
-      besselj_column<cplx>(rmul(kk, sqrt(vx * vx + vy * vy)), 2 * N - 2, s_w[warp], 1);
-    } else {
-      besselj_column<double>(kk * sqrt(vx * vx + vy * vy), 2 * N - 2, reinterpret_cast<double*>(s_w[warp]), 2);
-      for (int i = 0; i < 2 * N - 1; ++i) s_w[warp][i].im = 0.0;
-    }
+    besselj_column<T>(rmul(kk, sqrt(vx * vx + vy * vy)), 2 * N - 2, s_w[warp], 1);
   }
   __syncthreads();
   for (int col0 = (blockIdx.y * kUpWarps + warp) * NC; col0 < ncol; col0 += gridDim.y * kUpWarps * NC) {
@@ -699,11 +791,12 @@ __global__ void __launch_bounds__(32 * kUpWarps) k_tree_up(TreeArgs q, int l) {
         if (c >= nc) break;
         const cplx* m = reinterpret_cast<const cplx*>(a.coef) + (((size_t)(c0 + ch) * N + lane) * ncol + col0 + c) * 2;
         const cplx A = m[0], B = m[1];
-        s_sd[warp][2 * c][lane] = cplx{fma(A.re, cl, B.re * sl), fma(A.im, cl, B.im * sl)};
-        s_sd[warp][2 * c + 1][lane] = cplx{fma(B.im, cl, -A.im * sl), fma(A.re, sl, -B.re * cl)};
+        constexpr bool kC = IsCplx<T>::value;
+        rotate_in(A, B, cl, sl, &s_sd[warp][2 * c][lane], &s_sd[warp][2 * c + 1][lane],
+                  kC ? &s_ss[warp][kC ? 2 * c : 0][lane] : nullptr, kC ? &s_ss[warp][kC ? 2 * c + 1 : 0][lane] : nullptr);
       }
       __syncwarp();
-      translate<NC>(s_w[ch], s_sd[warp], N - 1, nc, lane, cl, sl, accA, accB);
+      translate<NC, T>(s_w[ch], s_sd[warp], s_ss[warp], N - 1, N - 1, nc, lane, cl, sl, accA, accB);
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -716,16 +809,16 @@ __global__ void __launch_bounds__(32 * kUpWarps) k_tree_up(TreeArgs q, int l) {
 }
 
 // The coefficient columns of one node or local expansion from its moments
-// [col][m][2] (m <= n): column set i is moment set `base`, itself or its
+// (m <= n; strides si of m, sab of A, B): column set i is moment set `base`, itself or its
 // derivative along x or y (the series of d/dx u has the coefficients
 //   A^x_m = (k/2)(A_{m+1} - A_{m-1}), B^x_m = (k/2)(B_{m+1} - B_{m-1}),
 //   A^y_m = (k/2)(B_{m+1} + B_{m-1}), B^y_m = -(k/2)(A_{m+1} + A_{m-1}),
 // A_0 counted twice).
-__device__ __forceinline__ void shifted_coef(const TreeArgs& a, int set, const cplx* mom, int stride, int n, int m,
-                                             cplx* out) {
+__device__ __forceinline__ void shifted_coef(const TreeArgs& a, int set, const cplx* mom, int si, int sab, int n,
+                                             int m, cplx* out) {
   auto at = [&](int i, int ab) {
     if (i < 0 || i > n) return cplx{0.0, 0.0};
-    return mom[i * stride + ab];
+    return mom[i * si + ab * sab];
   };
   const int sh = a.shift[set];
   if (sh == 0) {
@@ -787,7 +880,7 @@ __global__ void __launch_bounds__(64) k_tree_fold(TreeArgs a) {
   for (int i = threadIdx.x; i < a.ncset * (kTreeP + 1); i += 64) {
     const int cs = i / (kTreeP + 1), m = i - cs * (kTreeP + 1);
     if (a.base[cs] != set) continue;
-    shifted_coef(a, cs, &s_m[0][0], 2, kTreeP + 1, m,
+    shifted_coef(a, cs, &s_m[0][0], 2, 1, kTreeP + 1, m,
                  reinterpret_cast<cplx*>(a.coef) + (((size_t)id * (kTreeP + 2) + m) * a.ncset * a.nrhs + cs * a.nrhs + r) * 2);
   }
 }
@@ -800,27 +893,40 @@ __global__ void __launch_bounds__(64) k_tree_fold(TreeArgs a) {
 // d_m = i (A_m sin(m Theta) - B_m cos(m Theta)):
 //   S_q = sum_m s_m (H_{m-q} + (-1)^q H_{m+q}),  T_q = sum_m d_m (H_{m-q} - (-1)^q H_{m+q}),
 //   A'_q = cos(q Theta) S_q - i sin(q Theta) T_q,  B'_q = sin(q Theta) S_q + i cos(q Theta) T_q
-// (A'_0 halved).  One warp per node, lane = q: a tenth of the FP64 work of
-// taking the node through each of the block's 32 or 64 centres.
-// NC moment columns per CTA of kLocWarps warps.
-template <typename T, int NC, int kLocWarps>
-__global__ void __launch_bounds__(32 * kLocWarps) k_tree_local(TreeArgs q) {
+// (A'_0 halved).  Lane = q: a tenth of the FP64 work of taking the node through
+// each of the block's 32 or 64 centres.  A CTA takes a block and up to 8 groups
+// of 4 columns, a warp per group (with fewer groups the warps share the nodes).
+// The waves of 32 nodes at a time, one node per lane, serve all its columns:
+// formed by every warp for its own node and columns they were a quarter of the
+// FP64 work (12 curves, 24 columns: all of this kernel 22.4 ms, now 17.9 with the three-product form).
+constexpr int kLocWarps = 8, kLocCols = 4, kLocNodes = 32, kLocRow = 2 * kTreeP + 3;
+struct LocSmem {
+  cplx h[kLocNodes][kLocRow];
+  cplx sd[kLocWarps][2 * kLocCols][32];
+  double ss[kLocWarps][2 * kLocCols][32];
+  double2 dir[kLocNodes];
+};
+template <typename T>
+__global__ void __launch_bounds__(32 * kLocWarps, 2) k_tree_local(TreeArgs q) {
   const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
   if (blockIdx.x >= a.n_blk) return;
-  __shared__ cplx s_h[kLocWarps][2 * kTreeP + 2];
-  __shared__ cplx s_sd[kLocWarps][2 * NC][32];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  LocSmem& sm = *reinterpret_cast<LocSmem*>(smem_raw);
+  constexpr int NC = kLocCols;
   static_assert(kTreeP < 32, "one lane per order");
-  const int b = blockIdx.x, col0 = blockIdx.y * NC, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nc = min(NC, a.nset * a.nrhs - col0);
+  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int cnt = a.cnt[3 * b + 2];
+  const int nmom = a.nset * a.nrhs, g0 = blockIdx.y * kLocWarps, G = min(kLocWarps, (nmom + NC - 1) / NC - g0);
+  if (cnt == 0 || G <= 0) return;
+  const int parts = kLocWarps / G, part = warp / G;   // warps sharing the nodes of a column group
+  const int col0 = (g0 + warp % G) * NC, nc = min(NC, nmom - col0);
   int ccol[NC];   // coefficient column of each moment column
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    const int set = min(col0 + c, a.nset * a.nrhs - 1) / a.nrhs;
-    ccol[c] = a.plain[set] * a.nrhs + min(col0 + c, a.nset * a.nrhs - 1) - set * a.nrhs;
+    const int col = min(col0 + c, nmom - 1), set = col / a.nrhs;
+    ccol[c] = a.plain[set] * a.nrhs + col - set * a.nrhs;
   }
   const int ncol = a.ncset * a.nrhs;
-  const int cnt = a.cnt[3 * b + 2];
-  if (cnt == 0) return;
   const double* blk = a.node + 4 * (size_t)(a.off[a.lev] + b);
   const int2* loc = reinterpret_cast<const int2*>(a.loc) + (size_t)b * a.M;
   KW<T> kw;
@@ -828,70 +934,73 @@ __global__ void __launch_bounds__(32 * kLocWarps) k_tree_local(TreeArgs q) {
   cplx accA[NC], accB[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) accA[c] = accB[c] = cplx{0.0, 0.0};
-  for (int e = warp; e < cnt; e += kLocWarps) {
-    const int2 ent = loc[e];
-    const int om = ent.y & 0xff, oq = ent.y >> 8;
-    const double* nd = a.node + 4 * (size_t)ent.x;
-    double ct, st;
-    cplx h0, h1;
-    T twoz;
-    far_hankel<T>(kw, kw.kval(), blk[0], nd[0], blk[1], nd[1], ct, st, h0, h1, twoz);
-    double cl, sl;   // lane * Theta
-    lane_power(lane, ct, st, cl, sl);
-    __syncwarp();   // the previous node's tables are no longer read
-    if (lane == 0) s_h[warp][0] = h0;
-    T s = twoz;
-    for (int i = 1; i <= om + oq; ++i) {
-      if (lane == 0) s_h[warp][i] = h1;
-      const cplx h2 = hrec(s, h1, h0);
-      h0 = h1;
-      h1 = h2;
-      s = sadd(s, twoz);
-    }
-    if (lane <= om) {
-      const double2* co = reinterpret_cast<const double2*>(a.coef) + ((size_t)ent.x * (kTreeP + 2) + lane) * ncol * 2;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        if (c >= nc) break;
-        const double2 A = co[2 * ccol[c]], B = co[2 * ccol[c] + 1];
-        s_sd[warp][2 * c][lane] = cplx{fma(A.x, cl, B.x * sl), fma(A.y, cl, B.y * sl)};
-        s_sd[warp][2 * c + 1][lane] = cplx{fma(B.y, cl, -A.y * sl), fma(A.x, sl, -B.x * cl)};
-      }
-    }
-    __syncwarp();
-    if (lane <= oq) translate<NC>(s_h[warp], s_sd[warp], om, nc, lane, cl, sl, accA, accB);
-  }
-  // the warps' sums, in warp order
-  __shared__ cplx s_sum[2 * NC][32], s_mom[NC][kTreeP + 1][2];
-  for (int w = 0; w < kLocWarps; ++w) {
-    if (warp == w) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        if (w > 0) {
-          accA[c] = s_sum[2 * c][lane] + accA[c];
-          accB[c] = s_sum[2 * c + 1][lane] + accB[c];
-        }
-        s_sum[2 * c][lane] = accA[c];
-        s_sum[2 * c + 1][lane] = accB[c];
+  for (int e0 = 0; e0 < cnt; e0 += kLocNodes) {
+    __syncthreads();   // the previous nodes' waves are no longer read
+    if (warp == 0 && e0 + lane < cnt) {
+      const int2 ent = loc[e0 + lane];
+      const int n = (ent.y & 0xff) + (ent.y >> 8);
+      const double* nd = a.node + 4 * (size_t)ent.x;
+      double ct, st;
+      cplx h0, h1;
+      T twoz;
+      far_hankel<T>(kw, kw.kval(), blk[0], nd[0], blk[1], nd[1], ct, st, h0, h1, twoz);
+      sm.dir[lane] = make_double2(ct, st);
+      cplx* h = sm.h[lane];
+      h[0] = h0;
+      T s = twoz;
+      for (int i = 1; i <= n; ++i) {
+        h[i] = h1;
+        const cplx h2 = hrec(s, h1, h0);
+        h0 = h1;
+        h1 = h2;
+        s = sadd(s, twoz);
       }
     }
     __syncthreads();
-  }
-  if (warp == 0 && lane <= kTreeP) {
+    const int ne = part < parts ? min(kLocNodes, cnt - e0) : 0;
+    for (int e = part; e < ne; e += parts) {
+      const int2 ent = loc[e0 + e];
+      const int om = ent.y & 0xff, oq = ent.y >> 8;
+      const double2 dir = sm.dir[e];
+      double cl, sl;   // lane * Theta
+      lane_power(lane, dir.x, dir.y, cl, sl);
+      __syncwarp();   // the previous node's rows are no longer read
+      if (lane <= om) {
+        const double2* co = reinterpret_cast<const double2*>(a.coef) + ((size_t)ent.x * (kTreeP + 2) + lane) * ncol * 2;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      s_mom[c][lane][0] = (lane == 0 ? 0.5 : 1.0) * s_sum[2 * c][lane];
-      s_mom[c][lane][1] = lane == 0 ? cplx{0.0, 0.0} : s_sum[2 * c + 1][lane];
+        for (int c = 0; c < NC; ++c) {
+          if (c >= nc) break;
+          const double2 A = co[2 * ccol[c]], B = co[2 * ccol[c] + 1];
+          rotate_in(cplx{A.x, A.y}, cplx{B.x, B.y}, cl, sl, &sm.sd[warp][2 * c][lane], &sm.sd[warp][2 * c + 1][lane],
+                    &sm.ss[warp][2 * c][lane], &sm.ss[warp][2 * c + 1][lane]);
+        }
+      }
+      __syncwarp();
+      translate<NC, cplx>(sm.h[e], sm.sd[warp], sm.ss[warp], om, oq, nc, lane, cl, sl, accA, accB);
     }
+  }
+  // the sums of the warps of a column group, in warp order
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    sm.sd[warp][2 * c][lane] = accA[c];
+    sm.sd[warp][2 * c + 1][lane] = accB[c];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < G * 2 * NC * 32; i += 32 * kLocWarps) {
+    const int g = i / (2 * NC * 32), row = i / 32 % (2 * NC), m = i & 31;
+    cplx v = sm.sd[g][row][m];
+    for (int w = 1; w < parts; ++w) v = v + sm.sd[g + w * G][row][m];
+    sm.sd[g][row][m] = m > 0 ? v : row & 1 ? cplx{0.0, 0.0} : 0.5 * v;
   }
   __syncthreads();
   cplx* out = reinterpret_cast<cplx*>(a.coef) + (size_t)(a.off[a.lev] + b) * (kTreeP + 2) * ncol * 2;
-  for (int i = threadIdx.x; i < nc * a.ncset * (kTreeP + 1); i += 32 * kLocWarps) {
-    const int c = i / (a.ncset * (kTreeP + 1)), rem = i - c * a.ncset * (kTreeP + 1);
-    const int cs = rem / (kTreeP + 1), m = rem - cs * (kTreeP + 1);
-    const int set = (col0 + c) / a.nrhs, r = col0 + c - set * a.nrhs;
+  const int nmine = min(G * NC, nmom - g0 * NC), per = a.ncset * (kTreeP + 1);
+  for (int i = threadIdx.x; i < nmine * per; i += 32 * kLocWarps) {
+    const int c = i / per, rem = i - c * per, cs = rem / (kTreeP + 1), m = rem - cs * (kTreeP + 1);
+    const int col = g0 * NC + c, set = col / a.nrhs, r = col - set * a.nrhs;
     if (a.base[cs] == set)
-      shifted_coef(a, cs, &s_mom[c][0][0], 2, kTreeP, m, out + ((size_t)m * ncol + cs * a.nrhs + r) * 2);
+      shifted_coef(a, cs, &sm.sd[c / NC][2 * (c % NC)][0], 1, 32, kTreeP, m, out + ((size_t)m * ncol + cs * a.nrhs + r) * 2);
   }
 }
 
@@ -1494,7 +1603,7 @@ cudaError_t launch_far_ops(const TreeArgs& a, cudaStream_t st) {
 
 template <typename T>
 size_t moments_smem(int q_src) {
-  return (size_t)2 * (kTreeP + 4) * (q_src | 1) * sizeof(T);
+  return (size_t)((dipole_rows<T>(q_src) ? 4 * kTreeP + 12 : 2 * kTreeP + 8)) * (q_src | 1) * sizeof(T);
 }
 
 template <typename T>
@@ -1522,8 +1631,10 @@ cudaError_t launch_moments_t(const TreeArgs& a, cudaStream_t st, int n_inst) {
                      32 * kUpWarps, 0, st>>>(a, l);
   if (!a.up) k_tree_fold<<<dim3(a.off[a.lev], ncol), 64, 0, st>>>(a);
   if (a.n_blk == 0) return cudaGetLastError();
-  if (a.up) k_tree_local<T, 4, 4><<<dim3(a.n_blk, (ncol + 3) / 4, n_inst), 32 * 4, 0, st>>>(a);
-  else k_tree_local<T, 2, 8><<<dim3(a.n_blk, (ncol + 1) / 2, n_inst), 32 * 8, 0, st>>>(a);
+  cudaError_t e = cudaFuncSetAttribute(k_tree_local<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocSmem));
+  if (e != cudaSuccess) return e;
+  const int per = kLocWarps * kLocCols;
+  k_tree_local<T><<<dim3(a.n_blk, (ncol + per - 1) / per, n_inst), 32 * kLocWarps, sizeof(LocSmem), st>>>(a);
   return cudaGetLastError();
 }
 

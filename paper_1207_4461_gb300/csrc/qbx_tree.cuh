@@ -63,6 +63,9 @@ __device__ __forceinline__ int series_order(float kr, float z, float q, float da
   return last;
 }
 
+__device__ __forceinline__ double neg_if(bool neg, double v) {
+  return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
+}
 __device__ __forceinline__ cplx neg_if(bool neg, cplx v) {   // on the integer pipe
   const int m = neg ? 0x80000000 : 0;
   return cplx{__hiloint2double(__double2hiint(v.re) ^ m, __double2loint(v.re)),
