@@ -15,7 +15,10 @@
 // and the panels m = 4 blockIdx.y + g (mod 4 gridDim.y) for warp g; the
 // matrix is stored column-major
 // (entry (t, t') at t' n + t), so a warp writes 32 consecutive rows of one
-// column at a time.
+// column at a time.  From 16 panels on (and where the workspace holds it) only
+// the panels near a block of 32 targets go this way, the four warps of a CTA
+// sharing one panel's sources; the others by their moments (k_tree_matrix),
+// beside it on the plan's side stream.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
@@ -40,11 +43,15 @@ struct AsmArgs {
   const double* P;     // [q_src][q_tgt]
   cplx* out;           // [n_tgt][n_tgt] column-major
   const double* hk_tab;   // complex k: the amplitude table of this k's ray, or null
+  const int *near, *near_cnt;   // near panels of every 32-target block (stride M); null: every panel
 };
 
 template <typename T>
 __global__ void __launch_bounds__(kAsmLanes * kAsmWarps) k_assemble_cfie(AsmArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int share = a.near ? kAsmWarps : 1;   // warps that share a panel's sources
+  const int cnt = a.near ? a.near_cnt[3 * blockIdx.x] : a.M;
+  if ((int)blockIdx.y * (kAsmWarps / share) >= cnt) return;
   double* sP = reinterpret_cast<double*>(smem_raw);                  // [q_src][q_tgt]
   T* slot = reinterpret_cast<T*>(sP + a.q_src * a.q_tgt + (a.q_src * a.q_tgt & 1));
   const int p = a.p, P2 = (p + 2) * kAsmLanes;
@@ -85,11 +92,13 @@ __global__ void __launch_bounds__(kAsmLanes * kAsmWarps) k_assemble_cfie(AsmArgs
   const T kneg_j0 = rmul(sc_mul(kk, J0), -1.0), kneg_j0e = rmul(sc_mul(kk, J0e), -1.0);
   const cplx ieta = cplx{-a.eta_im, a.eta_re};   // i eta
   const double swt = sqrt(a.tw[tt]);
-  for (int m = (int)blockIdx.y * kAsmWarps + warp; m < a.M; m += kAsmWarps * (int)gridDim.y) {
+  const int part = warp % share, j0 = part * a.q_src / share, j1 = (part + 1) * a.q_src / share;
+  for (int e = (int)blockIdx.y * (kAsmWarps / share) + warp / share; e < cnt; e += kAsmWarps / share * (int)gridDim.y) {
+    const int m = a.near ? a.near[blockIdx.x * a.M + e] : e;
     cplx acc[kAsmQ];
 #pragma unroll
     for (int i = 0; i < kAsmQ; ++i) acc[i] = cplx{0.0, 0.0};
-    for (int j = 0; j < a.q_src; ++j) {
+    for (int j = j0; j < j1; ++j) {
       const int s = m * a.q_src + j;
       const double sx = a.sx[s], sy = a.sy[s], nx = a.snx[s], ny = a.sny[s];
       cplx GS, K, GA, GB, EX, EY, v{0.0, 0.0};
@@ -109,10 +118,24 @@ __global__ void __launch_bounds__(kAsmLanes * kAsmWarps) k_assemble_cfie(AsmArgs
         }
       }
     }
+    if (share > 1) {   // the warps' sums, in warp order; then each warp writes its columns
+      cplx* sA = reinterpret_cast<cplx*>(sLe + P2);   // [kAsmWarps][kAsmQ][32]
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < kAsmQ; ++i) sA[(warp * kAsmQ + i) * 32 + lane] = acc[i];
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < kAsmQ; ++i) {
+        acc[i] = sA[i * 32 + lane];
+#pragma unroll
+        for (int w = 1; w < kAsmWarps; ++w) acc[i] = acc[i] + sA[(w * kAsmQ + i) * 32 + lane];
+      }
+    }
     if (!active) continue;
 #pragma unroll
     for (int i = 0; i < kAsmQ; ++i) {
       if (i >= a.q_tgt) break;
+      if (share > 1 && (i & (kAsmWarps - 1)) != warp) continue;
       const int col = m * a.q_tgt + i;
       // (i/4)(1/2) acc, the 1/2 of the identity, the sqrt-weight scaling
       cplx e = cplx{-0.125 * acc[i].im, 0.125 * acc[i].re};
@@ -124,8 +147,9 @@ __global__ void __launch_bounds__(kAsmLanes * kAsmWarps) k_assemble_cfie(AsmArgs
 }
 
 template <typename T>
-size_t asm_smem(int p, int q_src, int q_tgt) {
-  return ((size_t)q_src * q_tgt + 1) * 8 + 4 * (size_t)(p + 2) * kAsmLanes * sizeof(T) + 16;
+size_t asm_smem(int p, int q_src, int q_tgt, bool near) {
+  return ((size_t)q_src * q_tgt + 1) * 8 + 4 * (size_t)(p + 2) * kAsmLanes * sizeof(T) + 16 +
+         (near ? (size_t)kAsmWarps * kAsmQ * 32 * 16 : 0);
 }
 
 int afail(int code, const char* what) {
@@ -182,23 +206,58 @@ extern "C" int qbx_assemble_cfie(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, q
   a.P = P;
   a.out = reinterpret_cast<cplx*>(A);
   const bool ck = k.im != 0.0;
-  const size_t smem = ck ? asm_smem<cplx>(p, q_src, q_tgt) : asm_smem<double>(p, q_src, q_tgt);
-  if (smem > 200 * 1024) return afail(QBX_EINVAL, "p too large");
-  // panel groups: about 8192 CTAs in all (some 18 waves of the resident
-  // CTAs), so that the last, partly filled wave costs little
-  const unsigned gx = (unsigned)((g->n_tgt + kAsmLanes - 1) / kAsmLanes);
-  const unsigned gy = (unsigned)std::max(1, std::min((g->M + kAsmWarps - 1) / kAsmWarps, (int)((8192 + gx - 1) / gx)));
-  const dim3 grid(gx, gy);
+  if ((ck ? asm_smem<cplx>(p, q_src, q_tgt, false) : asm_smem<double>(p, q_src, q_tgt, false)) > 200 * 1024)
+    return afail(QBX_EINVAL, "p too large");
   cudaStream_t st = (cudaStream_t)stream;
   a.hk_tab = host_plan_hk_table(plan, k, st, &e);
   if (e != cudaSuccess) return acuda(e, "complex-k amplitude table");
-  if (ck) {
-    e = cudaFuncSetAttribute(k_assemble_cfie<cplx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_assemble_cfie<cplx><<<grid, kAsmLanes * kAsmWarps, smem, st>>>(a);
-  } else {
-    e = cudaFuncSetAttribute(k_assemble_cfie<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_assemble_cfie<double><<<grid, kAsmLanes * kAsmWarps, smem, st>>>(a);
+  void* ws;
+  size_t ws_bytes;
+  int num_sms;
+  int* status;
+  host_plan_workspace(plan, &ws, &ws_bytes, &num_sms, &status);
+  MatrixFarArgs far;
+  const size_t need = matrix_tree_setup(&far, g, k, eta, p, a.hk_tab, nullptr);
+  const bool tree = need > 0 && need <= ws_bytes &&
+                    (ck ? asm_smem<cplx>(p, q_src, q_tgt, true) : asm_smem<double>(p, q_src, q_tgt, true)) <= 200 * 1024;
+  const size_t smem = ck ? asm_smem<cplx>(p, q_src, q_tgt, tree) : asm_smem<double>(p, q_src, q_tgt, tree);
+  // panel groups: about 8192 CTAs in all (some 18 waves of the resident
+  // CTAs), so that the last, partly filled wave costs little; near panels: one
+  // per CTA up to 32 per block
+  const unsigned gx = (unsigned)((g->n_tgt + kAsmLanes - 1) / kAsmLanes);
+  const unsigned gy = (unsigned)(tree ? std::min(g->M, 32)
+                                      : std::max(1, std::min((g->M + kAsmWarps - 1) / kAsmWarps, (int)((8192 + gx - 1) / gx))));
+  const dim3 grid(gx, gy);
+  auto pairs = [&](cudaStream_t s) {
+    cudaError_t le;
+    if (ck) {
+      le = cudaFuncSetAttribute(k_assemble_cfie<cplx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (le == cudaSuccess) k_assemble_cfie<cplx><<<grid, kAsmLanes * kAsmWarps, smem, s>>>(a);
+    } else {
+      le = cudaFuncSetAttribute(k_assemble_cfie<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (le == cudaSuccess) k_assemble_cfie<double><<<grid, kAsmLanes * kAsmWarps, smem, s>>>(a);
+    }
+    return le == cudaSuccess ? cudaGetLastError() : le;
+  };
+  if (!tree) {
+    e = pairs(st);
+    return e == cudaSuccess ? QBX_OK : acuda(e, "assembly kernel");
   }
-  if (e == cudaSuccess) e = cudaGetLastError();
-  return e == cudaSuccess ? QBX_OK : acuda(e, "assembly kernel");
+  matrix_tree_setup(&far, g, k, eta, p, a.hk_tab, static_cast<char*>(ws));
+  far.out = A;
+  cudaStream_t side;
+  cudaEvent_t fork, join;
+  host_plan_side(plan, &side, &fork, &join);
+  e = launch_tree_lists(far.t, st);
+  if (e == cudaSuccess) e = cudaEventRecord(fork, st);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork, 0);
+  if (e != cudaSuccess) return acuda(e, "panel lists");
+  a.near = far.t.near;
+  a.near_cnt = far.t.cnt;
+  e = pairs(side);
+  const cudaError_t ef = launch_matrix_far(far, g->src_w, P, st);
+  cudaError_t ej = cudaEventRecord(join, side);   // (joined also after an error)
+  if (ej == cudaSuccess) ej = cudaStreamWaitEvent(st, join, 0);
+  if (e == cudaSuccess) e = ef != cudaSuccess ? ef : ej;
+  return e == cudaSuccess ? QBX_OK : acuda(e, "assembly kernels");
 }

@@ -286,6 +286,7 @@ struct TreeArgs {
   int pl;                     // orders of the list entries (p, or kTreeLocal for near-only QBX)
   int nd;                     // derivatives taken on one side of a kernel (D, grad S: 1)
   double eta;                 // near-only QBX (> 0)
+  int only_loc;               // lists: leaves that do not go through the block's local expansion are near
   int M, q_src, n_src;        // leaves (halves of panels, or panels), sources per leaf, sources
   const double *sx, *sy, *snx, *sny;
   // adjoint sweeps: the nodes hold the discs of n_ctr_n centres (dcx, dcy) of
@@ -354,6 +355,15 @@ struct FarPointArgs {
   void* part;          // as FarArgs::part
 };
 cudaError_t launch_far_points(FarPointArgs a, cudaStream_t st);
+// Far entries of the assembled matrix (t: leaves are whole panels, columns the interpolation's)
+struct MatrixFarArgs {
+  TreeArgs t;
+  const double* tw;
+  void* out;           // [n_tgt][n_tgt] column-major
+};
+size_t matrix_tree_setup(MatrixFarArgs* q, const qbx_geom* g, qbx_c64 k, qbx_c64 eta, int p, const double* hk_tab,
+                         char* base);
+cudaError_t launch_matrix_far(const MatrixFarArgs& q, const double* sw, const double* P, cudaStream_t st);
 // nodes and coefficients only
 cudaError_t launch_tree_nodes(const TreeArgs& a, cudaStream_t st);
 // adjoint sweeps: the tree over the discs of the centres, evaluated at the

@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs q) {
         if (code) break;
       }
     }
+    if (a.only_loc && !(code >> 16 & 0xff)) code = 0;
     const bool is_near = j < a.M && !code;
     const bool is_node = code && (j & ((1 << l) - 1)) == 0, has_loc = (code >> 16 & 0xff) > 0;
     const bool is_far = is_node && !has_loc, is_loc = is_node && has_loc;
@@ -885,6 +886,28 @@ __global__ void __launch_bounds__(64) k_tree_fold(TreeArgs a) {
   }
 }
 
+// Waves H_0..H_{om+oq} and direction of one entry (node, orders om | oq << 8) of a local expansion about blk
+template <typename T>
+__device__ __forceinline__ void loc_waves(const KW<T>& kw, const double* blk, const double* node, int2 ent, cplx* h,
+                                          double2* dir) {
+  const int n = (ent.y & 0xff) + (ent.y >> 8);
+  const double* nd = node + 4 * (size_t)ent.x;
+  double ct, st;
+  cplx h0, h1;
+  T twoz;
+  far_hankel<T>(kw, kw.kval(), blk[0], nd[0], blk[1], nd[1], ct, st, h0, h1, twoz);
+  *dir = make_double2(ct, st);
+  h[0] = h0;
+  T s = twoz;
+  for (int i = 1; i <= n; ++i) {
+    h[i] = h1;
+    const cplx h2 = hrec(s, h1, h0);
+    h0 = h1;
+    h1 = h2;
+    s = sadd(s, twoz);
+  }
+}
+
 // Local expansions: the nodes that are far from a whole block of targets (its
 // radius included) are first gathered into one expansion about the block's
 // centre z_b, u = sum_q J_q(k d) [A'_q cos(q phi) + B'_q sin(q phi)], which then
@@ -936,26 +959,7 @@ __global__ void __launch_bounds__(32 * kLocWarps, 2) k_tree_local(TreeArgs q) {
   for (int c = 0; c < NC; ++c) accA[c] = accB[c] = cplx{0.0, 0.0};
   for (int e0 = 0; e0 < cnt; e0 += kLocNodes) {
     __syncthreads();   // the previous nodes' waves are no longer read
-    if (warp == 0 && e0 + lane < cnt) {
-      const int2 ent = loc[e0 + lane];
-      const int n = (ent.y & 0xff) + (ent.y >> 8);
-      const double* nd = a.node + 4 * (size_t)ent.x;
-      double ct, st;
-      cplx h0, h1;
-      T twoz;
-      far_hankel<T>(kw, kw.kval(), blk[0], nd[0], blk[1], nd[1], ct, st, h0, h1, twoz);
-      sm.dir[lane] = make_double2(ct, st);
-      cplx* h = sm.h[lane];
-      h[0] = h0;
-      T s = twoz;
-      for (int i = 1; i <= n; ++i) {
-        h[i] = h1;
-        const cplx h2 = hrec(s, h1, h0);
-        h0 = h1;
-        h1 = h2;
-        s = sadd(s, twoz);
-      }
-    }
+    if (warp == 0 && e0 + lane < cnt) loc_waves<T>(kw, blk, a.node, loc[e0 + lane], sm.h[lane], &sm.dir[lane]);
     __syncthreads();
     const int ne = part < parts ? min(kLocNodes, cnt - e0) : 0;
     for (int e = part; e < ne; e += parts) {
@@ -1013,6 +1017,155 @@ __host__ __device__ size_t far_warp_bytes(int pl) {
 template <typename T>
 __host__ __device__ size_t far_col_bytes(int pl) {
   return (size_t)(pl + 2) * 32 * sizeof(T);
+}
+
+// Matrix entries of the assembled combined field from the panels that are far
+// from a block of 32 targets: the panel's q_tgt columns of moments (one per
+// column of the interpolation) go into local expansions about the block's
+// centre, whose waves' truncated expansions about the two centres of a target
+// are the same for every panel: their sums C_q, S_q over both sides are formed
+// once per CTA, and an entry is sum_q (A'_q C_q + B'_q S_q).  A warp takes one
+// panel, four columns at a time (lane = q in the translation, then lane =
+// target).  FP64-bound: 4000 instructions per panel and block, pair by pair
+// 20700 (assembly at 72 panels, p = 10, 18 of them near a block: 5.7 -> 2.8 ms).
+struct MatrixSmem {
+  union {
+    LocSmem loc;
+    unsigned char setup[sizeof(LocSmem)];   // per side: J column, waves, orders (while C, S are formed)
+  };
+  cplx basis[kTreeP + 1][2][32];
+};
+template <typename T>
+__global__ void __launch_bounds__(32 * kLocWarps) k_tree_matrix(MatrixFarArgs q) {
+  const TreeArgs& a = q.t;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MatrixSmem& ms = *reinterpret_cast<MatrixSmem*>(smem_raw);
+  LocSmem& sm = ms.loc;
+  constexpr int NC = kLocCols;
+  const int b = blockIdx.x, split = blockIdx.y, nsplit = gridDim.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int cnt = a.cnt[3 * b + 2], mine = cnt > split ? (cnt - split + nsplit - 1) / nsplit : 0;
+  if (mine == 0) return;
+  const double* blk = a.node + 4 * (size_t)(a.off[a.lev] + b);
+  const int2* loc = reinterpret_cast<const int2*>(a.loc) + (size_t)b * a.M;
+  const bool active = b * 32 + lane < a.n_tgt;
+  const int t = active ? b * 32 + lane : a.n_tgt - 1;
+  KW<T> kw;
+  kw.init(a.kre, a.kim, a.hk_tab);
+  const T kk = kw.kval();
+  int oqmax = 0;
+  for (int e = lane; e < mine; e += 32) oqmax = max(oqmax, loc[split + nsplit * e].y >> 8);
+  oqmax = __reduce_max_sync(0xffffffffu, oqmax);
+  // the basis: the columns of a side by two warps of four, then all warps' pairs of orders on both sides
+  for (int phase = 0; phase < 3; ++phase) {
+    const int p = a.p;
+    for (int sd = phase < 2 ? warp >> 2 : 0; sd < (phase < 2 ? (warp >> 2) + 1 : 2); ++sd) {
+      const int c = sd * a.n_tgt + t;
+      unsigned char* set = ms.setup + sd * (far_col_bytes<T>(p) + far_warp_bytes<T>(p));
+      T* colJ = reinterpret_cast<T*>(set) + lane;
+      cplx* sH = reinterpret_cast<cplx*>(set + far_col_bytes<T>(p)) + lane;
+      T* sF = reinterpret_cast<T*>(sH - lane + (kTreeP + p + 2) * 32) + lane;
+      const double cx = a.cx[c], cy = a.cy[c];
+      double ux = a.tx[t] - cx, uy = a.ty[t] - cy;
+      const double r = hypot(ux, uy), vx = cx - blk[0], vy = cy - blk[1], rho = sqrt(fma(vx, vx, vy * vy));
+      ux /= r;
+      uy /= r;
+      const double ct = rho > 0.0 ? vx / rho : 1.0, st = rho > 0.0 ? vy / rho : 0.0;
+      if (phase == 0) {
+        if ((warp & 3) == 0) besselj_column<T>(rmul(kk, r), p + 1, colJ, 32);
+        if ((warp & 3) == 1) besselj_wave<T>(rmul(kk, rho), oqmax + p + 1, sH);
+        continue;
+      }
+      if (phase == 1) {
+        if ((warp & 3) == 0) far_orders<T>(fma(ux, ct, uy * st), fma(uy, ct, -ux * st), p, colJ, sF);
+        continue;
+      }
+      double cm = 1.0, sn = 0.0;
+      for (int m = 0; m <= oqmax; ++m) {
+        const double c1 = fma(cm, ct, -sn * st), s1 = fma(sn, ct, cm * st);
+        if (!(m & 1) && (m >> 1) % kLocWarps == warp) {
+          cplx X0, Y0, X1, Y1;
+          far_pair<T>(sH, sF, colJ[0], m, p, X0, Y0, X1, Y1);
+          auto add = [&](int n, const cplx fc, const cplx fs) {
+            ms.basis[n][0][lane] = sd ? ms.basis[n][0][lane] + fc : fc;
+            ms.basis[n][1][lane] = sd ? ms.basis[n][1][lane] + fs : fs;
+          };
+          add(m, lin2(cm, X0, -sn, Y0), lin2(sn, X0, cm, Y0));
+          if (m < oqmax) add(m + 1, lin2(c1, X1, -s1, Y1), lin2(s1, X1, c1, Y1));
+        }
+        cm = c1;
+        sn = s1;
+      }
+    }
+    __syncthreads();
+  }
+  const double swt = sqrt(q.tw[t]);
+  cplx* out = reinterpret_cast<cplx*>(q.out);
+  const int ncol = a.nrhs;
+  for (int e0 = 0; e0 < mine; e0 += kLocNodes) {
+    if (e0) __syncthreads();
+    if (warp == 0 && e0 + lane < mine) loc_waves<T>(kw, blk, a.node, loc[split + nsplit * (e0 + lane)], sm.h[lane], &sm.dir[lane]);
+    __syncthreads();
+    for (int e = warp; e < min(kLocNodes, mine - e0); e += kLocWarps) {
+      const int2 ent = loc[split + nsplit * (e0 + e)];
+      const int om = ent.y & 0xff, oq = ent.y >> 8;
+      const double2 dir = sm.dir[e];
+      double cl, sl;
+      lane_power(lane, dir.x, dir.y, cl, sl);
+      for (int c0 = 0; c0 < ncol; c0 += NC) {
+        const int nc = min(NC, ncol - c0);
+        __syncwarp();
+        if (lane <= om) {
+          const cplx* co = reinterpret_cast<const cplx*>(a.coef) + (((size_t)ent.x * (kTreeP + 2) + lane) * ncol + c0) * 2;
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            if (c >= nc) break;
+            rotate_in(co[2 * c], co[2 * c + 1], cl, sl, &sm.sd[warp][2 * c][lane], &sm.sd[warp][2 * c + 1][lane],
+                      &sm.ss[warp][2 * c][lane], &sm.ss[warp][2 * c + 1][lane]);
+          }
+        }
+        __syncwarp();
+        cplx accA[NC], accB[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) accA[c] = accB[c] = cplx{0.0, 0.0};
+        translate<NC, cplx>(sm.h[e], sm.sd[warp], sm.ss[warp], om, oq, nc, lane, cl, sl, accA, accB);
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          sm.sd[warp][2 * c][lane] = (lane == 0 ? 0.5 : 1.0) * accA[c];
+          sm.sd[warp][2 * c + 1][lane] = lane == 0 ? cplx{0.0, 0.0} : accB[c];
+        }
+        __syncwarp();
+        cplx v[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[c] = cplx{0.0, 0.0};
+        for (int m = 0; m <= oq; ++m) {
+          const cplx fc = ms.basis[m][0][lane], fs = ms.basis[m][1][lane];
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            cfma(v[c], sm.sd[warp][2 * c][m], fc);
+            cfma(v[c], sm.sd[warp][2 * c + 1][m], fs);
+          }
+        }
+        if (active) {
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            if (c >= nc) break;
+            const int col = ent.x * ncol + c0 + c;
+            const double sc = swt / sqrt(q.tw[col]);
+            out[(size_t)col * a.n_tgt + t] = cplx{sc * (-0.125 * v[c].im), sc * (0.125 * v[c].re)};
+          }
+        }
+      }
+    }
+  }
+}
+
+// the columns of the interpolation as weighted densities: wd[s][i] = w_s P[s mod q_src][i]
+__global__ void k_matrix_density(int n, int q_src, int q_tgt, const double* w, const double* P, cplx* wd) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n * q_tgt) return;
+  const int s = i / q_tgt;
+  wd[i] = cplx{w[s] * P[(s % q_src) * q_tgt + i - s * q_tgt], 0.0};
 }
 
 // Far sums: a warp holds 32 centres of one side (one per lane) and takes the
@@ -1686,6 +1839,73 @@ cudaError_t launch_tree_lists(const TreeArgs& a, cudaStream_t st, int n_inst) {
 
 cudaError_t launch_tree_moments(const TreeArgs& a, bool ck, cudaStream_t st, int n_inst) {
   return ck ? launch_moments_t<cplx>(a, st, n_inst) : launch_moments_t<double>(a, st, n_inst);
+}
+
+// Assembled matrix: the set-up of the tree over whole panels and its bytes
+// (base null: only those); 0 where the entries are formed pair by pair.
+size_t matrix_tree_setup(MatrixFarArgs* q, const qbx_geom* g, qbx_c64 k, qbx_c64 eta, int p, const double* hk_tab,
+                         char* base) {
+  *q = MatrixFarArgs{};
+  TreeArgs& t = q->t;
+  if (g->M < kTreeMinPanels || g->q_src > 128) return 0;
+  const bool ck = k.im != 0.0;
+  const size_t setup = 2 * (ck ? far_col_bytes<cplx>(p) + far_warp_bytes<cplx>(p) : far_col_bytes<double>(p) + far_warp_bytes<double>(p));
+  if (setup > sizeof(LocSmem) || (ck ? moments_smem<cplx>(g->q_src) : moments_smem<double>(g->q_src)) > 220 * 1024) return 0;
+  t.kre = k.re;
+  t.kim = k.im;
+  t.eta_re = eta.re;
+  t.eta_im = eta.im;
+  t.p = t.pl = p;
+  t.nd = 1;
+  t.only_loc = 1;
+  t.M = g->M;
+  t.q_src = g->q_src;
+  t.n_src = g->n_src;
+  t.lev = 1;
+  t.off[0] = 0;
+  t.off[1] = g->M;
+  t.sx = g->src_x;
+  t.sy = g->src_y;
+  t.snx = g->src_nx;
+  t.sny = g->src_ny;
+  t.n_tgt = g->n_tgt;
+  t.n_ctr = 2 * g->n_tgt;
+  t.cx = g->ctr_x;
+  t.cy = g->ctr_y;
+  t.tx = g->tgt_x;
+  t.ty = g->tgt_y;
+  t.hk_tab = hk_tab;
+  t.n_blk = (g->n_tgt + 31) / 32;
+  t.nrhs = g->q_tgt;
+  t.up = 1;
+  t.ops = OPB_C;
+  const int none[3] = {0, 0, 0};
+  tree_columns(&t, none);
+  size_t at = tree_layout(&t, base);
+  t.wd[0] = base ? base + at : nullptr;
+  at += host_align256((size_t)g->n_src * g->q_tgt * 16);
+  q->tw = g->tgt_w;
+  return at;
+}
+
+template <typename T>
+static cudaError_t launch_matrix_far_t(const MatrixFarArgs& q, const double* sw, const double* P, cudaStream_t st) {
+  const TreeArgs& a = q.t;
+  const int n = a.n_src * a.nrhs;
+  k_matrix_density<<<(n + 255) / 256, 256, 0, st>>>(a.n_src, a.q_src, a.nrhs, sw, P, (cplx*)a.wd[0]);
+  const size_t sm = moments_smem<T>(a.q_src);
+  cudaError_t e = cudaFuncSetAttribute(k_tree_moments<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_tree_matrix<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MatrixSmem));
+  if (e != cudaSuccess) return e;
+  k_tree_moments<T><<<dim3(a.M, 1, 1), 128, sm, st>>>(a);
+  // one CTA (8 warps) per SM
+  const unsigned ns = (unsigned)std::max(1, std::min((152 + a.n_blk - 1) / a.n_blk, (a.M + kLocWarps - 1) / kLocWarps));
+  k_tree_matrix<T><<<dim3(a.n_blk, ns), 32 * kLocWarps, sizeof(MatrixSmem), st>>>(q);
+  return cudaGetLastError();
+}
+cudaError_t launch_matrix_far(const MatrixFarArgs& q, const double* sw, const double* P, cudaStream_t st) {
+  return q.t.kim != 0.0 ? launch_matrix_far_t<cplx>(q, sw, P, st) : launch_matrix_far_t<double>(q, sw, P, st);
 }
 
 cudaError_t launch_far_clusters(TreeArgs a, cudaStream_t st) {

@@ -360,6 +360,20 @@ def test_non_finite_inputs_are_reported(cuda):
         qbx.qbx_sync_status(plan)
 
 
+@pytest.mark.parametrize("M,qt,qs,k,p,scale", [
+    (16, 16, 64, 5.0, 8, 1.0), (33, 16, 64, 9.0, 10, 1.0), (41, 5, 21, 7.0, 6, 1.0), (37, 9, 128, 4.0, 12, 1.0),
+    (37, 9, 127, 4 + 0.3j, 12, 1.0), (40, 12, 40, 6 + 0.5j, 9, 1.0), (40, 16, 64, 60.0, 12, 1.0),
+    (40, 16, 64, 1e-3, 1, 1.0), (40, 16, 16, 5.0, 20, 1e-4), (50, 16, 64, 5.0, 30, 1.0), (64, 1, 8, 3.0, 0, 1.0)])
+def test_assembled_matrix_clusters_match_pairs(cuda, M, qt, qs, k, p, scale):
+    """Every entry against the largest: the rows of a far panel are cut at 5e-17 of a kernel value."""
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(qt, qs, n_src=M * qs, n_ctr=2 * M * qt, ncoef=8, nrhs=qt)
+    g = geometry(plan, cur, cur.edges(M), scale)
+    got = qbx.qbx_assemble_cfie(plan, g, k / scale, (2.0 - 0.5j) / scale, p)
+    ref = qbx.qbx_assemble_cfie(qbx.Plan(qt, qs, workspace_bytes=4096), g, k / scale, (2.0 - 0.5j) / scale, p)
+    check(got, ref, "A")
+
+
 @pytest.mark.parametrize("k", [2 + 6j, 0.1 + 9j, 30 + 30j])
 def test_hankel_ray_at_strong_damping(cuda, k):
     """The amplitude table loses nothing to e^{2 Im z}: scipy's scaled Hankel
