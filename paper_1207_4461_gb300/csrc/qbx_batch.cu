@@ -316,6 +316,7 @@ int configure(qbx_batch* b, int rg, int chunk) {
     for (const TreeArgs& t : b->h_tree) {
       tr.M = std::max(tr.M, t.M);
       tr.n_blk = std::max(tr.n_blk, t.n_blk);
+      tr.n_sup = std::max(tr.n_sup, t.n_sup);
       if (t.off[t.lev] > tr.off[tr.lev]) {
         tr.lev = t.lev;
         for (int l = 0; l <= t.lev; ++l) tr.off[l] = t.off[l];

@@ -846,8 +846,9 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
       ns_far = std::max(1, std::min(4, (p->num_sms * 3 + units - 1) / units));
     } else {
       // a few CTAs per SM share a block's far nodes; few blocks: several warps to a node
+      // (16 blocks: 8 CTAs to a block 189 us, 19 CTAs 112)
       tr.nparts = std::max(1, std::min(4, p->num_sms * 8 / (units * 16)));
-      ns_far = std::max(2, std::min(8, (p->num_sms * 2 + units - 1) / units));
+      ns_far = std::max(2, std::min(20, (p->num_sms * 2 + units - 1) / units));
     }
     if (!(far_group ? far_group_fit(tr, ck, nsd) : far_clusters_fit(tr)) ||
         avail < tree_bytes + (size_t)(ns_far + 1) * per_split)
@@ -1077,7 +1078,7 @@ static int grad_d_impl(qbx_plan* p, const qbx_geom* g, int side, int limit, qbx_
       tree_levels(g->M, g->q_src, &tr);
       tree_bytes = tree_layout(&tr, nullptr);
       tr.nparts = std::max(1, std::min(4, p->num_sms * 8 / (units * 16)));
-      ns_far = std::max(2, std::min(8, (p->num_sms * 2 + units - 1) / units));
+      ns_far = std::max(2, std::min(20, (p->num_sms * 2 + units - 1) / units));
       if (!far_clusters_fit(tr) || p->ws_bytes < fixed + tree_bytes + (size_t)(ns_far + 1) * per_split) ns_far = 0;
     }
     const bool tree = ns_far > 0;

@@ -275,6 +275,7 @@ constexpr int kTreeLocal = 32;    // near-only QBX: orders of a centre's expansi
 constexpr int kTreeMinPanels = 16;   // fewer panels: every source pair by pair (no cluster of 8 is far from any block)
 constexpr int kTreeLevels = 16;
 constexpr int kTreeSets = 4;
+constexpr int kSupLevels = 7;
 // what a moment set is made of: the density itself, or dipoles along n_s, x, y
 enum { kSetMono = 0, kSetNormal = 1, kSetX = 2, kSetY = 3, kSetCombined = 4,
        kSetQuadX = 5, kSetQuadY = 6 };   // (the dipoles' derivatives along x, y)
@@ -299,12 +300,18 @@ struct TreeArgs {
   int lev;                    // levels; node (l, j) is off[l] + j
   int off[kTreeLevels + 1];   // off[lev]: node count
   int n_blk;                  // 32-target blocks
-  double* node;               // [nodes + n_blk][4]: centre x, y, radius; then the blocks
+  double* node;               // [nodes + n_blk + n_sup][4]: centre x, y, radius; then the blocks, super-blocks
   int* near;                  // [n_blk][M] near leaves
   int* far;                   // [n_blk][M + 1][2] far nodes: index, orders (cluster | centre << 8);
                               // last the block's local expansion (index nodes + block, bit 16 set)
   int* loc;                   // [n_blk][M][2] nodes of the local expansion: index, orders (cluster | block << 8)
   int* cnt;                   // [n_blk][3] counts: near, far, loc
+  // super-blocks (many columns): 2^B consecutive blocks, B = 1..sup_lev, index
+  // sup_off[B] + j; their entries follow the blocks' in node and coef
+  int n_sup, sup_lev, sup_c, sup_off[kSupLevels + 2], sup_stride;
+  int* sloc;                  // [n_sup][sup_stride][2] as loc
+  int* scnt;                  // [n_sup][2] entries, largest centre order
+  unsigned char* scov;        // [n_sup][M] leaves in the list of the super-block or of one above it
   int nset, nrhs;
   int kind[kTreeSets];
   int slot[kTreeSets];        // which of the call's densities
@@ -315,7 +322,7 @@ struct TreeArgs {
   void* mom;                  // few columns: [lev][M][nset nrhs][kTreeP + 2][2] leaf contributions
   int ncset;                  // coefficient column sets: a moment set, or its x, y derivative
   int base[2 * kTreeSets], shift[2 * kTreeSets], plain[kTreeSets];
-  void* coef;                 // [nodes + n_blk][kTreeP + 2][ncset nrhs][2] coefficients
+  void* coef;                 // [nodes + n_blk + n_sup][kTreeP + 2][ncset nrhs][2] coefficients
   // evaluation (launch_far_clusters)
   int ops;                    // OPB_* bits
   int set_s, set_d, set_g, set_gx, set_x;   // column sets (grad S: the density's, its x derivative; y after x)

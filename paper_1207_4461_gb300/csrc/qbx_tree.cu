@@ -85,11 +85,135 @@ __global__ void __launch_bounds__(256) k_tree_nodes(TreeArgs q) {
   }
 }
 
+// Super-blocks (many columns): a node that is far from 2^B consecutive blocks
+// of targets goes into one expansion about them all, which the blocks take up
+// as one more entry (k_tree_local), instead of into every block's own.  At 256
+// panels, k = 40: 49 entries per block become 8, and 20 per block in the super-
+// blocks (12 curves, 64 columns: 17.9 -> 11.4 ms of local expansions; teardrop,
+// k = 30: 4.4 -> 2.4).  First their discs: one CTA per super-block.
+__global__ void __launch_bounds__(256) k_tree_super(TreeArgs q) {
+  const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
+  __shared__ float s_red[8];
+  const int id = blockIdx.x;
+  if (id >= a.n_sup) return;
+  int B = 1;
+  while (id >= a.sup_off[B + 1]) ++B;
+  const int t0 = (id - a.sup_off[B]) * (32 << B), t1 = min(a.n_tgt, t0 + (32 << B));
+  const double x0 = a.tx[t0], y0 = a.ty[t0];
+  float xa = -INFINITY, xb = -INFINITY, ya = -INFINITY, yb = -INFINITY;
+  for (int t = t0 + threadIdx.x; t < t1; t += 256) {
+    const float x = (float)(a.tx[t] - x0), y = (float)(a.ty[t] - y0);
+    xa = fmaxf(xa, -x);
+    xb = fmaxf(xb, x);
+    ya = fmaxf(ya, -y);
+    yb = fmaxf(yb, y);
+  }
+  xa = block_reduce_max(xa, s_red, 8);
+  xb = block_reduce_max(xb, s_red, 8);
+  ya = block_reduce_max(ya, s_red, 8);
+  yb = block_reduce_max(yb, s_red, 8);
+  const double zx = x0 + (double)(0.5f * (xb - xa)), zy = y0 + (double)(0.5f * (yb - ya));
+  float rd = 0.0f, rm = 0.0f, bad = 0.0f;
+  for (int t = t0 + threadIdx.x; t < t1; t += 256)
+    for (int c = t; c < a.n_ctr; c += a.n_tgt) {
+      const float ex = (float)(a.tx[t] - a.cx[c]), ey = (float)(a.ty[t] - a.cy[c]);
+      const float ox = (float)(a.cx[c] - zx), oy = (float)(a.cy[c] - zy);
+      const float r = sqrtf(fmaf(ex, ex, ey * ey)) * 1.00001f, v = sqrtf(fmaf(ox, ox, oy * oy)) + r;
+      if (!(v < 1e30f)) bad = 1.0f;
+      rd = fmaxf(rd, v);
+      rm = fmaxf(rm, r);
+    }
+  rd = block_reduce_max(rd, s_red, 8);
+  rm = block_reduce_max(rm, s_red, 8);
+  bad = block_reduce_max(bad, s_red, 8);
+  if (threadIdx.x == 0) {
+    double* n = a.node + 4 * (size_t)(a.off[a.lev] + a.n_blk + id);
+    n[0] = zx;
+    n[1] = zy;
+    n[2] = bad > 0.0f ? INFINITY : (double)(rd * 1.00001f);   // (no node is far from such a one)
+    n[3] = rm;
+  }
+}
+
+// Their lists: for the super-blocks above this one and then itself, from the
+// largest down, the nodes of its own size and twice it that are far from all
+// its discs and not covered yet; its own go into its list in node order.
+// Every super-block goes through its ancestors' tests itself (same
+// instructions, same numbers), so all agree on what is covered.
+__global__ void __launch_bounds__(256) k_super_lists(TreeArgs q) {
+  const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
+  const int id = blockIdx.x;
+  if (id >= a.n_sup) return;
+  __shared__ int s_n[8], s_at, s_ol;
+  int B = 1;
+  while (id >= a.sup_off[B + 1]) ++B;
+  const int j = id - a.sup_off[B], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned char* cov = a.scov + (size_t)id * a.M;
+  int2* out = reinterpret_cast<int2*>(a.sloc) + (size_t)id * a.sup_stride;
+  const float ka = (float)sqrt(a.kre * a.kre + a.kim * a.kim), ki = (float)a.kim;
+  for (int i = threadIdx.x; i < a.M; i += 256) cov[i] = 0;
+  if (threadIdx.x == 0) s_at = s_ol = 0;
+  __syncthreads();
+  for (int Bb = a.sup_lev; Bb >= B; --Bb) {
+    const double* sb = a.node + 4 * (size_t)(a.off[a.lev] + a.n_blk + a.sup_off[Bb] + (j >> (Bb - B)));
+    const double bx = sb[0], by = sb[1];
+    const float rd = (float)sb[2] * 1.00001f, rm = (float)sb[3];
+    for (int l = min(Bb + a.sup_c + 1, a.lev - 1); l >= Bb + a.sup_c; --l) {
+      const int nl = a.off[l + 1] - a.off[l];
+      for (int i0 = 0; i0 < nl; i0 += 256) {
+        const int i = i0 + threadIdx.x;
+        int code = 0;
+        if (i < nl && !cov[i << l]) {
+          const double* n = a.node + 4 * (size_t)(a.off[l] + i);
+          const float dx = (float)(n[0] - bx), dy = (float)(n[1] - by), R = (float)n[2] * 1.00001f;
+          const float d = 0.99999f * sqrtf(fmaf(dx, dx, dy * dy)), dl = d - R, dm = d - rd, rho = dl - rd;
+          if (dl > 1.34f * rd && dm > 1.34f * R && rho > 1.34f * rm) {
+            const int oq = series_order(ka * rd, ka * dl, rd / dl, expf(2.0f * ki * rd), a.nd, kTreeP);
+            const int om = series_order(ka * R, ka * dm, R / dm, expf(2.0f * ki * R), a.nd, kTreeP);
+            int ol = rm > 0.0f ? series_order(ka * rm, ka * rho, rm / rho, expf(2.0f * ki * rm), a.nd, a.pl) : 0;
+            bool ok = oq <= kTreeP && om <= kTreeP;
+            if (a.eta > 0.0) ok = ok && rho >= 1.00001f * (float)a.eta * rm && ol <= a.pl;   // (all by the smooth rule)
+            else ol = min(ol, a.p);
+            // H of order om + ol and the moments of order om stay in FP64's range
+            const float no = (float)(om + max(ol, oq));
+            ok = ok && no * log10f(fmaxf(2.0f * no / (2.7f * ka * dm), 1.0f)) < 280.0f &&
+                 (float)om * log10f(fmaxf(2.0f * om / (2.7f * ka * R), 1.0f)) < 280.0f;
+            if (ok) code = om | oq << 8 | ol << 16 | 1 << 24;
+          }
+        }
+        if (Bb == B) {
+          const unsigned mine = __ballot_sync(0xffffffffu, code != 0);
+          if (lane == 0) s_n[warp] = __popc(mine);
+          __syncthreads();
+          int at = s_at;
+          for (int w = 0; w < warp; ++w) at += s_n[w];
+          if (code) {
+            out[at + __popc(mine & ((1u << lane) - 1))] = make_int2(a.off[l] + i, code & 0xffff);
+            atomicMax(&s_ol, code >> 16 & 0xff);
+          }
+          __syncthreads();
+          if (threadIdx.x == 0)
+            for (int w = 0; w < 8; ++w) s_at += s_n[w];
+          __syncthreads();
+        }
+        if (code)
+          for (int v = i << l; v < min(a.M, (i + 1) << l); ++v) cov[v] = 1;
+      }
+      __syncthreads();
+    }
+  }
+  if (threadIdx.x == 0) {
+    a.scnt[2 * id] = s_at;
+    a.scnt[2 * id + 1] = s_ol;
+  }
+}
+
 // Lists: one CTA per block of 32 targets, one thread per leaf.  A leaf's
 // thread looks from the largest node down for the first that is far from the
 // block; the first leaf of that node names it.  In leaf order, so the sums
 // do not depend on timing.
 constexpr int kListWarps = 8;
+constexpr int kSupMinLeaves = 128;   // fewer: no node of that size is far from a super-block
 __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs q) {
   const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
   if (blockIdx.x >= a.n_blk) return;
@@ -145,6 +269,8 @@ __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs q) {
   int* near = a.near + (size_t)b * a.M;
   int2* far = reinterpret_cast<int2*>(a.far) + (size_t)b * (a.M + 1);
   int2* loc = reinterpret_cast<int2*>(a.loc) + (size_t)b * a.M;
+
+  const unsigned char* cov = a.n_sup ? a.scov + (size_t)(a.sup_off[1] + (b >> 1)) * a.M : nullptr;   // by super-blocks
 
   // orders (cluster | centre << 8 | block << 16; block 0: not through the
   // block's local expansion) and bit 24 if the node is far from the block, else 0
@@ -207,14 +333,20 @@ __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs q) {
   for (int base = 0; base < a.M; base += 32 * kListWarps) {
     const int j = base + threadIdx.x;
     int code = 0, l = a.lev - 1;
-    if (j < a.M) {
+    const bool covered = cov && j < a.M && cov[j];
+    if (j < a.M && !covered) {
       for (; l >= 0; --l) {
+        if (cov) {   // no leaf of the node may be covered (covered are whole nodes of level sup_c + 1 and up)
+          bool hit = false;
+          for (int i = j >> l << l; i < min(a.M, ((j >> l) + 1) << l) && !hit; i += 2 << a.sup_c) hit = cov[i];
+          if (hit) continue;
+        }
         code = test(a.off[l] + (j >> l));
         if (code) break;
       }
     }
     if (a.only_loc && !(code >> 16 & 0xff)) code = 0;
-    const bool is_near = j < a.M && !code;
+    const bool is_near = j < a.M && !code && !covered;
     const bool is_node = code && (j & ((1 << l) - 1)) == 0, has_loc = (code >> 16 & 0xff) > 0;
     const bool is_far = is_node && !has_loc, is_loc = is_node && has_loc;
     const unsigned below = (1u << lane) - 1;
@@ -247,7 +379,15 @@ __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs q) {
   }
   if (threadIdx.x == 0) {
     int nf = s_at[1];
-    if (s_at[2] > 0)   // the block's local expansion, after the far nodes
+    bool sup = false;
+    for (int B = 1; a.n_sup && B <= a.sup_lev; ++B) {
+      const int* sc = a.scnt + 2 * (a.sup_off[B] + (b >> B));
+      if (sc[0] == 0) continue;
+      sup = true;
+      s_ord[0] = kTreeP;
+      s_ord[1] = max(s_ord[1], sc[1]);
+    }
+    if (s_at[2] > 0 || sup)   // the block's local expansion, after the far nodes
       far[nf++] = make_int2(a.off[a.lev] + b, s_ord[0] | s_ord[1] << 8 | 1 << 16);
     a.cnt[3 * b] = s_at[0];
     a.cnt[3 * b + 1] = nf;
@@ -917,11 +1057,13 @@ __device__ __forceinline__ void loc_waves(const KW<T>& kw, const double* blk, co
 //   S_q = sum_m s_m (H_{m-q} + (-1)^q H_{m+q}),  T_q = sum_m d_m (H_{m-q} - (-1)^q H_{m+q}),
 //   A'_q = cos(q Theta) S_q - i sin(q Theta) T_q,  B'_q = sin(q Theta) S_q + i cos(q Theta) T_q
 // (A'_0 halved).  Lane = q: a tenth of the FP64 work of taking the node through
-// each of the block's 32 or 64 centres.  A CTA takes a block and up to 8 groups
-// of 4 columns, a warp per group (with fewer groups the warps share the nodes).
-// The waves of 32 nodes at a time, one node per lane, serve all its columns:
-// formed by every warp for its own node and columns they were a quarter of the
-// FP64 work (12 curves, 24 columns: all of this kernel 22.4 ms, now 17.9 with the three-product form).
+// each of the block's 32 or 64 centres.  A CTA takes a block and four columns,
+// its warps the block's nodes in turn.  The waves of 32 nodes at a time are
+// formed with one node per lane (by every warp for its own node they were a
+// quarter of the FP64 work: 12 curves, 64 columns 22.4 -> 17.9 ms with the
+// three-product form).  Eight groups of columns to a CTA share the waves, but
+// leave few and long CTAs: 64 columns at 256 panels with super-blocks 4.8 ms
+// against 2.4, although the waves are then formed once per group (2 % of the work).
 constexpr int kLocWarps = 8, kLocCols = 4, kLocNodes = 32, kLocRow = 2 * kTreeP + 3;
 struct LocSmem {
   cplx h[kLocNodes][kLocRow];
@@ -930,19 +1072,28 @@ struct LocSmem {
   double2 dir[kLocNodes];
 };
 template <typename T>
-__global__ void __launch_bounds__(32 * kLocWarps, 2) k_tree_local(TreeArgs q) {
+__global__ void __launch_bounds__(32 * kLocWarps, 2) k_tree_local(TreeArgs q, bool super) {
   const TreeArgs& a = q.inst ? q.inst[blockIdx.z] : q;
-  if (blockIdx.x >= a.n_blk) return;
+  if (blockIdx.x >= (super ? a.n_sup : a.n_blk)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   LocSmem& sm = *reinterpret_cast<LocSmem*>(smem_raw);
   constexpr int NC = kLocCols;
   static_assert(kTreeP < 32, "one lane per order");
   const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int cnt = a.cnt[3 * b + 2];
-  const int nmom = a.nset * a.nrhs, g0 = blockIdx.y * kLocWarps, G = min(kLocWarps, (nmom + NC - 1) / NC - g0);
-  if (cnt == 0 || G <= 0) return;
-  const int parts = kLocWarps / G, part = warp / G;   // warps sharing the nodes of a column group
-  const int col0 = (g0 + warp % G) * NC, nc = min(NC, nmom - col0);
+  const int cnt = super ? a.scnt[2 * b] : a.cnt[3 * b + 2];
+  __shared__ int s_anc[kSupLevels];   // the super-blocks above the block with a list, as node entries
+  int nanc = 0;
+  if (!super && a.n_sup) {
+    for (int B = 1; B <= a.sup_lev; ++B) {
+      const int id = a.sup_off[B] + (b >> B);
+      if (a.scnt[2 * id] == 0) continue;
+      if (threadIdx.x == 0) s_anc[nanc] = a.off[a.lev] + a.n_blk + id;
+      ++nanc;
+    }
+  }
+  const int nmom = a.nset * a.nrhs, col0 = blockIdx.y * NC;
+  if (cnt + nanc == 0 || col0 >= nmom) return;
+  const int nc = min(NC, nmom - col0);
   int ccol[NC];   // coefficient column of each moment column
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
@@ -950,40 +1101,60 @@ __global__ void __launch_bounds__(32 * kLocWarps, 2) k_tree_local(TreeArgs q) {
     ccol[c] = a.plain[set] * a.nrhs + col - set * a.nrhs;
   }
   const int ncol = a.ncset * a.nrhs;
-  const double* blk = a.node + 4 * (size_t)(a.off[a.lev] + b);
-  const int2* loc = reinterpret_cast<const int2*>(a.loc) + (size_t)b * a.M;
+  const int own = a.off[a.lev] + (super ? a.n_blk : 0) + b;   // this expansion's entry
+  const double* blk = a.node + 4 * (size_t)own;
+  const int2* loc = super ? reinterpret_cast<const int2*>(a.sloc) + (size_t)b * a.sup_stride
+                          : reinterpret_cast<const int2*>(a.loc) + (size_t)b * a.M;
   KW<T> kw;
   kw.init(a.kre, a.kim, a.hk_tab);
   cplx accA[NC], accB[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) accA[c] = accB[c] = cplx{0.0, 0.0};
+  // rows s_m, d_m of this warp's columns of node or super-block id; cos, sin of lane * Theta
+  auto rows = [&](int id, int om, const double2 dir, double& cl, double& sl) {
+    lane_power(lane, dir.x, dir.y, cl, sl);
+    __syncwarp();   // the previous rows are no longer read
+    if (lane <= om) {
+      const double2* co = reinterpret_cast<const double2*>(a.coef) + ((size_t)id * (kTreeP + 2) + lane) * ncol * 2;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (c >= nc) break;
+        const double2 A = co[2 * ccol[c]], B = co[2 * ccol[c] + 1];
+        rotate_in(cplx{A.x, A.y}, cplx{B.x, B.y}, cl, sl, &sm.sd[warp][2 * c][lane], &sm.sd[warp][2 * c + 1][lane],
+                  &sm.ss[warp][2 * c][lane], &sm.ss[warp][2 * c + 1][lane]);
+      }
+    }
+    __syncwarp();
+  };
   for (int e0 = 0; e0 < cnt; e0 += kLocNodes) {
     __syncthreads();   // the previous nodes' waves are no longer read
     if (warp == 0 && e0 + lane < cnt) loc_waves<T>(kw, blk, a.node, loc[e0 + lane], sm.h[lane], &sm.dir[lane]);
     __syncthreads();
-    const int ne = part < parts ? min(kLocNodes, cnt - e0) : 0;
-    for (int e = part; e < ne; e += parts) {
+    for (int e = warp; e < min(kLocNodes, cnt - e0); e += kLocWarps) {
       const int2 ent = loc[e0 + e];
       const int om = ent.y & 0xff, oq = ent.y >> 8;
-      const double2 dir = sm.dir[e];
-      double cl, sl;   // lane * Theta
-      lane_power(lane, dir.x, dir.y, cl, sl);
-      __syncwarp();   // the previous node's rows are no longer read
-      if (lane <= om) {
-        const double2* co = reinterpret_cast<const double2*>(a.coef) + ((size_t)ent.x * (kTreeP + 2) + lane) * ncol * 2;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          if (c >= nc) break;
-          const double2 A = co[2 * ccol[c]], B = co[2 * ccol[c] + 1];
-          rotate_in(cplx{A.x, A.y}, cplx{B.x, B.y}, cl, sl, &sm.sd[warp][2 * c][lane], &sm.sd[warp][2 * c + 1][lane],
-                    &sm.ss[warp][2 * c][lane], &sm.ss[warp][2 * c + 1][lane]);
-        }
-      }
-      __syncwarp();
+      double cl, sl;
+      rows(ent.x, om, sm.dir[e], cl, sl);
       translate<NC, cplx>(sm.h[e], sm.sd[warp], sm.ss[warp], om, oq, nc, lane, cl, sl, accA, accB);
     }
   }
-  // the sums of the warps of a column group, in warp order
+  if (nanc > 0) {   // the expansions of the super-blocks: the same translation with J about the block's centre
+    __syncthreads();
+    if (warp == 0 && lane < nanc) {
+      const double* nd = a.node + 4 * (size_t)s_anc[lane];
+      const double vx = blk[0] - nd[0], vy = blk[1] - nd[1], d = sqrt(fma(vx, vx, vy * vy));
+      sm.dir[lane] = d > 0.0 ? make_double2(vx / d, vy / d) : make_double2(1.0, 0.0);
+      besselj_column<T>(rmul(kw.kval(), d), 2 * kTreeP + 1, reinterpret_cast<T*>(sm.h[lane]), 1);
+    }
+    __syncthreads();
+    for (int e = warp; e < nanc; e += kLocWarps) {
+      double cl, sl;
+      rows(s_anc[e], kTreeP, sm.dir[e], cl, sl);
+      translate<NC, T>(reinterpret_cast<const T*>(sm.h[e]), sm.sd[warp], sm.ss[warp], kTreeP, kTreeP, nc, lane, cl, sl,
+                       accA, accB);
+    }
+  }
+  // the warps' sums, in warp order
   __syncwarp();
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
@@ -991,20 +1162,20 @@ __global__ void __launch_bounds__(32 * kLocWarps, 2) k_tree_local(TreeArgs q) {
     sm.sd[warp][2 * c + 1][lane] = accB[c];
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < G * 2 * NC * 32; i += 32 * kLocWarps) {
-    const int g = i / (2 * NC * 32), row = i / 32 % (2 * NC), m = i & 31;
-    cplx v = sm.sd[g][row][m];
-    for (int w = 1; w < parts; ++w) v = v + sm.sd[g + w * G][row][m];
-    sm.sd[g][row][m] = m > 0 ? v : row & 1 ? cplx{0.0, 0.0} : 0.5 * v;
+  for (int i = threadIdx.x; i < 2 * NC * 32; i += 32 * kLocWarps) {
+    const int row = i >> 5, m = i & 31;
+    cplx v = sm.sd[0][row][m];
+    for (int w = 1; w < kLocWarps; ++w) v = v + sm.sd[w][row][m];
+    sm.sd[0][row][m] = m > 0 ? v : row & 1 ? cplx{0.0, 0.0} : 0.5 * v;
   }
   __syncthreads();
-  cplx* out = reinterpret_cast<cplx*>(a.coef) + (size_t)(a.off[a.lev] + b) * (kTreeP + 2) * ncol * 2;
-  const int nmine = min(G * NC, nmom - g0 * NC), per = a.ncset * (kTreeP + 1);
-  for (int i = threadIdx.x; i < nmine * per; i += 32 * kLocWarps) {
+  cplx* out = reinterpret_cast<cplx*>(a.coef) + (size_t)own * (kTreeP + 2) * ncol * 2;
+  const int per = a.ncset * (kTreeP + 1);
+  for (int i = threadIdx.x; i < nc * per; i += 32 * kLocWarps) {
     const int c = i / per, rem = i - c * per, cs = rem / (kTreeP + 1), m = rem - cs * (kTreeP + 1);
-    const int col = g0 * NC + c, set = col / a.nrhs, r = col - set * a.nrhs;
+    const int col = col0 + c, set = col / a.nrhs, r = col - set * a.nrhs;
     if (a.base[cs] == set)
-      shifted_coef(a, cs, &sm.sd[c / NC][2 * (c % NC)][0], 1, 32, kTreeP, m, out + ((size_t)m * ncol + cs * a.nrhs + r) * 2);
+      shifted_coef(a, cs, &sm.sd[0][2 * c][0], 1, 32, kTreeP, m, out + ((size_t)m * ncol + cs * a.nrhs + r) * 2);
   }
 }
 
@@ -1368,8 +1539,12 @@ __global__ void __launch_bounds__(128) k_far_clusters(TreeArgs a) {
 // rhs): a CTA of eight warps holds 32 targets; for every far node of the block
 // the warps form the values of H_m cos(m Theta), H_m sin(m Theta) through the
 // target's centre (or the average over its two centres) in shared memory, as
-// k_far_clusters does, and then multiply them into RG columns each.  A column
-// costs 8 FP64 instructions per order where the pairs of a leaf cost 96.
+// k_far_clusters does, and then multiply them into RG columns each, three real
+// products per complex one (the coefficients' Re + Im formed once per warp for
+// its 32 targets, five orders at a time in the place of the waves): a column costs 6 FP64 instructions per
+// order where the pairs of a leaf cost 96 (with four products, 8: 12 curves, 64
+// columns 9.5 ms, now 8.5).
+constexpr int kFgWarps = 8, kFgOrders = 5, kFgCols = 8;
 template <typename T>
 struct FarGroupSmem {
   static __host__ __device__ size_t rows(int pl) { return (size_t)kTreeP + pl + 2; }
@@ -1378,7 +1553,6 @@ struct FarGroupSmem {
            (size_t)2 * (kTreeP + 1) * 32 * 16;
   }
 };
-constexpr int kFgWarps = 8;
 
 template <typename T, int RG>
 __global__ void __launch_bounds__(32 * kFgWarps) k_far_group(TreeArgs q) {
@@ -1395,6 +1569,12 @@ __global__ void __launch_bounds__(32 * kFgWarps) k_far_group(TreeArgs q) {
   T* sF = sJ + (size_t)nsd * (pl + 2) * 32;                            // [side][pl][2][32]
   double* sT = reinterpret_cast<double*>(sF + (size_t)nsd * pl * 64);  // [side][2][32] Theta
   int* sL = reinterpret_cast<int*>(sT + nsd * 64);                     // [side][32] orders l by m
+  // per warp: coefficients of its columns, [order][column][A, B], and their Re + Im
+  // (where the waves of the first side were: at least kTreeP + 2 rows)
+  static_assert(RG <= kFgCols && kFgWarps * kFgOrders * kFgCols * 2 * 24 <= (kTreeP + 2) * 32 * 16, "columns of the warps");
+  double* mine = reinterpret_cast<double*>(sH) + (size_t)warp * kFgOrders * kFgCols * 6;
+  cplx* sC = reinterpret_cast<cplx*>(mine);
+  double* sS = mine + kFgOrders * kFgCols * 4;
   const bool active = blk * 32 + lane < a.n_tgt;
   const int t = active ? blk * 32 + lane : a.n_tgt - 1;
   KW<T> kw;
@@ -1419,9 +1599,9 @@ __global__ void __launch_bounds__(32 * kFgWarps) k_far_group(TreeArgs q) {
   // columns in the coefficient rows: S's set, then D's (or the combined one)
   const int set0 = (a.ops & OPB_S) ? a.set_s : a.set_d, set1 = a.set_d;
   for (int g0 = 0; g0 < ncols; g0 += kFgWarps * RG) {
-    cplx acc[RG];
+    double acc[RG][3];
 #pragma unroll
-    for (int i = 0; i < RG; ++i) acc[i] = cplx{0.0, 0.0};
+    for (int i = 0; i < RG; ++i) acc[i][0] = acc[i][1] = acc[i][2] = 0.0;
     const int mycol = g0 + warp * RG;
     for (int e = split; e < cnt; e += a.nsplit) {
       const int2 ent = far[cnt - 1 - e];
@@ -1469,20 +1649,31 @@ __global__ void __launch_bounds__(32 * kFgWarps) k_far_group(TreeArgs q) {
       __syncthreads();
       if (mycol < ncols) {
         const double2* co = reinterpret_cast<const double2*>(a.coef) + (size_t)ent.x * (kTreeP + 2) * ccol * 2;
-        int at[RG];
+        for (int m0 = 0; m0 <= om; m0 += kFgOrders) {
+          const int nm = min(kFgOrders, om + 1 - m0);
+          __syncwarp();
+          for (int v = lane; v < nm * RG * 2; v += 32) {
+            const int m = v / (RG * 2), i = v / 2 % RG, c = min(mycol + i, ncols - 1), comp = c / a.nrhs;
+            const double2 w = __ldg(co + (size_t)(m0 + m) * ccol * 2 +
+                                    2 * ((comp ? set1 : set0) * a.nrhs + c - comp * a.nrhs) + (v & 1));
+            sC[v] = cplx{w.x, w.y};
+            sS[v] = w.x + w.y;
+          }
+          __syncwarp();
+          for (int m = 0; m < nm; ++m) {
+            const cplx fc = sB[2 * (m0 + m) * 32 + lane], fs = sB[(2 * (m0 + m) + 1) * 32 + lane];
+            const double tc = fc.re + fc.im, ts = fs.re + fs.im;
 #pragma unroll
-        for (int i = 0; i < RG; ++i) {
-          const int c = min(mycol + i, ncols - 1), comp = c / a.nrhs;
-          at[i] = 2 * ((comp ? set1 : set0) * a.nrhs + c - comp * a.nrhs);
-        }
-        for (int m = 0; m <= om; ++m) {
-          const cplx fc = sB[(2 * m) * 32 + lane], fs = sB[(2 * m + 1) * 32 + lane];
-          const double2* v = co + (size_t)m * ccol * 2;
-#pragma unroll
-          for (int i = 0; i < RG; ++i) {
-            const double2 A = __ldg(v + at[i]), B = __ldg(v + at[i] + 1);
-            cfma(acc[i], cplx{A.x, A.y}, fc);
-            cfma(acc[i], cplx{B.x, B.y}, fs);
+            for (int i = 0; i < RG; ++i) {
+              const int v = (m * RG + i) * 2;
+              const cplx A = sC[v], B = sC[v + 1];
+              acc[i][0] = fma(A.re, fc.re, acc[i][0]);
+              acc[i][1] = fma(A.im, fc.im, acc[i][1]);
+              acc[i][2] = fma(sS[v], tc, acc[i][2]);
+              acc[i][0] = fma(B.re, fs.re, acc[i][0]);
+              acc[i][1] = fma(B.im, fs.im, acc[i][1]);
+              acc[i][2] = fma(sS[v + 1], ts, acc[i][2]);
+            }
           }
         }
       }
@@ -1491,7 +1682,8 @@ __global__ void __launch_bounds__(32 * kFgWarps) k_far_group(TreeArgs q) {
       cplx* part = reinterpret_cast<cplx*>(a.part) + ((size_t)(a.split0 + split) * a.n_tgt + t) * ncols;
 #pragma unroll
       for (int i = 0; i < RG; ++i)
-        if (mycol + i < ncols) part[mycol + i] = acc[i];
+        if (mycol + i < ncols)
+          part[mycol + i] = cplx{acc[i][0] - acc[i][1], acc[i][2] - acc[i][0] - acc[i][1]};
     }
   }
 }
@@ -1786,8 +1978,9 @@ cudaError_t launch_moments_t(const TreeArgs& a, cudaStream_t st, int n_inst) {
   if (a.n_blk == 0) return cudaGetLastError();
   cudaError_t e = cudaFuncSetAttribute(k_tree_local<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocSmem));
   if (e != cudaSuccess) return e;
-  const int per = kLocWarps * kLocCols;
-  k_tree_local<T><<<dim3(a.n_blk, (ncol + per - 1) / per, n_inst), 32 * kLocWarps, sizeof(LocSmem), st>>>(a);
+  const int ng = (ncol + kLocCols - 1) / kLocCols;
+  if (a.n_sup) k_tree_local<T><<<dim3(a.n_sup, ng, n_inst), 32 * kLocWarps, sizeof(LocSmem), st>>>(a, true);
+  k_tree_local<T><<<dim3(a.n_blk, ng, n_inst), 32 * kLocWarps, sizeof(LocSmem), st>>>(a, false);
   return cudaGetLastError();
 }
 
@@ -1820,12 +2013,29 @@ size_t tree_layout(TreeArgs* a, char* base) {
     at += host_align256(bytes);
     return v;
   };
-  const size_t nodes = (size_t)a->off[a->lev] + a->n_blk, ncol = (size_t)a->ncset * a->nrhs;
+  // Super-blocks for many columns (with few, the two more launches cost what
+  // they give), from kSupMinLeaves leaves on; nodes of a super-block's size are
+  // sup_c levels above it, by the number of leaves next to 32 targets
+  a->n_sup = a->sup_lev = a->sup_c = 0;
+  if (a->up && !a->discs && !a->only_loc && a->M >= kSupMinLeaves) {
+    for (double r = 32.0 * a->M / a->n_tgt; r > 1.5; r *= 0.5) ++a->sup_c;
+    a->sup_off[1] = 0;
+    for (int B = 1; B <= kSupLevels && B + a->sup_c < a->lev; ++B) {
+      a->sup_lev = B;
+      a->n_sup += (a->n_blk + (1 << B) - 1) >> B;
+      a->sup_off[B + 1] = a->n_sup;
+    }
+    a->sup_stride = (a->M >> (a->sup_c + 1)) + 2;
+  }
+  const size_t nodes = (size_t)a->off[a->lev] + a->n_blk + a->n_sup, ncol = (size_t)a->ncset * a->nrhs;
   a->node = (double*)take(nodes * 4 * 8);
   a->near = (int*)take((size_t)a->n_blk * a->M * 4);
   a->far = (int*)take((size_t)a->n_blk * (a->M + 1) * 8);
   a->loc = (int*)take((size_t)a->n_blk * a->M * 8);
   a->cnt = (int*)take((size_t)a->n_blk * 12);
+  a->sloc = (int*)take((size_t)a->n_sup * a->sup_stride * 8);
+  a->scnt = (int*)take((size_t)a->n_sup * 8);
+  a->scov = (unsigned char*)take((size_t)a->n_sup * a->M);
   a->mom = take(a->up ? 0 : (size_t)a->lev * a->M * a->nset * a->nrhs * (kTreeP + 2) * 2 * 16);
   a->coef = take(nodes * ncol * (kTreeP + 2) * 2 * 16);
   return at;
@@ -1833,6 +2043,10 @@ size_t tree_layout(TreeArgs* a, char* base) {
 
 cudaError_t launch_tree_lists(const TreeArgs& a, cudaStream_t st, int n_inst) {
   k_tree_nodes<<<dim3(a.off[a.lev], 1, n_inst), 256, 0, st>>>(a);
+  if (a.n_sup) {
+    k_tree_super<<<dim3(a.n_sup, 1, n_inst), 256, 0, st>>>(a);
+    k_super_lists<<<dim3(a.n_sup, 1, n_inst), 256, 0, st>>>(a);
+  }
   k_tree_lists<<<dim3(a.n_blk, 1, n_inst), 32 * kListWarps, 0, st>>>(a);
   return cudaGetLastError();
 }

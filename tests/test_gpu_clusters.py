@@ -114,13 +114,38 @@ def test_many_columns_match_pairs(cuda, case):
         check(a, b, (case, i))
 
 
+@pytest.mark.parametrize("case", [
+    (64, 16, 64, 5.0, 8, (0,), "int", 0, 16, None),              # fewest leaves with super-blocks
+    (131, 16, 64, 9.0, 10, (0, 1), "two", 0, 17, None),          # ragged at every level
+    (150, 5, 21, 7.0, 6, (1,), "ext", 1, 16, None),              # several panels per block, whole-panel leaves
+    (200, 16, 64, 40.0, 10, (0, 1), "int", 0, 16, None),         # k caps the nodes
+    (160, 16, 64, 4 + 0.3j, 9, (0, 1), "ext", 0, 16, None),
+    (160, 16, 64, 12.0, 10, (0, 1), "two", 0, 16, 6.0),          # near-only
+    (128, 16, 64, 1e-3, 8, (0,), "two", 0, 16, None),
+    (210, 16, 64, 11.0, 14, "cfie", "two", 0, 33, None),
+    (130, 16, 64, 3 + 3j, 10, "cfie", "two", 0, 4, None)])
+def test_super_blocks_match_pairs(cuda, case):
+    """Nodes far from many blocks at once; panels of very different sizes too."""
+    test_many_columns_match_pairs(cuda, case)
+    M, qt, qs, k, p, ops, side, limit, nrhs, eta = case
+    if qt != 16 or ops == "cfie" or eta:
+        return
+    edges = W.dyadic_edges(M, 6)
+    cur, M = W.teardrop(), len(edges) - 1
+    plan = qbx.Plan(qt, qs, n_src=M * qs, n_ctr=2 * M * qt, ncoef=4, nrhs=nrhs)
+    g = geometry(plan, cur, edges)
+    d = torch.as_tensor(W.complex_gaussian(M + p, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    got = qbx.qbx_apply_cfie(plan, g, k, 1.0, p, d)
+    check(got, qbx.qbx_apply_cfie(pair_plan(g, qt, qs, nrhs, 1), g, k, 1.0, p, d), case)
+
+
 @pytest.mark.parametrize("side,limit,ops,eta,ck", [("int", 1, (0, 1), 0.0, False), ("two", 0, (0, 1), 0.0, False),
                                                    ("ext", 0, (1,), 7.0, False), ("two", 0, (0,), 0.0, True)])
-def test_batch_clusters_match_single_curves(cuda, side, limit, ops, eta, ck):
+def test_batch_clusters_match_single_curves(cuda, side, limit, ops, eta, ck, Ms=(40, 9, 64, 16, 12, 33)):
     """A batch of curves with and without clusters (2 and 9 panels form none)
     against each curve alone, pair by pair; twice, for the kept counter."""
     side = {"int": qbx.SIDE_INT, "ext": qbx.SIDE_EXT, "two": qbx.SIDE_TWO}[side]
-    Ms, ks = (40, 9, 64, 16, 12, 33), [5.0, 9.0, 14.0, 3.0, 2.0, 7.0]
+    ks = [5.0, 9.0, 14.0, 3.0, 2.0, 7.0]
     if ck:
         ks = [v * (1 + 0.05j) if i % 2 else v for i, v in enumerate(ks)]
     nrhs, p = 12, 9
@@ -139,6 +164,11 @@ def test_batch_clusters_match_single_curves(cuda, side, limit, ops, eta, ck):
         ref = qbx.qbx_apply_ops(pair_plan(g, 16, 64, nrhs, len(ops)), g, ops, side, limit, k, p, d, eta=eta or None)
         for i in ops:
             check(o[i], ref[i], (g.M, i))
+
+
+def test_batch_super_blocks_match_single_curves(cuda):
+    """Curves with super-blocks of several levels beside curves with none."""
+    test_batch_clusters_match_single_curves(cuda, "two", 0, (0, 1), 0.0, False, Ms=(130, 9, 64, 16, 90, 63))
 
 
 @pytest.mark.parametrize("order", ["dyadic", "shuffled"])
