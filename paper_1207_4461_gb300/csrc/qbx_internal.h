@@ -306,7 +306,7 @@ struct TreeArgs {
                               // last the block's local expansion (index nodes + block, bit 16 set)
   int* loc;                   // [n_blk][M][2] nodes of the local expansion: index, orders (cluster | block << 8)
   int* cnt;                   // [n_blk][3] counts: near, far, loc
-  // super-blocks (many columns): 2^B consecutive blocks, B = 1..sup_lev, index
+  // super-blocks: 2^B consecutive blocks, B = 1..sup_lev, index
   // sup_off[B] + j; their entries follow the blocks' in node and coef
   int n_sup, sup_lev, sup_c, sup_off[kSupLevels + 2], sup_stride;
   int* sloc;                  // [n_sup][sup_stride][2] as loc

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256) k_tree_nodes(TreeArgs q) {
   }
 }
 
-// Super-blocks (many columns): a node that is far from 2^B consecutive blocks
+// Super-blocks: a node that is far from 2^B consecutive blocks
 // of targets goes into one expansion about them all, which the blocks take up
 // as one more entry (k_tree_local), instead of into every block's own.  At 256
 // panels, k = 40: 49 entries per block become 8, and 20 per block in the super-
@@ -2013,11 +2013,13 @@ size_t tree_layout(TreeArgs* a, char* base) {
     at += host_align256(bytes);
     return v;
   };
-  // Super-blocks for many columns (with few, the two more launches cost what
-  // they give), from kSupMinLeaves leaves on; nodes of a super-block's size are
-  // sup_c levels above it, by the number of leaves next to 32 targets
+  // Super-blocks: nodes of a super-block's size are sup_c levels above it, by
+  // the number of leaves next to 32 targets.  Many columns: from kSupMinLeaves
+  // leaves on; few: from 64 blocks on (complex k: 128), where they are worth
+  // their three launches (S + D + grad S, 128 blocks 3.25 -> 3.18 ms; shape step
+  // of S, 64 and 256 blocks 4.68 -> 4.43; 64 blocks, complex k 3.41 -> 3.44)
   a->n_sup = a->sup_lev = a->sup_c = 0;
-  if (a->up && !a->discs && !a->only_loc && a->M >= kSupMinLeaves) {
+  if (!a->only_loc && (a->up ? a->M >= kSupMinLeaves : a->n_blk >= (a->kim != 0.0 ? 128 : 64))) {
     for (double r = 32.0 * a->M / a->n_tgt; r > 1.5; r *= 0.5) ++a->sup_c;
     a->sup_off[1] = 0;
     for (int B = 1; B <= kSupLevels && B + a->sup_c < a->lev; ++B) {
