@@ -70,12 +70,14 @@ def flops_per_pair_ops(ops, p, nrhs=1):
 # (dram__bytes_read.sum + dram__bytes_write.sum); valid only for the kernel
 # sources it was taken with, identified by their hash.
 TRAFFIC = {"27706399748d3043": 1.667e6}   # profiles/k_apply_fused_S_D_gradS_starfish_M256_dram.md
-KERNEL_SOURCES = ["qbx_apply_impl.cuh", "qbx_device.cuh", "special_tables.h", "qbx_apply_real.cu"]
+KERNEL_SOURCES = ["qbx_apply_impl.cuh", "qbx_device.cuh", "special_tables.h", "qbx_apply_real.cu", "qbx_tree.cu",
+                  "qbx_tree.cuh"]
 GROUP_SOURCES = ["qbx_group_impl.cuh", "qbx_apply_impl.cuh", "qbx_device.cuh", "special_tables.h"]
-# Hardware-counted FP64 operations per (centre, source) pair, 2 DFMA + DMUL +
-# DADD from ncu's smsp__sass_thread_inst_executed_op_{dfma,dmul,dadd}_pred_on
-# counters divided by the pairs of the captured launch, for the kernel
-# sources with the given hash (profiles/fp64_counts_fused_M128_and_group_batch4.md).
+# Hardware-counted FP64 operations, 2 DFMA + DMUL + DADD from ncu's
+# smsp__sass_thread_inst_executed_op_{dfma,dmul,dadd}_pred_on counters, of all
+# launches between oversampling and finishing of one apply, divided by its
+# nominal (centre, source) pairs: near leaves pair by pair, distant sources by
+# their clusters' moments.  For the kernel sources with the given hash.
 HW_FP64_PER_PAIR = {"27706399748d3043": 434.9}         # fused S + D + grad S, p = 12, one rhs
 HW_FP64_PER_PAIR_GROUP = {"5b690bb633cedf23": 732.9}   # group kernel, S + D, p = 10, 32 rhs
 # sm__pipe_fp64_cycles_active (of peak) over the active and the elapsed
@@ -336,25 +338,29 @@ def run_gpu(args, wl):
         kname = "k_apply_fused, one launch per operator"
     else:
         fpp = flops_per_pair_ops(list(wl.ops), wl.p, wl.nrhs)
-        kname = "k_apply_fused, operators " + "+".join(wl.ops) + " in one pass"
+        kname = ("k_apply_fused (near leaves), k_tree_* and k_far_clusters (distant clusters), operators " +
+                 "+".join(wl.ops) + " in one pass")
     achieved = pairs * fpp / (kern_ms * 1e-3) / 1e9
     hw = None
     if not (args.separate or args.panels or args.ops or args.k):
         hw = hw_roofline(HW_FP64_PER_PAIR.get(kernel_source_hash()), pairs, kern_ms * 1e-3,
                          HW_FP64_PIPE.get(kernel_source_hash()))
-    # headline: hardware-counted FP64 flops (2 DFMA + DMUL + DADD per pair from
-    # ncu, for these kernel sources) per second against the FP64 peak; the
-    # algorithmic model beside it; the model alone when no count matches
-    roofline = {"bound": "alu", "achieved": hw["achieved"] if hw else achieved, "peak": FP64_PEAK_GFLOPS,
-                "unit": "GFLOP/s", "frac": hw["frac"] if hw else achieved / FP64_PEAK_GFLOPS,
-                "basis": "ncu-counted FP64 flops per pair" if hw else "algorithmic flop model per pair",
+    # headline: hardware-counted FP64 flops (2 DFMA + DMUL + DADD from ncu, for
+    # these kernel sources) per second against the FP64 peak; none when no
+    # count matches (the flops of taking every pair, beside it, are not done)
+    roofline = {"bound": "alu", "achieved": hw["achieved"] if hw else None, "peak": FP64_PEAK_GFLOPS,
+                "unit": "GFLOP/s", "frac": hw["frac"] if hw else None,
+                "basis": "ncu-counted FP64 flops of the apply's launches" if hw else
+                         "no FP64 count taken with these kernel sources",
                 "traffic": kernel_traffic(wl, args),
                 "kernel": kname, "kernel_ms": kern_ms,
                 "timing": "CUDA events recorded by the library around the kernel launch(es) of every "
                           "timed call, on the launching stream",
-                "flops_per_pair": hw["fp64_ops_per_pair"] if hw else fpp,
+                "flops_per_pair": hw["fp64_ops_per_pair"] if hw else None,
                 "peak_basis": "152 SMs x 4 FP64 flop/clk x 2.07 GHz",
-                "model": {"flops_per_pair": fpp, "achieved": achieved, "frac": achieved / FP64_PEAK_GFLOPS},
+                "every_pair": {"flops_per_pair": fpp, "equivalent": achieved,
+                               "note": "rate at which taking every (centre, source) pair would have to run for the "
+                                       "same time; distant sources go through their clusters' moments instead"},
                 "hw": hw}
 
     # ---- end to end through the public API with host buffers (pinned)
@@ -383,7 +389,10 @@ def run_gpu(args, wl):
     e2e = {"value": job_rate(world, terms_step, e2e_ms), "unit": "terms/s",
            "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms}
 
-    launches = (3 * len(wl.ops)) if args.separate else (2 + len(wl.ops))   # upsample, fused, finish(es)
+    # per call: upsample, pair kernel, finish(es); with clusters (16 panels or more) nodes, block lists, moments,
+    # their sums, local expansions, far evaluation; from 64 blocks of targets on three for the super-blocks
+    tree = 0 if wl.n_tgt < 16 * 16 else 9 if wl.n_tgt >= 64 * 32 else 6
+    launches = ((3 + tree) * len(wl.ops)) if args.separate else (2 + tree + len(wl.ops))
     line = {"metric": METRIC, "value": value, "unit": "terms/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": step_ms, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f64", "data": "synthetic", "config": config_dict(wl, args),
@@ -572,9 +581,10 @@ def run_batch_compare(args, qbx, torch, small=None):
             "items": {"model": dict(zip(("rhs_per_warp", "src_chunk", "items", "ctas"), model_cfg)),
                       "tuned": dict(zip(("rhs_per_warp", "src_chunk", "items", "ctas"), tuned_cfg)),
                       "tune_s": t_tune},
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
-                         "frac": achieved / FP64_PEAK_GFLOPS, "flops_per_pair": fpp,
-                         "kernel": "k_apply_group (persistent, longest-first items, CUDA graph)",
+            "roofline": {"bound": "alu", "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
+                         "every_pair": {"flops_per_pair": fpp, "equivalent": achieved},
+                         "kernel": "k_apply_group (near leaves; persistent, longest-first items, CUDA graph), "
+                                   "k_tree_* and k_far_group (distant clusters)",
                          "timing": "whole graph (oversampling, group kernel, finishing) per apply",
                          "hw": None if not full64 else hw_roofline(
                              HW_FP64_PER_PAIR_GROUP.get(source_hash(GROUP_SOURCES)), pairs, ms_batch * 1e-3,

@@ -114,7 +114,12 @@ int qbx_gauss_legendre(int q, double *nodes, double *weights);
  * uploads the per-panel interpolation matrix from the target to the source
  * nodes (Sec. 3.4.2), a device status word, and allocates `workspace_bytes`
  * of device workspace used by the split-source reductions (see
- * qbx_workspace_bytes) and a 29 KB buffer for the H0/H1 amplitude table of
+ * qbx_workspace_bytes), by the cluster arrays of calls on 16 panels or more
+ * (distant sources by their moments; with a workspace that holds the partial
+ * sums but not these arrays the call takes every pair instead, more slowly
+ * and to the same accuracy), a side stream on which such a call's near pairs
+ * run beside the rest (forked from and joined to the call's stream by events,
+ * also under stream capture), and a 29 KB buffer for the H0/H1 amplitude table of
  * the ray z = k rho, which calls with a complex k fill (on their stream)
  * when k differs from the last one.  *plan receives the handle.  Host call,
  * synchronous. */
@@ -123,8 +128,8 @@ int qbx_plan_destroy(qbx_plan *plan);
 
 /* Kernel timing (no counterpart in the paper; for measurement).  With timing
  * on, every qbx_apply / qbx_apply_ops call on the plan records two CUDA
- * events on its stream around its pair-sum launches (the fused or group
- * kernel, without oversampling and finishing); qbx_plan_kernel_ms waits for
+ * events on its stream around its sums (the pair kernels and the cluster
+ * kernels, without oversampling and finishing); qbx_plan_kernel_ms waits for
  * the second event and returns the elapsed milliseconds of the last call.
  * QBX_EINVAL if timing is off.  Host calls. */
 int qbx_plan_set_timing(qbx_plan *plan, int on);
@@ -391,8 +396,9 @@ int qbx_vec_combine(int n, int nrhs, int nv, const qbx_c64 *V, const qbx_c64 *y,
  * column-major into A (entry (t, t') at A[t' n_tgt + t]; 16 n_tgt^2 bytes,
  * caller-owned device memory).  Row t holds, for both centres of target t,
  * the truncated Graf sums against every source node carried back to the
- * target grid by the per-panel interpolation.  q_tgt <= 16.  Async on
- * stream.  qbx_solve_exterior_dirichlet_assembled then runs the same GMRES
+ * target grid by the per-panel interpolation.  q_tgt <= 16.  From 16 panels
+ * on the distant panels' columns go through moments held in the plan's
+ * workspace (too small a workspace: every pair).  Async on stream.  qbx_solve_exterior_dirichlet_assembled then runs the same GMRES
  * with one complex matrix product (qbx_matmul_cm) per iteration for all
  * right-hand sides, one Arnoldi step captured as a CUDA graph and launched
  * up to `restart` times per cycle without a host wait (steps after
@@ -432,6 +438,8 @@ size_t qbx_matmul_cm_work_bytes(int n, int nrhs);
  * at most `chunk` of its sources (equal ranges per curve; the ranges' partial
  * sums are added in a fixed order), taken longest first by persistent CTAs
  * through an atomic counter; no CTA ever waits for another.
+ * Curves of 16 panels or more (S, D, S + D) take distant sources by their
+ * clusters' moments; without device memory for those arrays, every pair.
  * qbx_batch_create allocates the batch's device memory (with, for every
  * curve of complex k, the H0/H1 amplitude table of its ray z = k rho), picks
  * the chunk with the smallest predicted makespan of that schedule (a model

@@ -850,6 +850,8 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
       tr.nparts = std::max(1, std::min(4, p->num_sms * 8 / (units * 16)));
       ns_far = std::max(2, std::min(20, (p->num_sms * 2 + units - 1) / units));
     }
+    // (a tight workspace: fewer CTAs share a block's far nodes)
+    while (ns_far > 1 && avail < tree_bytes + (size_t)(ns_far + 8) * per_split) --ns_far;
     if (!(far_group ? far_group_fit(tr, ck, nsd) : far_clusters_fit(tr)) ||
         avail < tree_bytes + (size_t)(ns_far + 1) * per_split)
       ns_far = 0;

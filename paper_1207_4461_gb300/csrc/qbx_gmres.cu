@@ -5,8 +5,8 @@
 // with unknowns scaled by the square roots of the target weights (Sec. 4.2:
 // sqrt-weight unknowns).  Every system (right-hand side) has its own Krylov
 // basis; the systems advance in lockstep so that one matvec call serves all.
-// Vectors are [n][nrhs] complex; bases [m+1][n][nrhs].  Reductions are
-// two-pass in fixed order, so results are deterministic.
+// Vectors are [n][nrhs] complex; bases [m+1][n][nrhs].  Reductions add in a
+// fixed order, so results are deterministic.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
@@ -201,9 +201,8 @@ int qbx_vec_combine(int n, int nrhs, int nv, const qbx_c64* V, const qbx_c64* y,
 // driven from the device.  Arnoldi by classical Gram-Schmidt with one
 // re-orthogonalisation (CGS2); the Hessenberg columns, the Givens rotations,
 // the residual estimates |g_{j+1}| / ||f||, the convergence test and the
-// back-substitution of each restart cycle run in small kernels on the device
-// (one thread per right-hand side), so the host waits for the device once
-// per restart cycle.  The kernels of an Arnoldi step read the step index and
+// back-substitution of each restart cycle run on the device, so the host waits
+// for it once per restart cycle.  The kernels of an Arnoldi step read the step index and
 // the state (done, matvec count) from a control block in device memory and
 // do nothing once the step is inactive (all systems converged, maxiter
 // reached or the cycle full); with the assembled matrix one step is
@@ -258,7 +257,7 @@ constexpr int kDotCluster = 8, kDotThreads = 256, kDotRows = 76;   // CTAs per v
 // take the vectors in turn.  FP64-bound from some 20 vectors on (4 multiply-
 // adds per element).  With 152 row ranges x (m + 1) vectors of CTAs, most of
 // which had nothing to do, and a second kernel for the 152 sums, the products
-// of one step at n = 1152, 16 right-hand sides took 23 us, now 8.
+// of one step at n = 1152, 16 right-hand sides took 28 us, now 8.
 __global__ void __cluster_dims__(kDotCluster, 1, 1) __launch_bounds__(kDotThreads)
 k_dots_step(int n, int nrhs, const cplx* __restrict__ V, const int* ctl, cplx* h) {
   if (!ctl[C_ACTIVE]) return;
@@ -360,8 +359,9 @@ __global__ void __launch_bounds__(kOrthThreads) k_orth_step(int n, int nrhs, cpl
 // the convergence test.  A rotation is (a, b) -> (conj(c) a + s b, c b - s a)
 // with s real (h(j+1) is); only a <- c b - s a is a chain, two multiply-adds
 // per rotation in one warp, the products around it are formed by all threads.
-// One thread per system for the whole column, with the column in global
-// memory, took 21 us at j = 30, in registers 14; now 4.
+// One thread per system for the whole column in its own launch took 21 us at
+// 60 steps of 16 systems, inside this kernel from registers 18 with norm and
+// scaling; now 10.
 constexpr int kRotItems = 1024, kRotRhs = 128;
 __global__ void __launch_bounds__(256) k_finish_step(int n, int nrhs, int m, cplx* __restrict__ V,
                                                      const double* __restrict__ part, int npart, const cplx* __restrict__ h1,
@@ -496,7 +496,7 @@ __global__ void k_fnorm(int nrhs, const cplx* hn, double* fnorm) {
 // y = H^{-1} g per system (upper triangular, jdone columns).  A CTA per system:
 // with y_i known every thread takes its rows' product from g, so that the chain
 // is one complex product and two barriers per column (one thread per system for
-// the whole triangle: 266 us at 60 columns).  y holds g, then y.
+// the whole triangle: 266 us at 60 columns, now 38).  y holds g, then y.
 __global__ void __launch_bounds__(128) k_backsolve(int nrhs, int m, const cplx* __restrict__ Hm,
                                                    const cplx* __restrict__ gv, cplx* y, const int* ctl) {
   const int r = blockIdx.x, jd = ctl[C_JDONE];

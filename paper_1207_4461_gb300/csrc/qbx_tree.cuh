@@ -23,8 +23,9 @@
 // Per target of the 256-panel starfish (p = 12, k = 20, S, D and grad S, both
 // sides) this leaves about 4.4 panels of pairs of 256 (146k FP64 instructions
 // of 8.5M), 9 nodes taken centre by centre and 33 gathered into the block's
-// local expansion (150k).  The apply: 63.2 ms -> 3.2 ms; k = 20 + 1i at 128
-// panels 26.9 -> 3.4 ms; S and D at 32 panels, p = 8: 751 -> 391 us.
+// local expansion (150k), most of these for several blocks at once
+// (k_tree_super).  The apply: 63.2 ms -> 3.2 ms; k = 20 + 1i at 128 panels
+// 26.9 -> 3.4 ms; S and D at 32 panels, p = 8: 751 -> 336 us.
 // The pair route stays for fewer than kTreeMinPanels panels (nothing is far)
 // and for workspaces without room for the arrays below.
 #pragma once
