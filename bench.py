@@ -65,11 +65,11 @@ def flops_per_pair_ops(ops, p, nrhs=1):
         (nrhs - 1) * sum(acc[o] for o in ops)
 
 
-# DRAM bytes (read + write) of one launch of the fused S + D + grad S kernel
-# on the full-size starfish workload, from one ncu capture
+# DRAM bytes (read + write) of the launches between oversampling and finishing
+# of one S + D + grad S apply on the full-size starfish workload, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum); valid only for the kernel
 # sources it was taken with, identified by their hash.
-TRAFFIC = {"27706399748d3043": 1.667e6}   # profiles/k_apply_fused_S_D_gradS_starfish_M256_dram.md
+TRAFFIC = {"e7ce47d256b09565": 1.512e+07}   # profiles/apply_S_D_gradS_starfish_M256_clusters.md
 KERNEL_SOURCES = ["qbx_apply_impl.cuh", "qbx_device.cuh", "special_tables.h", "qbx_apply_real.cu", "qbx_tree.cu",
                   "qbx_tree.cuh"]
 GROUP_SOURCES = ["qbx_group_impl.cuh", "qbx_apply_impl.cuh", "qbx_device.cuh", "special_tables.h"]
@@ -78,17 +78,15 @@ GROUP_SOURCES = ["qbx_group_impl.cuh", "qbx_apply_impl.cuh", "qbx_device.cuh", "
 # launches between oversampling and finishing of one apply, divided by its
 # nominal (centre, source) pairs: near leaves pair by pair, distant sources by
 # their clusters' moments.  For the kernel sources with the given hash.
-HW_FP64_PER_PAIR = {"27706399748d3043": 434.9}         # fused S + D + grad S, p = 12, one rhs
-HW_FP64_PER_PAIR_GROUP = {"5b690bb633cedf23": 732.9}   # group kernel, S + D, p = 10, 32 rhs
+HW_FP64_PER_PAIR = {"e7ce47d256b09565": 17.02}         # S + D + grad S, p = 12, one rhs: the same profile
+HW_FP64_PER_PAIR_GROUP = {}   # batches: none taken with clusters
 # sm__pipe_fp64_cycles_active (of peak) over the active and the elapsed
-# cycles, from the same captures (fused: 128-panel starfish, one wave;
-# group: the first 4 curves of the batch)
-HW_FP64_PIPE = {"27706399748d3043": (0.922, 0.880)}
-HW_FP64_PIPE_GROUP = {"5b690bb633cedf23": (0.949, 0.926)}
-# the fused S + D + grad S apply at the complex wavenumber 20 + 1i (same
-# capture set-up: 128-panel starfish, p = 12, one rhs)
-HW_FP64_PER_PAIR_CPLX = {"27706399748d3043": 726.4}
-HW_FP64_PIPE_CPLX = {"27706399748d3043": (0.923, 0.878)}
+# cycles, from the same captures, weighted by the launches' times
+HW_FP64_PIPE = {"e7ce47d256b09565": (0.799, 0.723)}
+HW_FP64_PIPE_GROUP = {}
+# the same at the complex wavenumber 20 + 1i: none taken with clusters
+HW_FP64_PER_PAIR_CPLX = {}
+HW_FP64_PIPE_CPLX = {}
 
 
 def source_hash(names=KERNEL_SOURCES):
