@@ -114,14 +114,15 @@ int qbx_gauss_legendre(int q, double *nodes, double *weights);
  * uploads the per-panel interpolation matrix from the target to the source
  * nodes (Sec. 3.4.2), a device status word, and allocates `workspace_bytes`
  * of device workspace used by the split-source reductions (see
- * qbx_workspace_bytes), by the cluster arrays of calls on 16 panels or more
- * (distant sources by their moments; with a workspace that holds the partial
- * sums but not these arrays the call takes every pair instead, more slowly
- * and to the same accuracy), a side stream on which such a call's near pairs
- * run beside the rest (forked from and joined to the call's stream by events,
- * also under stream capture), and a 29 KB buffer for the H0/H1 amplitude table of
- * the ray z = k rho, which calls with a complex k fill (on their stream)
- * when k differs from the last one.  *plan receives the handle.  Host call,
+ * qbx_workspace_bytes) and by the cluster arrays of calls on 16 panels or more
+ * (with many right-hand sides 20 to 64): distant sources by their moments.
+ * With a workspace that holds the partial sums but not these arrays the call
+ * takes every pair instead, more slowly and to the same accuracy.  The plan
+ * also holds a side stream on which such a call's near pairs run beside the
+ * rest (forked from and joined to the call's stream by events, also under
+ * stream capture), and a 29 KB buffer for the H0/H1 amplitude table of the ray
+ * z = k rho, which calls with a complex k fill (on their stream) when k
+ * differs from the last one.  *plan receives the handle.  Host call,
  * synchronous. */
 int qbx_plan_create(qbx_plan **plan, int device, int q_tgt, int q_src, size_t workspace_bytes);
 int qbx_plan_destroy(qbx_plan *plan);

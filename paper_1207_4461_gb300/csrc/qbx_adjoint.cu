@@ -140,7 +140,10 @@ extern "C" int qbx_apply_adjoint(qbx_plan* plan, const qbx_geom* g, int op, int 
   // distant centres through cluster moments (S: value; D: gradient along n_s), few columns
   TreeArgs tr;
   const int fops = op == QBX_OP_S ? 1 << QBX_OP_S : 1 << QBX_OP_GRAD_S;
-  size_t b_tree = nrhs <= 8 ? adj_tree_setup(&tr, g, c0, nc, k, p, fops, op == QBX_OP_D ? 1 : 0, nrhs, nullptr, nullptr,
+  // (clusters: S at 24, 32 and 48 panels 304, 444 and 462 us, pair by pair 255,
+  // 441 and 762; five rhs at 48 and 64 813 and 935, pairs 765 and 1140)
+  const bool clusters = nrhs <= 8 && (double)nc * g->n_src >= 1.05e6 * (1.0 + 0.4 * (nrhs - 1));
+  size_t b_tree = clusters ? adj_tree_setup(&tr, g, c0, nc, k, p, fops, op == QBX_OP_D ? 1 : 0, nrhs, nullptr, nullptr,
                                              num_sms, nullptr)
                             : 0;
   if (ws_bytes < fixed + b_tree + 256 + 2 * per_split) b_tree = 0;

@@ -354,6 +354,11 @@ int prepare_tree(qbx_batch* b, size_t budget) {
   b->tree = false;
   for (GroupInst& in : b->h_inst) in.near = nullptr;
   if (b->ops == (QBX_OPS_S | QBX_OPS_D | QBX_OPS_GRAD_S)) return QBX_OK;
+  // (the clusters' chain of launches is repaid from about 2.3e6 pairs on: one
+  // curve of 48 panels, 32 rhs, S + D; up to 16 rhs from 1e6)
+  double pairs = 0.0;
+  for (const GroupInst& in : b->h_inst) pairs += (double)in.n_ctr * in.n_src;
+  if (pairs < (b->nrhs <= 16 ? 1.0e6 : 2.3e6)) return QBX_OK;
   const int none[3] = {0, 0, 0};
   std::vector<TreeArgs> v(b->n_inst);
   size_t total = 0;

@@ -822,7 +822,18 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   size_t tree_bytes = 0;
   int ns_far = 0;
   const bool far_group = group && ops != 7;   // many columns: far values formed once for all
-  if (g->M >= kTreeMinPanels) {
+  // Many columns: the clusters' chain of launches (0.5 ms at 16 panels and 16
+  // rhs, 1.3 ms at 48 and 32, one side) has to be repaid: S + D of 16 rhs at 24
+  // and 32 panels 594 and 731 us, pair by pair 547 and 829; of 32 rhs at 32 and
+  // 48 panels 1086 and 1322, pairs 833 and 1760; D - i eta S of 8 rhs at 16 and
+  // 24 panels 606 and 689, pairs 439 and 767, of 32 rhs at 24 and 32 881 and
+  // 991, pairs 771 and 1220; S + D + grad S (no far values for all columns at once) of 16 rhs at 32 and
+  // 48 panels 1979 and 2406, pairs 1406 and 3056, of 32 rhs at 64 5039 and 5241.
+  double tree_pairs = 0.0;
+  if (cf) tree_pairs = nrhs <= 8 ? 1.15e6 : 2.0e6;
+  else if (group && ops == 7) tree_pairs = 1.25e5 * nrhs;
+  else if (group) tree_pairs = nrhs > 16 ? 2.3e6 : nc > g->n_tgt ? 0.8e6 : 1.0e6;
+  if (g->M >= kTreeMinPanels && (double)nc * g->n_src >= tree_pairs) {
     tr.kre = k.re;
     tr.kim = k.im;
     tr.p = pp;
@@ -841,6 +852,13 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     }
     tree_columns(&tr, slot_of);
     tree_levels(g->M, g->q_src, &tr);
+    // A level of k_tree_up takes 120 us however small; up to about 128 leaves of
+    // 64 columns summing the sources again at every level costs less (and one
+    // launch), where the workspace holds the leaf contributions
+    if (far_group && (long)tr.M * tr.nset * nrhs <= 8192) {
+      tr.up = 0;
+      if (avail < tree_layout(&tr, nullptr) + 5 * per_split) tr.up = 1;
+    }
     tree_bytes = tree_layout(&tr, nullptr);
     if (far_group) {
       ns_far = std::max(1, std::min(4, (p->num_sms * 3 + units - 1) / units));
@@ -860,7 +878,10 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   if (!tree) tree_bytes = 0;
   // (with clusters a block's near leaves are some six panels; down to two dozen sources a CTA)
   const int ns_near =
-      host_choose_split_waves(p->num_sms, occ, units, tree ? std::min(g->n_src, (group ? 8 : 16) * g->q_src) : g->n_src,
+      host_choose_split_waves(p->num_sms, occ, units,
+                              tree ? std::min(g->n_src, (group ? 8 : 16) * g->q_src)
+                                   : (group && nsd == 2 ? 2 : 1) * g->n_src,   // both sides in one item: half as long
+                              // (20 panels, S + D of 32 rhs, both sides 780 -> 583 us)
                               per_split, avail - tree_bytes - ns_far * per_split, waves);
   if (ns_near < 1) return fail(QBX_ENOMEM, "workspace too small for the apply partial sums");
   const int ns = ns_near + ns_far;
