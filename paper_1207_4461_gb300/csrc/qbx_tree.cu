@@ -661,6 +661,16 @@ __device__ __forceinline__ void rotate_in(const cplx A, const cplx B, double cl,
   }
 }
 
+// Whether a node of radius R (kr = |k| R) gets moments: it may be in a list (at
+// no distance do kTreeP orders do beyond |k| R = 7.23), or, moments carried
+// upward, its parent's come from it.  A node's points lie in the disc of every
+// node above it, but its own radius is about the centre of its bounding box and
+// up to (1 + sqrt 2)/2 = 1.207 times that disc's (half a circle: 1.118 circles).
+__device__ __forceinline__ bool has_moments(const TreeArgs& a, float kr) {
+  if (a.up) kr *= 0.8f;
+  return kr < 64.0f && series_order(kr, 1e4f * kr + 1e4f, 1e-4f, 1.0f, 0, kTreeP) <= kTreeP;
+}
+
 // whether k_tree_moments has room for the dipoles' columns (complex k: up to 99 sources a leaf)
 template <typename T>
 __host__ __device__ constexpr bool dipole_rows(int q) {
@@ -693,8 +703,7 @@ __global__ void __launch_bounds__(128) k_tree_moments(TreeArgs b) {
   KW<T> kw;
   kw.init(a.kre, a.kim, a.hk_tab);
   const T kk = kw.kval();
-  const float kr = (float)sc_abs(kk) * (float)n[2];   // orders at any distance beyond kTreeP: in no list
-  if (!(kr < 64.0f) || series_order(kr, 1e4f * kr + 1e4f, 1e-4f, 1.0f, 0, kTreeP) > kTreeP) return;
+  if (!has_moments(a, (float)sc_abs(kk) * (float)n[2])) return;
   for (int i = threadIdx.x; i < q; i += 128) {
     const double dx = a.sx[panel * q + i] - zx, dy = a.sy[panel * q + i] - zy;
     const double rho = sqrt(dx * dx + dy * dy);
@@ -829,8 +838,7 @@ __global__ void __launch_bounds__(32) k_tree_disc_moments(TreeArgs a) {
   KW<T> kw;
   kw.init(a.kre, a.kim, a.hk_tab);
   const T kk = kw.kval();
-  const float kr = (float)sc_abs(kk) * (float)n[2];   // orders at any distance beyond kTreeP: in no list
-  if (!(kr < 64.0f) || series_order(kr, 1e4f * kr + 1e4f, 1e-4f, 1.0f, 0, kTreeP) > kTreeP) return;
+  if (!has_moments(a, (float)sc_abs(kk) * (float)n[2])) return;
   const int nside = a.n_ctr_n / a.n_src, nc = a.q_src * nside, ncol = a.nset * a.nrhs;
   cplx* out = reinterpret_cast<cplx*>(a.mom) + (size_t)(l * a.M + leaf) * ncol * (P + 2) * 2;
   for (int c0 = 0; c0 < nc; c0 += 32) {
@@ -907,8 +915,7 @@ __global__ void __launch_bounds__(32 * kUpWarps) k_tree_up(TreeArgs q, int l) {
   kw.init(a.kre, a.kim, a.hk_tab);
   const T kk = kw.kval();
   const double* z = a.node + 4 * (size_t)id;
-  const float kr = (float)sc_abs(kk) * (float)z[2];
-  if (!(kr < 64.0f) || series_order(kr, 1e4f * kr + 1e4f, 1e-4f, 1.0f, 0, kTreeP) > kTreeP) return;   // in no list
+  if (!has_moments(a, (float)sc_abs(kk) * (float)z[2])) return;
   if (warp < nch && lane == 0) {
     const double* y = a.node + 4 * (size_t)(c0 + warp);
     const double vx = z[0] - y[0], vy = z[1] - y[1];

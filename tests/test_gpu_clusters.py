@@ -416,3 +416,43 @@ def test_hankel_ray_at_strong_damping(cuda, k):
     for n, h in ((0, h0), (1, h1)):
         ref = sp.hankel1e(n, z) * np.exp(1j * z)
         assert np.all(np.abs(h.cpu().numpy() - ref) <= 8e-14 * np.abs(ref)), n
+
+
+class Circles:
+    """n unit circles in a row, 3 apart, one after another in the parameter."""
+
+    def __init__(self, n):
+        self.n = n
+
+    def __call__(self, t):
+        j = np.minimum(np.floor(t / (2 * np.pi)), self.n - 1)
+        c, s = np.cos(t), np.sin(t)
+        return np.stack([3.0 * j + c, s], -1), np.stack([-s, c], -1)
+
+    def edges(self, M):
+        return np.linspace(0.0, 2 * np.pi * self.n, M + 1)
+
+
+def test_parent_node_smaller_than_its_children(cuda):
+    """Circles of 8 panels, two sides, 16 columns: at k = 6.5 the node of a
+    circle (k R = 6.5) is in the lists of distant blocks, the nodes of its
+    halves, whose radius about the centre of their bounding box is 1.118, are
+    beyond every list's limit (7.23).  A first call leaves NaN in every row."""
+    M, nrhs, p, ops = 256, 16, 10, (0, 1)
+    assert 2 * M * len(ops) * nrhs > 8192   # moments carried upward
+    cur = Circles(32)
+    plan = qbx.Plan(16, 64, n_src=M * 64, n_ctr=2 * M * 16, ncoef=4, nrhs=nrhs)
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(3, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    qbx.qbx_apply_ops(plan, g, ops, qbx.SIDE_TWO, 0, 1.0, p, torch.full_like(d, float("nan")))
+    with pytest.raises(qbx.QBXError):
+        qbx.qbx_sync_status(plan)
+    got = qbx.qbx_apply_ops(plan, g, ops, qbx.SIDE_TWO, 0, 6.5, p, d)
+    qbx.qbx_sync_status(plan)
+    ref = qbx.qbx_apply_ops(pair_plan(g, 16, 64, nrhs, 2), g, ops, qbx.SIDE_TWO, 0, 6.5, p, d)
+    b = qbx.Batch(plan, [g], [6.5], p, ops, qbx.SIDE_TWO, 0, [d])
+    out = b.apply()[0]
+    b.status()
+    for o in ops:
+        check(got[o], ref[o], ("apply", o))
+        check(out[o], ref[o], ("batch", o))
