@@ -484,6 +484,7 @@ int qbx_form_locals(qbx_plan* p, const qbx_geom* g, int kind, int side, qbx_c64 
     tr.kre = k.re;
     tr.kim = k.im;
     tr.p = tr.pl = pp;
+    tr.all_l = 1;
     tr.nd = kind == QBX_OP_D ? 1 : 0;
     tr.n_tgt = g->n_tgt;
     tr.n_ctr = nc;

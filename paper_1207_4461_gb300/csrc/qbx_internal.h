@@ -288,6 +288,7 @@ struct TreeArgs {
   int nd;                     // derivatives taken on one side of a kernel (D, grad S: 1)
   double eta;                 // near-only QBX (> 0)
   int only_loc;               // lists: leaves that do not go through the block's local expansion are near
+  int all_l;                  // stored coefficients: far nodes are evaluated for every order l <= p
   int M, q_src, n_src;        // leaves (halves of panels, or panels), sources per leaf, sources
   const double *sx, *sy, *snx, *sny;
   // adjoint sweeps: the nodes hold the discs of n_ctr_n centres (dcx, dcy) of

@@ -323,7 +323,8 @@ __global__ void __launch_bounds__(32 * kListWarps) k_tree_lists(TreeArgs q) {
       ol = min(ol, a.p);
     }
     // H of order om + ol and the moments of order om stay in FP64's range
-    const float no = (float)(om + max(ol, oq));
+    // (stored coefficients: a node taken directly goes into every order l <= p)
+    const float no = (float)(om + (a.all_l && !oq ? a.p : max(ol, oq)));
     if (!(no * log10f(fmaxf(2.0f * no / (2.7f * ka * dm), 1.0f)) < 280.0f) ||
         !((float)om * log10f(fmaxf(2.0f * om / (2.7f * ka * R), 1.0f)) < 280.0f))
       return 0;

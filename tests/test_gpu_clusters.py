@@ -456,3 +456,19 @@ def test_parent_node_smaller_than_its_children(cuda):
     for o in ops:
         check(got[o], ref[o], ("apply", o))
         check(out[o], ref[o], ("batch", o))
+
+
+@pytest.mark.parametrize("M,k,p,kind", [(40, 1e-3, 40, 0), (40, 1e-4, 24, 1), (40, 3e-4, 30, 0), (40, 1e-4, 30, 0),
+                                        (130, 1e-3, 40, 1), (40, 1e-3 + 1e-3j, 40, 0)])
+def test_locals_at_low_frequency_stay_finite(cuda, M, k, p, kind):
+    """Every order l <= p from distant nodes, whose waves H_{om + l} reach 1e344
+    where H_p of the pairs stays below 1e270."""
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(16, 64, n_src=M * 64, n_ctr=M * 16, ncoef=2 * p + 1, nrhs=1)
+    g = geometry(plan, cur, cur.edges(M))
+    w = torch.as_tensor(W.complex_gaussian(M + p, g.n_src).reshape(g.n_src, 1), device="cuda")
+    pp = qbx.Plan(16, 64, workspace_bytes=g.n_tgt * (2 * p + 1) * 16 * 2 + 1024)
+    got, ref = (qbx.qbx_form_locals(pl, g, kind, qbx.SIDE_INT, k, p, w) for pl in (plan, pp))
+    qbx.qbx_sync_status(plan)
+    for l in range(2 * p + 1):
+        check(got[:, l], ref[:, l], (M, p, l - p))
