@@ -397,7 +397,11 @@ __global__ void __launch_bounds__(kFormThreads) k_form(FormArgs a) {
     v0 = (int)(n * blockIdx.y / a.nsplit);
     v1 = (int)(n * (blockIdx.y + 1) / a.nsplit);
   }
-  const double2* wd = reinterpret_cast<const double2*>(a.wd) + a.rhs0;
+  const cplx* wd = reinterpret_cast<const cplx*>(a.wd) + a.rhs0;   // the caller's: 8-byte aligned
+  auto weight = [&](int s, int rr) {
+    const cplx* w = wd + (size_t)s * a.nrhs + rr;
+    return cplx{__ldg(&w->re), __ldg(&w->im)};
+  };
   for (int v = v0 + warp; v < v1; v += kFormThreads / 32) {
     int s = v;
     if (near) {
@@ -411,8 +415,7 @@ __global__ void __launch_bounds__(kFormThreads) k_form(FormArgs a) {
     cplx Hm, H;   // H_{n-1}, H_n
     T twoz;
     if constexpr (ONE) {
-      const double2 w = __ldg(wd + (size_t)s * a.nrhs);
-      kw.hankel_w(rho, inv, yq, cplx{w.x, w.y}, Hm, H, twoz);
+      kw.hankel_w(rho, inv, yq, weight(s, 0), Hm, H, twoz);
     } else {
       kw.hankel(rho, inv, yq, Hm, H, twoz);
     }
@@ -423,9 +426,8 @@ __global__ void __launch_bounds__(kFormThreads) k_form(FormArgs a) {
         if constexpr (ONE) {
           *A = *A + v_;
         } else {
-          const double2 w = __ldg(wd + (size_t)s * a.nrhs + rr);
           cplx u = *A;
-          cfma(u, cplx{w.x, w.y}, v_);
+          cfma(u, weight(s, rr), v_);
           *A = u;
         }
       }

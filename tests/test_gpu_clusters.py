@@ -472,3 +472,26 @@ def test_locals_at_low_frequency_stay_finite(cuda, M, k, p, kind):
     qbx.qbx_sync_status(plan)
     for l in range(2 * p + 1):
         check(got[:, l], ref[:, l], (M, p, l - p))
+
+
+@pytest.mark.parametrize("M", [8, 40])
+@pytest.mark.parametrize("nrhs", [1, 3])
+def test_weighted_density_at_an_odd_8_byte_address(cuda, M, nrhs):
+    """qbx_c64 asks for the alignment of a double only: the same bits from an
+    array 8 bytes off, pair by pair and through clusters."""
+    k, p = 6.0, 9
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(16, 64, n_src=M * 64, n_ctr=2 * M * 16, ncoef=2 * p + 1, nrhs=nrhs)
+    g = geometry(plan, cur, cur.edges(M))
+    w = torch.as_tensor(W.complex_gaussian(M, g.n_src * nrhs).reshape(g.n_src, nrhs), device="cuda")
+    flat = torch.zeros(2 * g.n_src * nrhs + 1, dtype=torch.float64, device="cuda")
+    flat[1:] = torch.view_as_real(w).reshape(-1)
+    ptr = flat.data_ptr() + 8
+    assert ptr % 16 == 8
+    for kind in (qbx.OP_S, qbx.OP_D):
+        ref = qbx.qbx_form_locals(plan, g, kind, qbx.SIDE_INT, k, p, w)
+        out = torch.empty_like(ref)
+        stream = torch.cuda.current_stream().cuda_stream
+        assert qbx.lib().qbx_form_locals(plan.handle, g.ref(), kind, qbx.SIDE_INT, qbx.c64(k, 0.0), p, ptr, nrhs,
+                                         out.data_ptr(), stream) == 0
+        assert torch.equal(out, ref)
