@@ -120,9 +120,9 @@ int qbx_gauss_legendre(int q, double *nodes, double *weights);
  * takes every pair instead, more slowly and to the same accuracy.  The plan
  * also holds a side stream on which such a call's near pairs run beside the
  * rest (forked from and joined to the call's stream by events, also under
- * stream capture), and a 29 KB buffer for the H0/H1 amplitude table of the ray
- * z = k rho, which calls with a complex k fill (on their stream) when k
- * differs from the last one.  *plan receives the handle.  Host call,
+ * stream capture), and two 29 KB tables of H0/H1 amplitudes along the ray
+ * z = k rho: one that calls with a complex k fill (on their stream) when k
+ * differs from the last one, and one that captured calls fill in their graph.  *plan receives the handle.  Host call,
  * synchronous. */
 int qbx_plan_create(qbx_plan **plan, int device, int q_tgt, int q_src, size_t workspace_bytes);
 int qbx_plan_destroy(qbx_plan *plan);

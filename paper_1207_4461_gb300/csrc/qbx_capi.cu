@@ -30,8 +30,8 @@ struct qbx_plan {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // waves of resident CTAs the split choice aims for (qbx_plan_set_min_waves)
   int min_waves = 1;
-  // H0/H1 amplitude table of the ray z = k rho for the last complex k
-  // (tab_kim = 0: none made yet)
+  // H0/H1 amplitude tables of the ray z = k rho: first that of the last complex
+  // k (tab_kim = 0: none made yet), then the one that captured calls fill
   double* d_hk_tab;
   double tab_kre, tab_kim;
   // the pair sums run here, beside the cluster moments on the caller's stream
@@ -233,9 +233,20 @@ void host_plan_info(const qbx_plan* plan, int* device, int* q_tgt, int* q_src, c
 
 // The plan's amplitude table for complex k (made on `st` when k changes;
 // later calls on the plan's streams see it in stream order), or null for real k.
+// A captured call makes its own in a second table, as a part of its graph (56
+// us of each replay): which k the first one holds when the graph is replayed
+// is not known, nor does a captured fill run before the replay.
 const double* host_plan_hk_table(qbx_plan* plan, qbx_c64 k, cudaStream_t st, cudaError_t* err) {
   *err = cudaSuccess;
   if (k.im == 0.0) return nullptr;
+  cudaStreamCaptureStatus capture;
+  *err = cudaStreamIsCapturing(st, &capture);
+  if (*err != cudaSuccess) return nullptr;
+  if (capture != cudaStreamCaptureStatusNone) {
+    double* tab = plan->d_hk_tab + hk_table_doubles();
+    *err = launch_hk_table(k.re, k.im, tab, st);
+    return *err == cudaSuccess ? tab : nullptr;
+  }
   if (plan->tab_kre != k.re || plan->tab_kim != k.im) {
     *err = launch_hk_table(k.re, k.im, plan->d_hk_tab, st);
     if (*err != cudaSuccess) return nullptr;
@@ -339,7 +350,7 @@ int qbx_plan_create(qbx_plan** plan, int device, int q_tgt, int q_src, size_t wo
   if (e == cudaSuccess) e = cudaMalloc(&p->d_wgl_src, q_src * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_status, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_diff, Dx.size() * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&p->d_hk_tab, (size_t)hk_table_doubles() * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&p->d_hk_tab, 2 * (size_t)hk_table_doubles() * sizeof(double));
   if (e == cudaSuccess && workspace_bytes > 0) e = cudaMalloc(&p->ws, workspace_bytes);
   if (e == cudaSuccess) e = cudaMemcpy(p->d_diff, Dx.data(), Dx.size() * sizeof(double), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(p->d_interp, Mx.data(), Mx.size() * sizeof(double), cudaMemcpyHostToDevice);

@@ -257,8 +257,8 @@ void host_plan_side(const qbx_plan* plan, cudaStream_t* side, cudaEvent_t* fork,
 void host_plan_workspace(const qbx_plan* plan, void** ws, size_t* bytes, int* num_sms, int** status);
 cudaError_t adjoint_sums(AdjArgs& a, TreeArgs* tr, qbx_plan* plan, const qbx_geom* g, int c0, int nc, qbx_c64 k,
                          int fops, int nd, int mode, int num_sms, char* tree_base, cudaStream_t st);
-// The plan's amplitude table for complex k (made on st when k changes), or
-// null for real k.
+// The plan's amplitude table for complex k (made on st when k changes, or in
+// every captured call), or null for real k.
 const double* host_plan_hk_table(qbx_plan* plan, qbx_c64 k, cudaStream_t st, cudaError_t* err);
 
 }  // namespace qbx

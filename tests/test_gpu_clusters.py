@@ -495,3 +495,41 @@ def test_weighted_density_at_an_odd_8_byte_address(cuda, M, nrhs):
         assert qbx.lib().qbx_form_locals(plan.handle, g.ref(), kind, qbx.SIDE_INT, qbx.c64(k, 0.0), p, ptr, nrhs,
                                          out.data_ptr(), stream) == 0
         assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("call", ["apply", "locals", "grad_d_stored"])
+def test_captured_calls_at_complex_k_keep_their_k(cuda, call):
+    """A graph replayed after a call at another k, and calls at that k after the
+    replay, on one plan: each takes the amplitudes of its own k."""
+    M, p, k1, k2 = 24, 8, 5 + 0.5j, 9 + 0.3j
+    nrhs = 4 if call == "grad_d_stored" else 1
+    plan = qbx.Plan(16, 64, n_src=M * 64, n_ctr=2 * M * 16, ncoef=2 * p + 1, nrhs=nrhs)
+    cur = W.starfish(0.2, 3)
+    g = geometry(plan, cur, cur.edges(M))
+    n = g.n_src if call == "locals" else g.n_tgt
+    d = torch.as_tensor(W.complex_gaussian(4, n * nrhs).reshape(n, nrhs), device="cuda")
+
+    def run(k):
+        if call == "locals":
+            return qbx.qbx_form_locals(plan, g, qbx.OP_D, qbx.SIDE_INT, k, p, d)
+        return qbx.qbx_apply(plan, g, qbx.OP_S if call == "apply" else qbx.OP_GRAD_D, qbx.SIDE_INT, 0, k, p, d)
+
+    r2, r1 = run(k2).clone(), run(k1).clone()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = run(k1)
+    assert torch.equal(run(k1), r1)   # (the captured table fill has not run yet)
+    assert torch.equal(run(k2), r2)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, r1)
+    assert torch.equal(run(k2), r2)
+    fresh = torch.cuda.CUDAGraph()
+    k3 = 4 + 1j
+    with torch.cuda.graph(fresh):
+        out3 = run(k3)
+    now = run(k3)   # (a new k, captured before it was ever made)
+    fresh.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out3, now) and torch.isfinite(torch.view_as_real(now)).all()
