@@ -148,7 +148,9 @@ int qbx_plan_set_min_waves(qbx_plan *plan, int waves);
 /* Workspace a call needs: for qbx_apply / qbx_far / qbx_form_locals with the
  * given sizes.  n_ctr = number of centres (or far targets) processed, ncoef =
  * coefficients per centre (1 for S/D values, 2 for grad S, 2p+1 for
- * form_locals).  Host, pure function. */
+ * form_locals).  It holds the cluster arrays too (up to 8 GB of them); for
+ * panels of fewer than 16 source nodes pass n_src as 16 per panel.  Host, pure
+ * function. */
 size_t qbx_workspace_bytes(int n_src, int n_ctr, int ncoef, int nrhs);
 
 /* Read (and clear) the plan's device status word: QBX_OK or QBX_ENONFINITE.
@@ -526,6 +528,11 @@ int qbx_apply_static_status(void *stream);
  * Im z == 0), and J_0..J_nmax (Miller) at z[n].  For tests. */
 int qbx_debug_hankel01(const qbx_c64 *z, int n, qbx_c64 *h0, qbx_c64 *h1, void *stream);
 int qbx_debug_besselj(const qbx_c64 *z, int n, int nmax, qbx_c64 *j, void *stream);
+/* Route of the plan's last apply, grad D, stored coefficients or adjoint:
+ * clusters = 1 if distant sources went through moments (0: every pair),
+ * upward = 1 if these were carried up level by level, super_blocks = how many
+ * super-blocks were formed.  Host.  For tests. */
+int qbx_debug_route(const qbx_plan *plan, int *clusters, int *upward, int *super_blocks);
 /* H0, H1 at z = k rho[i] (rho > 0, n values) as the pair kernels evaluate
  * them for this k: for Im k > 0 through the plan's amplitude table of the ray
  * z = k rho (fitted once per k) where |z| >= 2, the direct evaluation

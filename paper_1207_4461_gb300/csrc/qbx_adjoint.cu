@@ -147,6 +147,7 @@ extern "C" int qbx_apply_adjoint(qbx_plan* plan, const qbx_geom* g, int op, int 
                                              num_sms, nullptr)
                             : 0;
   if (ws_bytes < fixed + b_tree + 256 + 2 * per_split) b_tree = 0;
+  host_plan_route(plan, b_tree ? &tr : nullptr);
   const int tiles = (g->n_src + kGrpCentres - 1) / kGrpCentres;
   int ns = std::max(1, (num_sms * 6 + tiles - 1) / tiles);
   ns = std::min(ns, std::max(1, (b_tree ? std::min(nc, 12 * q_tgt * nsides) : nc) / kGrpTile));

@@ -38,6 +38,7 @@ struct qbx_plan {
   // (forked from it and joined to it by events within every call)
   cudaStream_t side;
   cudaEvent_t fork, join;
+  int route[3];   // of the last call (qbx_debug_route): clusters, carried upward, super-blocks
 };
 
 namespace {
@@ -223,6 +224,12 @@ void host_plan_side(const qbx_plan* plan, cudaStream_t* side, cudaEvent_t* fork,
   *join = plan->join;
 }
 
+void host_plan_route(qbx_plan* plan, const TreeArgs* t) {
+  plan->route[0] = t != nullptr;
+  plan->route[1] = t ? t->up : 0;
+  plan->route[2] = t ? t->n_sup : 0;
+}
+
 void host_plan_info(const qbx_plan* plan, int* device, int* q_tgt, int* q_src, const double** interp) {
   *device = plan->device;
   *q_tgt = plan->q_tgt;
@@ -321,10 +328,31 @@ int qbx_gauss_legendre(int q, double* nodes, double* weights) {
   return QBX_OK;
 }
 
+// Densities, 64 splits' partial sums, and a bound of the cluster arrays
+// (tree_layout) of any call with these sizes: leaves hold 16 sources or more
+// (panels of fewer source nodes: see qbx.h), a curve has no more targets than
+// sources; ncoef 1 to 4 are S or D; S + D or a gradient; one of them and grad
+// S; all three, each of its own density at worst; more: stored coefficients,
+// clusters for up to 8 rhs.  The lists grow with blocks times leaves (25 bytes
+// each: 0.4 GB at 4096 panels of 16/64 nodes), so the bound ends at 8 GB, from
+// where on a call that needs more takes every pair.
 size_t qbx_workspace_bytes(int n_src, int n_ctr, int ncoef, int nrhs) {
   if (n_src < 0 || n_ctr < 0 || ncoef < 0 || nrhs < 0) return 0;
-  return 3 * align256((size_t)n_src * nrhs * 16) +
-         align256((size_t)kMaxSplit * n_ctr * ncoef * nrhs * 16) + 512;
+  const size_t pairs = 3 * align256((size_t)n_src * nrhs * 16) +
+                       align256((size_t)kMaxSplit * n_ctr * ncoef * nrhs * 16) + 512;
+  if (ncoef > 4 && nrhs > 8) return pairs;
+  const size_t leaves = (size_t)n_src / 16 + 1, blocks = (size_t)std::min(n_src, n_ctr) / 32 + 2;
+  size_t levels = 1;
+  while (levels < (size_t)kTreeLevels && (leaves >> levels) >= 8) ++levels;
+  const size_t entries = 2 * leaves + levels + 2 * blocks + kSupLevels;   // nodes, blocks, super-blocks
+  const size_t nset = ncoef == 4 ? 3 : ncoef == 2 || ncoef == 3 ? 2 : 1;
+  const size_t ncset = ncoef >= 2 && ncoef <= 4 ? (size_t)ncoef + 1 : 1;
+  size_t leaf_cols = leaves * nset * nrhs;
+  if (ncoef == 1 && nrhs >= 16) leaf_cols = std::min<size_t>(leaf_cols, kTreeUpCols);
+  const size_t order_bytes = (size_t)(kTreeP + 2) * 2 * 16;
+  const size_t clusters = entries * (32 + ncset * nrhs * order_bytes) + levels * leaf_cols * order_bytes +
+                          blocks * (25 * leaves + 64) + (size_t)8 * 1024;
+  return pairs + std::min(align256(clusters), (size_t)8 << 30);
 }
 
 int qbx_plan_create(qbx_plan** plan, int device, int q_tgt, int q_src, size_t workspace_bytes) {
@@ -511,6 +539,7 @@ int qbx_form_locals(qbx_plan* p, const qbx_geom* g, int kind, int side, qbx_c64 
     if (!form_far_fit(tr) || avail < tree_bytes + (size_t)(ns_far + 1) * per_split) ns_far = 0;
   }
   const bool tree = ns_far > 0;
+  host_plan_route(p, tree ? &tr : nullptr);
   if (!tree) tree_bytes = 0;
   const int ns_near = choose_split(p, tree ? units / 2 + 1 : units, tree ? std::min(g->n_src, 16 * g->q_src) : g->n_src,
                                    per_split, avail - tree_bytes - ns_far * per_split);
@@ -867,7 +896,7 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     // A level of k_tree_up takes 120 us however small; up to about 128 leaves of
     // 64 columns summing the sources again at every level costs less (and one
     // launch), where the workspace holds the leaf contributions
-    if (far_group && (long)tr.M * tr.nset * nrhs <= 8192) {
+    if (far_group && (long)tr.M * tr.nset * nrhs <= kTreeUpCols) {
       tr.up = 0;
       if (avail < tree_layout(&tr, nullptr) + 5 * per_split) tr.up = 1;
     }
@@ -887,6 +916,7 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
       ns_far = 0;
   }
   const bool tree = ns_far > 0;
+  host_plan_route(p, tree ? &tr : nullptr);
   if (!tree) tree_bytes = 0;
   // (with clusters a block's near leaves are some six panels; down to two dozen sources a CTA)
   const int ns_near =
@@ -1117,6 +1147,7 @@ static int grad_d_impl(qbx_plan* p, const qbx_geom* g, int side, int limit, qbx_
       if (!far_clusters_fit(tr) || p->ws_bytes < fixed + tree_bytes + (size_t)(ns_far + 1) * per_split) ns_far = 0;
     }
     const bool tree = ns_far > 0;
+    host_plan_route(p, tree ? &tr : nullptr);
     if (!tree) tree_bytes = 0;
     const int ns_near = host_choose_split_waves(
         p->num_sms, occ, units, tree ? std::min(g->n_src, 16 * g->q_src) : g->n_src, per_split,
@@ -1324,6 +1355,14 @@ int qbx_assign_centres(qbx_plan* p, const qbx_geom* g, int side, int n, const do
   CK(cudaSetDevice(p->device), "cudaSetDevice");
   CK(launch_assign(n, xy, nc, g->ctr_x + c0, g->ctr_y + c0, g->ctr_r + c0, out, (cudaStream_t)stream),
      "assign kernel");
+  return QBX_OK;
+}
+
+int qbx_debug_route(const qbx_plan* p, int* clusters, int* upward, int* super_blocks) {
+  if (!p || !clusters || !upward || !super_blocks) return fail(QBX_EINVAL, "NULL argument");
+  *clusters = p->route[0];
+  *upward = p->route[1];
+  *super_blocks = p->route[2];
   return QBX_OK;
 }
 

@@ -254,6 +254,8 @@ cudaError_t launch_adjoint_real(const AdjArgs& a, cudaStream_t st);
 cudaError_t launch_adjoint_cplx(const AdjArgs& a, cudaStream_t st);
 // the plan's side stream and the events that fork it from and join it to a call's stream
 void host_plan_side(const qbx_plan* plan, cudaStream_t* side, cudaEvent_t* fork, cudaEvent_t* join);
+// what qbx_debug_route reports of the call (t: its clusters, or null)
+void host_plan_route(qbx_plan* plan, const TreeArgs* t);
 void host_plan_workspace(const qbx_plan* plan, void** ws, size_t* bytes, int* num_sms, int** status);
 cudaError_t adjoint_sums(AdjArgs& a, TreeArgs* tr, qbx_plan* plan, const qbx_geom* g, int c0, int nc, qbx_c64 k,
                          int fops, int nd, int mode, int num_sms, char* tree_base, cudaStream_t st);
@@ -274,6 +276,7 @@ constexpr int kTreeP = 30;
 constexpr int kTreeLocal = 32;    // near-only QBX: orders of a centre's expansion that stands for the smooth rule
 constexpr int kTreeMinPanels = 16;   // fewer panels: every source pair by pair (no cluster of 8 is far from any block)
 constexpr int kTreeLevels = 16;
+constexpr int kTreeUpCols = 8192;   // leaf columns up to which every level sums the sources again (TreeArgs::up = 0)
 constexpr int kTreeSets = 4;
 constexpr int kSupLevels = 7;
 // what a moment set is made of: the density itself, or dipoles along n_s, x, y

@@ -619,6 +619,7 @@ static int shape_impl(int op, qbx_plan* plan, const qbx_geom* g, int side, qbx_c
     if (!b_ta || ws_bytes < L0.total + 512 + b_tf + b_ta + (size_t)(ns_far + 2) * per_fwd + 2 * per_adj) b_tf = b_ta = 0;
   }
   const bool tree = b_tf > 0;
+  host_plan_route(plan, tree ? &tf : nullptr);
   if (!tree) ns_far = 0;
   const size_t avail = ws_bytes - L0.total - 512 - b_tf - b_ta - (tree ? (size_t)ns_far * per_fwd + per_adj : 0);
   const int occ = opD ? 3

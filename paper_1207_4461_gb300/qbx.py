@@ -131,6 +131,8 @@ def lib():
             L.qbx_matmul_cm_work_bytes.restype = ctypes.c_size_t
             L.qbx_apply_static_status.argtypes = [_P]
             L.qbx_apply_static_status.restype = I
+            L.qbx_debug_route.argtypes = [_P, ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(I)]
+            L.qbx_debug_route.restype = I
             L.qbx_vec_dots.argtypes = [I, I, I, _P, _P, _P, _P, _P]
             L.qbx_vec_dots.restype = I
             L.qbx_vec_dots_work_bytes.argtypes = [I, I]
@@ -718,6 +720,13 @@ def qbx_assign_centres(plan: Plan, g: Geometry, side, xy):
     _check(lib().qbx_assign_centres(plan.handle, g.ref(), side, xy.shape[0], _ptr(xy.contiguous()),
                                     _ptr(out), _stream()))
     return out
+
+
+def qbx_debug_route(plan: Plan):
+    """(clusters, carried upward, super-blocks) of the plan's last call."""
+    v = [ctypes.c_int(0) for _ in range(3)]
+    _check(lib().qbx_debug_route(plan.handle, *[ctypes.byref(x) for x in v]))
+    return tuple(x.value for x in v)
 
 
 def qbx_debug_hankel01(z):

@@ -76,3 +76,33 @@ def test_shape_adjoint_workspace_bytes():
     assert qbx.qbx_shape_adjoint_workspace_bytes(M, 16, 64, p, 2) > b
     assert qbx.qbx_shape_adjoint_workspace_bytes(0, 16, 64, p, 1) == 0
     assert qbx.qbx_shape_adjoint_workspace_bytes(M, 16, 64, -1, 1) == 0
+
+
+def test_workspace_bytes_hold_the_cluster_arrays():
+    """Beside 64 splits: node entries, coefficients (1 KB per node, column set
+    and rhs), leaf contributions (1 KB per leaf, level, set and rhs) and lists
+    (20 bytes per block and leaf), for one side and for two; the bound of these
+    arrays ends at 8 GB."""
+    for q_tgt, q_src in ((16, 64), (8, 32), (12, 40), (16, 16)):
+        for M in (16, 100, 256, 1024, 4096):
+            for sides in (1, 2):
+                for ncoef, nset, ncset in ((1, 1, 1), (2, 2, 2), (2, 1, 3), (3, 2, 4), (4, 3, 5)):
+                    for nrhs in (1, 3):
+                        n_src, n_ctr = M * q_src, sides * M * q_tgt
+                        leaves = M * (2 if q_src >= 32 and q_src % 2 == 0 else 1)
+                        blocks = (M * q_tgt + 31) // 32
+                        lev, nodes = 0, 0
+                        while lev == 0 or leaves >> lev >= 8:
+                            nodes += (leaves + (1 << lev) - 1) >> lev
+                            lev += 1
+                        supers = blocks + 7 if blocks >= 64 else 0
+                        entries = nodes + blocks + supers
+                        need = (entries * (32 + ncset * nrhs * 1024) + lev * leaves * nset * nrhs * 1024
+                                + 20 * blocks * leaves + 20 * blocks + 5 * supers * leaves + 24 * supers + 10 * 256)
+                        pairs = 3 * n_src * nrhs * 16 + 64 * n_ctr * ncoef * nrhs * 16
+                        b = qbx.qbx_workspace_bytes(n_src, n_ctr, ncoef, nrhs)
+                        assert pairs + need <= b < pairs + 4096 + 8 * 2**30, (q_tgt, q_src, M, sides, ncoef, nrhs)
+    assert qbx.qbx_workspace_bytes(1 << 22, 1 << 20, 1, 1) <= 3 * 16 * 2**22 + 64 * 16 * 2**20 + 8 * 2**30 + 4096
+    a, b, c = (ctypes.c_int() for _ in range(3))
+    L = qbx.lib()
+    assert L.qbx_debug_route(None, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)) == 1

@@ -533,3 +533,40 @@ def test_captured_calls_at_complex_k_keep_their_k(cuda, call):
     fresh.replay()
     torch.cuda.synchronize()
     assert torch.equal(out3, now) and torch.isfinite(torch.view_as_real(now)).all()
+
+
+@pytest.mark.parametrize("M,ops,nrhs", [(16, (0,), 1), (128, (0,), 1), (256, (1,), 1), (256, (0, 1), 1), (256, (2,), 1),
+                                        (128, (0, 1), 3), (1024, (0,), 1), (1024, (0, 1, 2), 1), (256, (1,), 16),
+                                        (96, (0, 1), 16)])
+def test_documented_workspace_holds_the_clusters(cuda, M, ops, nrhs):
+    """qbx_workspace_bytes for one side and the operators' components: distant
+    sources through moments, with the bits of a plan of twice the room."""
+    k, p = 0.05 * M, 8
+    ncoef = sum(2 if o == 2 else 1 for o in ops)
+    cur = W.starfish(0.2, 3)
+    size = qbx.qbx_workspace_bytes(M * 64, M * 16, ncoef, nrhs)
+    plan, big = (qbx.Plan(16, 64, workspace_bytes=b) for b in (size, 2 * size + (64 << 20)))
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    got = qbx.qbx_apply_ops(plan, g, ops, qbx.SIDE_INT, 0, k, p, d)
+    assert qbx.qbx_debug_route(plan)[0] == 1
+    ref = qbx.qbx_apply_ops(big, g, ops, qbx.SIDE_INT, 0, k, p, d)
+    assert qbx.qbx_debug_route(plan) == qbx.qbx_debug_route(big)
+    for o in ops:
+        assert torch.equal(got[o], ref[o])
+
+
+def test_documented_workspace_holds_separate_densities_and_grad_d(cuda):
+    M, k, p = 256, 12.0, 8
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(16, 64, workspace_bytes=qbx.qbx_workspace_bytes(M * 64, M * 16, 4, 1))
+    g = geometry(plan, cur, cur.edges(M))
+    d = {o: torch.as_tensor(W.complex_gaussian(o, g.n_tgt).reshape(-1, 1), device="cuda") for o in (0, 1, 2)}
+    qbx.qbx_apply_ops(plan, g, (0, 1, 2), qbx.SIDE_INT, 0, k, p, d)
+    assert qbx.qbx_debug_route(plan)[0] == 1
+    plan = qbx.Plan(16, 64, workspace_bytes=qbx.qbx_workspace_bytes(M * 64, M * 16, 2, 1))
+    qbx.qbx_apply(plan, g, qbx.OP_GRAD_D, qbx.SIDE_INT, 0, k, p, d[0])
+    assert qbx.qbx_debug_route(plan)[0] == 1
+    plan = qbx.Plan(16, 64, workspace_bytes=qbx.qbx_workspace_bytes(M * 64, M * 16, 2 * p + 1, 1))
+    qbx.qbx_form_locals(plan, g, qbx.OP_D, qbx.SIDE_INT, k, p, qbx.qbx_upsample(plan, g, d[0]))
+    assert qbx.qbx_debug_route(plan)[0] == 1
