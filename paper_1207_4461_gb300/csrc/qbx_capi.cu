@@ -863,17 +863,38 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   size_t tree_bytes = 0;
   int ns_far = 0;
   const bool far_group = group && ops != 7;   // many columns: far values formed once for all
-  // Many columns: the clusters' chain of launches (0.5 ms at 16 panels and 16
-  // rhs, 1.3 ms at 48 and 32, one side) has to be repaid: S + D of 16 rhs at 24
-  // and 32 panels 594 and 731 us, pair by pair 547 and 829; of 32 rhs at 32 and
-  // 48 panels 1086 and 1322, pairs 833 and 1760; D - i eta S of 8 rhs at 16 and
-  // 24 panels 606 and 689, pairs 439 and 767, of 32 rhs at 24 and 32 881 and
-  // 991, pairs 771 and 1220; S + D + grad S (no far values for all columns at once) of 16 rhs at 32 and
-  // 48 panels 1979 and 2406, pairs 1406 and 3056, of 32 rhs at 64 5039 and 5241.
+  // Many columns: the clusters' chain of launches has to be repaid.  By pairs,
+  // between the sizes where either side is the faster one; measured at 16/64
+  // nodes a panel and k = 0.15 / 0.4 times the panels, clusters against pairs, us:
+  //  S + D, 16 rhs, one side, 24 and 32 panels 599/640 and 735/818 against 508 and 826;
+  //    32 rhs, 40 and 48 panels 1202/1471 and 1318/1677 against 1268 and 1711;
+  //  D - i eta S, 8 rhs, 20 and 28 panels 623/700 and 736/744 against 483 and 846;
+  //    32 rhs, 28 and 32 panels 959/1010 and 997/1093 against 849 and 1072;
+  //  S + D + grad S (no far values for all columns at once: the clusters' time
+  //    goes with the rhs, the pairs' with passes of 32 or 64), one side, 16 rhs,
+  //    40 and 48 panels 2111/2947 and 2421/3493 against 2199 and 3064; 32 rhs, 64
+  //    and 96 panels 5037/7635 and 7748/12678 against 5302 and 11739; both sides,
+  //    16 rhs, 40 and 48 panels 3514/5288 and 3698/6230 against 4228 and 5964;
+  //  near-only (the pairs beyond eta r are cheap), eta = 10: S + D, 16 rhs, one
+  //    side, 32 and 40 panels 0.89/1.02 and 0.80/0.95 of the pairs' time, 32 rhs,
+  //    48 and 64 panels 1.02/1.24 and 0.81/0.98, both sides, 32 and 40 panels
+  //    1.10/1.12 and 0.92/0.94; with grad S, 16 rhs, one side, 48 and 64 panels
+  //    0.98/1.24 and 0.61/0.97;
+  //  grad S alone (pairs in passes of 8 rhs), 8 rhs, one side, 48 and 64 panels
+  //    1.03/1.48 and 0.67/1.10, both sides, 48 and 64 panels 0.81/1.43 and 0.60/1.23.
+  // Leaves of few sources cost the clusters as much and save less: D - i eta S
+  // of 16 rhs at 1.4e6 pairs of 4/8 nodes 1589 against 782, at 1.2e6 of 8/32 1081
+  // against 632, at 2.1e6 of 8/32 1130 against 1069.
+  const bool half_leaves = g->q_src % 2 == 0 && g->q_src >= 32, both = nc > g->n_tgt;
+  const double leaf = std::max(1.0, 20.0 / (half_leaves ? g->q_src / 2 : g->q_src));
   double tree_pairs = 0.0;
-  if (cf) tree_pairs = nrhs <= 8 ? 1.15e6 : 2.0e6;
-  else if (group && ops == 7) tree_pairs = 1.25e5 * nrhs;
-  else if (group) tree_pairs = nrhs > 16 ? 2.3e6 : nc > g->n_tgt ? 0.8e6 : 1.0e6;
+  if (cf) tree_pairs = leaf * (nrhs <= 8 ? 1.15e6 : 2.0e6);
+  else if (group && ops == 7)
+    tree_pairs = (both ? 1.6 : 1.0) * (local ? 1.6 : 1.0) *
+                 (2.3e6 + 0.21e6 * (nrhs <= 32 ? nrhs - 16 : std::min(std::max(0.6 * nrhs - 16.0, 4.0), 22.0)));
+  else if (group && local) tree_pairs = leaf * (both ? 3.2e6 : nrhs > 16 ? 3.6e6 : 1.8e6);
+  else if (group) tree_pairs = leaf * (nrhs > 16 ? 2.3e6 : both ? 0.8e6 : 1.0e6);
+  else if (ops == QBX_OPS_GRAD_S && nrhs > 3) tree_pairs = (both ? 1.6 : 1.0) * 0.45e6 * nrhs / ((nrhs + 7) / 8);
   if (g->M >= kTreeMinPanels && (double)nc * g->n_src >= tree_pairs) {
     tr.kre = k.re;
     tr.kim = k.im;

@@ -570,3 +570,45 @@ def test_documented_workspace_holds_separate_densities_and_grad_d(cuda):
     plan = qbx.Plan(16, 64, workspace_bytes=qbx.qbx_workspace_bytes(M * 64, M * 16, 2 * p + 1, 1))
     qbx.qbx_form_locals(plan, g, qbx.OP_D, qbx.SIDE_INT, k, p, qbx.qbx_upsample(plan, g, d[0]))
     assert qbx.qbx_debug_route(plan)[0] == 1
+
+
+ROUTES = [
+    # M, q_tgt, q_src, ops, side, nrhs, eta, clusters: either side of the rules by pairs, columns and sources per leaf
+    (32, 16, 64, (0, 1, 2), "two", 16, None, 0), (48, 16, 64, (0, 1, 2), "two", 16, None, 1),   # the far values anew for 2 rhs
+    (48, 16, 64, (0, 1, 2), "int", 16, None, 1), (64, 16, 64, (0, 1, 2), "int", 32, None, 0),
+    (96, 16, 64, (0, 1, 2), "int", 32, None, 1), (64, 16, 64, (0, 1, 2), "two", 32, None, 0),
+    (24, 16, 64, "cfie", "two", 8, None, 1), (48, 8, 32, "cfie", "two", 8, None, 0),            # leaves of 16 sources
+    (200, 4, 8, "cfie", "two", 1, None, 0), (220, 4, 8, "cfie", "two", 1, None, 1),             # of 8
+    (32, 16, 64, "cfie", "two", 32, None, 1), (64, 8, 32, "cfie", "two", 32, None, 0),
+    (20, 16, 64, (0, 1), "two", 16, None, 1), (40, 16, 16, (0, 1), "two", 16, None, 0),
+    (150, 4, 8, (0, 1), "two", 16, None, 0), (200, 4, 8, (0,), "int", 16, None, 0),
+    (96, 8, 32, (0, 1), "int", 32, None, 0), (48, 16, 64, (0, 1), "int", 32, None, 1),
+    (32, 16, 64, (0, 1), "two", 16, 6.0, 0), (40, 16, 64, (0, 1), "two", 16, 6.0, 1),           # the pairs beyond eta r are cheap
+    (24, 16, 64, (0, 1), "int", 16, 10.0, 0), (48, 16, 64, (0, 1), "int", 32, 10.0, 0), (64, 16, 64, (0, 1), "int", 32, 10.0, 1),
+    (48, 16, 64, (0, 1, 2), "int", 16, 10.0, 0), (64, 16, 64, (0, 1, 2), "int", 16, 10.0, 1),
+    (45, 12, 40, (2,), "int", 16, None, 0), (64, 16, 64, (2,), "int", 16, None, 1),
+    (48, 16, 64, (2,), "two", 8, None, 0), (64, 16, 64, (2,), "two", 8, None, 1), (24, 16, 64, (2,), "two", 3, None, 1),
+    (16, 16, 64, (0, 1, 2), "int", 1, None, 1), (15, 16, 64, (0, 1, 2), "int", 1, None, 0),     # few columns: by panels alone
+]
+
+
+@pytest.mark.parametrize("case", ROUTES)
+def test_route_rules(cuda, case):
+    """Which calls go through clusters, and that both routes agree there."""
+    M, qt, qs, ops, side, nrhs, eta, want = case
+    side = {"int": qbx.SIDE_INT, "two": qbx.SIDE_TWO}[side]
+    k, p = M * qs / 64 * 0.15, 8
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(qt, qs, n_src=M * qs, n_ctr=2 * M * qt, ncoef=4, nrhs=nrhs)
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M + nrhs, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    ncomp = 1 if ops == "cfie" else sum(2 if o == 2 else 1 for o in ops)
+    pp = pair_plan(g, qt, qs, nrhs, ncomp)
+    run = lambda pl: ([qbx.qbx_apply_cfie(pl, g, k, k - 0.5j, p, d)] if ops == "cfie" else
+                      list(qbx.qbx_apply_ops(pl, g, ops, side, 0, k, p, d, eta=eta).values()))
+    got = run(plan)
+    assert qbx.qbx_debug_route(plan)[0] == want
+    ref = run(pp)
+    assert qbx.qbx_debug_route(pp) == (0, 0, 0)
+    for i, (a, b) in enumerate(zip(got, ref)):
+        check(a, b, (case, i))
