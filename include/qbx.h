@@ -528,7 +528,7 @@ int qbx_apply_static_status(void *stream);
  * Im z == 0), and J_0..J_nmax (Miller) at z[n].  For tests. */
 int qbx_debug_hankel01(const qbx_c64 *z, int n, qbx_c64 *h0, qbx_c64 *h1, void *stream);
 int qbx_debug_besselj(const qbx_c64 *z, int n, int nmax, qbx_c64 *j, void *stream);
-/* Route of the plan's last apply, grad D, stored coefficients or adjoint:
+/* Route of the plan's last apply, grad D, stored coefficients, adjoint or assembly:
  * clusters = 1 if distant sources went through moments (0: every pair),
  * upward = 1 if these were carried up level by level, super_blocks = how many
  * super-blocks were formed.  Host.  For tests. */

@@ -140,9 +140,12 @@ extern "C" int qbx_apply_adjoint(qbx_plan* plan, const qbx_geom* g, int op, int 
   // distant centres through cluster moments (S: value; D: gradient along n_s), few columns
   TreeArgs tr;
   const int fops = op == QBX_OP_S ? 1 << QBX_OP_S : 1 << QBX_OP_GRAD_S;
-  // (clusters: S at 24, 32 and 48 panels 304, 444 and 462 us, pair by pair 255,
-  // 441 and 762; five rhs at 48 and 64 813 and 935, pairs 765 and 1140)
-  const bool clusters = nrhs <= 8 && (double)nc * g->n_src >= 1.05e6 * (1.0 + 0.4 * (nrhs - 1));
+  // (clusters: S, one side, 24, 32 and 48 panels 304, 444 and 462 us, pair by
+  // pair 255, 441 and 762; at k = 0.15 / 0.4 times the panels, of the pairs' time:
+  // three rhs at 40 and 48 panels 1.10/1.31 and 0.82/1.06, eight at 64 and 96
+  // 0.91/1.30 and 0.50/0.70; D, both sides, one rhs at 20 and 28 1.03/1.17 and
+  // 0.72/0.91, three at 28 and 40 0.98/1.17 and 0.72/0.87)
+  const bool clusters = nrhs <= 8 && (double)nc * g->n_src >= 1.2e6 + 0.55e6 * (nrhs - 1);
   size_t b_tree = clusters ? adj_tree_setup(&tr, g, c0, nc, k, p, fops, op == QBX_OP_D ? 1 : 0, nrhs, nullptr, nullptr,
                                              num_sms, nullptr)
                             : 0;

@@ -220,6 +220,7 @@ extern "C" int qbx_assemble_cfie(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, q
   const size_t need = matrix_tree_setup(&far, g, k, eta, p, a.hk_tab, nullptr);
   const bool tree = need > 0 && need <= ws_bytes &&
                     (ck ? asm_smem<cplx>(p, q_src, q_tgt, true) : asm_smem<double>(p, q_src, q_tgt, true)) <= 200 * 1024;
+  host_plan_route(plan, tree ? &far.t : nullptr);
   const size_t smem = ck ? asm_smem<cplx>(p, q_src, q_tgt, tree) : asm_smem<double>(p, q_src, q_tgt, tree);
   // panel groups: about 8192 CTAs in all (some 18 waves of the resident
   // CTAs), so that the last, partly filled wave costs little; near panels: one

@@ -612,7 +612,11 @@ static int shape_impl(int op, qbx_plan* plan, const qbx_geom* g, int side, qbx_c
     tf.split0 = split0;
     return tree_layout(&tf, at);
   };
-  if (g->M >= kTreeMinPanels && nrhs <= 8) {
+  // (S of several rhs: the clusters' chains have to be repaid; one side, three
+  // rhs at 32 and 40 panels 1.12/1.30 and 0.82/1.05 of the pairs' time at k = 0.15
+  // / 0.4 times the panels, eight at 32 and 48 1.33/1.49 and 0.76/1.04)
+  if (g->M >= kTreeMinPanels && nrhs <= 8 &&
+      (opD || nrhs == 1 || (double)nc * n_src >= 0.9e6 + 0.08e6 * nrhs)) {
     b_tf = set_fwd_tree(nullptr, nullptr, nullptr, nullptr, 0);
     if (!far_clusters_fit(tf)) b_tf = 0;
     if (b_tf) b_ta = adj_tree_setup(&ta, g, c0, nc, k, p, aops, opD ? 2 : 1, nrhs, nullptr, nullptr, num_sms, nullptr);

@@ -2071,7 +2071,10 @@ size_t matrix_tree_setup(MatrixFarArgs* q, const qbx_geom* g, qbx_c64 k, qbx_c64
                          char* base) {
   *q = MatrixFarArgs{};
   TreeArgs& t = q->t;
-  if (g->M < kTreeMinPanels || g->q_src > 128) return 0;
+  // (a panel's q_tgt columns of moments against its q_src sources: at 16/16 nodes
+  // 1.25 to 1.42 times the pairs' time, 80 panels; at 16/64 0.36 to 0.99, at 8/32
+  // 0.31 to 1.04)
+  if (g->M < kTreeMinPanels || g->q_src > 128 || g->q_src < 2 * g->q_tgt) return 0;
   const bool ck = k.im != 0.0;
   const size_t setup = 2 * (ck ? far_col_bytes<cplx>(p) + far_warp_bytes<cplx>(p) : far_col_bytes<double>(p) + far_warp_bytes<double>(p));
   if (setup > sizeof(LocSmem) || (ck ? moments_smem<cplx>(g->q_src) : moments_smem<double>(g->q_src)) > 220 * 1024) return 0;

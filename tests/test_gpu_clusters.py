@@ -612,3 +612,31 @@ def test_route_rules(cuda, case):
     assert qbx.qbx_debug_route(pp) == (0, 0, 0)
     for i, (a, b) in enumerate(zip(got, ref)):
         check(a, b, (case, i))
+
+
+@pytest.mark.parametrize("call,M,q_tgt,q_src,side,nrhs,want", [
+    ("adjoint", 33, 16, 64, "int", 1, 0), ("adjoint", 35, 16, 64, "int", 1, 1), ("adjoint", 48, 16, 64, "int", 3, 1),
+    ("adjoint", 32, 16, 64, "two", 3, 0), ("adjoint", 64, 16, 64, "int", 8, 0), ("adjoint", 72, 16, 64, "int", 8, 1),
+    ("shape_s", 16, 16, 64, "int", 1, 1), ("shape_s", 32, 16, 64, "int", 3, 0), ("shape_s", 40, 16, 64, "int", 3, 1),
+    ("shape_s", 38, 16, 64, "int", 8, 0), ("shape_s", 48, 16, 64, "int", 8, 1), ("shape_d", 20, 16, 64, "int", 8, 1),
+    ("locals", 16, 16, 64, "int", 1, 1), ("locals", 200, 4, 8, "int", 1, 0), ("locals", 200, 4, 8, "two", 1, 1),
+    ("assemble", 40, 16, 16, "two", 1, 0), ("assemble", 40, 16, 64, "two", 1, 1), ("assemble", 40, 8, 32, "two", 1, 1)])
+def test_route_rules_of_adjoints_locals_and_the_matrix(cuda, call, M, q_tgt, q_src, side, nrhs, want):
+    side = {"int": qbx.SIDE_INT, "two": qbx.SIDE_TWO}[side]
+    k, p = M * q_src / 64 * 0.15, 8
+    cur = W.starfish(0.2, 3)
+    size = max(qbx.qbx_workspace_bytes(M * q_src, 2 * M * q_tgt, 2 * p + 1, nrhs),
+               qbx.qbx_workspace_bytes(M * q_src, 2 * M * q_tgt, 4, max(nrhs, q_tgt)),
+               qbx.qbx_shape_adjoint_workspace_bytes(M, q_tgt, q_src, p, nrhs))
+    plan = qbx.Plan(q_tgt, q_src, workspace_bytes=size)
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    if call == "adjoint":
+        qbx.qbx_apply_adjoint(plan, g, qbx.OP_S, side, 0, k, p, d)
+    elif call == "locals":
+        qbx.qbx_form_locals(plan, g, qbx.OP_S, side, k, p, qbx.qbx_upsample(plan, g, d))
+    elif call == "assemble":
+        qbx.qbx_assemble_cfie(plan, g, k, k, p)
+    else:
+        qbx.qbx_apply_shape_adjoint(plan, g, side, k, p, d, d, op=qbx.OP_S if call == "shape_s" else qbx.OP_D)
+    assert qbx.qbx_debug_route(plan)[0] == want
