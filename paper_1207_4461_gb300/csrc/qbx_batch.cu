@@ -203,8 +203,11 @@ double lpt_makespan(const std::vector<GroupInst>& inst, const std::vector<GroupI
   return *std::max_element(heap.begin(), heap.end());
 }
 
-// smallest source range of an item (with clusters a block has few hundred sources in all)
-int min_chunk(const qbx_batch* b) { return b->tree ? 64 : 512; }
+// smallest source range of an item (with clusters a block has few hundred
+// sources in all; both sides of a target in one item take twice as long per
+// source: one curve of 16 panels, S, both sides, 32 rhs 2289 us with 512,
+// 1460 with one side per item)
+int min_chunk(const qbx_batch* b) { return b->tree ? 64 : 512 / b->nsd; }
 
 // The source chunk the model prefers: the smallest predicted makespan over
 // chunks 2^j * 32 (and all sources), ties to the larger chunk (fewer

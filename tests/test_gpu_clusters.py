@@ -640,3 +640,21 @@ def test_route_rules_of_adjoints_locals_and_the_matrix(cuda, call, M, q_tgt, q_s
     else:
         qbx.qbx_apply_shape_adjoint(plan, g, side, k, p, d, d, op=qbx.OP_S if call == "shape_s" else qbx.OP_D)
     assert qbx.qbx_debug_route(plan)[0] == want
+
+
+@pytest.mark.parametrize("M,q_tgt,q_src,ops,nrhs", [(16, 16, 64, (0,), 32), (31, 12, 40, (0,), 4), (12, 16, 64, (0, 1), 32)])
+def test_batch_of_one_small_curve_on_both_sides(cuda, M, q_tgt, q_src, ops, nrhs):
+    """Both sides of a target are one item, twice as long per source: ranges down
+    to 256 sources there, so that there are no fewer items than one side at a time has."""
+    plan = qbx.Plan(q_tgt, q_src, n_src=M * q_src, n_ctr=2 * M * q_tgt, ncoef=2, nrhs=nrhs)
+    cur = W.starfish(0.2, 3)
+    g = qbx.qbx_geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    b = qbx.Batch(plan, [g], [3.0], 7, ops, qbx.SIDE_TWO, 0, [d])
+    one = qbx.Batch(plan, [g], [3.0], 7, ops, qbx.SIDE_INT, 0, [d])
+    assert b.info()[1] == one.info()[1] // 2 and b.info()[2] >= 2 * ((g.n_tgt + 31) // 32) * (g.n_src // 512)
+    out = b.apply()[0]
+    b.status()
+    ref = qbx.qbx_apply_ops(pair_plan(g, q_tgt, q_src, nrhs, len(ops)), g, ops, qbx.SIDE_TWO, 0, 3.0, 7, d)
+    for o in ops:
+        check(out[o], ref[o], o)
