@@ -156,8 +156,10 @@ int block_sources(const GroupInst& in) {
   return in.near ? std::min(in.n_src, 6 * (in.n_src / in.M)) : in.n_src;
 }
 
-// Work items of a configuration: 32 targets of one curve x a range of at
-// most `chunk` of its sources (equal ranges per curve), longest first.
+// Work items of a configuration: 32 rows of one curve (with a near list: of one
+// side, otherwise across the sides: both sides of 400 centres are 25 blocks, not
+// 26) x a range of at most `chunk` of its sources (equal ranges per curve),
+// longest first.
 std::vector<GroupItem> make_items(const std::vector<GroupInst>& inst, int chunk, std::vector<int>& nsplit) {
   std::vector<GroupItem> items;
   nsplit.assign(inst.size(), 1);
@@ -167,14 +169,15 @@ std::vector<GroupItem> make_items(const std::vector<GroupInst>& inst, int chunk,
     const int len = (n + ns - 1) / ns;
     ns = (n + len - 1) / len;   // every range non-empty
     nsplit[i] = ns;
-    for (int sd = 0; sd < inst[i].n_row / inst[i].n_tgt; ++sd)
-      for (int t = 0; t < inst[i].n_tgt; t += kGrpCentres)
+    const int run = inst[i].near ? inst[i].n_tgt : inst[i].n_row;
+    for (int r = 0; r < inst[i].n_row; r += run)
+      for (int c = r; c < r + run; c += kGrpCentres)
         for (int k = 0; k < ns; ++k)
-          items.push_back(GroupItem{(int)i, t, sd, k, k * len, std::min(n, (k + 1) * len)});
+          items.push_back(GroupItem{(int)i, c, std::min(r + run, c + kGrpCentres), k, k * len, std::min(n, (k + 1) * len)});
   }
   std::stable_sort(items.begin(), items.end(), [&](const GroupItem& x, const GroupItem& y) {
-    const long cx = (long)std::min(kGrpCentres, inst[x.inst].n_tgt - x.t0) * (x.src1 - x.src0);
-    const long cy = (long)std::min(kGrpCentres, inst[y.inst].n_tgt - y.t0) * (y.src1 - y.src0);
+    const long cx = (long)(x.row1 - x.row0) * (x.src1 - x.src0);
+    const long cy = (long)(y.row1 - y.row0) * (y.src1 - y.src0);
     return cx > cy;
   });
   return items;
@@ -191,12 +194,12 @@ size_t part_bytes(const std::vector<GroupInst>& inst, const std::vector<int>& ns
 // Predicted makespan (in pair units) of the persistent grid taking the items
 // in list order: each of `slots` CTAs takes the next item when it finishes
 // (the atomic counter), an item costs its pairs plus a fixed set-up share.
-double lpt_makespan(const std::vector<GroupInst>& inst, const std::vector<GroupItem>& items, int slots) {
+double lpt_makespan(const std::vector<GroupItem>& items, int slots) {
   std::vector<double> heap(std::max(1, slots), 0.0);   // min-heap of finish times
   auto cmp = [](double x, double y) { return x > y; };
   for (const GroupItem& it : items) {
     std::pop_heap(heap.begin(), heap.end(), cmp);
-    const double pairs = (double)std::min(kGrpCentres, inst[it.inst].n_tgt - it.t0) * (it.src1 - it.src0);
+    const double pairs = (double)(it.row1 - it.row0) * (it.src1 - it.src0);
     heap.back() += pairs + 32.0 * kGrpTile;   // + one tile's worth of set-up per item
     std::push_heap(heap.begin(), heap.end(), cmp);
   }
@@ -222,7 +225,7 @@ int model_chunk(const qbx_batch* b, int slots, size_t budget) {
   for (int c : cand) {
     std::vector<GroupItem> items = make_items(b->h_inst, c, ns);
     if (part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs) > budget) break;
-    const double t = lpt_makespan(b->h_inst, items, slots);
+    const double t = lpt_makespan(items, slots);
     if (t < bt * 0.995) {
       bt = t;
       best = c;

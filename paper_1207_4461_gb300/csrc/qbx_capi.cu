@@ -940,9 +940,10 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   const bool tree = ns_far > 0;
   host_plan_route(p, tree ? &tr : nullptr);
   if (!tree) tree_bytes = 0;
+  const int pair_units = group && !tree ? (nrow + kGrpCentres - 1) / kGrpCentres : units;   // (across the sides)
   // (with clusters a block's near leaves are some six panels; down to two dozen sources a CTA)
   const int ns_near =
-      host_choose_split_waves(p->num_sms, occ, units,
+      host_choose_split_waves(p->num_sms, occ, pair_units,
                               tree ? std::min(g->n_src, (group ? 8 : 16) * g->q_src)
                                    : (group && nsd == 2 ? 2 : 1) * g->n_src,   // both sides in one item: half as long
                               // (20 panels, S + D of 32 rhs, both sides 780 -> 583 us)
@@ -1058,15 +1059,15 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     in.near_cnt = a.near_cnt;
     in.near_stride = a.near_stride;
     in.near_q = a.near_q_src;
-    ga.st_units = units;
+    ga.st_units = pair_units;
     ga.st_nsplit = ns_near;
     ga.st_split_len = split_len(g->n_src, ns_near);
     ga.eta2 = a.eta2;
   }
   auto pair_sums = [&](cudaStream_t s) {
     if (group) {
-      if (local) return launch_group_local(ga, ck, rg, units * ns_near, s);
-      return ck ? launch_group_cplx(ga, rg, units * ns_near, s) : launch_group_real(ga, rg, units * ns_near, s);
+      if (local) return launch_group_local(ga, ck, rg, pair_units * ns_near, s);
+      return ck ? launch_group_cplx(ga, rg, pair_units * ns_near, s) : launch_group_real(ga, rg, pair_units * ns_near, s);
     }
     cudaError_t e = cudaSuccess;
     for (int r0 = 0; r0 < nrhs && e == cudaSuccess; r0 += chunk) {

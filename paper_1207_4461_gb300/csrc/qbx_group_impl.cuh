@@ -10,7 +10,7 @@
 // Kernel generation is therefore paid once per pair however many densities
 // there are, and each thread keeps only RG accumulators per component.
 //
-// Items (32 targets x a source range) come either from blockIdx (one curve,
+// Items (32 rows x a source range) come either from blockIdx (one curve,
 // static split of the sources) or from a longest-first item list through an
 // atomic counter (a batch: persistent CTAs, no waits between CTAs).  With a
 // near list (qbx_tree.cu) an item's sources are its share of the block's near
@@ -105,22 +105,27 @@ k_apply_group(GroupArgs a) {
     if (dynamic) {
       item = a.items[it];
     } else {
-      // rank r of the launch takes the 32-target blocks' splits near-field
+      // rank r of the launch takes the 32-row blocks' splits near-field
       // first, as the fused apply
-      const int blks = (a.inst0.n_tgt + kGrpCentres - 1) / kGrpCentres;
       item.inst = 0;
       const int unit = it % a.st_units, rank = it / a.st_units;
       const int q_t = a.inst0.n_tgt / a.inst0.M, q_s = a.inst0.n_src / a.inst0.M;
-      item.side = unit / blks;
-      item.t0 = (unit - item.side * blks) * kGrpCentres;
-      item.split = a.inst0.near ? rank
-                                : near_first_split(rank, min(item.t0 + kGrpCentres / 2, a.inst0.n_tgt - 1), q_t, q_s,
-                                                   a.st_split_len, a.st_nsplit);
+      if (a.inst0.near) {   // (a list belongs to 32 targets of one side)
+        const int blks = (a.inst0.n_tgt + kGrpCentres - 1) / kGrpCentres, side = unit / blks;
+        item.row0 = side * a.inst0.n_tgt + (unit - side * blks) * kGrpCentres;
+        item.row1 = min((side + 1) * a.inst0.n_tgt, item.row0 + kGrpCentres);
+        item.split = rank;
+      } else {
+        item.row0 = unit * kGrpCentres;
+        item.row1 = min(a.inst0.n_row, item.row0 + kGrpCentres);
+        item.split = near_first_split(rank, min(item.row0 + kGrpCentres / 2, a.inst0.n_row - 1) % a.inst0.n_tgt, q_t,
+                                      q_s, a.st_split_len, a.st_nsplit);
+      }
       item.src0 = item.split * a.st_split_len;
       item.src1 = min(a.inst0.n_src, item.src0 + a.st_split_len);
     }
     const GroupInst& in = dynamic ? a.inst[item.inst] : a.inst0;
-    const int blk = item.t0 / kGrpCentres;
+    const int blk = item.row0 % in.n_tgt / kGrpCentres;
     const int* near = in.near ? in.near + (size_t)blk * in.near_stride : nullptr;
     if (near) {
       const long n = (long)in.near_cnt[3 * blk] * in.near_q;
@@ -129,9 +134,9 @@ k_apply_group(GroupArgs a) {
     }
 
     // ---- per-target set-up: warp sd forms side sd's geometry and columns ----
-    const bool active = item.t0 + lane < in.n_tgt;
-    const int t = active ? item.t0 + lane : in.n_tgt - 1;
-    const int c = item.side * in.n_tgt + t;   // row of the partial sums
+    const bool active = item.row0 + lane < item.row1;
+    const int c = active ? item.row0 + lane : item.row1 - 1;   // row of the partial sums
+    const int t = c % in.n_tgt;
     KW<T> kw;
     kw.init(in.kre, in.kim, in.hk_tab);
     const T kk = kw.kval();

@@ -200,11 +200,12 @@ struct GroupInst {
   void* out[3];                   // per operator (S, D, grad S) outputs, for the finish
   const double* hk_tab;           // complex k: the amplitude table of this curve's k, or null
 };
-// A work item: 32 targets from t0 of instance inst, one side's centres (both
-// when merged: side 0), sources [src0, src1) or the split's share of the near
+// A work item: the rows [row0, row1) of the partial sums of instance inst, 32
+// at most (centres: of one side, as a near list's block, or across the sides;
+// merged: targets), sources [src0, src1) or the split's share of the near
 // leaves, partial-sum slot `split`.
 struct GroupItem {
-  int inst, t0, side, split, src0, src1;
+  int inst, row0, row1, split, src0, src1;
 };
 struct GroupArgs {
   int ops, p, nrhs;

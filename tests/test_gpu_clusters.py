@@ -658,3 +658,27 @@ def test_batch_of_one_small_curve_on_both_sides(cuda, M, q_tgt, q_src, ops, nrhs
     ref = qbx.qbx_apply_ops(pair_plan(g, q_tgt, q_src, nrhs, len(ops)), g, ops, qbx.SIDE_TWO, 0, 3.0, 7, d)
     for o in ops:
         check(out[o], ref[o], o)
+
+
+@pytest.mark.parametrize("q_tgt,q_src,M,nrhs", [(10, 100, 40, 4), (4, 8, 100, 16), (5, 21, 9, 3), (3, 16, 7, 17)])
+def test_group_blocks_across_the_sides(cuda, q_tgt, q_src, M, nrhs):
+    """400, 400, 45 and 21 targets (no multiple of 32), S + D + grad S on both
+    sides: pair by pair 32 centres to a block across the sides, in a batch and
+    (from 16 rhs on) in one apply; against single right-hand sides."""
+    plan = qbx.Plan(q_tgt, q_src, n_src=M * q_src, n_ctr=2 * M * q_tgt, ncoef=4, nrhs=nrhs)
+    cur, k, p, ops = W.starfish(0.2, 3), 3.0, 7, (0, 1, 2)
+    g = qbx.qbx_geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    b = qbx.Batch(plan, [g, g], [k, k], p, ops, qbx.SIDE_TWO, 0, [d, d])
+    n = b.info()[2]
+    assert n % (2 * ((2 * g.n_tgt + 31) // 32)) == 0   # items: blocks of both sides together, times equal ranges
+    outs = b.apply()
+    b.status()
+    got = qbx.qbx_apply_ops(plan, g, ops, qbx.SIDE_TWO, 0, k, p, d)
+    for r in range(0, nrhs, 3):
+        pp = pair_plan(g, q_tgt, q_src, 1, 4)
+        ref = qbx.qbx_apply_ops(pp, g, ops, qbx.SIDE_TWO, 0, k, p, d[:, r:r + 1].contiguous())
+        for o in ops:
+            check(got[o][..., r:r + 1], ref[o], ("apply", o, r))
+            for out in outs:
+                check(out[o][..., r:r + 1], ref[o], ("batch", o, r))
