@@ -533,6 +533,7 @@ int qbx_debug_besselj(const qbx_c64 *z, int n, int nmax, qbx_c64 *j, void *strea
  * upward = 1 if these were carried up level by level, super_blocks = how many
  * super-blocks were formed.  Host.  For tests. */
 int qbx_debug_route(const qbx_plan *plan, int *clusters, int *upward, int *super_blocks);
+int qbx_debug_batch_route(const qbx_batch *batch, int *clusters);
 /* H0, H1 at z = k rho[i] (rho > 0, n values) as the pair kernels evaluate
  * them for this k: for Im k > 0 through the plan's amplitude table of the ray
  * z = k rho (fitted once per k) where |z| >= 2, the direct evaluation

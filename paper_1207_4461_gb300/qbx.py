@@ -133,6 +133,8 @@ def lib():
             L.qbx_apply_static_status.restype = I
             L.qbx_debug_route.argtypes = [_P, ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(I)]
             L.qbx_debug_route.restype = I
+            L.qbx_debug_batch_route.argtypes = [_P, ctypes.POINTER(I)]
+            L.qbx_debug_batch_route.restype = I
             L.qbx_vec_dots.argtypes = [I, I, I, _P, _P, _P, _P, _P]
             L.qbx_vec_dots.restype = I
             L.qbx_vec_dots_work_bytes.argtypes = [I, I]
@@ -669,6 +671,12 @@ class Batch:
         v = [ctypes.c_int(0) for _ in range(4)]
         _check(lib().qbx_batch_info(self.handle, *[ctypes.byref(x) for x in v]))
         return tuple(x.value for x in v)
+
+    def debug_route(self):
+        """1 if the curves of 16 panels or more take distant sources through moments."""
+        v = ctypes.c_int(0)
+        _check(lib().qbx_debug_batch_route(self.handle, ctypes.byref(v)))
+        return v.value
 
     def status(self):
         _check(lib().qbx_batch_status(self.handle, _stream()))

@@ -682,3 +682,26 @@ def test_group_blocks_across_the_sides(cuda, q_tgt, q_src, M, nrhs):
             check(got[o][..., r:r + 1], ref[o], ("apply", o, r))
             for out in outs:
                 check(out[o][..., r:r + 1], ref[o], ("batch", o, r))
+
+
+@pytest.mark.parametrize("Ms,q_tgt,q_src,side,ops,nrhs,eta,want", [
+    ((31,), 16, 64, "int", (0, 1), 4, 0.0, 0), ((32,), 16, 64, "int", (0, 1), 4, 0.0, 1),
+    ((47,), 16, 64, "int", (0, 1), 32, 0.0, 0), ((40, 30, 9), 16, 64, "int", (0, 1), 32, 0.0, 1),
+    ((100,) * 12, 4, 8, "int", (0, 1), 32, 0.0, 0), ((150,) * 12, 4, 8, "int", (0, 1), 32, 0.0, 1),
+    ((64,), 8, 32, "int", (0,), 16, 0.0, 0), ((32,), 16, 64, "two", (0,), 12, 8.0, 0), ((40,), 16, 64, "two", (0,), 12, 8.0, 1)])
+def test_batch_route_rules(cuda, Ms, q_tgt, q_src, side, ops, nrhs, eta, want):
+    side, k, p = {"int": qbx.SIDE_INT, "two": qbx.SIDE_TWO}[side], 4.0, 7
+    cur = W.starfish(0.15, 3)
+    plan = qbx.Plan(q_tgt, q_src, n_src=q_src * max(Ms), n_ctr=2 * q_tgt * max(Ms), ncoef=2, nrhs=nrhs)
+    gs = [qbx.qbx_geometry(plan, cur, cur.edges(M)) for M in Ms]
+    ds = [torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+          for M, g in zip(Ms, gs)]
+    b = qbx.Batch(plan, gs, [k] * len(Ms), p, ops, side, 0, ds)
+    if eta:
+        b.set_eta(eta)
+    assert b.debug_route() == want
+    out = b.apply()
+    b.status()
+    ref = qbx.qbx_apply_ops(pair_plan(gs[0], q_tgt, q_src, nrhs, len(ops)), gs[0], ops, side, 0, k, p, ds[0], eta=eta or None)
+    for o in ops:
+        check(out[0][o], ref[o], o)
