@@ -461,8 +461,8 @@ int qbx_batch_status(qbx_batch *batch, void *stream);
  * rebuilds the batch with the fastest; *rg, *chunk (may be NULL) receive the
  * choice.  Writes the outputs as an apply does.  Host call, synchronous.
  * The choice is cached in the process per (device, p, operators, side,
- * nrhs, real/complex k, and power-of-two buckets of the largest curve's
- * sources, the total pairs and the curve count); qbx_batch_create starts
+ * nrhs, real/complex k, with clusters or without, and power-of-two buckets of
+ * the largest curve's sources, the total pairs and the curve count); qbx_batch_create starts
  * from a cached choice when one matches. */
 int qbx_batch_tune(qbx_batch *batch, void *stream, int *rg, int *chunk);
 /* Near-only QBX for the whole batch (as qbx_apply_local, Sec. 5 remark):

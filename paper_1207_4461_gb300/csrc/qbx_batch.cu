@@ -435,10 +435,11 @@ int prepare_tree(qbx_batch* b, size_t budget) {
 }
 
 // Tuned configurations, cached per (device, p, operators, side, nrhs, real or
-// complex k, global or near-only, and the power-of-two buckets of the largest
-// curve, the total pairs and the curve count): a batch created later with the
-// same key starts from the measured choice instead of the model's.
-typedef std::tuple<int, int, int, int, int, int, int, int, int, int> TuneKey;
+// complex k, global or near-only, with clusters or without (whose thresholds
+// lie inside the buckets), and the power-of-two buckets of the largest curve,
+// the total pairs and the curve count): a batch created later with the same key
+// starts from the measured choice instead of the model's.
+typedef std::tuple<int, int, int, int, int, int, int, int, int, int, int> TuneKey;
 std::mutex g_tune_mu;
 std::map<TuneKey, std::pair<int, int>> g_tune_cache;
 
@@ -448,7 +449,7 @@ TuneKey tune_key(const qbx_batch* b) {
   double pairs = 0.0;
   for (const GroupInst& in : b->h_inst) pairs += (double)in.n_ctr * in.n_src;
   return TuneKey{b->device, b->p, b->ops, b->side, b->nrhs, b->ck ? 1 : 0, b->eta2 > 0.0 ? 1 : 0,
-                 log2i(b->max_src), log2i(pairs), log2i(b->n_inst)};
+                 b->tree ? 1 : 0, log2i(b->max_src), log2i(pairs), log2i(b->n_inst)};
 }
 
 // partial-sum budget: a quarter of the free device memory

@@ -705,3 +705,25 @@ def test_batch_route_rules(cuda, Ms, q_tgt, q_src, side, ops, nrhs, eta, want):
     ref = qbx.qbx_apply_ops(pair_plan(gs[0], q_tgt, q_src, nrhs, len(ops)), gs[0], ops, side, 0, k, p, ds[0], eta=eta or None)
     for o in ops:
         check(out[0][o], ref[o], o)
+
+
+def test_batch_tuning_is_kept_apart_for_clusters_and_pairs(cuda):
+    """Two batches whose pairs lie in one power-of-two bucket on either side of
+    the clusters' threshold: tuning one leaves the other its own items."""
+    nrhs, p, ops = 12, 7, (0,)
+    cur = W.starfish(0.15, 3)
+    plan = qbx.Plan(16, 64, n_src=64 * 32, n_ctr=32 * 32, ncoef=2, nrhs=nrhs)
+
+    def batch(Ms):
+        gs = [qbx.qbx_geometry(plan, cur, cur.edges(M)) for M in Ms]
+        ds = [torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+              for M, g in zip(Ms, gs)]
+        return qbx.Batch(plan, gs, [4.0, 3.0], p, ops, qbx.SIDE_INT, 0, ds)
+
+    pairs, clusters = (30, 8), (30, 10)   # 0.99e6 and 1.02e6 pairs, between 2^19 and 2^20
+    a, b = batch(pairs), batch(clusters)
+    assert a.debug_route() == 0 and b.debug_route() == 1
+    own = a.info()
+    b.tune()
+    assert batch(pairs).info() == own
+    assert a.info() == own and own[1] >= 512
