@@ -256,7 +256,7 @@ extern "C" int qbx_assemble_cfie(qbx_plan* plan, const qbx_geom* g, qbx_c64 k, q
   a.near = far.t.near;
   a.near_cnt = far.t.cnt;
   e = pairs(side);
-  const cudaError_t ef = launch_matrix_far(far, g->src_w, P, st);
+  const cudaError_t ef = launch_matrix_far(far, g->src_w, P, num_sms, st);
   cudaError_t ej = cudaEventRecord(join, side);   // (joined also after an error)
   if (ej == cudaSuccess) ej = cudaStreamWaitEvent(st, join, 0);
   if (e == cudaSuccess) e = ef != cudaSuccess ? ef : ej;

@@ -375,7 +375,7 @@ struct MatrixFarArgs {
 };
 size_t matrix_tree_setup(MatrixFarArgs* q, const qbx_geom* g, qbx_c64 k, qbx_c64 eta, int p, const double* hk_tab,
                          char* base);
-cudaError_t launch_matrix_far(const MatrixFarArgs& q, const double* sw, const double* P, cudaStream_t st);
+cudaError_t launch_matrix_far(const MatrixFarArgs& q, const double* sw, const double* P, int num_sms, cudaStream_t st);
 // nodes and coefficients only
 cudaError_t launch_tree_nodes(const TreeArgs& a, cudaStream_t st);
 // adjoint sweeps: the tree over the discs of the centres, evaluated at the

@@ -2116,7 +2116,8 @@ size_t matrix_tree_setup(MatrixFarArgs* q, const qbx_geom* g, qbx_c64 k, qbx_c64
 }
 
 template <typename T>
-static cudaError_t launch_matrix_far_t(const MatrixFarArgs& q, const double* sw, const double* P, cudaStream_t st) {
+static cudaError_t launch_matrix_far_t(const MatrixFarArgs& q, const double* sw, const double* P, int num_sms,
+                                       cudaStream_t st) {
   const TreeArgs& a = q.t;
   const int n = a.n_src * a.nrhs;
   k_matrix_density<<<(n + 255) / 256, 256, 0, st>>>(a.n_src, a.q_src, a.nrhs, sw, P, (cplx*)a.wd[0]);
@@ -2127,12 +2128,12 @@ static cudaError_t launch_matrix_far_t(const MatrixFarArgs& q, const double* sw,
   if (e != cudaSuccess) return e;
   k_tree_moments<T><<<dim3(a.M, 1, 1), 128, sm, st>>>(a);
   // one CTA (8 warps) per SM
-  const unsigned ns = (unsigned)std::max(1, std::min((152 + a.n_blk - 1) / a.n_blk, (a.M + kLocWarps - 1) / kLocWarps));
+  const unsigned ns = (unsigned)std::max(1, std::min((num_sms + a.n_blk - 1) / a.n_blk, (a.M + kLocWarps - 1) / kLocWarps));
   k_tree_matrix<T><<<dim3(a.n_blk, ns), 32 * kLocWarps, sizeof(MatrixSmem), st>>>(q);
   return cudaGetLastError();
 }
-cudaError_t launch_matrix_far(const MatrixFarArgs& q, const double* sw, const double* P, cudaStream_t st) {
-  return q.t.kim != 0.0 ? launch_matrix_far_t<cplx>(q, sw, P, st) : launch_matrix_far_t<double>(q, sw, P, st);
+cudaError_t launch_matrix_far(const MatrixFarArgs& q, const double* sw, const double* P, int num_sms, cudaStream_t st) {
+  return q.t.kim != 0.0 ? launch_matrix_far_t<cplx>(q, sw, P, num_sms, st) : launch_matrix_far_t<double>(q, sw, P, num_sms, st);
 }
 
 cudaError_t launch_far_clusters(TreeArgs a, cudaStream_t st) {
