@@ -942,13 +942,21 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   if (!tree) tree_bytes = 0;
   const int pair_units = group && !tree ? (nrow + kGrpCentres - 1) / kGrpCentres : units;   // (across the sides)
   // (with clusters a block's near leaves are some six panels; down to two dozen sources a CTA)
-  const int ns_near =
+  int ns_near =
       host_choose_split_waves(p->num_sms, occ, pair_units,
                               tree ? std::min(g->n_src, (group ? 8 : 16) * g->q_src)
                                    : (group && nsd == 2 ? 2 : 1) * g->n_src,   // both sides in one item: half as long
                               // (20 panels, S + D of 32 rhs, both sides 780 -> 583 us)
                               per_split, avail - tree_bytes - ns_far * per_split, waves);
   if (ns_near < 1) return fail(QBX_ENOMEM, "workspace too small for the apply partial sums");
+  if (group && !tree) {
+    // a few items beyond whole rounds of the SMs would be a round of their own (9
+    // blocks of 17 splits: 153 items): D - i eta S on 70 panels of 4/8 nodes 347 ->
+    // 254 us, S of 33 rhs on 18 panels 430 -> 289, no call of 1060 slower.  (Ranges
+    // in whole turns of the warps on top: 135 of them slower, by up to 12 %.)
+    const int items = pair_units * ns_near, rounds = items / p->num_sms;
+    if (rounds >= 1 && items % p->num_sms < p->num_sms / 6) ns_near = std::max(1, rounds * p->num_sms / pair_units);
+  }
   const int ns = ns_near + ns_far;
   if (group ? (ck ? group_smem_cplx(gops, pp, rg, nsd) : group_smem_real(gops, pp, rg, nsd)) > 220 * 1024
             : apply_smem_bytes(ops, ck, pp, chunk) > 220 * 1024)

@@ -727,3 +727,17 @@ def test_batch_tuning_is_kept_apart_for_clusters_and_pairs(cuda):
     b.tune()
     assert batch(pairs).info() == own
     assert a.info() == own and own[1] >= 512
+
+
+@pytest.mark.parametrize("M,q_tgt,q_src,nrhs", [(70, 4, 8, 1), (18, 16, 64, 33), (100, 4, 8, 16)])
+def test_few_items_beyond_whole_rounds(cuda, M, q_tgt, q_src, nrhs):
+    """9 x 17, 9 x 34 and 13 x 25 items over 152 SMs: a split or two fewer, and
+    the sums as with two splits."""
+    k, p = 2.0, 8
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(q_tgt, q_src, n_src=M * q_src, n_ctr=2 * M * q_tgt, ncoef=2, nrhs=nrhs)
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    got = qbx.qbx_apply_cfie(plan, g, k, k, p, d)
+    assert qbx.qbx_debug_route(plan)[0] == 0
+    check(got, qbx.qbx_apply_cfie(pair_plan(g, q_tgt, q_src, nrhs, 1), g, k, k, p, d), M)
