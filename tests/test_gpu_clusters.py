@@ -741,3 +741,47 @@ def test_few_items_beyond_whole_rounds(cuda, M, q_tgt, q_src, nrhs):
     got = qbx.qbx_apply_cfie(plan, g, k, k, p, d)
     assert qbx.qbx_debug_route(plan)[0] == 0
     check(got, qbx.qbx_apply_cfie(pair_plan(g, q_tgt, q_src, nrhs, 1), g, k, k, p, d), M)
+
+
+MANY = [
+    # M, q_tgt, q_src, k, p, ops, side, limit, nrhs, eta, (carried upward, super-blocks)
+    (32, 16, 64, 5.0, 8, (0,), "int", 0, 16, None, (0, 0)),            # smallest
+    (75, 12, 40, 9.0, 10, (1,), "ext", 1, 17, None, (0, 0)),           # blocks across panels, a ragged column group
+    (75, 7, 33, 7.0, 6, (0, 1), "two", 0, 33, None, (0, 0)),           # whole-panel leaves, 66 columns: two passes
+    (131, 7, 33, 7.0, 6, (0, 1), "two", 0, 33, None, (1, 1)),
+    (63, 16, 64, 9.0, 10, (0, 1), "two", 0, 33, None, (1, 0)),         # upward, a leaf short of super-blocks
+    (64, 16, 64, 9.0, 10, (0, 1), "two", 0, 33, None, (1, 1)),         # fewest leaves with them
+    (62, 16, 64, 9.0, 10, (0, 1), "two", 0, 33, None, (0, 0)),         # 8184 leaf columns
+    (64, 16, 64, 6.0, 40, (0, 1), "int", 1, 33, None, (1, 1)),         # highest order
+    (64, 16, 64, 6.0, 0, (0, 1), "two", 0, 33, None, (1, 1)),          # lowest
+    (128, 16, 64, 9.0, 9, (0,), "int", 0, 16, None, (0, 1)),           # super-blocks by blocks, not upward
+    (128, 16, 64, 9 + 0.5j, 9, (0,), "int", 0, 16, None, (0, 0)),      # (complex k: from 128 blocks on)
+    (128, 16, 64, 1e-3, 8, (0,), "two", 0, 33, None, (1, 1)),          # Laplace-like
+    (200, 5, 21, 7.0, 6, (1,), "ext", 1, 48, None, (1, 1)),            # several panels per block
+    (96, 16, 64, 12.0, 10, (0, 1), "two", 0, 48, 6.0, (1, 1)),         # near-only
+    (130, 16, 64, 3 + 3j, 10, "cfie", "two", 0, 40, None, (1, 1)),
+    (131, 16, 64, 30.0, 12, "cfie", "two", 0, 65, None, (1, 1)),
+]
+
+
+@pytest.mark.parametrize("case", MANY)
+def test_many_columns_by_route(cuda, case):
+    """Sums at every level and moments carried upward, with and without
+    super-blocks: the route that each size stands for, and the pairs' result."""
+    M, qt, qs, k, p, ops, side, limit, nrhs, eta, (up, sup) = case
+    side = {"int": qbx.SIDE_INT, "ext": qbx.SIDE_EXT, "two": qbx.SIDE_TWO}[side]
+    cur = W.starfish(0.2, 3)
+    plan = qbx.Plan(qt, qs, n_src=M * qs, n_ctr=2 * M * qt, ncoef=4, nrhs=nrhs)
+    g = geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M + p, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    pp = pair_plan(g, qt, qs, nrhs, 1 if ops == "cfie" else len(ops))
+    run = lambda pl: ([qbx.qbx_apply_cfie(pl, g, k, k - 0.5j, p, d)] if ops == "cfie" else
+                      list(qbx.qbx_apply_ops(pl, g, ops, side, limit, k, p, d, eta=eta).values()))
+    got = run(plan)
+    qbx.qbx_sync_status(plan)
+    r = qbx.qbx_debug_route(plan)
+    assert r[:2] == (1, up) and (r[2] > 0) == bool(sup)
+    ref = run(pp)
+    assert qbx.qbx_debug_route(pp)[0] == 0
+    for i, (a, b) in enumerate(zip(got, ref)):
+        check(a, b, (case, i))
