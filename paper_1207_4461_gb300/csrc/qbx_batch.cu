@@ -159,13 +159,17 @@ int block_sources(const GroupInst& in) {
 // Work items of a configuration: 32 rows of one curve (with a near list: of one
 // side, otherwise across the sides: both sides of 400 centres are 25 blocks, not
 // 26) x a range of at most `chunk` of its sources (equal ranges per curve),
-// longest first.
-std::vector<GroupItem> make_items(const std::vector<GroupInst>& inst, int chunk, std::vector<int>& nsplit) {
+// longest first.  Both sides of a target in one item take twice as long per
+// source: a curve without a near list has twice the ranges then (one curve of
+// 16 panels, S, both sides, 32 rhs: 1460 us; with the ranges of one side 2289;
+// with one side per item 1442).
+std::vector<GroupItem> make_items(const std::vector<GroupInst>& inst, int nsd, int chunk, std::vector<int>& nsplit) {
   std::vector<GroupItem> items;
   nsplit.assign(inst.size(), 1);
   for (size_t i = 0; i < inst.size(); ++i) {
     const int n = block_sources(inst[i]);
     int ns = std::max(1, (n + chunk - 1) / chunk);
+    if (nsd == 2 && !inst[i].near) ns = std::min(2 * ns, std::max(1, n / 16));
     const int len = (n + ns - 1) / ns;
     ns = (n + len - 1) / len;   // every range non-empty
     nsplit[i] = ns;
@@ -206,11 +210,11 @@ double lpt_makespan(const std::vector<GroupItem>& items, int slots) {
   return *std::max_element(heap.begin(), heap.end());
 }
 
-// smallest source range of an item (with clusters a block has few hundred
-// sources in all; both sides of a target in one item take twice as long per
-// source: one curve of 16 panels, S, both sides, 32 rhs 2289 us with 512,
-// 1460 with one side per item)
-int min_chunk(const qbx_batch* b) { return b->tree ? 64 : 512 / b->nsd; }
+// smallest source range of an item (with clusters a block has few hundred sources in all)
+int min_chunk(const qbx_batch* b) { return b->tree ? 64 : 512; }
+
+// sources of an item that has the range `chunk` (make_items)
+int item_sources(const qbx_batch* b, int chunk) { return b->nsd == 2 && !b->tree ? (chunk + 1) / 2 : chunk; }
 
 // The source chunk the model prefers: the smallest predicted makespan over
 // chunks 2^j * 32 (and all sources), ties to the larger chunk (fewer
@@ -223,7 +227,7 @@ int model_chunk(const qbx_batch* b, int slots, size_t budget) {
   double bt = 1e300;
   std::vector<int> ns;
   for (int c : cand) {
-    std::vector<GroupItem> items = make_items(b->h_inst, c, ns);
+    std::vector<GroupItem> items = make_items(b->h_inst, b->nsd, c, ns);
     if (part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs) > budget) break;
     const double t = lpt_makespan(items, slots);
     if (t < bt * 0.995) {
@@ -240,7 +244,7 @@ int configure(qbx_batch* b, int rg, int chunk) {
   cudaError_t e = cudaSetDevice(b->device);
   if (e != cudaSuccess) return bcuda(e, "device");
   std::vector<int> ns;
-  std::vector<GroupItem> items = make_items(b->h_inst, chunk, ns);
+  std::vector<GroupItem> items = make_items(b->h_inst, b->nsd, chunk, ns);
   const size_t pb = part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs);
   if (pb > b->part_cap) {
     cudaFree(b->d_part);
@@ -368,7 +372,7 @@ int prepare_tree(qbx_batch* b, size_t budget) {
   for (const GroupInst& in : b->h_inst) pairs += (double)in.n_ctr * in.n_src;
   const bool many = b->nrhs > 16, half_leaves = b->q_src % 2 == 0 && b->q_src >= 32;
   const double leaf = std::max(1.0, 20.0 / (half_leaves ? b->q_src / 2 : b->q_src));
-  if (pairs < leaf * (b->eta2 > 0.0 ? (b->side == QBX_SIDE_TWO ? 3.2e6 : many ? 3.6e6 : 1.8e6) : many ? 2.3e6 : 1.0e6))
+  if (pairs < leaf * (b->eta2 > 0.0 ? (b->side == QBX_SIDE_TWO ? 3.2e6 : many ? 3.6e6 : 2.0e6) : many ? 2.3e6 : 1.0e6))
     return QBX_OK;
   const int none[3] = {0, 0, 0};
   std::vector<TreeArgs> v(b->n_inst);
@@ -603,7 +607,7 @@ int qbx_batch_create(qbx_batch** batch, qbx_plan* plan, int n_inst, const qbx_ge
   }
   if (chunk > 0) {   // a cached choice, if its partial sums fit
     std::vector<int> ns;
-    make_items(b->h_inst, chunk, ns);
+    make_items(b->h_inst, b->nsd, chunk, ns);
     if (part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs) > part_budget(b->device)) chunk = 0;
   }
   if (chunk == 0) {
@@ -644,7 +648,7 @@ int qbx_batch_tune(qbx_batch* b, void* stream, int* rg_out, int* chunk_out) {
   for (int rg : rgs) {
     for (int c : chunks) {
       std::vector<int> ns;
-      make_items(b->h_inst, c, ns);
+      make_items(b->h_inst, b->nsd, c, ns);
       if (part_bytes(b->h_inst, ns, b->ns_far, b->ncomp, b->nrhs) > budget) continue;
       if ((rc = configure(b, rg, c))) break;
       // one untimed launch, then one timed
@@ -676,7 +680,7 @@ int qbx_batch_tune(qbx_batch* b, void* stream, int* rg_out, int* chunk_out) {
     g_tune_cache[tune_key(b)] = std::make_pair(best_rg, best_chunk);
   }
   if (rg_out) *rg_out = best_rg;
-  if (chunk_out) *chunk_out = best_chunk;
+  if (chunk_out) *chunk_out = item_sources(b, best_chunk);
   return QBX_OK;
 }
 
@@ -694,7 +698,7 @@ int qbx_batch_set_eta(qbx_batch* b, double eta) {
 int qbx_batch_info(const qbx_batch* b, int* rg, int* chunk, int* n_items, int* grid) {
   if (!b) return bfail(QBX_EINVAL, "batch is NULL");
   if (rg) *rg = b->rg;
-  if (chunk) *chunk = b->chunk;
+  if (chunk) *chunk = item_sources(b, b->chunk);
   if (n_items) *n_items = b->n_items;
   if (grid) *grid = b->grid;
   return QBX_OK;

@@ -893,7 +893,7 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
   else if (group && ops == 7)
     tree_pairs = (both ? 1.6 : 1.0) * (local ? 1.6 : 1.0) *
                  (2.3e6 + 0.21e6 * (nrhs <= 32 ? nrhs - 16 : std::min(std::max(0.6 * nrhs - 16.0, 4.0), 22.0)));
-  else if (group && local) tree_pairs = leaf * (both ? 3.2e6 : nrhs > 16 ? 3.6e6 : 1.8e6);
+  else if (group && local) tree_pairs = leaf * (both ? 3.2e6 : nrhs > 16 ? 3.6e6 : 2.0e6);
   else if (group) tree_pairs = leaf * (nrhs > 16 ? 2.3e6 : both ? 0.8e6 : 1.0e6);
   else if (ops == QBX_OPS_GRAD_S && nrhs > 3) tree_pairs = (both ? 1.6 : 1.0) * 0.45e6 * nrhs / ((nrhs + 7) / 8);
   if (g->M >= kTreeMinPanels && (double)nc * g->n_src >= tree_pairs) {

@@ -785,3 +785,22 @@ def test_many_columns_by_route(cuda, case):
     assert qbx.qbx_debug_route(pp)[0] == 0
     for i, (a, b) in enumerate(zip(got, ref)):
         check(a, b, (case, i))
+
+
+@pytest.mark.parametrize("M,q_tgt,q_src", [(16, 4, 8), (20, 16, 64), (100, 4, 8), (2, 5, 7)])
+def test_batch_items_of_both_sides_are_as_many_as_of_one_each(cuda, M, q_tgt, q_src):
+    """64, 320, 400 and 10 targets: as many items as both sides one by one have,
+    also where a side's sources are a single range."""
+    nrhs, k, p = 4, 2.0, 7
+    plan = qbx.Plan(q_tgt, q_src, n_src=M * q_src, n_ctr=2 * M * q_tgt, ncoef=2, nrhs=nrhs)
+    cur = W.starfish(0.2, 3)
+    g = qbx.qbx_geometry(plan, cur, cur.edges(M))
+    d = torch.as_tensor(W.complex_gaussian(M, g.n_tgt * nrhs).reshape(g.n_tgt, nrhs), device="cuda")
+    one, b = (qbx.Batch(plan, [g], [k], p, (0,), s, 0, [d]) for s in (qbx.SIDE_INT, qbx.SIDE_TWO))
+    assert one.debug_route() == b.debug_route() == 0
+    if g.n_src >= 32:
+        assert b.info()[2] >= 2 * one.info()[2]
+    out = b.apply()[0]
+    b.status()
+    ref = qbx.qbx_apply_ops(pair_plan(g, q_tgt, q_src, nrhs, 1), g, (0,), qbx.SIDE_TWO, 0, k, p, d)
+    check(out[0], ref[0], M)
