@@ -69,7 +69,7 @@ def flops_per_pair_ops(ops, p, nrhs=1):
 # of one S + D + grad S apply on the full-size starfish workload, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum); valid only for the kernel
 # sources it was taken with, identified by their hash.
-TRAFFIC = {"e7ce47d256b09565": 1.512e+07}   # profiles/apply_S_D_gradS_starfish_M256_clusters.md
+TRAFFIC = {"36031c1ffce96e4f": 1.513e+07}   # profiles/apply_S_D_gradS_starfish_M256_clusters.md
 KERNEL_SOURCES = ["qbx_apply_impl.cuh", "qbx_device.cuh", "special_tables.h", "qbx_apply_real.cu", "qbx_tree.cu",
                   "qbx_tree.cuh"]
 GROUP_SOURCES = ["qbx_group_impl.cuh", "qbx_apply_impl.cuh", "qbx_device.cuh", "special_tables.h"]
@@ -78,11 +78,11 @@ GROUP_SOURCES = ["qbx_group_impl.cuh", "qbx_apply_impl.cuh", "qbx_device.cuh", "
 # launches between oversampling and finishing of one apply, divided by its
 # nominal (centre, source) pairs: near leaves pair by pair, distant sources by
 # their clusters' moments.  For the kernel sources with the given hash.
-HW_FP64_PER_PAIR = {"e7ce47d256b09565": 17.02}         # S + D + grad S, p = 12, one rhs: the same profile
+HW_FP64_PER_PAIR = {"36031c1ffce96e4f": 17.02}         # S + D + grad S, p = 12, one rhs: the same profile
 HW_FP64_PER_PAIR_GROUP = {}   # batches: none taken with clusters
 # sm__pipe_fp64_cycles_active (of peak) over the active and the elapsed
 # cycles, from the same captures, weighted by the launches' times
-HW_FP64_PIPE = {"e7ce47d256b09565": (0.799, 0.723)}
+HW_FP64_PIPE = {"36031c1ffce96e4f": (0.798, 0.721)}
 HW_FP64_PIPE_GROUP = {}
 # the same at the complex wavenumber 20 + 1i: none taken with clusters
 HW_FP64_PER_PAIR_CPLX = {}

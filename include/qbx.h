@@ -113,11 +113,13 @@ int qbx_gauss_legendre(int q, double *nodes, double *weights);
 /* Create a plan on CUDA device `device` for the grid pair (q_tgt, q_src):
  * uploads the per-panel interpolation matrix from the target to the source
  * nodes (Sec. 3.4.2), a device status word, and allocates `workspace_bytes`
- * of device workspace used by the split-source reductions (see
- * qbx_workspace_bytes) and by the cluster arrays of calls on 16 panels or more
- * (with many right-hand sides 20 to 64): distant sources by their moments.
- * With a workspace that holds the partial sums but not these arrays the call
- * takes every pair instead, more slowly and to the same accuracy.  The plan
+ * of device workspace used by the split-source reductions and by the cluster
+ * arrays of calls that take distant sources by their moments: on 16 panels or
+ * more, and where centres times sources repay it (few right-hand sides: at
+ * once, points off the curve from 4e6; many: 0.8e6 to 14e6 by operators,
+ * columns, sides and sources per panel).  qbx_workspace_bytes has room for
+ * both; with a workspace that holds the partial sums but not these arrays the
+ * call takes every pair instead, more slowly and to the same accuracy.  The plan
  * also holds a side stream on which such a call's near pairs run beside the
  * rest (forked from and joined to the call's stream by events, also under
  * stream capture), and two 29 KB tables of H0/H1 amplitudes along the ray
@@ -400,8 +402,10 @@ int qbx_vec_combine(int n, int nrhs, int nv, const qbx_c64 *V, const qbx_c64 *y,
  * caller-owned device memory).  Row t holds, for both centres of target t,
  * the truncated Graf sums against every source node carried back to the
  * target grid by the per-panel interpolation.  q_tgt <= 16.  From 16 panels
- * on the distant panels' columns go through moments held in the plan's
- * workspace (too small a workspace: every pair).  Async on stream.  qbx_solve_exterior_dirichlet_assembled then runs the same GMRES
+ * on, and with q_src >= 2 q_tgt, the distant panels' columns go through moments
+ * held in the plan's workspace (qbx_workspace_bytes(n_src, 2 n_tgt, 1, q_tgt)
+ * holds them; too small a workspace: every pair).  Async on stream.
+ * qbx_solve_exterior_dirichlet_assembled then runs the same GMRES
  * with one complex matrix product (qbx_matmul_cm) per iteration for all
  * right-hand sides, one Arnoldi step captured as a CUDA graph and launched
  * up to `restart` times per cycle without a host wait (steps after
@@ -442,7 +446,10 @@ size_t qbx_matmul_cm_work_bytes(int n, int nrhs);
  * sums are added in a fixed order), taken longest first by persistent CTAs
  * through an atomic counter; no CTA ever waits for another.
  * Curves of 16 panels or more (S, D, S + D) take distant sources by their
- * clusters' moments; without device memory for those arrays, every pair.
+ * clusters' moments where the batch's centres times sources, over all curves,
+ * repay it (1e6; 2.3e6 for more than 16 right-hand sides; more near-only and
+ * for few sources per panel); without device memory for those arrays, every
+ * pair.  Both sides of a target may be one item, of half as many sources.
  * qbx_batch_create allocates the batch's device memory (with, for every
  * curve of complex k, the H0/H1 amplitude table of its ray z = k rho), picks
  * the chunk with the smallest predicted makespan of that schedule (a model

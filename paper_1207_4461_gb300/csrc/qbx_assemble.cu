@@ -15,7 +15,7 @@
 // and the panels m = 4 blockIdx.y + g (mod 4 gridDim.y) for warp g; the
 // matrix is stored column-major
 // (entry (t, t') at t' n + t), so a warp writes 32 consecutive rows of one
-// column at a time.  From 16 panels on (and where the workspace holds it) only
+// column at a time.  From 16 panels on (with q_src >= 2 q_tgt, and where the workspace holds it) only
 // the panels near a block of 32 targets go this way, the four warps of a CTA
 // sharing one panel's sources; the others by their moments (k_tree_matrix),
 // beside it on the plan's side stream.

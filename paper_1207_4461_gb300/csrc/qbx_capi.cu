@@ -34,7 +34,7 @@ struct qbx_plan {
   // k (tab_kim = 0: none made yet), then the one that captured calls fill
   double* d_hk_tab;
   double tab_kre, tab_kim;
-  // the pair sums run here, beside the cluster moments on the caller's stream
+  // the near pairs run here where the cluster moments run on the caller's stream
   // (forked from it and joined to it by events within every call)
   cudaStream_t side;
   cudaEvent_t fork, join;
@@ -1086,8 +1086,11 @@ static int apply_impl(qbx_plan* p, const qbx_geom* g, int ops, int side, int lim
     return e;
   };
   if (tree) {
-    // near pairs on the side stream, clusters on the caller's: the moments'
-    // and the far sums' short launches fill in where the pair kernel leaves room
+    // near pairs on the side stream, clusters on the caller's.  On a large curve
+    // the two barely overlap (256 panels, S + D + grad S: launches of 3.21 ms one
+    // after another, 3.17 ms in the call: the pair kernel's CTAs are queued first);
+    // on a small one the chain of short launches runs beside the pairs (32
+    // panels: 0.25 and 0.15 ms in a call of 0.34)
     CK(cudaEventRecord(p->fork, st), "fork event");
     CK(cudaStreamWaitEvent(p->side, p->fork, 0), "fork");
     const cudaError_t en = pair_sums(p->side);

@@ -26,8 +26,12 @@
 // local expansion (150k), most of these for several blocks at once
 // (k_tree_super).  The apply: 63.2 ms -> 3.2 ms; k = 20 + 1i at 128 panels
 // 26.9 -> 3.4 ms; S and D at 32 panels, p = 8: 751 -> 336 us.
-// The pair route stays for fewer than kTreeMinPanels panels (nothing is far)
-// and for workspaces without room for the arrays below.
+// The pair route stays for fewer than kTreeMinPanels panels (nothing is far),
+// for workspaces without room for the arrays below, and where the clusters'
+// chain of launches is not repaid: by pairs, columns, sources per leaf and
+// operators, with both sides measured, at the calls (qbx_capi.cu: applies of
+// many columns, stored coefficients, points off the curve; qbx_batch.cu,
+// qbx_adjoint.cu, qbx_shape.cu; matrix_tree_setup for the assembled matrix).
 #pragma once
 #include <cuda_runtime.h>
 #include "qbx_apply_impl.cuh"
